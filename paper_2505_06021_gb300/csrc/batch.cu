@@ -299,10 +299,11 @@ rpa_status batch_enqueue(rpa_ctx* ctx, SideStreams& bc, const Plan& p, const rpa
       CholTask* dp = reinterpret_cast<CholTask*>(ws + g.task_off);
       CKB(cudaMemcpyAsync(dp, hp, sizeof(CholTask) * (tc.size() + tr.size()), cudaMemcpyHostToDevice, s));
       prof_begin(ctx, pex, s);
-      CKB(launch_cholesky_ragged(1, dp, (int)tc.size(), s));
-      CKB(launch_cholesky_ragged(0, dp + tc.size(), (int)tr.size(), s));
-      prof_end(ctx, pex, s, RPA_K_LOGDET, (tc.empty() ? 0 : 1) + (tr.empty() ? 0 : 1));
-      ctx->launches += (tc.empty() ? 0 : 1) + (tr.empty() ? 0 : 1);
+      int lc = 0, lr = 0;
+      CKB(launch_cholesky_ragged(1, dp, tc.data(), (int)tc.size(), s, &lc));
+      CKB(launch_cholesky_ragged(0, dp + tc.size(), tr.data(), (int)tr.size(), s, &lr));
+      prof_end(ctx, pex, s, RPA_K_LOGDET, lc + lr);
+      ctx->launches += lc + lr;
       for (int i = g.j0; i < g.j1; ++i)
         if (jobs[i].prec == RPA_PREC_MIXED)
           if (rpa_status st = finish_job(i, s)) return st;

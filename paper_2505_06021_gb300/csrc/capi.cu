@@ -509,14 +509,14 @@ static rpa_status vside_factor(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
   prof_begin(ctx, pex, s);
   CK(launch_cholesky(j->is_complex, j->n_aux, nq, b.L, mstride, 1, b.Vc ? b.ldV + q0 : nullptr, b.status,
                      (1 << 29) + q0, s));
-  prof_end(ctx, pex, s, RPA_K_VFACTOR, cholesky_launches(j->n_aux, nq));
-  ctx->launches += cholesky_launches(j->n_aux, nq);
+  prof_end(ctx, pex, s, RPA_K_VFACTOR, cholesky_launches(j->n_aux, nq, 1));
+  ctx->launches += cholesky_launches(j->n_aux, nq, 1);
   if (b.Vc) {
     // inverse form: -V^-1 per q (X = L^-1 in T's storage, then -(X^H X) over L)
     prof_begin(ctx, pex, s);
     CK(launch_vinv(j->is_complex, j->n_aux, nq, b.L, b.T, b.L, s));
-    prof_end(ctx, pex, s, RPA_K_VFACTOR, 2);
-    ctx->launches += 2;
+    prof_end(ctx, pex, s, RPA_K_VFACTOR, trinv_launches(j->n_aux) + 1);
+    ctx->launches += trinv_launches(j->n_aux) + 1;
   }
   return RPA_OK;
 }
@@ -539,8 +539,8 @@ static rpa_status stage_logdet(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
     prof_begin(ctx, pex, s);
     CK(launch_cholesky(j->is_complex, j->n_aux, nq * j->n_w, b.chi, mstride, 2, b.parts + (size_t)2 * q0 * j->n_w,
                        b.status, q0 * j->n_w, s, b.L, b.Vc, b.ldV + q0, j->n_w));
-    prof_end(ctx, pex, s, RPA_K_LOGDET, cholesky_launches(j->n_aux, nq * j->n_w));
-    ctx->launches += cholesky_launches(j->n_aux, nq * j->n_w);
+    prof_end(ctx, pex, s, RPA_K_LOGDET, cholesky_launches(j->n_aux, nq * j->n_w, 2));
+    ctx->launches += cholesky_launches(j->n_aux, nq * j->n_w, 2);
     return RPA_OK;
   }
   // Y = -(L^H chi L) (lower triangle), overwriting chi's storage
@@ -552,8 +552,8 @@ static rpa_status stage_logdet(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
   prof_begin(ctx, pex, s);
   CK(launch_cholesky(j->is_complex, j->n_aux, nq * j->n_w, b.chi, mstride, 0, b.parts + (size_t)2 * q0 * j->n_w,
                      b.status, q0 * j->n_w, s));
-  prof_end(ctx, pex, s, RPA_K_LOGDET, cholesky_launches(j->n_aux, nq * j->n_w));
-  ctx->launches += cholesky_launches(j->n_aux, nq * j->n_w);
+  prof_end(ctx, pex, s, RPA_K_LOGDET, cholesky_launches(j->n_aux, nq * j->n_w, 0));
+  ctx->launches += cholesky_launches(j->n_aux, nq * j->n_w, 0);
   return RPA_OK;
 }
 
@@ -1079,15 +1079,16 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   prof_begin(ctx, &ex, s);
   CK(launch_cholesky(job->is_complex, job->n_aux, 1, b.L, (long)(NN * (es / 8)), 1, nullptr, b.status,
                      (1 << 29) + q, s));
-  prof_end(ctx, &ex, s, RPA_K_VFACTOR, 1);
+  const int nv = cholesky_launches(job->n_aux, 1, 1), nd = cholesky_launches(job->n_aux, job->n_w, 0);
+  prof_end(ctx, &ex, s, RPA_K_VFACTOR, nv);
   prof_begin(ctx, &ex, s);
   CK(launch_sandwich(job->is_complex, job->n_aux, job->n_w, job->n_w, (const double*)chi, b.L, b.T, b.chi, s));
   prof_end(ctx, &ex, s, RPA_K_SANDWICH, 2);
   prof_begin(ctx, &ex, s);
   CK(launch_cholesky(job->is_complex, job->n_aux, job->n_w, b.chi, (long)(NN * (es / 8)), 0, b.parts, b.status, 0,
                      s));
-  prof_end(ctx, &ex, s, RPA_K_LOGDET, 1);
-  ctx->launches += 4;
+  prof_end(ctx, &ex, s, RPA_K_LOGDET, nd);
+  ctx->launches += nv + 2 + nd;
   if (!ex.hres.reserve(64 + sizeof(double) * 2 * job->n_w)) return RPA_E_NOMEM;
   CK(cudaMemcpyAsync(ex.results(), b.parts, sizeof(double) * 2 * job->n_w, cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&ex.status_word(), b.status, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -56,9 +56,8 @@ cudaError_t launch_cholesky(int cplx, int N, int n_mat, double* mats, long bstri
                             int* status, int status_base, cudaStream_t s, const double* Wn = nullptr,
                             const double* Vc = nullptr, const double* ldV = nullptr, int n_w = 0);
 
-// Kernel launches launch_cholesky makes for n_mat matrices of size N (1, or 2
-// when a short last wave goes to clusters).
-int cholesky_launches(int N, int n_mat);
+// Kernel launches launch_cholesky makes for n_mat matrices of size N.
+int cholesky_launches(int N, int n_mat, int mode);
 
 // One matrix of a ragged Cholesky launch (matrices of different sizes).
 struct CholTask {
@@ -70,11 +69,18 @@ struct CholTask {
   int* status;        // set to `code` on a non-positive pivot (if still 0)
   int N, mode, code, pad;
 };
-// Tasks in device memory, one CTA each; `cplx` selects complex128 or float64.
-cudaError_t launch_cholesky_ragged(int cplx, const CholTask* tasks, int n_tasks, cudaStream_t s);
+// Tasks in device memory, all of one mode and sorted by N, largest first;
+// `host` is the same table in host memory (the launches are shaped from it
+// before the call returns).  `cplx` selects complex128 or float64.
+cudaError_t launch_cholesky_ragged(int cplx, const CholTask* tasks, const CholTask* host, int n_tasks, cudaStream_t s,
+                                   int* n_launch);
 
+// X[q] = L[q]^-1 (lower triangular, strict upper triangle zero) and the
+// launches it takes.
+cudaError_t launch_trinv(int cplx, int N, int n_q, const double* L, double* X, cudaStream_t s);
+int trinv_launches(int N);
 // Wn[q] = -V(q)^-1 (lower triangle) from the Cholesky factors L[q]: X = L^-1
-// by block forward substitution into X[q], then -(X^H X).
+// into X[q], then -(X^H X).
 cudaError_t launch_vinv(int cplx, int N, int n_q, const double* L, double* X, double* Wn, cudaStream_t s);
 
 // ---- AO -> MO transform (kernels_ao.cu) -----------------------------------
