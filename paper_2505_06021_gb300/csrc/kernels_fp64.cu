@@ -63,16 +63,17 @@ __global__ void dtab_kernel(BatchGeom g, const double* __restrict__ eps_occ, con
 
 // --------------------------------------------------------------- chi0 -----
 // Grid: one CTA per (q in batch, lower tile pair (I, J), frequency group).
-// Tile 32 x 32 outputs, 256 threads, each thread a 2 x 2 block of outputs
-// (rows ty, ty+16; columns tx, tx+16) for G frequencies.
+// Tile 16 U x 16 U outputs, 256 threads, each thread U x U outputs (rows
+// ty + 16 u, columns tx + 16 v) for G frequencies.  An output's sum does not
+// depend on U or G.
 
-constexpr int CT = 32;  // output tile edge
 constexpr int TK = 16;  // t-chunk
 
-template <bool C, int G>
+template <bool C, int G, int U>
 __global__ void __launch_bounds__(256, 1)
     chi0_fp64_kernel(BatchGeom g, const double* const* __restrict__ Cptrs, const double* __restrict__ dtab,
                      double* __restrict__ chi, int n_tiles, int n_wg) {
+  constexpr int CT = 16 * U;  // output tile edge
   __shared__ Elem<C> As[TK][CT];
   __shared__ Elem<C> Bs[TK][CT];
   __shared__ double Ds[G][TK];
@@ -88,11 +89,11 @@ __global__ void __launch_bounds__(256, 1)
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int N = g.n_aux, n_ov = g.n_ov;
 
-  Elem<C> acc[G][4];
+  Elem<C> acc[G][U * U];
 #pragma unroll
   for (int k = 0; k < G; ++k)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) acc[k][m] = zero_elem<C>();
+    for (int m = 0; m < U * U; ++m) acc[k][m] = zero_elem<C>();
 
   for (int j = 0; j < g.n_k; ++j) {
     const double* Cj = Cptrs[qb * g.n_k + j];
@@ -111,27 +112,29 @@ __global__ void __launch_bounds__(256, 1)
       __syncthreads();
 #pragma unroll 4
       for (int tt = 0; tt < TK; ++tt) {
-        const Elem<C> a0 = As[tt][ty], a1 = As[tt][ty + 16];
-        const Elem<C> b0 = Bs[tt][tx], b1 = Bs[tt][tx + 16];
         // p = conj(a) * b
-        Elem<C> p[4];
-        const Elem<C> aa[2] = {a0, a1}, bb[2] = {b0, b1};
+        Elem<C> p[U * U], aa[U], bb[U];
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+        for (int u = 0; u < U; ++u) {
+          aa[u] = As[tt][ty + 16 * u];
+          bb[u] = Bs[tt][tx + 16 * u];
+        }
 #pragma unroll
-          for (int v = 0; v < 2; ++v) {
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int v = 0; v < U; ++v) {
             if constexpr (C) {
-              p[2 * u + v].re = fma(aa[u].re, bb[v].re, aa[u].im * bb[v].im);
-              p[2 * u + v].im = fma(aa[u].re, bb[v].im, -aa[u].im * bb[v].re);
+              p[U * u + v].re = fma(aa[u].re, bb[v].re, aa[u].im * bb[v].im);
+              p[U * u + v].im = fma(aa[u].re, bb[v].im, -aa[u].im * bb[v].re);
             } else {
-              p[2 * u + v].re = aa[u].re * bb[v].re;
+              p[U * u + v].re = aa[u].re * bb[v].re;
             }
           }
 #pragma unroll
         for (int k = 0; k < G; ++k) {
           const double d = Ds[k][tt];
 #pragma unroll
-          for (int m = 0; m < 4; ++m) {
+          for (int m = 0; m < U * U; ++m) {
             acc[k][m].re = fma(d, p[m].re, acc[k][m].re);
             if constexpr (C) acc[k][m].im = fma(d, p[m].im, acc[k][m].im);
           }
@@ -148,12 +151,12 @@ __global__ void __launch_bounds__(256, 1)
     if (w >= g.n_w) break;
     double* out = chi + ((long)qb * g.n_w + w) * NN * (C ? 2 : 1);
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int v = 0; v < 2; ++v) {
+      for (int v = 0; v < U; ++v) {
         const int P = I * CT + ty + 16 * u, Q = J * CT + tx + 16 * v;
         if (P >= N || Q >= N || Q > P) continue;
-        Elem<C> e = acc[k][2 * u + v];
+        Elem<C> e = acc[k][U * u + v];
         if (P == Q) {
           if constexpr (C) e.im = 0.0;
           st_elem<C>(out, (long)P * N + Q, e);
@@ -165,48 +168,62 @@ __global__ void __launch_bounds__(256, 1)
   }
 }
 
-template <bool C, int G>
+template <bool C, int G, int U>
 cudaError_t chi0_launch_g(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
                           cudaStream_t s) {
-  const int nt = (g.n_aux + CT - 1) / CT;
+  const int nt = (g.n_aux + 16 * U - 1) / (16 * U);
   const int n_tiles = nt * (nt + 1) / 2;
   const int n_wg = (g.n_w + G - 1) / G;
   const long blocks = (long)n_tiles * n_wg * g.n_qb;
   if (blocks > 0x7fffffffL) return cudaErrorInvalidConfiguration;
-  chi0_fp64_kernel<C, G><<<(unsigned)blocks, 256, 0, s>>>(g, Cptrs, dtab, chi, n_tiles, n_wg);
+  chi0_fp64_kernel<C, G, U><<<(unsigned)blocks, 256, 0, s>>>(g, Cptrs, dtab, chi, n_tiles, n_wg);
   return cudaGetLastError();
 }
 
-// Frequency group size: minimises FP64 instructions per (P, Q, t),
-// 4 * ceil(n_w / G) (products, complex) + 2 * G * ceil(n_w / G) (weights).
-int pick_group(int n_w) {
-  const int cand[4] = {4, 5, 8, 10};
-  int best = 8;
-  long best_cost = -1;
-  for (int c : cand) {
-    const long ng = (n_w + c - 1) / c;
-    const long cost = 4 * ng + 2 * (long)c * ng;
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = c;
-    }
-  }
-  return best;
-}
-
+// Tile edge and frequency group.  A CTA issues (4 + 2 G) FP64 instructions
+// per complex (P, Q, t) (1 + G real) for G frequencies, and its SM's FP64
+// pipe serves all CTAs that sit there, so the choice minimises the number of
+// CTAs the fullest SM gets times a CTA's work: large groups share the product
+// conj(C_P) C_Q when there is work for every SM, small tiles and groups spread
+// a small response (a 32 x 32 tile of 8 frequencies holds the pipe for 4.6k
+// clocks per 1000 real t).  Measured at N_aux 64, 112 t, 16 frequencies, real:
+// 272 us with 32 x 32 tiles of 8 frequencies (6 CTAs), see the table in the
+// design notes for the present time.
 template <bool C>
 cudaError_t chi0_dispatch(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
                           cudaStream_t s) {
-  switch (pick_group(g.n_w)) {
-    case 4:
-      return chi0_launch_g<C, 4>(g, Cptrs, dtab, chi, s);
-    case 5:
-      return chi0_launch_g<C, 5>(g, Cptrs, dtab, chi, s);
-    case 10:
-      return chi0_launch_g<C, 10>(g, Cptrs, dtab, chi, s);
+  const int Gs[6] = {10, 8, 5, 4, 2, 1};
+  const long sms = num_sms_fp64();
+  int bG = 8, bU = 2;
+  double best = 1e300;
+  for (int U = 2; U >= 1; --U)
+    for (int G : Gs) {
+      const long nt = (g.n_aux + 16 * U - 1) / (16 * U);
+      const long blocks = nt * (nt + 1) / 2 * ((g.n_w + G - 1) / G) * g.n_qb;
+      const double work = (C ? 4.0 + 2.0 * G : 1.0 + G) * U * U;
+      // the last wave counts as a whole one while there are few
+      const double waves = blocks >= 16 * sms ? (double)blocks / sms : (double)((blocks + sms - 1) / sms);
+      const double cost = waves * work * (U == 1 ? 1.05 : 1.0);  // smaller tiles read the operands more often
+      if (cost < best) {
+        best = cost;
+        bG = G;
+        bU = U;
+      }
+    }
+#define RPA_CHI0_G(G)                                                   \
+  case G:                                                               \
+    return bU == 2 ? chi0_launch_g<C, G, 2>(g, Cptrs, dtab, chi, s)     \
+                   : chi0_launch_g<C, G, 1>(g, Cptrs, dtab, chi, s)
+  switch (bG) {
+    RPA_CHI0_G(10);
+    RPA_CHI0_G(5);
+    RPA_CHI0_G(4);
+    RPA_CHI0_G(2);
+    RPA_CHI0_G(1);
     default:
-      return chi0_launch_g<C, 8>(g, Cptrs, dtab, chi, s);
+      return bU == 2 ? chi0_launch_g<C, 8, 2>(g, Cptrs, dtab, chi, s) : chi0_launch_g<C, 8, 1>(g, Cptrs, dtab, chi, s);
   }
+#undef RPA_CHI0_G
 }
 
 // ----------------------------------------------------------- sandwich -----
