@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "batch_internal.h"
+#include "g64.h"
 #include "rpa_internal.h"
 #include "rpa_runtime.h"
 
@@ -72,7 +73,7 @@ std::vector<uint64_t> signature(const rpa_job* jobs, int n, int n_slices) {
 
 }  // namespace
 
-std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget) {
+std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget, bool g64) {
   std::unique_ptr<Plan> p(new Plan);
   p->jobs.resize(n);
   size_t pin = 0;
@@ -80,6 +81,12 @@ std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_
     JobPlan& jp = p->jobs[i];
     jp.L = plan_layout(&jobs[i], jobs[i].n_q, n_slices, 0, false);
     jp.mixed = 0;
+    jp.g64 = 0;
+    if (g64 && jobs[i].prec == RPA_PREC_FP64) {
+      BatchGeom ga = geom_q(jobs[i]);
+      ga.n_qb = jobs[i].n_q;
+      if (chi0_g64_use(ga) && a1k(jp.L.total) + chi0_g64_bytes(ga) + 2048 <= budget) jp.g64 = a1k(chi0_g64_bytes(ga));
+    }
     if (jobs[i].prec == RPA_PREC_MIXED) {
       const size_t per_q = a1k(mixed_workspace_bytes(geom_q(jobs[i]), n_slices, kBatchSliceCap));
       jp.mixed = per_q * (size_t)jobs[i].n_q;
@@ -95,21 +102,22 @@ std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_
   int i = 0;
   while (i < n) {
     Group g{i, i, 0, 0, 0, 0, 0, 0, 0};
-    size_t fp = 0, mx = 0;
+    size_t fp = 0, mx = 0, mg = 0;  // mg: the FP64 jobs' chi0 run one after another before the mixed ones'
     while (g.j1 < n) {
       const JobPlan& jp = p->jobs[g.j1];
-      const size_t f2 = fp + a1k(jp.L.total), m2 = mx + jp.mixed;
-      if (g.j1 > g.j0 && f2 + m2 + 1024 > budget) break;
+      const size_t f2 = fp + a1k(jp.L.total), m2 = mx + jp.mixed, g2 = std::max(mg, jp.g64);
+      if (g.j1 > g.j0 && f2 + std::max(m2, g2) + 1024 > budget) break;
       p->jobs[g.j1].ws_off = fp;
       fp = f2;
       mx = m2;
+      mg = g2;
       ++g.j1;
     }
     for (int k = g.j0; k < g.j1; ++k)
       if (jobs[k].prec == RPA_PREC_MIXED) (jobs[k].is_complex ? g.n_task_c : g.n_task_r) += jobs[k].n_q * jobs[k].n_w;
     const size_t tbytes = a1k(sizeof(CholTask) * (size_t)(g.n_task_c + g.n_task_r));
     g.mixed_off = fp;
-    g.mixed_bytes = mx ? mx + 1024 : 0;
+    g.mixed_bytes = std::max(mx ? mx + 1024 : 0, mg);
     g.task_off = fp + g.mixed_bytes;
     g.pin_task = pin;
     pin += tbytes;
@@ -219,10 +227,15 @@ rpa_status batch_enqueue(rpa_ctx* ctx, SideStreams& bc, const Plan& p, const rpa
       } else {
         BatchGeom ga = g1;
         ga.n_qb = j.n_q;
+        uint64_t nl = 1;
         prof_begin(ctx, pex, s);
-        CKB(launch_chi0_fp64(ga, (const double* const*)B[i].Cptrs, B[i].dtab, B[i].chi, s));
-        prof_end(ctx, pex, s, RPA_K_CHI0, 1);
-        ctx->launches++;
+        if (p.jobs[i].g64)
+          CKB(launch_chi0_g64(ga, (const double* const*)B[i].Cptrs, B[i].dtab, B[i].chi, ws + g.mixed_off, g.mixed_bytes,
+                              B[i].status, &nl, s));
+        else
+          CKB(launch_chi0_fp64(ga, (const double* const*)B[i].Cptrs, B[i].dtab, B[i].chi, s));
+        prof_end(ctx, pex, s, RPA_K_CHI0, (int)nl);
+        ctx->launches += nl;
       }
     }
     if (!mq.empty()) {
@@ -355,7 +368,7 @@ extern "C" rpa_status rpa_energy_batch(rpa_ctx* ctx, const rpa_job* jobs, int n_
   const bool known = bc.plan && bc.plan->exec && bc.plan->sig == sig;
   const bool replay = known && !ctx->prof;
   if (!known) {
-    bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap);
+    bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap, true);
     bc.plan->sig = sig;
   }
   Plan& p = *bc.plan;

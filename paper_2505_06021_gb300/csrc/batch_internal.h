@@ -20,6 +20,7 @@ struct JobPlan {
   size_t tab_off;  // pinned tables
   size_t res_off;  // pinned results: [status | pad to 64 | Ec | eps | parts]
   size_t mixed;    // mixed-path workspace of all its q
+  size_t g64;      // FP64 job: chi0 workspace on the tensor cores (0: the FP64 kernel)
 };
 
 struct Group {
@@ -55,8 +56,11 @@ struct SideStreams {
   void release();
 };
 
-// Plan for n jobs; groups of jobs whose workspace fits `budget`.
-std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget);
+// Plan for n jobs; groups of jobs whose workspace fits `budget`.  g64: FP64
+// jobs may take chi0 to the tensor cores (their planes share the mixed region;
+// not set by the serving lanes, whose admission counts the FP64 kernel's
+// workspace).
+std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget, bool g64 = false);
 // Writes every job's small tables into the pinned buffer (tables_bytes each).
 void batch_fill_tables(const Plan& p, const rpa_job* jobs, int n, char* pin);
 // Issues the batch on `s` (tables already filled); results land in `pin` at

@@ -16,6 +16,7 @@
 
 #include "rpa_internal.h"
 #include "ao_internal.h"
+#include "g64.h"
 #include "rpa_runtime.h"
 
 using namespace rpa;
@@ -244,7 +245,8 @@ static size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 // Workspace cap of the synchronous calls (the serving lanes use a smaller one).
 size_t sync_ws_cap(rpa_ctx* ctx) { return std::min<size_t>(ctx->cap, (size_t)192 << 30); }
 
-Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt, const BinJob* bj) {
+Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt, const BinJob* bj,
+                   bool g64) {
   Layout L{};
   if (qt < qb) qt = qb;
   const size_t es = j->is_complex ? 16 : 8;
@@ -279,13 +281,24 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
   if (binned) L.binmeta = al(bj->meta_bytes);
   L.total = L.meta + L.dtab + L.chi + L.T + L.L + L.Vc + 2 * (L.stageC + L.stageV) + L.eps + L.mixed + L.ao +
             L.binmeta;
+  if (g64 && j->prec == RPA_PREC_FP64) {
+    // the FP64 chi0 on the tensor cores, where its planes fit under the cap
+    BatchGeom g{j->is_complex, j->n_aux, j->n_occ, j->n_virt, (int)nov, j->n_k, j->n_w, qb};
+    if (chi0_g64_use(g)) {
+      const size_t m = al(chi0_g64_bytes(g));
+      if (L.total + m <= ws_cap) {
+        L.mixed = m;
+        L.total += m;
+      }
+    }
+  }
   if (mixed_ws && binned) {
     // the frequency-batched chi0 takes what the cap leaves (pipelined when that suffices)
     BatchGeom g{j->is_complex, j->n_aux, j->n_occ, j->n_virt, (int)nov, j->n_k, j->n_w, 1};
     const size_t budget = ws_cap > L.total ? ws_cap - L.total : 0;
     L.mixed = al(binned_workspace_bytes(g, bj->plan, bj->Kt_max, bj->np_max, n_slices, budget));
     L.total += L.mixed;
-  } else if (L.mixed && qb >= 2) {
+  } else if (L.mixed && j->prec == RPA_PREC_MIXED && qb >= 2) {
     // two alternating regions (the next q's operand written during the
     // current q's tensor-core launch) when they fit under the cap
     BatchGeom g{j->is_complex, j->n_aux, j->n_occ, j->n_virt, (int)nov, j->n_k, j->n_w, 1};
@@ -629,10 +642,15 @@ static rpa_status run_chi(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const Bufs&
                              pex ? &hook : nullptr));
     ctx->launches += nl;
   } else {
+    uint64_t nl = 1;
     prof_begin(ctx, pex, s);
-    CK(launch_chi0_fp64(g, (const double* const*)(b.Cptrs + (size_t)q0 * nk), b.dtab, chi, s));
-    prof_end(ctx, pex, s, RPA_K_CHI0, 1);
-    ctx->launches++;
+    if (b.mixed_bytes)
+      CK(launch_chi0_g64(g, (const double* const*)(b.Cptrs + (size_t)q0 * nk), b.dtab, chi, b.mixed, b.mixed_bytes,
+                         b.status, &nl, s));
+    else
+      CK(launch_chi0_fp64(g, (const double* const*)(b.Cptrs + (size_t)q0 * nk), b.dtab, chi, s));
+    prof_end(ctx, pex, s, RPA_K_CHI0, (int)nl);
+    ctx->launches += nl;
   }
   return RPA_OK;
 }
@@ -723,7 +741,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
     if (rpa_status stb = bin_job_build(ctx, ex, job, bj)) return stb;
   const int qb = choose_qb(job, ctx->n_slices, ws_cap, &bj);
   const int qt = choose_qt(job, qb, ctx->n_slices, ws_cap, &bj);
-  Layout L = plan_layout(job, qb, ctx->n_slices, ws_cap, true, qt, &bj);
+  Layout L = plan_layout(job, qb, ctx->n_slices, ws_cap, true, qt, &bj, allow_bin);
   if (!ex.ensure_ws(L.total)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
     return RPA_E_NOMEM;
@@ -982,7 +1000,7 @@ rpa_status rpa_chi0(rpa_ctx* ctx, const rpa_job* job, int q, void* chi_out, void
   cudaStream_t s = (cudaStream_t)stream;
   BinJob bj;
   if (rpa_status stb = bin_job_build(ctx, ex, job, bj)) return stb;
-  Layout L = plan_layout(job, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, &bj);
+  Layout L = plan_layout(job, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, &bj, true);
   if (!ex.ensure_ws(L.total)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
     return RPA_E_NOMEM;

@@ -72,7 +72,7 @@ constexpr int TK = 16;  // t-chunk
 template <bool C, int G, int U>
 __global__ void __launch_bounds__(256, 1)
     chi0_fp64_kernel(BatchGeom g, const double* const* __restrict__ Cptrs, const double* __restrict__ dtab,
-                     double* __restrict__ chi, int n_tiles, int n_wg) {
+                     double* __restrict__ chi, int n_tiles, int n_wg, const int* __restrict__ only) {
   constexpr int CT = 16 * U;  // output tile edge
   __shared__ Elem<C> As[TK][CT];
   __shared__ Elem<C> Bs[TK][CT];
@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(256, 1)
   bid /= n_wg;
   const int tile = bid % n_tiles;
   const int qb = bid / n_tiles;
+  if (only && !only[qb]) return;
   int I, J;
   tri_index(tile, I, J);
   const int w0 = wg * G;
@@ -170,13 +171,13 @@ __global__ void __launch_bounds__(256, 1)
 
 template <bool C, int G, int U>
 cudaError_t chi0_launch_g(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
-                          cudaStream_t s) {
+                          cudaStream_t s, const int* only) {
   const int nt = (g.n_aux + 16 * U - 1) / (16 * U);
   const int n_tiles = nt * (nt + 1) / 2;
   const int n_wg = (g.n_w + G - 1) / G;
   const long blocks = (long)n_tiles * n_wg * g.n_qb;
   if (blocks > 0x7fffffffL) return cudaErrorInvalidConfiguration;
-  chi0_fp64_kernel<C, G, U><<<(unsigned)blocks, 256, 0, s>>>(g, Cptrs, dtab, chi, n_tiles, n_wg);
+  chi0_fp64_kernel<C, G, U><<<(unsigned)blocks, 256, 0, s>>>(g, Cptrs, dtab, chi, n_tiles, n_wg, only);
   return cudaGetLastError();
 }
 
@@ -191,7 +192,7 @@ cudaError_t chi0_launch_g(const BatchGeom& g, const double* const* Cptrs, const 
 // design notes for the present time.
 template <bool C>
 cudaError_t chi0_dispatch(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
-                          cudaStream_t s) {
+                          cudaStream_t s, const int* only) {
   const int Gs[6] = {10, 8, 5, 4, 2, 1};
   const long sms = num_sms_fp64();
   int bG = 8, bU = 2;
@@ -212,8 +213,8 @@ cudaError_t chi0_dispatch(const BatchGeom& g, const double* const* Cptrs, const 
     }
 #define RPA_CHI0_G(G)                                                   \
   case G:                                                               \
-    return bU == 2 ? chi0_launch_g<C, G, 2>(g, Cptrs, dtab, chi, s)     \
-                   : chi0_launch_g<C, G, 1>(g, Cptrs, dtab, chi, s)
+    return bU == 2 ? chi0_launch_g<C, G, 2>(g, Cptrs, dtab, chi, s, only)     \
+                   : chi0_launch_g<C, G, 1>(g, Cptrs, dtab, chi, s, only)
   switch (bG) {
     RPA_CHI0_G(10);
     RPA_CHI0_G(5);
@@ -221,7 +222,7 @@ cudaError_t chi0_dispatch(const BatchGeom& g, const double* const* Cptrs, const 
     RPA_CHI0_G(2);
     RPA_CHI0_G(1);
     default:
-      return bU == 2 ? chi0_launch_g<C, 8, 2>(g, Cptrs, dtab, chi, s) : chi0_launch_g<C, 8, 1>(g, Cptrs, dtab, chi, s);
+      return bU == 2 ? chi0_launch_g<C, 8, 2>(g, Cptrs, dtab, chi, s, only) : chi0_launch_g<C, 8, 1>(g, Cptrs, dtab, chi, s, only);
   }
 #undef RPA_CHI0_G
 }
@@ -352,8 +353,8 @@ cudaError_t launch_dtab(const BatchGeom& g, const double* eps_occ, const double*
 }
 
 cudaError_t launch_chi0_fp64(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
-                             cudaStream_t s) {
-  return g.cplx ? chi0_dispatch<true>(g, Cptrs, dtab, chi, s) : chi0_dispatch<false>(g, Cptrs, dtab, chi, s);
+                             cudaStream_t s, const int* only) {
+  return g.cplx ? chi0_dispatch<true>(g, Cptrs, dtab, chi, s, only) : chi0_dispatch<false>(g, Cptrs, dtab, chi, s, only);
 }
 
 namespace {

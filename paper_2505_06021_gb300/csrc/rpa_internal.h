@@ -37,8 +37,9 @@ cudaError_t launch_dtab(const BatchGeom& g, const double* eps_occ, const double*
                         const int* kqidx, const double* omega, double zeta_k, double* dtab, cudaStream_t s);
 
 // chi[qb][w] (N x N, full Hermitian) = sum_j sum_t conj(C[qb*n_k+j][P,t]) C[..][Q,t] d[qb][j][w][t].
+// only: null, or device flags per q of the batch; q with a zero flag are left as they are.
 cudaError_t launch_chi0_fp64(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
-                             cudaStream_t s);
+                             cudaStream_t s, const int* only = nullptr);
 
 // In-place Cholesky of n_mat matrices (stride bstride doubles).
 //   mode 0: input Y = -Pi (lower triangle), factorises 1 + Y = 1 - Pi and writes

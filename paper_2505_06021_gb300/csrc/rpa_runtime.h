@@ -165,7 +165,7 @@ void prof_collect(rpa_ctx* ctx, Exec* ex);
 // mixed_ws: include the split-precision chi0 workspace (a batch supplies its own).
 // qt: q per tail batch (0: qt = qb).  bj: the job's frequency-batched chi0, if any.
 Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt = 0,
-                   const BinJob* bj = nullptr);
+                   const BinJob* bj = nullptr, bool g64 = false);
 int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj = nullptr);
 int choose_qt(const rpa_job* j, int qb, int n_slices, size_t cap, const BinJob* bj = nullptr);
 // Builds the frequency-batched plan of a split-precision job (band energies
