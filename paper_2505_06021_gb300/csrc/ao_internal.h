@@ -25,6 +25,18 @@ struct AoPlan {
   size_t off_hocc = 0, off_hvirt = 0, off_c = 0, bytes = 0;
 };
 
+// The tensor-core form of the transforms (digit products, g64.cu): panel sizes
+// and its workspace, a region of its own outside AoPlan's.
+struct AoG64 {
+  bool half = false, assemble = false;
+  int k_batch = 1;       // k-points per half-transform batch
+  int rows = 0;          // PADF columns per panel (a multiple of 128, or S)
+  size_t a = 0, b = 0;   // bytes of the left and right planes
+  size_t e = 0;          // bytes of one exponent array (left and right each)
+  size_t bytes = 0;      // 0: the FP64 kernels throughout
+};
+AoG64 ao_g64_plan(const rpa_job* j, const AoPlan& p);
+
 // RPA_OK or RPA_E_INVAL with a message; j->ao must be non-null.
 int ao_validate(const rpa_job* j, char* msg, size_t len);
 // qb: q whose MO-basis coefficients the region holds at once.
@@ -35,8 +47,9 @@ size_t ao_region_bytes(const rpa_job* j, int qb);
 size_t ao_input_bytes(const rpa_job* j);
 // Fit table upload and half-transforms of the k-points used by q (q < 0: by
 // every q) into `region`.
+// gws: the AoG64 workspace, or null (FP64 kernels); status: device status word.
 rpa_status ao_enqueue_half(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p, char* region, int q,
-                           cudaStream_t s);
+                           cudaStream_t s, char* gws = nullptr, int* status = nullptr);
 // With overlap matrices: the periodic projector's c~ of every k-point into the
 // region (synchronises s); without: nothing.
 rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p, char* region, cudaStream_t s);
@@ -44,6 +57,6 @@ rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p
 const double* ao_mo(const rpa_job* j, const AoPlan& p, const char* region, int k);
 // C(q, k_j), j = 0..n_k-1, into out + j * cblk (half-transforms in place).
 rpa_status ao_enqueue_assemble(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p, const char* region, int q,
-                               char* out, cudaStream_t s);
+                               char* out, cudaStream_t s, char* gws = nullptr, int* status = nullptr);
 
 }  // namespace rpa

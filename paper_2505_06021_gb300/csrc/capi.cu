@@ -281,6 +281,13 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
   if (binned) L.binmeta = al(bj->meta_bytes);
   L.total = L.meta + L.dtab + L.chi + L.T + L.L + L.Vc + 2 * (L.stageC + L.stageV) + L.eps + L.mixed + L.ao +
             L.binmeta;
+  if (g64 && j->ao) {
+    const size_t m = al(ao_g64_plan(j, ao_plan(j, qb)).bytes);
+    if (L.total + m <= ws_cap) {
+      L.aog = m;
+      L.total += m;
+    }
+  }
   if (g64 && j->prec == RPA_PREC_FP64) {
     // the FP64 chi0 on the tensor cores, where its planes fit under the cap
     BatchGeom g{j->is_complex, j->n_aux, j->n_occ, j->n_virt, (int)nov, j->n_k, j->n_w, qb};
@@ -429,6 +436,8 @@ Bufs carve(void* ws, const rpa_job* j, const Layout& L) {
   b.ao = L.ao ? p : nullptr;
   p += L.ao;
   b.binmeta = L.binmeta ? p : nullptr;
+  p += L.binmeta;
+  b.aog = L.aog ? p : nullptr;
   return b;
 }
 
@@ -781,7 +790,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
   }
   if (job->ao) {
     if (rpa_status st1 = ao_project(ctx, &ex, job, aop, b.ao, s)) return st1;
-    if (rpa_status st1 = ao_enqueue_half(ctx, &ex, job, aop, b.ao, -1, s)) return st1;
+    if (rpa_status st1 = ao_enqueue_half(ctx, &ex, job, aop, b.ao, -1, s, b.aog, b.status)) return st1;
   }
 
   const double* eo = job->eps_occ;
@@ -819,7 +828,8 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
     if (host) CK(cudaStreamWaitEvent(s, ex.ready[slot], 0));
     for (int qi = 0; job->ao && qi < nq; ++qi)
       if (rpa_status st1 = ao_enqueue_assemble(ctx, &ex, job, aop, b.ao, q0 + qi,
-                                               b.ao + aop.off_c + (size_t)qi * job->n_k * cblk, s))
+                                               b.ao + aop.off_c + (size_t)qi * job->n_k * cblk, s, b.aog,
+                                               b.status))
         return st1;
     if (rpa_status st = run_chi(ctx, &ex, job, b, q0, nq, eo, ev, s, b.chi + (size_t)lo * job->n_w * NN * (es / 8),
                                 ctx->n_slices, &bj))
@@ -1019,8 +1029,9 @@ rpa_status rpa_chi0(rpa_ctx* ctx, const rpa_job* job, int q, void* chi_out, void
   CK(cudaStreamWaitEvent(s, ex.done, 0));
   if (job->ao) {
     if (rpa_status st1 = ao_project(ctx, &ex, job, aop, b.ao, s)) return st1;
-    if (rpa_status st1 = ao_enqueue_half(ctx, &ex, job, aop, b.ao, q, s)) return st1;
-    if (rpa_status st1 = ao_enqueue_assemble(ctx, &ex, job, aop, b.ao, q, b.ao + aop.off_c, s)) return st1;
+    if (rpa_status st1 = ao_enqueue_half(ctx, &ex, job, aop, b.ao, q, s, b.aog, b.status)) return st1;
+    if (rpa_status st1 = ao_enqueue_assemble(ctx, &ex, job, aop, b.ao, q, b.ao + aop.off_c, s, b.aog, b.status))
+      return st1;
   }
   if (rpa_status st = run_chi(ctx, &ex, job, b, q, 1, job->eps_occ, job->eps_virt, s, (double*)chi_out,
                               ctx->n_slices, &bj))
@@ -1051,20 +1062,30 @@ rpa_status rpa_ao2mo(rpa_ctx* ctx, const rpa_job* job, int q, void* C_out, void*
   Exec& ex = ctx->ex;
   cudaStream_t s = (cudaStream_t)stream;
   const AoPlan aop = ao_plan(job, 1);
-  // only the AO region is used: fit table and half-transforms
-  if (!ex.ensure_ws(aop.off_c + 256)) {
+  // only the AO region is used (fit table and half-transforms), and the digit
+  // planes of the tensor-core form where they fit
+  const size_t base = al(aop.off_c + 256);
+  size_t gb = ao_g64_plan(job, aop).bytes;
+  if (base + gb > sync_ws_cap(ctx) || (gb && !ex.ensure_ws(base + gb))) gb = 0;
+  if (!ex.ensure_ws(base)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", aop.off_c);
     return RPA_E_NOMEM;
   }
   char* region = (char*)ex.ws;
   if (rpa_status st = ao_project(ctx, &ex, job, aop, region, s)) return st;
-  if (rpa_status st = ao_enqueue_half(ctx, &ex, job, aop, region, q, s)) return st;
-  if (rpa_status st = ao_enqueue_assemble(ctx, &ex, job, aop, region, q, (char*)C_out, s)) return st;
+  char* gws = gb ? region + base : nullptr;
+  int* status = gws ? (int*)(gws + 512) : nullptr;
+  ex.status_word() = 0;
+  if (status) CK(cudaMemsetAsync(status, 0, sizeof(int), s));
+  if (rpa_status st = ao_enqueue_half(ctx, &ex, job, aop, region, q, s, gws, status)) return st;
+  if (rpa_status st = ao_enqueue_assemble(ctx, &ex, job, aop, region, q, (char*)C_out, s, gws, status)) return st;
+  if (status) CK(cudaMemcpyAsync(&ex.status_word(), status, sizeof(int), cudaMemcpyDeviceToHost, s));
   // the workspace is reused by the next call on this context
   CK(cudaEventRecord(ex.done, s));
   rpa_status wst = wait_event(ctx, ex.done, ctx->timeout_s + 600.0);
   prof_collect(ctx, &ex);
-  return wst;
+  if (wst) return wst;
+  return decode_status(ctx, ex.status_word(), job->n_w);
 }
 
 rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, double* out, void* stream) {

@@ -25,9 +25,10 @@
 // formed one k-point at a time by padf_k_kernel just before its
 // half-transforms (HBM-bound: n_R real reads and one complex write per entry).
 //
-// The transform kernels are FP64 (DFMA): the result feeds the FP64 chi0 path directly
-// and the split-precision path through its own 31-bit slicing.  GB300 issues
-// about two DFMA per clock per SM, so the kernels are organised only to keep
+// The transforms run as digit products on the tensor cores (ao.cu, g64.cu) where
+// their planes fit; the kernels here are the FP64 (DFMA) form for small atoms,
+// tight workspaces and rows whose spread the split cannot hold.  GB300 issues
+// about two DFMA per clock per SM, so they are organised only to keep
 // that pipe busy: a 32 x 32 output tile per CTA, 2 x 2 outputs per thread,
 // operands staged through shared memory in K-steps of 16 with coalesced row
 // loads, every complex multiply-add four DFMAs.
@@ -74,7 +75,8 @@ __device__ __forceinline__ void tile_tn(int K, const LA& la, const LB& lb, Elem<
 template <bool C>
 __global__ void __launch_bounds__(256) ao_half_kernel(int n_bas, int S, int n_mo, const double* __restrict__ P,
                                                       const double* __restrict__ c, int n0, int ncols,
-                                                      double* __restrict__ H, int n_tn) {
+                                                      double* __restrict__ H, int n_tn, const int* __restrict__ only) {
+  if (only && !*only) return;
   __shared__ Elem<C> As[AK][AT];
   __shared__ Elem<C> Bs[AK][AT];
   const int ts = blockIdx.x / n_tn, tn = blockIdx.x % n_tn;
@@ -105,7 +107,8 @@ __global__ void __launch_bounds__(256) ao_half_kernel(int n_bas, int S, int n_mo
 template <bool C>
 __global__ void __launch_bounds__(256)
     ao_assemble_kernel(const __grid_constant__ AoPairs pr, const int4* __restrict__ fit, int n_aux, int n_occ,
-                       int n_virt, int n_mo, int n_ti, int n_ta) {
+                       int n_virt, int n_mo, int n_ti, int n_ta, const int* __restrict__ only) {
+  if (only && !*only) return;
   __shared__ Elem<C> As[AK][AT];
   __shared__ Elem<C> Bs[AK][AT];
   long bid = blockIdx.x;
@@ -196,29 +199,29 @@ cudaError_t launch_padf_k(int cplx, const PadfLattice& L, const double* kfrac, l
 }
 
 cudaError_t launch_ao_half(int cplx, int n_bas, int S, int n_mo, const double* P, const double* c, int n0, int ncols,
-                           double* H, cudaStream_t s) {
+                           double* H, cudaStream_t s, const int* only) {
   if (S <= 0 || ncols <= 0) return cudaSuccess;
   const int n_ts = (S + AT - 1) / AT, n_tn = (ncols + AT - 1) / AT;
   const long blocks = (long)n_ts * n_tn;
   if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
   if (cplx)
-    ao_half_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(n_bas, S, n_mo, P, c, n0, ncols, H, n_tn);
+    ao_half_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(n_bas, S, n_mo, P, c, n0, ncols, H, n_tn, only);
   else
-    ao_half_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(n_bas, S, n_mo, P, c, n0, ncols, H, n_tn);
+    ao_half_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(n_bas, S, n_mo, P, c, n0, ncols, H, n_tn, only);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ao_assemble(int cplx, const AoPairs& pr, int n_pairs, const int4* fit, int n_aux, int n_occ,
-                               int n_virt, int n_mo, cudaStream_t s) {
+                               int n_virt, int n_mo, cudaStream_t s, const int* only) {
   if (n_pairs <= 0) return cudaSuccess;
   if (n_pairs > AoPairs::kMax) return cudaErrorInvalidValue;
   const int n_ti = (n_occ + AT - 1) / AT, n_ta = (n_virt + AT - 1) / AT;
   const long blocks = (long)n_pairs * n_aux * n_ti * n_ta;
   if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
   if (cplx)
-    ao_assemble_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(pr, fit, n_aux, n_occ, n_virt, n_mo, n_ti, n_ta);
+    ao_assemble_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(pr, fit, n_aux, n_occ, n_virt, n_mo, n_ti, n_ta, only);
   else
-    ao_assemble_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(pr, fit, n_aux, n_occ, n_virt, n_mo, n_ti, n_ta);
+    ao_assemble_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(pr, fit, n_aux, n_occ, n_virt, n_mo, n_ti, n_ta, only);
   return cudaGetLastError();
 }
 

@@ -88,9 +88,10 @@ cudaError_t launch_vinv(int cplx, int N, int n_q, const double* L, double* X, do
 
 // H[s][n] = sum_nu P[nu][s] c[nu][n0 + n], s < S, n < ncols: the half-
 // transform of one k-point's PADF array P (n_bas x S) with the MO columns
-// [n0, n0 + ncols) of c (n_bas x n_mo).  H is S x ncols.
+// [n0, n0 + ncols) of c (n_bas x n_mo).  H is S x ncols.  only: null, or a
+// device word; nothing is done when it is zero.
 cudaError_t launch_ao_half(int cplx, int n_bas, int S, int n_mo, const double* P, const double* c, int n0, int ncols,
-                           double* H, cudaStream_t s);
+                           double* H, cudaStream_t s, const int* only = nullptr);
 
 // Lattice form of the PADF coefficients: n_R integer lattice vectors and the
 // device arrays of their real cell-pair coefficients.
@@ -118,7 +119,7 @@ struct AoPairs {
 // fit[gamma] = (first basis function of gamma's atom, basis functions on it,
 // PADF column of (its first basis function, gamma), fit functions on it).
 cudaError_t launch_ao_assemble(int cplx, const AoPairs& pr, int n_pairs, const int4* fit, int n_aux, int n_occ,
-                               int n_virt, int n_mo, cudaStream_t s);
+                               int n_virt, int n_mo, cudaStream_t s, const int* only = nullptr);
 
 // ---- periodic projector (kernels_proj.cu) --------------------------------
 
