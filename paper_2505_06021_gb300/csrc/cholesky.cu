@@ -2,17 +2,28 @@
 // 1 - Pi' and V^-1 - chi0 with their log-determinants and traces, and the
 // inverse of the V factors.
 //
-// What bounds it.  An SM issues two DFMA lanes per clock, so one complex
-// N = 768 factorisation is 151e6 clocks (73 ms) of one SM's FP64 pipe but
+// What bounds it.  An SM's FP64 pipe takes 64 clocks per warp instruction on
+// each of its four sub-partitions (two DFMA lanes per clock and SM), so one
+// complex N = 768 factorisation is 151e6 clocks (73 ms) of one SM's pipe but
 // 0.5 ms of all 152: a matrix that stays on one SM, or on a cluster of eight,
 // is bound by that pipe and by its own serial phases, whatever else is idle.
 // Every panel step is therefore spread over the whole GPU: a launch covers
-// the panel rows (16 or 64 per CTA) or the trailing 32 x 32 tiles of every
-// matrix, and the kernel boundary is the only synchronisation.  The tile that
-// holds the next diagonal block factors it at once, so a panel costs two
-// launches.  Per matrix the arithmetic and its order do not depend on the
-// batch, so a matrix gives the same bits alone, in a batch or in a ragged
-// launch.  Matrices up to 64 stay in one CTA's shared memory, one launch in all.
+// the panel rows or the trailing tiles of every matrix, and the kernel boundary is
+// the only synchronisation.  The tile that holds the next diagonal block factors it at
+// once, so a panel costs two launches.  Matrices up to 64 stay in one CTA's
+// shared memory, one launch in all.
+//
+// Panel width.  Few matrices are bound by the chain of a panel: diagonal
+// block, rows, update of the next diagonal block.  Its FP64 instructions per
+// column grow with the panel width (every warp instruction is 64 clocks however
+// few lanes it has), so panels of 16 columns, 16 lanes per row and 16 x 16
+// tiles are about 22 us, two of them 44 where one of 32 columns took 95.  The FP64 modes
+// always take 16 columns (with many matrices the FP64 pipe bounds either
+// width); per matrix the arithmetic and its order do not depend on the batch,
+// the lanes per row or the tile, so a matrix gives the same bits alone, in a
+// batch or in a ragged launch.  The inverse form takes 32 columns when its
+// trailing tiles fill the GPU, since each panel converts and adds the whole
+// trailing matrix in FP64.
 //
 // Measured on GB300, one CTA or an 8-CTA cluster per matrix before, panel
 // launches now: one complex N = 768 factor of V 19.9 -> 2.4 ms; 16 matrices of
@@ -36,9 +47,8 @@
 namespace rpa {
 namespace {
 
-constexpr int CB = 32;                   // panel width and trailing tile edge
+constexpr int CB = 32;                   // block edge of the triangular inverse
 constexpr int SMALL_N = 64;              // largest matrix of the one-launch kernel
-constexpr int TRI = CB * (CB + 1) / 2;   // elements of a diagonal block's lower triangle
 constexpr int INIT_BLOCKS = 32;          // CTAs per matrix that form V^-1 - chi (<= SMALL_N)
 
 // Lower-triangular index -> (i, j), j <= i.
@@ -113,38 +123,61 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;
 }
 
-template <bool C>
+// 1 / x for a normal positive x: the hardware approximation and two
+// Newton-Raphson steps r += r (1 - x r), four FP64 instructions on the serial
+// chain of a panel; other values go through the division.
+__device__ __forceinline__ double fast_rcp(double x) {
+  const int hi = __double2hiint(x);
+  if (hi < (2 << 20) || hi >= (2044 << 20)) return 1.0 / x;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
+template <bool C, int NB>
 struct DiagShared {
-  Elem<C> col[2][CB];  // the current column (unscaled), double-buffered
+  Elem<C> col[2][NB];  // the current column (unscaled), double-buffered
   double rd[2];        // reciprocal of the current pivot
-  double piv[CB];      // pivots (mode 0: pivot - 1)
-  double l[CB], rs[CB];
+  double piv[NB];      // pivots (mode 0: pivot - 1)
+  double l[NB], rs[NB];
   int bad;
 };
 
 // Factor of the diagonal block D (lower triangle, nb x nb, shared memory) by
-// the CTA's 256 threads; L goes to Lout (leading dimension ld).  Each thread
-// keeps two or three elements of the triangle in registers, in column order,
-// so that whole warps retire as the columns do.  A column costs one barrier:
-// the columns stay unscaled (x_rc -= x_rk conj(x_ck) / d_k), which leaves one
+// the CTA's 256 threads; L goes to Lout (leading dimension ld).  The first
+// column needs no update; the others' elements stay in registers, in column
+// order, so that whole warps retire as the columns do (NB = 16: one element
+// per thread of four warps, one per sub-partition).  A column costs one
+// barrier: the columns stay unscaled (x_rc -= x_rk conj(x_ck) / d_k), which leaves one
 // reciprocal on the serial chain; all square roots, logarithms and scalings
 // follow at the end, one per thread.  Returns (thread 0) the block's share of
-// the log-determinant, NaN and *S.bad on a non-positive pivot.
-template <bool C>
-__device__ double diag_factor(Elem<C> (*D)[CB + 1], DiagShared<C>& S, int nb, int mode, double* Lout, long ld) {
+// the log-determinant, NaN and S.bad on a non-positive pivot.
+template <bool C, int NB>
+__device__ double diag_factor(Elem<C> (*D)[CB + 1], DiagShared<C, NB>& S, int nb, int mode, double* Lout, long ld) {
+  constexpr int UPD = NB * (NB - 1) / 2;  // elements of columns 1 ..
+  constexpr int E = (UPD + 255) / 256;
   const int tid = threadIdx.x;
-  Elem<C> x[3];
-  int er[3], ec[3];
+  Elem<C> x[E];
+  int er[E], ec[E];
   if (tid == 0) S.bad = 0;
+  auto publish = [&](int r, int c, const Elem<C>& v, int buf) {
+    S.col[buf][r] = v;
+    if (r == c) {
+      const double u = v.re;
+      S.piv[r] = u;
+      S.rd[buf] = fast_rcp(mode == 0 ? 1.0 + u : u);
+    }
+  };
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; k < E; ++k) {
     const int e = tid + 256 * k;
     er[k] = ec[k] = -1;
     x[k] = zero_elem<C>();
-    if (e < TRI) {
+    if (e < UPD) {
       int i, j;
-      tri_ij(TRI - 1 - e, i, j);
-      const int r = CB - 1 - j, c = CB - 1 - i;
+      tri_ij(UPD - 1 - e, i, j);
+      const int r = NB - 1 - j, c = NB - 1 - i;
       if (r < nb) {
         er[k] = r;
         ec[k] = c;
@@ -152,24 +185,20 @@ __device__ double diag_factor(Elem<C> (*D)[CB + 1], DiagShared<C>& S, int nb, in
       }
     }
   }
-  auto publish = [&](int k, int buf) {
-    S.col[buf][er[k]] = x[k];
-    if (er[k] == ec[k]) {
-      const double u = x[k].re;
-      S.piv[er[k]] = u;
-      S.rd[buf] = 1.0 / (mode == 0 ? 1.0 + u : u);
-    }
-  };
-  if (ec[0] == 0) publish(0, 0);
+  Elem<C> x0 = zero_elem<C>();  // column 0, one element per thread
+  if (tid < nb) {
+    x0 = D[tid][0];
+    publish(tid, 0, x0, 0);
+  }
   __syncthreads();
-  for (int c = 0; c < nb; ++c) {
+  for (int c = 0; c + 1 < nb; ++c) {
     const int buf = c & 1;
     const double rd = S.rd[buf];
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < E; ++k)
       if (ec[k] > c) {
         msub_conj<C>(x[k], scale<C>(S.col[buf][er[k]], rd), S.col[buf][ec[k]]);
-        if (ec[k] == c + 1) publish(k, buf ^ 1);
+        if (ec[k] == c + 1) publish(er[k], c + 1, x[k], buf ^ 1);
       }
     __syncthreads();
   }
@@ -180,21 +209,23 @@ __device__ double diag_factor(Elem<C> (*D)[CB + 1], DiagShared<C>& S, int nb, in
     const bool ok = p > 0.0;
     const double l = sqrt(p);
     S.l[tid] = l;
-    S.rs[tid] = 1.0 / l;
+    S.rs[tid] = fast_rcp(l);
     lg = !ok ? nan("") : mode == 0 ? log1p(u) : log(p);
     if (!ok) S.bad = 1;
   }
   __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    if (ec[k] >= 0) {
-      Elem<C> v = scale<C>(x[k], S.rs[ec[k]]);
-      if (er[k] == ec[k]) {
-        v = zero_elem<C>();
-        v.re = S.l[er[k]];
-      }
-      st_elem<C>(Lout, er[k] * ld + ec[k], v);
+  auto put = [&](int r, int c, const Elem<C>& v) {
+    Elem<C> w = scale<C>(v, S.rs[c]);
+    if (r == c) {
+      w = zero_elem<C>();
+      w.re = S.l[r];
     }
+    st_elem<C>(Lout, r * ld + c, w);
+  };
+  if (tid < nb) put(tid, 0, x0);
+#pragma unroll
+  for (int k = 0; k < E; ++k)
+    if (ec[k] >= 0) put(er[k], ec[k], x[k]);
   return tid < 32 ? warp_sum(lg) : 0.0;
 }
 
@@ -208,31 +239,32 @@ __device__ __forceinline__ void diag_report(const CholTask& t, double lg, int ba
   t.out[0] = v;
 }
 
-// Rows of a panel: X L_kk^H = A_panel, four lanes per row (lane g of a row
-// owns columns c = 4 j + g), so that the serial chain of a row is 32 short
-// steps and a warp's FP64 instructions carry eight rows.  Ls[c][c'] holds
-// L_kk[c'][c], rs the reciprocal diagonal.  `row` is this quad's row (invalid
-// rows take part in the shuffles).
-template <bool C, class ST>
-__device__ __forceinline__ void panel_row(const double* A, long ld, bool valid, const Elem<C> (*Ls)[CB + 1],
+// Rows of a panel: X L_kk^H = A_panel, LPR lanes per row (lane g of a row
+// owns columns c = LPR j + g).  16 lanes keep a row's serial chain short (a
+// column is six FP64 instructions of its warp), 4 lanes use fewer instructions
+// per row.  Ls[c][c'] holds L_kk[c'][c], rs the reciprocal diagonal.  `A` is
+// this row's panel (invalid rows take part in the shuffles).
+template <bool C, int NB, int LPR, class ST>
+__device__ __forceinline__ void panel_row(const double* A, bool valid, const Elem<C> (*Ls)[CB + 1],
                                           const double* rs, const ST& store) {
-  const int lane = threadIdx.x & 31, g = lane & 3, q0 = lane & ~3;
-  Elem<C> x[CB / 4];
+  constexpr int J = NB / LPR;
+  const int lane = threadIdx.x & 31, g = lane & (LPR - 1), q0 = lane & ~(LPR - 1);
+  Elem<C> x[J];
 #pragma unroll
-  for (int j = 0; j < CB / 4; ++j) x[j] = valid ? ld_elem<C>(A, 4 * j + g) : zero_elem<C>();
+  for (int j = 0; j < J; ++j) x[j] = valid ? ld_elem<C>(A, LPR * j + g) : zero_elem<C>();
 #pragma unroll
-  for (int c = 0; c < CB; ++c) {
-    Elem<C> v = scale<C>(x[c / 4], rs[c]);
-    v.re = __shfl_sync(0xffffffffu, v.re, q0 | (c & 3));
-    if constexpr (C) v.im = __shfl_sync(0xffffffffu, v.im, q0 | (c & 3));
-    if (g == (c & 3)) x[c / 4] = v;
+  for (int c = 0; c < NB; ++c) {
+    Elem<C> v = scale<C>(x[c / LPR], rs[c]);
+    v.re = __shfl_sync(0xffffffffu, v.re, q0 | (c & (LPR - 1)));
+    if constexpr (C) v.im = __shfl_sync(0xffffffffu, v.im, q0 | (c & (LPR - 1)));
+    if (g == (c & (LPR - 1))) x[c / LPR] = v;
 #pragma unroll
-    for (int j = c / 4; j < CB / 4; ++j)
-      if (j > c / 4 || g > (c & 3)) msub_conj<C>(x[j], v, Ls[c][4 * j + g]);
+    for (int j = c / LPR; j < J; ++j)
+      if (j > c / LPR || g > (c & (LPR - 1))) msub_conj<C>(x[j], v, Ls[c][LPR * j + g]);
   }
   if (valid)
 #pragma unroll
-    for (int j = 0; j < CB / 4; ++j) store(4 * j + g, x[j]);
+    for (int j = 0; j < J; ++j) store(LPR * j + g, x[j]);
 }
 
 // --------------------------------------------------- per-panel kernels ----
@@ -276,13 +308,13 @@ __global__ void __launch_bounds__(256) chol_init_kernel(const __grid_constant__ 
 
 // The first diagonal block of every matrix, and the traces (mode 0: Tr Pi =
 // -sum Y_jj; mode 2: the partial sums of chol_init_kernel).
-template <bool C>
+template <bool C, int NB>
 __global__ void __launch_bounds__(256) chol_first_kernel(const __grid_constant__ CholBatch B, int nblk) {
-  __shared__ Elem<C> D[CB][CB + 1];
-  __shared__ DiagShared<C> S;
+  __shared__ Elem<C> D[NB][CB + 1];
+  __shared__ DiagShared<C, NB> S;
   __shared__ double red[8];
   const CholTask t = task_of<C>(B, blockIdx.x);
-  const int N = t.N, tid = threadIdx.x, nb = min(CB, N);
+  const int N = t.N, tid = threadIdx.x, nb = min(NB, N);
   if (t.mode != 1) {
     double s = 0.0;
     if (t.mode == 0) {
@@ -293,149 +325,161 @@ __global__ void __launch_bounds__(256) chol_first_kernel(const __grid_constant__
     s = block_sum(s, red);
     if (tid == 0) t.out[1] = s;
   }
-  for (int i = tid; i < CB * CB; i += 256) {
-    const int r = i / CB, c = i % CB;
+  for (int i = tid; i < NB * NB; i += 256) {
+    const int r = i / NB, c = i % NB;
     if (r < nb && c <= r) D[r][c] = ld_elem<C>(t.A, (long)r * N + c);
   }
   __syncthreads();
-  const double lg = diag_factor<C>(D, S, nb, t.mode, t.A, N);
-  if (tid == 0) diag_report(t, lg, S.bad, true, N <= CB);
+  const double lg = diag_factor<C, NB>(D, S, nb, t.mode, t.A, N);
+  if (tid == 0) diag_report(t, lg, S.bad, true, N <= NB);
 }
 
-// Panel rows below the diagonal block at kb (full panels only: kb + CB < N).
+// Panel rows below the diagonal block at kb (full panels only: kb + NB < N).
 // Mode 2 also stores the float-float copy of L_{i,kb+c} at (row kb + c, column
 // i) of the free strict upper triangle, where a trailing tile's operand rows
 // are contiguous.
-template <bool C, int WARPS>
+template <bool C, int NB, int LPR, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS) chol_panel_kernel(const __grid_constant__ CholBatch B, int kb, int per) {
-  __shared__ Elem<C> Ls[CB][CB + 1];
-  __shared__ double rs[CB];
+  __shared__ Elem<C> Ls[NB][CB + 1];
+  __shared__ double rs[NB];
   const int b = blockIdx.x / per, blk = blockIdx.x % per;
   const CholTask t = task_of<C>(B, b);
   const int N = t.N, tid = threadIdx.x;
-  const int r0 = kb + CB + blk * 8 * WARPS;
+  const int r0 = kb + NB + blk * (32 / LPR) * WARPS;
   if (r0 >= N) return;
-  for (int i = tid; i < CB * CB; i += 32 * WARPS) {
-    const int r = i / CB, c = i % CB;
-    if (c <= r) Ls[c][r] = ld_elem<C>(t.A, (long)(kb + r) * N + kb + c);
+  for (int i = tid; i < NB * NB; i += 32 * WARPS) {
+    const int r = i / NB, c = i % NB;
+    if (c <= r) {
+      const Elem<C> e = ld_elem<C>(t.A, (long)(kb + r) * N + kb + c);
+      Ls[c][r] = e;
+      if (c == r) rs[r] = fast_rcp(e.re);
+    }
   }
   __syncthreads();
-  if (tid < CB) rs[tid] = 1.0 / Ls[tid][tid].re;
-  __syncthreads();
-  const int i = r0 + (tid >> 2);
+  const int i = r0 + tid / LPR;
   const bool valid = i < N;
   double* row = t.A + ((long)i * N + kb) * (C ? 2 : 1);
   double* A = t.A;
   const bool ff = t.mode == 2;
-  panel_row<C>(row, N, valid, Ls, rs, [&](int c, const Elem<C>& v) {
+  panel_row<C, NB, LPR>(row, valid, Ls, rs, [&](int c, const Elem<C>& v) {
     st_elem<C>(row, c, v);
     if (ff) st_ff<C>(A, (long)(kb + c) * N + i, to_ff<C>(v));
   });
 }
 
-// Trailing update with the panel at kb: 32 x 32 tiles of the lower triangle
-// beyond it, 2 x 2 outputs per thread; FP64 (FF = false) or, on the
+// Trailing update with the panel at kb: tiles of edge 16 U of the lower
+// triangle beyond it, U x U outputs per thread; FP64 (FF = false) or, on the
 // split-precision path, float-float on the FP32 pipe (about 2^-45 of the
 // update, five times the FP64 pipe's rate).  Tile (0, 0) goes on to factor
 // the next diagonal block.
-template <bool C, bool FF>
+template <bool C, bool FF, int NB, int U>
 __global__ void __launch_bounds__(256, FF ? 3 : 2)
     chol_update_kernel(const __grid_constant__ CholBatch B, int kb, int per) {
-  __shared__ Elem<C> S1[CB][CB + 1];
-  __shared__ Elem<C> S2[CB][CB + 1];
-  __shared__ DiagShared<C> S;
+  static_assert(NB <= 16 * U, "the first tile holds the next diagonal block");
+  constexpr int T = 16 * U, SR = NB > T ? NB : T;
+  __shared__ Elem<C> S1[SR][CB + 1];
+  __shared__ Elem<C> S2[NB][CB + 1];
+  __shared__ DiagShared<C, NB> S;
   const int b = blockIdx.x / per, tile = blockIdx.x % per;
   const CholTask t = task_of<C>(B, b);
-  const int N = t.N, m0 = kb + CB, m = N - m0;
+  const int N = t.N, m0 = kb + NB, m = N - m0;
   if (m <= 0) return;
-  const int nt = (m + CB - 1) / CB;
+  const int nt = (m + T - 1) / T;
   if (tile >= nt * (nt + 1) / 2) return;
   int TI, TJ;
   tri_ij(tile, TI, TJ);
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   double* A = t.A;
-  Elem<C> o[2][2];  // the tile's own values, in flight during the product
+  Elem<C> o[U][U];  // the tile's own values, in flight during the product
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
+  for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const int r = m0 + TI * CB + ty + 16 * u, c = m0 + TJ * CB + tx + 16 * v;
+    for (int v = 0; v < U; ++v) {
+      const int r = m0 + TI * T + ty + 16 * u, c = m0 + TJ * T + tx + 16 * v;
       o[u][v] = (r < N && c <= r) ? ld_elem<C>(A, (long)r * N + c) : zero_elem<C>();
     }
   if constexpr (FF) {
     FFE<C>(*F1)[CB + 1] = reinterpret_cast<FFE<C>(*)[CB + 1]>(S1);
     FFE<C>(*F2)[CB + 1] = reinterpret_cast<FFE<C>(*)[CB + 1]>(S2);
-    for (int i = tid; i < CB * CB; i += 256) {
-      const int r = i % CB, c = i / CB;
-      const int ri = m0 + TI * CB + r, rj = m0 + TJ * CB + r;
+    for (int i = tid; i < NB * T; i += 256) {
+      const int r = i % T, c = i / T;
+      const int ri = m0 + TI * T + r, rj = m0 + TJ * T + r;
       const long up = (long)(kb + c) * N;
       F1[c][r] = ri < N ? ld_ff<C>(A, up + ri) : FFE<C>{};
       F2[c][r] = rj < N ? conj_ff<C>(ld_ff<C>(A, up + rj)) : FFE<C>{};
     }
     __syncthreads();
-    FFE<C> acc[2][2] = {};
+    FFE<C> acc[U][U] = {};
 #pragma unroll 2
-    for (int c = 0; c < CB; ++c) {
-      const FFE<C> a0 = F1[c][ty], a1 = F1[c][ty + 16];
-      const FFE<C> b0 = F2[c][tx], b1 = F2[c][tx + 16];
-      ff_mac_e<C>(acc[0][0], a0, b0);
-      ff_mac_e<C>(acc[0][1], a0, b1);
-      ff_mac_e<C>(acc[1][0], a1, b0);
-      ff_mac_e<C>(acc[1][1], a1, b1);
+    for (int c = 0; c < NB; ++c) {
+      FFE<C> fa[U], fb[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        fa[u] = F1[c][ty + 16 * u];
+        fb[u] = F2[c][tx + 16 * u];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v) ff_mac_e<C>(acc[u][v], fa[u], fb[v]);
     }
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int v = 0; v < 2; ++v) {
+      for (int v = 0; v < U; ++v) {
         o[u][v].re -= (double)acc[u][v].rh + (double)acc[u][v].rl;
         if constexpr (C) o[u][v].im -= (double)acc[u][v].ih + (double)acc[u][v].il;
       }
   } else {
-    for (int i = tid; i < CB * CB; i += 256) {
-      const int r = i / CB, c = i % CB;
-      const int ri = m0 + TI * CB + r, rj = m0 + TJ * CB + r;
+    for (int i = tid; i < NB * T; i += 256) {
+      const int r = i / NB, c = i % NB;
+      const int ri = m0 + TI * T + r, rj = m0 + TJ * T + r;
       S1[c][r] = ri < N ? ld_elem<C>(A, (long)ri * N + kb + c) : zero_elem<C>();
       S2[c][r] = rj < N ? ld_elem<C>(A, (long)rj * N + kb + c) : zero_elem<C>();
     }
     __syncthreads();
 #pragma unroll 4
-    for (int c = 0; c < CB; ++c) {
-      const Elem<C> a0 = S1[c][ty], a1 = S1[c][ty + 16];
-      const Elem<C> b0 = S2[c][tx], b1 = S2[c][tx + 16];
-      msub_conj<C>(o[0][0], a0, b0);
-      msub_conj<C>(o[0][1], a0, b1);
-      msub_conj<C>(o[1][0], a1, b0);
-      msub_conj<C>(o[1][1], a1, b1);
+    for (int c = 0; c < NB; ++c) {
+      Elem<C> a[U], bv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a[u] = S1[c][ty + 16 * u];
+        bv[u] = S2[c][tx + 16 * u];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v) msub_conj<C>(o[u][v], a[u], bv[v]);
     }
   }
-  if (tile == 0) {
-    __syncthreads();  // S1 is read no more
+  const bool diag = tile == 0;
+  if (diag) __syncthreads();  // S1 is read no more
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+  for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int v = 0; v < 2; ++v) S1[ty + 16 * u][tx + 16 * v] = o[u][v];
-    __syncthreads();
-    const int nb = min(CB, m);
-    const double lg = diag_factor<C>(S1, S, nb, t.mode, A + ((long)m0 * N + m0) * (C ? 2 : 1), N);
-    if (tid == 0) diag_report(t, lg, S.bad, false, m <= CB);
-    return;
-  }
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const int r = m0 + TI * CB + ty + 16 * u, c = m0 + TJ * CB + tx + 16 * v;
-      if (r < N && c <= r) st_elem<C>(A, (long)r * N + c, o[u][v]);
+    for (int v = 0; v < U; ++v) {
+      const int lr = ty + 16 * u, lc = tx + 16 * v;
+      const int r = m0 + TI * T + lr, c = m0 + TJ * T + lc;
+      if (diag && lr < NB && lc < NB)
+        S1[lr][lc] = o[u][v];
+      else if (r < N && c <= r)
+        st_elem<C>(A, (long)r * N + c, o[u][v]);
     }
+  if (!diag) return;
+  __syncthreads();
+  const int nb = min(NB, m);
+  const double lg = diag_factor<C, NB>(S1, S, nb, t.mode, A + ((long)m0 * N + m0) * (C ? 2 : 1), N);
+  if (tid == 0) diag_report(t, lg, S.bad, false, m <= NB);
 }
 
 // N <= 64: the whole matrix in one CTA's shared memory, all modes, one launch
-// (two panels: diagonal block, rows, trailing block, diagonal block).
+// (up to four panels of 16 columns: diagonal block, rows, trailing elements).
 template <bool C>
 __global__ void __launch_bounds__(256) chol_small_kernel(const __grid_constant__ CholBatch B) {
   extern __shared__ __align__(16) double m_raw[];  // SMALL_N x (SMALL_N + 1) elements
-  __shared__ Elem<C> D[CB][CB + 1];
-  __shared__ DiagShared<C> S;
+  constexpr int NB = 16;
+  __shared__ Elem<C> D[NB][CB + 1];
+  __shared__ DiagShared<C, NB> S;
   __shared__ double red[8];
   constexpr long LD = SMALL_N + 1;
   const CholTask t = task_of<C>(B, blockIdx.x);
@@ -459,38 +503,36 @@ __global__ void __launch_bounds__(256) chol_small_kernel(const __grid_constant__
   }
   s = block_sum(s, red);  // its barriers also order the loads before the factor
   if (tid == 0 && t.mode != 1) t.out[1] = s;
-  for (int kb = 0; kb < N; kb += CB) {
-    const int nb = min(CB, N - kb), m0 = kb + nb;
-    for (int i = tid; i < CB * CB; i += 256) {
-      const int r = i / CB, c = i % CB;
+  for (int kb = 0; kb < N; kb += NB) {
+    const int nb = min(NB, N - kb), m0 = kb + nb, m = N - m0;
+    for (int i = tid; i < NB * NB; i += 256) {
+      const int r = i / NB, c = i % NB;
       if (r < nb && c <= r) D[r][c] = ld_elem<C>(m_raw, (kb + r) * LD + kb + c);
     }
     __syncthreads();
-    const double lg = diag_factor<C>(D, S, nb, t.mode, m_raw + (kb * LD + kb) * (C ? 2 : 1), LD);
-    if (tid == 0) diag_report(t, lg, S.bad, kb == 0, m0 >= N);
+    const double lg = diag_factor<C, NB>(D, S, nb, t.mode, m_raw + (kb * LD + kb) * (C ? 2 : 1), LD);
+    if (tid == 0) diag_report(t, lg, S.bad, kb == 0, m <= 0);
     __syncthreads();
-    if (m0 >= N) break;
-    for (int i = tid; i < CB * CB; i += 256) {
-      const int r = i / CB, c = i % CB;
-      if (c <= r) D[c][r] = ld_elem<C>(m_raw, r * LD + c);
+    if (m <= 0) break;
+    for (int i = tid; i < NB * NB; i += 256) {
+      const int r = i / NB, c = i % NB;
+      if (c <= r) D[c][r] = ld_elem<C>(m_raw, (kb + r) * LD + kb + c);
     }
     __syncthreads();
-    // at most 32 rows: the first four warps
-    if (tid < 128) {
+    // at most 48 rows, four lanes each
+    if (tid < 192) {
       const int i = m0 + (tid >> 2);
-      double* row = m_raw + (long)min(i, N - 1) * LD * (C ? 2 : 1);
-      panel_row<C>(row, LD, i < N, D, S.rs, [&](int c, const Elem<C>& v) { st_elem<C>(row, c, v); });
+      double* row = m_raw + ((long)min(i, N - 1) * LD + kb) * (C ? 2 : 1);
+      panel_row<C, NB, 4>(row, i < N, D, S.rs, [&](int c, const Elem<C>& v) { st_elem<C>(row, c, v); });
     }
     __syncthreads();
-    const int m = N - m0;
-    for (int e = tid; e < TRI; e += 256) {
+    for (int e = tid; e < m * (m + 1) / 2; e += 256) {
       int r, c;
       tri_ij(e, r, c);
-      if (r >= m) continue;
       const long ro = (m0 + r) * LD, co = (m0 + c) * LD;
       Elem<C> x = ld_elem<C>(m_raw, ro + m0 + c);
 #pragma unroll 4
-      for (int k = 0; k < CB; ++k) msub_conj<C>(x, ld_elem<C>(m_raw, ro + k), ld_elem<C>(m_raw, co + k));
+      for (int k = 0; k < NB; ++k) msub_conj<C>(x, ld_elem<C>(m_raw, ro + kb + k), ld_elem<C>(m_raw, co + kb + k));
       st_elem<C>(m_raw, ro + m0 + c, x);
     }
     __syncthreads();
@@ -560,38 +602,40 @@ __global__ void __launch_bounds__(128) trinv_diag_kernel(int N, const double* __
 // the mirrored block (rows of block 1, columns of block 2: the strict upper
 // triangle, free until the end), transposed; PASS 1: X21 = -X22 T21.
 // K ranges skip the operands' zero triangles.
-template <bool C, int PASS>
+template <bool C, int PASS, int U>
 __global__ void __launch_bounds__(256) trinv_join_kernel(int N, int s, const double* __restrict__ Lb,
                                                          double* __restrict__ Xb, int tiles, int n_pairs) {
-  __shared__ Elem<C> S1[CB][CB + 1];
-  __shared__ Elem<C> S2[CB][CB + 1];
-  const int nt = s / CB;
+  constexpr int T = 16 * U;  // tile edge
+  __shared__ Elem<C> S1[CB][T + 1];
+  __shared__ Elem<C> S2[CB][T + 1];
+  const int nt = s / T;
   int bid = blockIdx.x;
   const int tile = bid % tiles;
   bid /= tiles;
   const int p = bid % n_pairs, b = bid / n_pairs;
   const int TI = tile / nt, TJ = tile % nt;
   const int c0 = 2 * s * p, r0 = c0 + s;  // block 1 (columns), block 2 (rows)
-  const int row0 = r0 + TI * CB, col0 = c0 + TJ * CB;
+  const int row0 = r0 + TI * T, col0 = c0 + TJ * T;
   if (row0 >= N) return;
   const long NN = (long)N * N * (C ? 2 : 1);
   const double* L = Lb + b * NN;
   double* X = Xb + b * NN;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  Elem<C> o[2][2];
+  Elem<C> o[U][U];
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
+  for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int v = 0; v < 2; ++v) o[u][v] = zero_elem<C>();
+    for (int v = 0; v < U; ++v) o[u][v] = zero_elem<C>();
   // PASS 0: sum over k of L[row][k] X[k][col], k in block 1 from the column's tile on
   // PASS 1: sum over k of X[row][k] T[k][col], k in block 2 up to the row's tile
-  const int ka = PASS == 0 ? col0 : r0, kz = PASS == 0 ? r0 : min(row0 + CB, N);
+  const int ka = PASS == 0 ? col0 / CB * CB : r0, kz = PASS == 0 ? r0 : min(row0 + T, N);
   for (int k0 = ka; k0 < kz; k0 += CB) {
-    for (int i = tid; i < CB * CB; i += 256) {
+    for (int i = tid; i < CB * T; i += 256) {
       const int r = i / CB, c = i % CB;
       if (PASS == 0) {
+        const int kr = i / T, kc = i % T;
         S1[c][r] = row0 + r < N ? ld_elem<C>(L, (long)(row0 + r) * N + k0 + c) : zero_elem<C>();
-        S2[r][c] = ld_elem<C>(X, (long)(k0 + r) * N + col0 + c);
+        S2[kr][kc] = ld_elem<C>(X, (long)(k0 + kr) * N + col0 + kc);
       } else {
         S1[c][r] = (row0 + r < N && k0 + c < N) ? ld_elem<C>(X, (long)(row0 + r) * N + k0 + c) : zero_elem<C>();
         // T[k][col] is stored at X[col][k]
@@ -601,19 +645,23 @@ __global__ void __launch_bounds__(256) trinv_join_kernel(int N, int s, const dou
     __syncthreads();
 #pragma unroll 4
     for (int c = 0; c < CB; ++c) {
-      const Elem<C> a0 = S1[c][ty], a1 = S1[c][ty + 16];
-      const Elem<C> b0 = S2[c][tx], b1 = S2[c][tx + 16];
-      mac<C>(o[0][0], a0, b0);
-      mac<C>(o[0][1], a0, b1);
-      mac<C>(o[1][0], a1, b0);
-      mac<C>(o[1][1], a1, b1);
+      Elem<C> a[U], bv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a[u] = S1[c][ty + 16 * u];
+        bv[u] = S2[c][tx + 16 * u];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v) mac<C>(o[u][v], a[u], bv[v]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
+  for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
+    for (int v = 0; v < U; ++v) {
       const int r = row0 + ty + 16 * u, c = col0 + tx + 16 * v;
       if (r >= N) continue;
       Elem<C> e = o[u][v];
@@ -652,6 +700,13 @@ cudaError_t small_attr() {
   return e;
 }
 
+// Inverse form: panels of 32 columns once the trailing tiles of half the
+// matrix's panels fill the GPU several times over.
+bool panel32(int N, long n_mat) {
+  const long h = (N / 2 + 31) / 32;
+  return n_mat * h * (h + 1) / 2 >= 8L * device_sm_count();
+}
+
 // Launches of one batch whose largest matrix is N (tasks sorted by size,
 // largest first, when ragged: Ns[b] is task b's size, so that each panel
 // covers only the prefix that still has one).
@@ -668,25 +723,49 @@ cudaError_t chol_run(const CholBatch& B, int N, int n_mat, const int* Ns, int mo
     chol_init_kernel<C><<<n_mat * INIT_BLOCKS, 256, 0, s>>>(B, INIT_BLOCKS);
     ++nl;
   }
-  chol_first_kernel<C><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS);
+  const bool wide = mode == 2 && panel32(N, n_mat);
+  if (wide)
+    chol_first_kernel<C, 32><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS);
+  else
+    chol_first_kernel<C, 16><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS);
   ++nl;
-  const int sms = device_sm_count();
+  const long sms = device_sm_count();
+  const int NB = wide ? 32 : 16;
   int live = n_mat;
-  for (int kb = 0; kb + CB < N; kb += CB) {
-    while (Ns && live > 0 && Ns[live - 1] <= kb + CB) --live;
-    const int m = N - kb - CB;
-    // 16 rows per CTA while 64 would leave SMs idle (a CTA's rows queue on
-    // its SM's FP64 pipe: 64 rows are 34 us, 16 are 9)
-    const int per64 = (m + 63) / 64, per16 = (m + 15) / 16;
-    if ((long)live * per64 >= 2L * sms)
-      chol_panel_kernel<C, 8><<<(unsigned)(live * per64), 256, 0, s>>>(B, kb, per64);
-    else
-      chol_panel_kernel<C, 2><<<(unsigned)(live * per16), 64, 0, s>>>(B, kb, per16);
-    const int nt = (m + CB - 1) / CB, per = nt * (nt + 1) / 2;
-    if (mode == 2)
-      chol_update_kernel<C, true><<<(unsigned)(live * per), 256, 0, s>>>(B, kb, per);
-    else
-      chol_update_kernel<C, false><<<(unsigned)(live * per), 256, 0, s>>>(B, kb, per);
+  for (int kb = 0; kb + NB < N; kb += NB) {
+    while (Ns && live > 0 && Ns[live - 1] <= kb + NB) --live;
+    const int m = N - kb - NB;
+    // rows: 8 per CTA with 16 lanes each while that leaves SMs free, else 64
+    // with four lanes each (80 instead of 128 FP64 instructions per row)
+    const int per64 = (m + 63) / 64, per8 = (m + 7) / 8;
+    const bool few = (long)live * per8 <= 4 * sms;
+    if (wide) {
+      if (few)
+        chol_panel_kernel<C, 32, 16, 4><<<(unsigned)(live * per8), 128, 0, s>>>(B, kb, per8);
+      else
+        chol_panel_kernel<C, 32, 4, 8><<<(unsigned)(live * per64), 256, 0, s>>>(B, kb, per64);
+    } else {
+      if (few)
+        chol_panel_kernel<C, 16, 16, 4><<<(unsigned)(live * per8), 128, 0, s>>>(B, kb, per8);
+      else
+        chol_panel_kernel<C, 16, 4, 8><<<(unsigned)(live * per64), 256, 0, s>>>(B, kb, per64);
+    }
+    const long n32 = (m + 31) / 32, n16 = (m + 15) / 16;
+    const int per32 = (int)(n32 * (n32 + 1) / 2), per16 = (int)(n16 * (n16 + 1) / 2);
+    // 16 x 16 tiles until 32 x 32 ones give every SM two (they read less)
+    const bool t32 = live * (long)per32 >= 2 * sms;
+    if (mode == 2) {
+      if (wide)
+        chol_update_kernel<C, true, 32, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32);
+      else if (t32)
+        chol_update_kernel<C, true, 16, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32);
+      else
+        chol_update_kernel<C, true, 16, 1><<<(unsigned)(live * per16), 256, 0, s>>>(B, kb, per16);
+    } else if (t32) {
+      chol_update_kernel<C, false, 16, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32);
+    } else {
+      chol_update_kernel<C, false, 16, 1><<<(unsigned)(live * per16), 256, 0, s>>>(B, kb, per16);
+    }
     nl += 2;
   }
   if (n_launch) *n_launch = nl;
@@ -701,7 +780,7 @@ cudaError_t launch_cholesky(int cplx, int N, int n_mat, double* mats, long bstri
   if (n_mat == 0) return cudaSuccess;
   if (mode == 2 && (!Wn || !Vc || !ldV || n_w <= 0)) return cudaErrorInvalidValue;
   if (mode != 1 && !out) return cudaErrorInvalidValue;
-  const long nt = (N + CB - 1) / CB;
+  const long nt = (N + 15) / 16;
   if ((long)n_mat * std::max<long>(nt * (nt + 1) / 2, INIT_BLOCKS) > 0x7fffffffL) return cudaErrorInvalidValue;
   const CholBatch B{nullptr, mats, bstride, out, status, Wn, Vc, ldV, N, mode, status_base, std::max(n_w, 1)};
   return cplx ? chol_run<true>(B, N, n_mat, nullptr, mode, s, nullptr)
@@ -711,7 +790,7 @@ cudaError_t launch_cholesky(int cplx, int N, int n_mat, double* mats, long bstri
 int cholesky_launches(int N, int n_mat, int mode) {
   if (n_mat <= 0) return 0;
   if (N <= SMALL_N) return 1;
-  return (mode != 0 ? 2 : 1) + 2 * ((N - 1) / CB);
+  return (mode != 0 ? 2 : 1) + 2 * ((N - 1) / (mode == 2 && panel32(N, n_mat) ? 32 : 16));
 }
 
 cudaError_t launch_cholesky_ragged(int cplx, const CholTask* tasks, const CholTask* host, int n_tasks, cudaStream_t s,
@@ -746,11 +825,20 @@ namespace {
 template <bool C>
 cudaError_t trinv_run(int N, int n_q, const double* L, double* X, cudaStream_t s) {
   const int nt = (N + CB - 1) / CB;
+  const long sms = device_sm_count();
   trinv_diag_kernel<C><<<n_q * nt, 128, 0, s>>>(N, L, X);
   for (int sz = CB; sz < N; sz *= 2) {
-    const int tiles = (sz / CB) * (sz / CB), pairs = (N - sz + 2 * sz - 1) / (2 * sz);
-    trinv_join_kernel<C, 0><<<n_q * pairs * tiles, 256, 0, s>>>(N, sz, L, X, tiles, pairs);
-    trinv_join_kernel<C, 1><<<n_q * pairs * tiles, 256, 0, s>>>(N, sz, L, X, tiles, pairs);
+    const int pairs = (N - sz + 2 * sz - 1) / (2 * sz);
+    // 16 x 16 tiles (a quarter of the FP64 work each, the same sums) while 32 x 32 ones leave SMs idle
+    if ((long)n_q * pairs * (sz / 32) * (sz / 32) >= 2 * sms) {
+      const int tiles = (sz / 32) * (sz / 32);
+      trinv_join_kernel<C, 0, 2><<<n_q * pairs * tiles, 256, 0, s>>>(N, sz, L, X, tiles, pairs);
+      trinv_join_kernel<C, 1, 2><<<n_q * pairs * tiles, 256, 0, s>>>(N, sz, L, X, tiles, pairs);
+    } else {
+      const int tiles = (sz / 16) * (sz / 16);
+      trinv_join_kernel<C, 0, 1><<<n_q * pairs * tiles, 256, 0, s>>>(N, sz, L, X, tiles, pairs);
+      trinv_join_kernel<C, 1, 1><<<n_q * pairs * tiles, 256, 0, s>>>(N, sz, L, X, tiles, pairs);
+    }
   }
   if (N > CB) clear_upper_kernel<C><<<n_q * N, 256, 0, s>>>(N, X);
   return cudaGetLastError();

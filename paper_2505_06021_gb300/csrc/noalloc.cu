@@ -11,8 +11,8 @@
 // calls.
 //
 // Limits: n_aux <= RPA_NOALLOC_MAX_NAUX (384).  The array holds three
-// n_aux x n_aux complex128 matrices (the Cholesky factor of V, chi L and
-// -L^H chi L for one frequency at a time) plus a status word: 7,078,144 bytes.
+// n_aux x n_aux complex128 matrices (the Cholesky factor of V, then chi L and
+// -L^H chi L of as many frequencies as fit) plus a status word: 7,078,144 bytes.
 //
 // Calls share the array: two calls whose work overlaps on the GPU (different
 // streams, or different host threads, on one device) race and corrupt each
@@ -126,18 +126,25 @@ rpa_status rpa_logdet_noalloc(int is_complex, int n_aux, int n_w, const void* V,
   const size_t es = is_complex ? 16 : 8;
   const size_t NN = (size_t)n_aux * n_aux;
   double* L = reinterpret_cast<double*>(base);
-  double* T = reinterpret_cast<double*>(base + RPA_NOALLOC_MAT_BYTES);
-  double* Y = reinterpret_cast<double*>(base + 2 * RPA_NOALLOC_MAT_BYTES);
+  // as many frequencies at a time as the scratch holds chi L and -L^H chi L of
+  // (1 at n_aux 384, 4 at 201, 53 at 64): a factorisation's panels are serial, so
+  // frequencies side by side cost little more than one (12 of n_aux 201: 9.4 ms
+  // one by one)
+  const size_t mat = (es * NN + 255) & ~(size_t)255;
+  const int nbat = (int)((3 * RPA_NOALLOC_MAT_BYTES - mat) / (2 * mat));
+  double* T = reinterpret_cast<double*>(base + mat);
+  double* Y = reinterpret_cast<double*>(base + mat * (size_t)(1 + nbat));
   int* status = reinterpret_cast<int*>(base + 3 * RPA_NOALLOC_MAT_BYTES);
   cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(L, V, es * NN, cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess)
     e = rpa::launch_cholesky(is_complex, n_aux, 1, L, (long)(NN * (es / 8)), 1, nullptr, status, 1 << 29, s);
   const double* chib = static_cast<const double*>(chi);
-  for (int w = 0; w < n_w && e == cudaSuccess; ++w) {
-    e = rpa::launch_sandwich(is_complex, n_aux, 1, 1, chib + (size_t)w * NN * (es / 8), L, T, Y, s);
+  for (int w = 0; w < n_w && e == cudaSuccess; w += nbat) {
+    const int nb = n_w - w < nbat ? n_w - w : nbat;
+    e = rpa::launch_sandwich(is_complex, n_aux, nb, nb, chib + (size_t)w * NN * (es / 8), L, T, Y, s);
     if (e == cudaSuccess)
-      e = rpa::launch_cholesky(is_complex, n_aux, 1, Y, (long)(NN * (es / 8)), 0, out + 2 * w, status, w, s);
+      e = rpa::launch_cholesky(is_complex, n_aux, nb, Y, (long)(NN * (es / 8)), 0, out + 2 * w, status, w, s);
   }
   int st = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, s);
