@@ -314,7 +314,7 @@ rpa_status ao_enqueue_half(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPl
       const G64Op A = op_of(c, 0, R, p.n_bas, pl, pl + g.a + g.b);
       G64Src sa = src_of(0, 1, R, p.n_bas, p.S, nb);  // conjugated: the product conjugates its left side
       for (int b = 0; b < nb; ++b) sa.tab[b] = Ps[b] + (long)r0 * cs;
-      CKA(g64_slice(c, 0, sa, A, flag, s));
+      CKA(g64_slice(c, 0, sa, A, flag, 0, s));
       nl += 2;
       for (int side = 0; side < 2; ++side) {
         const int n0 = side ? j->n_occ : 0, nc = side ? j->n_virt : j->n_occ;
@@ -339,9 +339,9 @@ rpa_status ao_enqueue_half(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPl
         }
         if (sb.nb == 0) continue;
         const G64Op B = op_of(c, 1, nc, p.n_bas, pl + g.a, pl + g.a + g.b + g.e);
-        CKA(g64_slice(c, 1, sb, B, flag, s));
+        CKA(g64_slice(c, 1, sb, B, flag, 0, s));
         nl += 2;
-        CKA(g64_product(c, A, B, G64Index{ia.data(), nullptr, 1, 1}, o, sb.nb, 0, nullptr, 0, nullptr, status, &nl, s));
+        CKA(g64_product(c, A, B, G64Index{ia.data(), nullptr, 1, 1}, o, sb.nb, 0, nullptr, 0, flag, 0, status, &nl, s));
       }
     }
     n += (int)nl;
@@ -446,13 +446,13 @@ rpa_status ao_enqueue_assemble(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
           o2.C = gc * j->n_occ;
           o2.add = 1;
           const G64Op A1 = op_of(c, 0, a1.R, t.nb, pl, ea), B1 = op_of(c, 1, b1.R, t.nb, pl + g.a, eb);
-          CKA(g64_slice(c, 0, a1, A1, flag, s));
-          CKA(g64_slice(c, 1, b1, B1, flag, s));
-          CKA(g64_product(c, A1, B1, G64Index{nullptr, nullptr, 1, 1}, o1, np, 0, nullptr, 0, nullptr, status, &nl, s));
+          CKA(g64_slice(c, 0, a1, A1, flag, 0, s));
+          CKA(g64_slice(c, 1, b1, B1, flag, 0, s));
+          CKA(g64_product(c, A1, B1, G64Index{nullptr, nullptr, 1, 1}, o1, np, 0, nullptr, 0, flag, 0, status, &nl, s));
           const G64Op A2 = op_of(c, 0, a2.R, t.nb, pl, ea), B2 = op_of(c, 1, b2.R, t.nb, pl + g.a, eb);
-          CKA(g64_slice(c, 0, a2, A2, flag, s));
-          CKA(g64_slice(c, 1, b2, B2, flag, s));
-          CKA(g64_product(c, A2, B2, G64Index{nullptr, nullptr, 1, 1}, o2, np, 0, nullptr, 0, nullptr, status, &nl, s));
+          CKA(g64_slice(c, 0, a2, A2, flag, 0, s));
+          CKA(g64_slice(c, 1, b2, B2, flag, 0, s));
+          CKA(g64_product(c, A2, B2, G64Index{nullptr, nullptr, 1, 1}, o2, np, 0, nullptr, 0, flag, 0, status, &nl, s));
           nl += 8;
         }
     }

@@ -82,10 +82,16 @@ std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_
     jp.L = plan_layout(&jobs[i], jobs[i].n_q, n_slices, 0, false);
     jp.mixed = 0;
     jp.g64 = 0;
+    jp.tail = 0;
+    if (g64) {
+      // the tails run side by side, each with planes of its own
+      const size_t m = a1k(tail_region_bytes(&jobs[i], jobs[i].n_q));
+      if (m && a1k(jp.L.total) + m + 2048 <= budget / 2) jp.tail = m;
+    }
     if (g64 && jobs[i].prec == RPA_PREC_FP64) {
       BatchGeom ga = geom_q(jobs[i]);
       ga.n_qb = jobs[i].n_q;
-      if (chi0_g64_use(ga) && a1k(jp.L.total) + chi0_g64_bytes(ga) + 2048 <= budget) jp.g64 = a1k(chi0_g64_bytes(ga));
+      if (chi0_g64_use(ga) && a1k(jp.L.total) + jp.tail + chi0_g64_bytes(ga) + 2048 <= budget) jp.g64 = a1k(chi0_g64_bytes(ga));
     }
     if (jobs[i].prec == RPA_PREC_MIXED) {
       const size_t per_q = a1k(mixed_workspace_bytes(geom_q(jobs[i]), n_slices, kBatchSliceCap));
@@ -105,7 +111,7 @@ std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_
     size_t fp = 0, mx = 0, mg = 0;  // mg: the FP64 jobs' chi0 run one after another before the mixed ones'
     while (g.j1 < n) {
       const JobPlan& jp = p->jobs[g.j1];
-      const size_t f2 = fp + a1k(jp.L.total), m2 = mx + jp.mixed, g2 = std::max(mg, jp.g64);
+      const size_t f2 = fp + a1k(jp.L.total) + jp.tail, m2 = mx + jp.mixed, g2 = std::max(mg, jp.g64);
       if (g.j1 > g.j0 && f2 + std::max(m2, g2) + 1024 > budget) break;
       p->jobs[g.j1].ws_off = fp;
       fp = f2;
@@ -206,6 +212,10 @@ rpa_status batch_enqueue(rpa_ctx* ctx, SideStreams& bc, const Plan& p, const rpa
   for (const Group& g : p.groups) {
     for (int i = g.j0; i < g.j1; ++i) {
       B[i] = carve(ws + p.jobs[i].ws_off, &jobs[i], p.jobs[i].L);
+      if (p.jobs[i].tail) {
+        B[i].tail = ws + p.jobs[i].ws_off + a1k(p.jobs[i].L.total);
+        B[i].tail_bytes = p.jobs[i].tail;
+      }
       if (rpa_status st = enqueue_table_copies(ctx, &jobs[i], B[i], pin + p.jobs[i].tab_off, s)) return st;
       if (rpa_status st = stage_dtab(ctx, pex, &jobs[i], B[i], 0, jobs[i].n_q, jobs[i].eps_occ,
                                      jobs[i].eps_virt, s))

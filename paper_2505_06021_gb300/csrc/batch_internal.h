@@ -20,6 +20,7 @@ struct JobPlan {
   size_t tab_off;  // pinned tables
   size_t res_off;  // pinned results: [status | pad to 64 | Ec | eps | parts]
   size_t mixed;    // mixed-path workspace of all its q
+  size_t tail;     // tail products on the tensor cores, after L.total (0: the FP64 kernels)
   size_t g64;      // FP64 job: chi0 workspace on the tensor cores (0: the FP64 kernel)
 };
 

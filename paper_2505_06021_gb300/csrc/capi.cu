@@ -245,6 +245,14 @@ static size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 // Workspace cap of the synchronous calls (the serving lanes use a smaller one).
 size_t sync_ws_cap(rpa_ctx* ctx) { return std::min<size_t>(ctx->cap, (size_t)192 << 30); }
 
+size_t tail_region_bytes(const rpa_job* j, int nq) {
+  // the sandwich of an FP64 job (per q and frequency), the Gram product of the
+  // inverse form otherwise (per q)
+  const bool f64 = j->prec == RPA_PREC_FP64;
+  if (!tail_g64_use(j->is_complex, j->n_aux, f64 ? j->n_w : nq)) return 0;
+  return al(tail_g64_bytes(j->is_complex, j->n_aux, f64 ? nq * j->n_w : nq));
+}
+
 Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt, const BinJob* bj,
                    bool g64) {
   Layout L{};
@@ -285,6 +293,13 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
     const size_t m = al(ao_g64_plan(j, ao_plan(j, qb)).bytes);
     if (L.total + m <= ws_cap) {
       L.aog = m;
+      L.total += m;
+    }
+  }
+  if (g64) {
+    const size_t m = tail_region_bytes(j, qt);
+    if (L.total + m <= ws_cap) {
+      L.tail = m;
       L.total += m;
     }
   }
@@ -438,6 +453,9 @@ Bufs carve(void* ws, const rpa_job* j, const Layout& L) {
   b.binmeta = L.binmeta ? p : nullptr;
   p += L.binmeta;
   b.aog = L.aog ? p : nullptr;
+  p += L.aog;
+  b.tail = L.tail ? p : nullptr;
+  b.tail_bytes = L.tail;
   return b;
 }
 
@@ -536,9 +554,16 @@ static rpa_status vside_factor(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
   if (b.Vc) {
     // inverse form: -V^-1 per q (X = L^-1 in T's storage, then -(X^H X) over L)
     prof_begin(ctx, pex, s);
-    CK(launch_vinv(j->is_complex, j->n_aux, nq, b.L, b.T, b.L, s));
-    prof_end(ctx, pex, s, RPA_K_VFACTOR, trinv_launches(j->n_aux) + 1);
-    ctx->launches += trinv_launches(j->n_aux) + 1;
+    uint64_t nl = trinv_launches(j->n_aux);
+    CK(launch_trinv(j->is_complex, j->n_aux, nq, b.L, b.T, s));
+    if (b.tail) {
+      CK(launch_gram_g64(j->is_complex, j->n_aux, nq, b.T, b.L, b.tail, b.tail_bytes, b.status, &nl, s));
+    } else {
+      CK(launch_gram(j->is_complex, j->n_aux, nq, b.T, b.L, s));
+      ++nl;
+    }
+    prof_end(ctx, pex, s, RPA_K_VFACTOR, (int)nl);
+    ctx->launches += nl;
   }
   return RPA_OK;
 }
@@ -547,6 +572,14 @@ rpa_status stage_vside(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const Bufs& b,
                        const void* const* Vdev, cudaStream_t s) {
   if (rpa_status st = vside_copy(ctx, j, b, 0, nq, Vdev, s)) return st;
   return vside_factor(ctx, pex, j, b, q0, nq, s);
+}
+
+// Y = -(L^H chi L), lower triangles, of n matrices (n_w per q), T as scratch.
+static cudaError_t sandwich(int cplx, int N, int n, int n_w, const Bufs& b, const double* chi, double* Y, uint64_t* nl,
+                            cudaStream_t s) {
+  if (b.tail) return launch_sandwich_g64(cplx, N, n, n_w, chi, b.L, b.T, Y, b.tail, b.tail_bytes, b.status, nl, s);
+  *nl += 2;
+  return launch_sandwich(cplx, N, n, n_w, chi, b.L, b.T, Y, s);
 }
 
 // Log-det of every (q, w), q in [q0, q0+nq) held in slots 0..nq-1 of chi, L
@@ -567,9 +600,10 @@ static rpa_status stage_logdet(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
   }
   // Y = -(L^H chi L) (lower triangle), overwriting chi's storage
   prof_begin(ctx, pex, s);
-  CK(launch_sandwich(j->is_complex, j->n_aux, nq * j->n_w, j->n_w, b.chi, b.L, b.T, b.chi, s));
-  prof_end(ctx, pex, s, RPA_K_SANDWICH, 2);
-  ctx->launches += 2;
+  uint64_t nl = 0;
+  CK(sandwich(j->is_complex, j->n_aux, nq * j->n_w, j->n_w, b, b.chi, b.chi, &nl, s));
+  prof_end(ctx, pex, s, RPA_K_SANDWICH, (int)nl);
+  ctx->launches += nl;
   // 1 - Pi' = 1 + Y: Cholesky, ln det, Tr
   prof_begin(ctx, pex, s);
   CK(launch_cholesky(j->is_complex, j->n_aux, nq * j->n_w, b.chi, mstride, 0, b.parts + (size_t)2 * q0 * j->n_w,
@@ -1105,7 +1139,8 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   cudaStream_t s = (cudaStream_t)stream;
   rpa_job j1 = *job;
   j1.prec = RPA_PREC_FP64;
-  Layout L = plan_layout(&j1, 1, ctx->n_slices, sync_ws_cap(ctx), true);
+  j1.ao = nullptr;  // only the tail's buffers are used
+  Layout L = plan_layout(&j1, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, nullptr, true);
   if (!ex.ensure_ws(L.total)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
     return RPA_E_NOMEM;
@@ -1121,13 +1156,14 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   const int nv = cholesky_launches(job->n_aux, 1, 1), nd = cholesky_launches(job->n_aux, job->n_w, 0);
   prof_end(ctx, &ex, s, RPA_K_VFACTOR, nv);
   prof_begin(ctx, &ex, s);
-  CK(launch_sandwich(job->is_complex, job->n_aux, job->n_w, job->n_w, (const double*)chi, b.L, b.T, b.chi, s));
-  prof_end(ctx, &ex, s, RPA_K_SANDWICH, 2);
+  uint64_t nsw = 0;
+  CK(sandwich(job->is_complex, job->n_aux, job->n_w, job->n_w, b, (const double*)chi, b.chi, &nsw, s));
+  prof_end(ctx, &ex, s, RPA_K_SANDWICH, (int)nsw);
   prof_begin(ctx, &ex, s);
   CK(launch_cholesky(job->is_complex, job->n_aux, job->n_w, b.chi, (long)(NN * (es / 8)), 0, b.parts, b.status, 0,
                      s));
   prof_end(ctx, &ex, s, RPA_K_LOGDET, nd);
-  ctx->launches += nv + 2 + nd;
+  ctx->launches += nv + nsw + nd;
   if (!ex.hres.reserve(64 + sizeof(double) * 2 * job->n_w)) return RPA_E_NOMEM;
   CK(cudaMemcpyAsync(ex.results(), b.parts, sizeof(double) * 2 * job->n_w, cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&ex.status_word(), b.status, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1137,6 +1173,7 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   const int sw = ex.status_word();
   if (sw) {
     const int code = sw - 1;
+    if (code >= (1 << 30)) return decode_status(ctx, sw, job->n_w);
     if (code >= (1 << 29))
       ctx_set_error(ctx, "V(q=%d) is not positive definite", q);
     else

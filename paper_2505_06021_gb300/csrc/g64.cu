@@ -17,10 +17,13 @@
 // Error: the dropped levels and the rounding of F, about 2^-56 max|a| max|b|
 // sqrt(K) per output, against 2^-53 sqrt(K) (partial sums) for a chain of
 // DFMA.  Emulated on Gaussian rows: 1.3e-16 against 3.2e-16 (norm, relative)
-// for K = 128, 1.1e-16 against 2.0e-15 for K = 4096.  The split has an absolute
-// error per row, so rows whose entries differ by so much that this would exceed the
-// DFMA chain's are flagged (row_exponent) and the callers keep the FP64
-// kernels' result.
+// for K = 128, 1.1e-16 against 2.0e-15 for K = 4096.  The dropped levels scale
+// with the rows' largest entries, so where one stands far out of its row's root
+// mean square (row_flags), the seven pairs of level 8 are multiplied too; the
+// error left is the rounding of F, 2^-56 (max|a| |b| + |a| max|b|).  Rows whose
+// typical entry lies so far below the largest that even this could exceed the
+// DFMA chain's error, and rows with an infinity or NaN or outside 2^+-60, are
+// flagged, and the callers keep the FP64 kernels' result.
 //
 // Tile: 128 rows x 64 real columns.  Complex data is embedded as real rows
 // X = (re_0, im_0, ...) on the left and X over Y = (im_0, -re_0, ...) on the
@@ -85,13 +88,15 @@ __device__ __forceinline__ long long fix55_mul(unsigned long long cb, unsigned l
 constexpr unsigned long long DIGIT_BIAS = 64ull | 64ull << 7 | 64ull << 14 | 64ull << 21 | 64ull << 28 | 64ull << 35 |
                                           64ull << 42 | 64ull << 49;
 
-// Digit of plane P of G = F + DIGIT_BIAS as FP32 bits (exact, |d| <= 64).
+// Digit d of plane P of G = F + DIGIT_BIAS as the FP32 bits of d 2^(-7 P) (exact,
+// |d| <= 64).
 template <int P>
 __device__ __forceinline__ uint32_t digit_bits(unsigned long long G) {
   constexpr int s = 7 * (7 - P);
   const uint32_t v = (uint32_t)(G >> s);
   const uint32_t f = (P == 0 ? v : (v & 127u)) | 0x4B000000u;
-  return __float_as_uint(__uint_as_float(f) - 8388672.0f);
+  constexpr float sc = 1.0f / (float)(1ull << (7 * P));
+  return __float_as_uint(fmaf(__uint_as_float(f), sc, -8388672.0f * sc));
 }
 
 // Digit planes of 16 consecutive real k of one row: G in order.  Left: row
@@ -132,68 +137,91 @@ __device__ __forceinline__ uint32_t abs_bits32(unsigned long long b) {
   return __funnelshift_l(lo, hi, 3) - (896u << 23);
 }
 
-// Exponent of a row from its largest |x| (FP32, truncated) and sum of squares;
-// raises *flag where the split could be less exact than DFMA: (max / rms)^2
-// above `spread` sqrt(K / 128), or values outside 2^+-60.
-constexpr float SPREAD = 60.f;         // as given
-constexpr float SPREAD_WEIGHTED = 160.f;  // times the smooth frequency weights (a factor 2 to 3 of spread of their own)
-constexpr float TINY = 8.7e-19f;       // 2^-60
-__device__ __forceinline__ int row_exponent(uint32_t mbits, float ss, float K, float spread, int* flag) {
-  if (mbits == 0) return E_ZERO;
-  const float m = __uint_as_float(mbits);
-  if (mbits == 0xffffffffu || !(m < 1.1e18f) || !(m > TINY) || !(m * m <= spread * sqrtf(K * (1.0f / 128.0f)) * ss / K)) {
-    atomicOr(flag, 1);
-    if (mbits == 0xffffffffu) return 1100;
+// What decides a row's exponent and its flags: largest |x| (FP32 bits, truncated),
+// sum of squares, sum of the FP32 exponents and count of the nonzero entries.
+struct RowStat {
+  uint32_t m = 0;
+  float ss = 0.f;
+  int es = 0, nz = 0;
+  __device__ __forceinline__ void add(uint32_t v) {
+    m = max(m, v);
+    ss = fmaf(__uint_as_float(v), __uint_as_float(v), ss);
+    es += (int)(v >> 23);
+    nz += v != 0;
   }
-  return (int)(__float_as_uint(m * 1.000001f) >> 23) - 126;
+  __device__ __forceinline__ void join(const RowStat& o) {
+    m = max(m, o.m);
+    ss += o.ss;
+    es += o.es;
+    nz += o.nz;
+  }
+  __device__ __forceinline__ void warp_join() {
+    m = __reduce_max_sync(0xffffffffu, m);
+    es = __reduce_add_sync(0xffffffffu, es);
+    nz = __reduce_add_sync(0xffffffffu, nz);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  }
+};
+
+// Bit 0 (FP64 kernels): an infinity, a NaN, values outside 2^+-60, or a mean
+// binary exponent more than 1.5 + log2(K) / 2 below the largest entry's: then
+// 2^-56 max|a| |b| can exceed the DFMA chain's error, about 2^-53 sqrt(K) / 5
+// of |a| |b| for typical entries.  (Gaussian rows: 3 at K = 128, 3.2 at 34560.
+// Sums of less than 64 terms, the short ends of triangular operands: 8, as
+// their few exponents scatter.)
+// Bit 1 (level 8 too): (max / rms)^2 above `spread` sqrt(K / 128), where the
+// dropped levels could exceed it.
+constexpr float SPREAD = 40.f;            // as given: Gaussian rows reach 20
+constexpr float SPREAD_WEIGHTED = 100.f;  // times the smooth frequency weights (a factor 2 of spread of their own)
+constexpr float TINY = 8.7e-19f;          // 2^-60
+__device__ __forceinline__ int row_flags(const RowStat& r, float spread) {
+  const float m = __uint_as_float(r.m), n = (float)max(r.nz, 1);
+  if (r.m >= 0x7f800000u || !(m < 1.1e18f) || !(m > TINY)) return 1;
+  if ((float)(r.m >> 23) - (float)r.es / n > (n < 64.f ? 8.f : 1.5f + 0.5f * log2f(n))) return 1;
+  return m * m <= spread * sqrtf(n * (1.0f / 128.0f)) * r.ss / n ? 0 : 2;
+}
+// The row's exponent; raises its flags.
+__device__ __forceinline__ int row_exponent(const RowStat& r, float spread, int* flag, int nflag = 1) {
+  if (r.m == 0) return E_ZERO;
+  if (const int bits = row_flags(r, spread))
+    for (int i = 0; i < nflag; ++i) atomicOr(flag + i, bits);
+  if (r.m >= 0x7f800000u) return 1100;
+  return (int)(__float_as_uint(__uint_as_float(r.m) * 1.000001f) >> 23) - 126;
 }
 
-// Largest |x| and sum of squares of every row of every matrix: one warp per
+// Exponent and flags of every row of every matrix: one warp per
 // row (by rows), or 32 rows per CTA with eight warps along k (by columns).
 template <bool C>
 __global__ void __launch_bounds__(256) g64_exp_kernel(const __grid_constant__ G64Src src, int Rpad, int* __restrict__ e,
-                                                      int* __restrict__ flag) {
-  __shared__ uint32_t sm[8][32];
-  __shared__ float sq[8][32];
+                                                      int* __restrict__ flag, int frep) {
+  __shared__ RowStat sr[8][32];
   const int rows = src.by_rows ? 8 : 32, nblk = (Rpad + rows - 1) / rows;
   const int b = blockIdx.x / nblk, r0 = (blockIdx.x % nblk) * rows;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double* p = src_ptr<C>(src, b);
   const int r = r0 + (src.by_rows ? warp : lane);
-  uint32_t m = 0;
-  float ss = 0.f;
+  RowStat st;
   if (r < src.R) {
     const int k0 = src.by_rows ? lane : warp, dk = src.by_rows ? 32 : 8;
     for (int k = k0; k < src.K; k += dk) {
+      if (src.no_diag && k == r) continue;
       const Elem<C> x = ld_elem<C>(p, src.by_rows ? (long)r * src.ld + k : (long)k * src.ld + r);
-      const uint32_t v = abs_bits32((unsigned long long)__double_as_longlong(x.re));
-      m = max(m, v);
-      ss = fmaf(__uint_as_float(v), __uint_as_float(v), ss);
-      if constexpr (C) {
-        const uint32_t w = abs_bits32((unsigned long long)__double_as_longlong(x.im));
-        m = max(m, w);
-        ss = fmaf(__uint_as_float(w), __uint_as_float(w), ss);
-      }
+      st.add(abs_bits32((unsigned long long)__double_as_longlong(x.re)));
+      if constexpr (C) st.add(abs_bits32((unsigned long long)__double_as_longlong(x.im)));
     }
   }
   if (src.by_rows) {
-    m = __reduce_max_sync(0xffffffffu, m);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    st.warp_join();
     if (lane != 0) return;
   } else {
-    sm[warp][lane] = m;
-    sq[warp][lane] = ss;
+    sr[warp][lane] = st;
     __syncthreads();
     if (warp != 0) return;
-    ss = 0.f;
-    for (int w = 0; w < 8; ++w) {
-      m = max(m, sm[w][lane]);
-      ss += sq[w][lane];
-    }
+    for (int w = 1; w < 8; ++w) st.join(sr[w][lane]);
   }
   if (r < Rpad)
-    e[(long)b * Rpad + r] = r < src.R ? row_exponent(m, ss, (float)src.K * (C ? 2.f : 1.f), SPREAD, flag) : E_ZERO;
+    e[(long)b * Rpad + r] = r < src.R ? row_exponent(st, SPREAD, flag + (long)b * frep, max(frep, 1)) : E_ZERO;
 }
 
 // One thread per (matrix, row, K-block); consecutive threads take consecutive
@@ -214,7 +242,7 @@ __global__ void __launch_bounds__(256) g64_slice_kernel(const __grid_constant__ 
     for (int v = 0; v < kpb; ++v) {
       const int k = kb * kpb + v;
       Elem<C> x = zero_elem<C>();
-      if (r < src.R && k < src.K) x = ld_elem<C>(p, src.by_rows ? (long)r * src.ld + k : (long)k * src.ld + r);
+      if (r < src.R && k < src.K && !(src.no_diag && k == r)) x = ld_elem<C>(p, src.by_rows ? (long)r * src.ld + k : (long)k * src.ld + r);
       if constexpr (C) {
         if (src.conj) x.im = -x.im;
         G[2 * v] = (unsigned long long)fix55(x.re, e) + DIGIT_BIAS;
@@ -239,9 +267,11 @@ struct G64Params {
   int nb, nI, nJ, tri, n_tiles, n_split, cps;  // cps: chunks per split
   int kmode, n_items;
   longlong2* part;
-  const int* skip;  // a nonzero word: nothing to do
+  const int* flag;  // null, the operands' one flag word, or (per_b) a word per matrix
+  int per_b;
   int* status;
   G64Out out;
+  G64Diag diag;
 };
 
 // One MMA: left plane i, right planes j .. j + n - 1, accumulators g .. g + n - 1.
@@ -342,13 +372,26 @@ __device__ __forceinline__ double to_f64(long long hi, long long lo, int ex) {
   return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
 }
 
-// Writes one thread's 16 complex (32 real) outputs of row r: columns c0 + u.
 template <bool C>
+__device__ __forceinline__ Elem<C> src_at(const G64Src& s, int b, int r, int k) {
+  Elem<C> x = ld_elem<C>(s.base + b * s.stride * (C ? 2 : 1), s.by_rows ? (long)r * s.ld + k : (long)k * s.ld + r);
+  if (s.conj) x = conj_e<C>(x);
+  return x;
+}
+// v += conj(A(r, k)) B(c, k) for k = r and k = c.
+template <bool C>
+__device__ __forceinline__ void add_diag(const G64Diag& d, int ia, int ib, int r, int c, Elem<C>& v) {
+  mac<C>(v, conj_e<C>(src_at<C>(d.A, ia, r, r)), src_at<C>(d.B, ib, c, r));
+  if (r != c) mac<C>(v, conj_e<C>(src_at<C>(d.A, ia, r, c)), src_at<C>(d.B, ib, c, c));
+}
+
+// Writes one thread's 16 complex (32 real) outputs of row r: columns c0 + u.
+template <bool C, bool DIAG>
 __device__ __forceinline__ void g_store(const G64Params& p, const GItem& it, int row, int half, const long long (&hi)[32],
                                         const long long (&lo)[32]) {
   const G64Out& o = p.out;
   const int r = it.I * 128 + row;
-  if (r >= o.R) return;
+  if (r >= o.R || (p.per_b && (p.flag[it.b] & 1))) return;
   double* out = o.use_tab ? o.tab[it.b] : o.base + it.b * o.stride * (C ? 2 : 1);
   const int eA = p.eA[(long)it.ia * p.RpA + r];
   const int* eB = p.eB + (long)it.ib * p.RpB;
@@ -363,6 +406,7 @@ __device__ __forceinline__ void g_store(const G64Params& p, const GItem& it, int
     Elem<C> v;
     v.re = to_f64(hi[u], lo[u], ex);
     if constexpr (C) v.im = to_f64(hi[16 + u], lo[16 + u], ex);
+    if constexpr (DIAG) add_diag<C>(p.diag, it.ia, it.ib, r, c, v);
     if (o.neg) {
       v.re = -v.re;
       if constexpr (C) v.im = -v.im;
@@ -382,7 +426,7 @@ __device__ __forceinline__ void g_store(const G64Params& p, const GItem& it, int
 
 // One producer thread (bulk copies), one MMA thread, eight epilogue warps; a
 // persistent CTA per SM.  Epilogue warp w: rows 32 (w & 3) .., column half.
-template <bool C>
+template <bool C, bool DIAG>
 __global__ void __launch_bounds__(G_THREADS, 1) g64_kernel(const __grid_constant__ G64Params p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -393,7 +437,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) g64_kernel(const __grid_constant
   uint64_t* drain = acc_empty + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  if (p.skip && *p.skip) return;  // the same word for every thread
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int ERR = 1 + (1 << 30);
   if (threadIdx.x == 0) {
@@ -458,6 +501,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) g64_kernel(const __grid_constant
       const uint64_t d0 = sdesc(smem_u32(smem));
       for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
         const GItem it = g_item<C>(p, item);
+        const bool more = p.flag && (p.flag[p.per_b ? it.b : 0] & 2);
         for (int c0 = it.kb0; c0 < it.kb1 && ok; c0 += KBC) {
           const int c1 = min(it.kb1, c0 + KBC);
           ok = mbar_wait(acc_empty, acc_phase ^ 1u, abort_flag, p.status, ERR + 22);
@@ -474,6 +518,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) g64_kernel(const __grid_constant
               mma(tmem + 64u * (uint32_t)kG[m].g, da + (uint64_t)((kG[m].i * 128 * KBLK * 2) >> 4),
                   db + (uint64_t)((kG[m].j * 64 * KBLK * 2) >> 4), idesc(64u * (uint32_t)kG[m].n),
                   !(kb == c0 && (m == 0 || m == 4)));
+            if (more) {  // level 8, into level 7's accumulator
+#pragma unroll
+              for (int i = 1; i < NP; ++i)
+                mma(tmem + 64u * 7u, da + (uint64_t)((i * 128 * KBLK * 2) >> 4),
+                    db + (uint64_t)(((8 - i) * 64 * KBLK * 2) >> 4), idesc(64u), true);
+            }
             mma_commit(&empty[stage]);
             if (++stage == G_STAGES) {
               stage = 0;
@@ -516,11 +566,13 @@ __global__ void __launch_bounds__(G_THREADS, 1) g64_kernel(const __grid_constant
           tmem_wait_ld();
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
-            long long h = (long long)__float2int_rn(v[3][w]), q = (long long)__float2int_rn(v[7][w]);
+            // level l holds its integer sum times 2^(-7 l)
+            long long h = 0, q = 0;
 #pragma unroll
-            for (int l = 0; l < 3; ++l) {
-              h += (long long)__float2int_rn(v[l][w]) * (long long)(1 << (7 * (3 - l)));
-              q += (long long)__float2int_rn(v[4 + l][w]) * (long long)(1 << (7 * (3 - l)));
+            for (int l = 0; l < 4; ++l) {
+              h += (long long)__float2int_rn(v[l][w] * (float)(1ull << (7 * l))) * (long long)(1 << (7 * (3 - l)));
+              q += (long long)__float2int_rn(v[4 + l][w] * (float)(1ull << (7 * (4 + l)))) *
+                   (long long)(1 << (7 * (3 - l)));
             }
             hi[u + w] += h;
             lo[u + w] += q;
@@ -532,7 +584,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) g64_kernel(const __grid_constant
       }
       if (!ok) break;
       if (p.n_split == 1) {
-        g_store<C>(p, it, row, half, hi, lo);
+        g_store<C, DIAG>(p, it, row, half, hi, lo);
       } else {
         longlong2* d = p.part + (long)item * (32 * 256) + (threadIdx.x - 64);
 #pragma unroll
@@ -551,7 +603,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) g64_kernel(const __grid_constant
 // Sum of the split-K partials (exact) and the store, one CTA per tile.
 template <bool C>
 __global__ void __launch_bounds__(256) g64_reduce_kernel(const __grid_constant__ G64Params p) {
-  if (p.skip && *p.skip) return;
   const int per = p.nb * p.n_tiles;
   const GItem it = g_item<C>(p, blockIdx.x);
   long long hi[32], lo[32];
@@ -567,7 +618,7 @@ __global__ void __launch_bounds__(256) g64_reduce_kernel(const __grid_constant__
     }
   }
   const int warp = (threadIdx.x >> 5) + 2;
-  g_store<C>(p, it, (warp & 3) * 32 + (threadIdx.x & 31), (warp - 2) >> 2, hi, lo);
+  g_store<C, false>(p, it, (warp & 3) * 32 + (threadIdx.x & 31), (warp - 2) >> 2, hi, lo);
 }
 
 cudaError_t g64_attr() {
@@ -578,9 +629,9 @@ cudaError_t g64_attr() {
   if (dev < 0 || dev >= MAX_DEVICES) dev = 0;
   std::lock_guard<std::mutex> lk(mu);
   if (done[dev]) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(g64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(g64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM);
+  cudaError_t e = cudaSuccess;
+  for (auto* k : {g64_kernel<true, false>, g64_kernel<false, false>, g64_kernel<true, true>, g64_kernel<false, true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM);
   done[dev] = e == cudaSuccess;
   return e;
 }
@@ -601,18 +652,18 @@ size_t g64_plane_bytes(int cplx, int role, int R, int K, int nb) {
   return blocks * g64_nkb(cplx, K) * (role == 0 ? A_BLOCK : B_BLOCK) * nb;
 }
 
-cudaError_t g64_slice(int cplx, int role, const G64Src& src, const G64Op& op, int* flag, cudaStream_t s) {
+cudaError_t g64_slice(int cplx, int role, const G64Src& src, const G64Op& op, int* flag, int frep, cudaStream_t s) {
   const int rows = src.by_rows ? 8 : 32;
   const unsigned gb = (unsigned)((long)src.nb * ((op.Rpad + rows - 1) / rows));
   const unsigned gs = grid_for((long)op.Rpad * op.n_kb * src.nb, 16);
   if (cplx) {
-    g64_exp_kernel<true><<<gb, 256, 0, s>>>(src, op.Rpad, op.e, flag);
+    g64_exp_kernel<true><<<gb, 256, 0, s>>>(src, op.Rpad, op.e, flag, frep);
     if (role == 0)
       g64_slice_kernel<true, 0><<<gs, 256, 0, s>>>(src, op);
     else
       g64_slice_kernel<true, 1><<<gs, 256, 0, s>>>(src, op);
   } else {
-    g64_exp_kernel<false><<<gb, 256, 0, s>>>(src, op.Rpad, op.e, flag);
+    g64_exp_kernel<false><<<gb, 256, 0, s>>>(src, op.Rpad, op.e, flag, frep);
     if (role == 0)
       g64_slice_kernel<false, 0><<<gs, 256, 0, s>>>(src, op);
     else
@@ -622,8 +673,8 @@ cudaError_t g64_slice(int cplx, int role, const G64Src& src, const G64Op& op, in
 }
 
 cudaError_t g64_product(int cplx, const G64Op& A, const G64Op& B, const G64Index& ix, const G64Out& out, int nb,
-                        int kmode, void* part, size_t part_bytes, const int* skip, int* status, uint64_t* n_launch,
-                        cudaStream_t s) {
+                        int kmode, void* part, size_t part_bytes, const int* flag, int per_b, int* status,
+                        uint64_t* n_launch, cudaStream_t s, const G64Diag* diag) {
   if (nb <= 0) return cudaSuccess;
   if (A.n_kb != B.n_kb || ((ix.ta || ix.tb || out.use_tab) && nb > G64_TAB)) return cudaErrorInvalidValue;
   if (cudaError_t e = g64_attr()) return e;
@@ -659,7 +710,7 @@ cudaError_t g64_product(int cplx, const G64Op& A, const G64Op& B, const G64Index
   // its drain as the unit, half a unit per item, one per split for the reduction
   const int chunks = (p.n_kb + KBC - 1) / KBC;
   int ns = 1;
-  if (part && kmode == 0) {
+  if (part && kmode == 0 && !diag) {
     double best = 1e300;
     for (int k = 1; k <= std::min(chunks, 64); ++k) {
       const int cps = (chunks + k - 1) / k, kk = (chunks + cps - 1) / cps;
@@ -679,14 +730,15 @@ cudaError_t g64_product(int cplx, const G64Op& A, const G64Op& B, const G64Index
   p.kmode = kmode;
   p.n_items = (int)(items * ns);
   p.part = (longlong2*)part;
-  p.skip = skip;
+  p.flag = flag;
+  p.per_b = flag && per_b;
   p.status = status;
   p.out = out;
+  if (diag) p.diag = *diag;
   const unsigned grid = (unsigned)std::min<long>(p.n_items, sms);
-  if (cplx)
-    g64_kernel<true><<<grid, G_THREADS, G_SMEM, s>>>(p);
-  else
-    g64_kernel<false><<<grid, G_THREADS, G_SMEM, s>>>(p);
+  auto* kern = diag ? (cplx ? g64_kernel<true, true> : g64_kernel<false, true>)
+                    : (cplx ? g64_kernel<true, false> : g64_kernel<false, false>);
+  kern<<<grid, G_THREADS, G_SMEM, s>>>(p);
   if (n_launch) *n_launch += 1;
   if (ns > 1) {
     if (cplx)
@@ -695,6 +747,153 @@ cudaError_t g64_product(int cplx, const G64Op& A, const G64Op& B, const G64Index
       g64_reduce_kernel<false><<<(unsigned)items, 256, 0, s>>>(p);
     if (n_launch) *n_launch += 1;
   }
+  return cudaGetLastError();
+}
+
+// ------------------------------------------------ products of the tail ----
+
+namespace {
+
+size_t al1k(size_t x) { return (x + 1023) & ~(size_t)1023; }
+
+// Bytes of the planes of one matrix of the sandwich: one left and one right
+// operand per (q, w), and one of L per q (at least as large as its share).
+struct TailBytes {
+  size_t a, b, ea, eb, one;
+};
+TailBytes tail_bytes(int cplx, int N) {
+  TailBytes t;
+  t.a = g64_plane_bytes(cplx, 0, N, N, 1);
+  t.b = g64_plane_bytes(cplx, 1, N, N, 1);
+  t.ea = al1k(sizeof(int) * (size_t)g64_rpad(cplx, 0, N));
+  t.eb = al1k(sizeof(int) * (size_t)g64_rpad(cplx, 1, N));
+  t.one = t.a + t.b + t.ea + t.eb;
+  return t;
+}
+
+// Square matrices at a stride N^2, by rows or columns, without their diagonals.
+G64Src square(const double* base, int N, int nb, int by_rows, int conj) {
+  G64Src s{};
+  s.base = base;
+  s.stride = (long)N * N;
+  s.ld = N;
+  s.by_rows = by_rows;
+  s.conj = conj;
+  s.nb = nb;
+  s.R = s.K = N;
+  s.no_diag = 1;
+  return s;
+}
+
+G64Op square_op(int cplx, int role, int N, char* planes, char* e) {
+  G64Op o{};
+  o.planes = (uint16_t*)planes;
+  o.e = (int*)e;
+  o.stride = (long)(g64_plane_bytes(cplx, role, N, N, 1) / 2);
+  o.Rpad = g64_rpad(cplx, role, N);
+  o.n_kb = g64_nkb(cplx, N);
+  return o;
+}
+
+G64Out square_out(double* base, int N, int neg, int tri) {
+  G64Out o{};
+  o.base = base;
+  o.stride = (long)N * N;
+  o.s0 = N;
+  o.t0 = 1;
+  o.rd = o.cd = 1 << 30;
+  o.R = o.C = N;
+  o.neg = neg;
+  o.tri = tri;
+  return o;
+}
+
+}  // namespace
+
+// Measured: the sandwich of 16 matrices of N = 768 40.6 ms in FP64 (its pipe
+// needs 33), 1.9 ms here; 48 of N = 150 1.69 -> 0.40 ms; V^-1 = X^H X of 16 of N =
+// 512 3.5 -> 0.45 ms.  Small matrices leave the tiles (128 rows) mostly padding; below 2.5e7 complex
+// multiply-adds per q (N = 150, 12 frequencies: 0.42 ms in FP64) the FP64 kernels
+// take little more than the launches.
+bool tail_g64_use(int cplx, int N, int n) {
+  return N >= 128 && (cplx ? 1.0 : 0.25) * N * (double)N * N * n >= 2.5e7;
+}
+
+size_t tail_g64_bytes(int cplx, int N, int n_mat) {
+  const size_t one = tail_bytes(cplx, N).one;
+  return al1k(sizeof(int) * (size_t)n_mat) + std::max(2 * one, std::min<size_t>((size_t)1 << 30, one * (size_t)n_mat));
+}
+
+cudaError_t launch_sandwich_g64(int cplx, int N, int n_batch, int n_w, const double* chi, const double* L, double* T,
+                                double* Y, void* work, size_t work_bytes, int* status, uint64_t* n_launch,
+                                cudaStream_t s) {
+  const TailBytes t = tail_bytes(cplx, N);
+  const long NN = (long)N * N, cs = cplx ? 2 : 1;
+  const size_t fb = al1k(sizeof(int) * (size_t)n_batch);
+  int* flag = (int*)work;
+  char* p = (char*)work + fb;
+  const int room = (int)std::min<size_t>((size_t)n_batch, (work_bytes - fb) / t.one);
+  if (work_bytes < fb + t.one) return cudaErrorInvalidValue;
+  if (cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int) * (size_t)n_batch, s)) return e;
+  uint64_t nl = 0;
+  // passes over whole q, or over some matrices of one
+  for (int b0 = 0; b0 < n_batch;) {
+    const int q = b0 / n_w, nq = std::max(1, std::min(room / n_w, (n_batch - b0) / n_w));
+    const int nb = std::min({room, nq * n_w, (q + nq) * n_w - b0});
+    const int rep = std::min(nb, n_w);                 // matrices of a pass that share an L
+    char *pb = p + t.a * (size_t)nb, *ea = pb + t.b * (size_t)nb, *eb = ea + t.ea * (size_t)nb;
+    const double *X = chi + b0 * NN * cs, *Lq = L + q * NN * cs;
+    double *Tb = T + b0 * NN * cs, *Yb = Y + b0 * NN * cs;
+    const G64Op A = square_op(cplx, 0, N, p, ea), B = square_op(cplx, 1, N, pb, eb);
+    // T = chi L: conj(A)(P, R) = chi[P][R], B(Q, R) = L[R][Q], R >= Q
+    const G64Diag d1{1, square(X, N, nb, 1, 1), square(Lq, N, nq, 0, 0)};
+    if (cudaError_t e = g64_slice(cplx, 0, d1.A, A, flag + b0, 1, s)) return e;
+    if (cudaError_t e = g64_slice(cplx, 1, d1.B, B, flag + b0, rep, s)) return e;
+    if (cudaError_t e = g64_product(cplx, A, B, G64Index{nullptr, nullptr, 1, rep}, square_out(Tb, N, 0, 0), nb, 1,
+                                    nullptr, 0, flag + b0, 1, status, &nl, s, &d1))
+      return e;
+    // Y = -L^H T: A(P, R) = L[R][P], B(Q, R) = T[R][Q], R >= P, lower triangle
+    const G64Diag d2{1, square(Lq, N, nq, 0, 0), square(Tb, N, nb, 0, 0)};
+    if (cudaError_t e = g64_slice(cplx, 0, d2.A, A, flag + b0, rep, s)) return e;
+    if (cudaError_t e = g64_slice(cplx, 1, d2.B, B, flag + b0, 1, s)) return e;
+    // (Y may be chi, which the FP64 kernels need: flagged matrices are not stored)
+    if (cudaError_t e = g64_product(cplx, A, B, G64Index{nullptr, nullptr, rep, 1}, square_out(Yb, N, 1, 2), nb, 2,
+                                    nullptr, 0, flag + b0, 1, status, &nl, s, &d2))
+      return e;
+    if (cudaError_t e = launch_sandwich(cplx, N, nb, rep, X, Lq, Tb, Yb, s, flag + b0)) return e;
+    nl += 10;
+    b0 += nb;
+  }
+  if (n_launch) *n_launch += nl;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gram_g64(int cplx, int N, int n_q, const double* X, double* Wn, void* work, size_t work_bytes,
+                            int* status, uint64_t* n_launch, cudaStream_t s) {
+  const TailBytes t = tail_bytes(cplx, N);
+  const long NN = (long)N * N, cs = cplx ? 2 : 1;
+  const size_t fb = al1k(sizeof(int) * (size_t)n_q);
+  int* flag = (int*)work;
+  char* p = (char*)work + fb;
+  if (work_bytes < fb + t.one) return cudaErrorInvalidValue;
+  const int room = (int)std::min<size_t>((size_t)n_q, (work_bytes - fb) / t.one);
+  if (cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int) * (size_t)n_q, s)) return e;
+  uint64_t nl = 0;
+  for (int q0 = 0; q0 < n_q; q0 += room) {
+    const int nb = std::min(room, n_q - q0);
+    char *pb = p + t.a * (size_t)nb, *ea = pb + t.b * (size_t)nb, *eb = ea + t.ea * (size_t)nb;
+    const G64Op A = square_op(cplx, 0, N, p, ea), B = square_op(cplx, 1, N, pb, eb);
+    const G64Src sx = square(X + q0 * NN * cs, N, nb, 0, 0);
+    if (cudaError_t e = g64_slice(cplx, 0, sx, A, flag + q0, 1, s)) return e;
+    if (cudaError_t e = g64_slice(cplx, 1, sx, B, flag + q0, 1, s)) return e;
+    const G64Diag d{1, sx, sx};
+    if (cudaError_t e = g64_product(cplx, A, B, G64Index{nullptr, nullptr, 1, 1}, square_out(Wn + q0 * NN * cs, N, 1, 2), nb,
+                                    2, nullptr, 0, flag + q0, 1, status, &nl, s, &d))
+      return e;
+    if (cudaError_t e = launch_gram(cplx, N, nb, X + q0 * NN * cs, Wn + q0 * NN * cs, s, flag + q0)) return e;
+    nl += 5;
+  }
+  if (n_launch) *n_launch += nl;
   return cudaGetLastError();
 }
 
@@ -708,27 +907,21 @@ namespace {
 
 constexpr int CHI_W = 8;  // frequencies per pass of the exponent kernel
 
-// Largest |C_Pt| or |C_Pt d_t(w)| and sum of squares over a part of the panel:
+// Statistics of |C_Pt| or |C_Pt d_t(w)| over a part of the panel:
 // one warp per row, the FP32 weights of 256 t staged for the CTA's 8 rows;
 // blockIdx.z = 0: no weight (the right operand), z > 0: frequencies
 // [w0 + 8 (z - 1), ...).  part[slot][kp][P], slot 0 unweighted, 1 + w.
 template <bool C>
 __global__ void __launch_bounds__(256) chi_exp_kernel(int N, int Npad, int n_ov, int n_w, int w0, int G, long t0, long t1,
                                                       const double* const* __restrict__ Cp,
-                                                      const double* __restrict__ dtab, float2* __restrict__ part,
+                                                      const double* __restrict__ dtab, RowStat* __restrict__ part,
                                                       int* __restrict__ flag) {
   __shared__ float ds[CHI_W][256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int P = blockIdx.x * 8 + warp, kp = blockIdx.y, KP = gridDim.y;
   const int z = blockIdx.z, g0 = z == 0 ? 0 : (z - 1) * CHI_W, ng = z == 0 ? 1 : min(CHI_W, G - g0);
   const long len = t1 - t0, a = t0 + len * kp / KP, b = t0 + len * (kp + 1) / KP;
-  uint32_t m[CHI_W];
-  float ss[CHI_W];
-#pragma unroll
-  for (int g = 0; g < CHI_W; ++g) {
-    m[g] = 0;
-    ss[g] = 0.f;
-  }
+  RowStat st[CHI_W];
   for (long tb = a; tb < b; tb += 256) {
     __syncthreads();
     for (int i = threadIdx.x; i < ng * 256; i += 256) {
@@ -761,42 +954,32 @@ __global__ void __launch_bounds__(256) chi_exp_kernel(int N, int Npad, int n_ov,
       for (int g = 0; g < CHI_W; ++g) {
         if (g >= ng) break;
         const float d = ds[g][u];
-        const float pr = xr * d, pi = xi * d;
         // non-negative floats order like their bits; a NaN sorts above all
-        m[g] = max(m[g], max(__float_as_uint(pr) & 0x7fffffffu, __float_as_uint(pi) & 0x7fffffffu));
-        ss[g] = fmaf(pr, pr, fmaf(pi, pi, ss[g]));
+        st[g].add(__float_as_uint(xr * d) & 0x7fffffffu);
+        if constexpr (C) st[g].add(__float_as_uint(xi * d) & 0x7fffffffu);
       }
     }
   }
 #pragma unroll
   for (int g = 0; g < CHI_W; ++g) {
     if (g >= ng) break;
-    const uint32_t mm = __reduce_max_sync(0xffffffffu, m[g]);
-    float s = ss[g];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    st[g].warp_join();
     const int slot = z == 0 ? 0 : 1 + g0 + g;
-    if (lane == 0 && P < Npad) part[((long)slot * KP + kp) * Npad + P] = make_float2(__uint_as_float(mm), s);
+    if (lane == 0 && P < Npad) part[((long)slot * KP + kp) * Npad + P] = st[g];
   }
 }
 
 // Exponents from the parts, in part order: eB[P] (slot 0) and eA[w][P].
 __global__ void __launch_bounds__(256) chi_exp_final_kernel(int N, int NpadA, int NpadB, int Npad, int G, int KP,
-                                                            float K, const float2* __restrict__ part, int* eA, int* eB,
+                                                            const RowStat* __restrict__ part, int* eA, int* eB,
                                                             int* flag) {
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= (G + 1) * Npad) return;
   const int slot = i / Npad, P = i % Npad;
-  uint32_t m = 0;
-  float ss = 0.f;
+  RowStat st;
   if (P < N)
-    for (int kp = 0; kp < KP; ++kp) {
-      const float2 v = part[((long)slot * KP + kp) * Npad + P];
-      m = max(m, __float_as_uint(v.x));
-      ss += v.y;
-    }
-  // products that left the FP32 range (infinity or NaN bits) have no exponent
-  const int e = row_exponent(m >= 0x7f800000u ? 0xffffffffu : m, ss, K, slot ? SPREAD_WEIGHTED : SPREAD, flag);
+    for (int kp = 0; kp < KP; ++kp) st.join(part[((long)slot * KP + kp) * Npad + P]);
+  const int e = row_exponent(st, slot ? SPREAD_WEIGHTED : SPREAD, flag);
   if (slot == 0) {
     if (P < NpadB) eB[P] = e;
   } else if (P < NpadA) {
@@ -900,8 +1083,6 @@ struct ChiPanel {
   long T;        // transitions per panel
   size_t a, b, ea, eb, ep, part, flag, total;
 };
-size_t al1k(size_t x) { return (x + 1023) & ~(size_t)1023; }
-
 // The panel depends on the geometry of one q alone, so the result does not
 // depend on what shares the workspace.
 ChiPanel chi0_panel(const BatchGeom& g) {
@@ -924,7 +1105,7 @@ ChiPanel chi0_panel(const BatchGeom& g) {
   L.b = al1k(g64_plane_bytes(g.cplx, 1, g.n_aux, K, 1));
   L.ea = al1k(sizeof(int) * (size_t)RA * L.G);
   L.eb = al1k(sizeof(int) * (size_t)RB);
-  L.ep = al1k(sizeof(float2) * (size_t)(L.G + 1) * L.KP * std::max(RA, RB));
+  L.ep = al1k(sizeof(RowStat) * (size_t)(L.G + 1) * L.KP * std::max(RA, RB));
   L.flag = al1k(sizeof(int) * (size_t)std::max(1, g.n_qb));
   const long nI = RA / 128, nJ = RB / (g.cplx ? 32 : 64);
   long tiles = 0;
@@ -950,7 +1131,7 @@ cudaError_t chi0_g64_run(const BatchGeom& g, const double* const* Cptrs, const d
   p += L.ea;
   B.e = (int*)p;
   p += L.eb;
-  float2* ep = (float2*)p;
+  RowStat* ep = (RowStat*)p;
   p += L.ep;
   A.Rpad = g64_rpad(C, 0, g.n_aux);
   B.Rpad = g64_rpad(C, 1, g.n_aux);
@@ -971,9 +1152,8 @@ cudaError_t chi0_g64_run(const BatchGeom& g, const double* const* Cptrs, const d
         const int G = std::min(L.G, g.n_w - w0);
         chi_exp_kernel<C><<<dim3((unsigned)((Npad + 7) / 8), (unsigned)L.KP, (unsigned)(1 + (G + CHI_W - 1) / CHI_W)), 256, 0,
                          s>>>(g.n_aux, Npad, g.n_ov, g.n_w, w0, G, t0, t1, Cq, dq, ep, flag + q);
-        chi_exp_final_kernel<<<((G + 1) * Npad + 255) / 256, 256, 0, s>>>(g.n_aux, A.Rpad, B.Rpad, Npad, G, L.KP,
-                                                                         (float)K * (C ? 2.f : 1.f), ep, A.e, B.e,
-                                                                         flag + q);
+        chi_exp_final_kernel<<<((G + 1) * Npad + 255) / 256, 256, 0, s>>>(g.n_aux, A.Rpad, B.Rpad, Npad, G, L.KP, ep, A.e,
+                                                                         B.e, flag + q);
         if (w0 == 0)
           chi_slice_b_kernel<C><<<grid_for((long)B.Rpad * B.n_kb, 16), 256, 0, s>>>(g.n_aux, g.n_ov, t0, t1, Cq, B);
         chi_slice_a_kernel<C><<<grid_for((long)A.Rpad * A.n_kb, 16), 256, 0, s>>>(g.n_aux, g.n_ov, g.n_w, w0, G, t0, t1, Cq,
@@ -989,7 +1169,7 @@ cudaError_t chi0_g64_run(const BatchGeom& g, const double* const* Cptrs, const d
         o.add = t0 > 0;
         o.tri = 1;
         G64Index ix{nullptr, nullptr, 1, 1 << 30};
-        if (cudaError_t e = g64_product(C, A, B, ix, o, G, 0, p, L.part, flag + q, status, &nl, s)) return e;
+        if (cudaError_t e = g64_product(C, A, B, ix, o, G, 0, p, L.part, flag + q, 0, status, &nl, s)) return e;
       }
     }
   }

@@ -76,7 +76,7 @@ template <bool C>
 __global__ void __launch_bounds__(256) ao_half_kernel(int n_bas, int S, int n_mo, const double* __restrict__ P,
                                                       const double* __restrict__ c, int n0, int ncols,
                                                       double* __restrict__ H, int n_tn, const int* __restrict__ only) {
-  if (only && !*only) return;
+  if (only && !(*only & 1)) return;
   __shared__ Elem<C> As[AK][AT];
   __shared__ Elem<C> Bs[AK][AT];
   const int ts = blockIdx.x / n_tn, tn = blockIdx.x % n_tn;
@@ -108,7 +108,7 @@ template <bool C>
 __global__ void __launch_bounds__(256)
     ao_assemble_kernel(const __grid_constant__ AoPairs pr, const int4* __restrict__ fit, int n_aux, int n_occ,
                        int n_virt, int n_mo, int n_ti, int n_ta, const int* __restrict__ only) {
-  if (only && !*only) return;
+  if (only && !(*only & 1)) return;
   __shared__ Elem<C> As[AK][AT];
   __shared__ Elem<C> Bs[AK][AT];
   long bid = blockIdx.x;

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256, 1)
   bid /= n_wg;
   const int tile = bid % n_tiles;
   const int qb = bid / n_tiles;
-  if (only && !only[qb]) return;
+  if (only && !(only[qb] & 1)) return;
   int I, J;
   tri_index(tile, I, J);
   const int w0 = wg * G;
@@ -240,11 +240,12 @@ constexpr int GK = 16;
 template <bool C, int MODE, int U>
 __global__ void __launch_bounds__(256)
     sandwich_kernel(int N, int n_w, const double* __restrict__ Xb, const double* __restrict__ Lb,
-                    double* __restrict__ Ob, int n_tiles_row, int tiles_per_mat) {
+                    double* __restrict__ Ob, int n_tiles_row, int tiles_per_mat, const int* __restrict__ only) {
   constexpr int GT = 16 * U;
   __shared__ Elem<C> As[GK][GT];
   __shared__ Elem<C> Bs[GK][GT];
   const int b = blockIdx.x / tiles_per_mat;
+  if (only && !(only[b] & 1)) return;
   const int tile = blockIdx.x % tiles_per_mat;
   int I, J;
   if (MODE == 0) {
@@ -359,11 +360,12 @@ cudaError_t launch_chi0_fp64(const BatchGeom& g, const double* const* Cptrs, con
 
 namespace {
 template <bool C, int MODE, int U>
-cudaError_t sandwich_pass_u(int N, int n_batch, int n_w, const double* X, const double* L, double* O, cudaStream_t s) {
+cudaError_t sandwich_pass_u(int N, int n_batch, int n_w, const double* X, const double* L, double* O, cudaStream_t s,
+                            const int* only) {
   const int nt = (N + 16 * U - 1) / (16 * U);
   const int per = MODE == 0 ? nt * nt : nt * (nt + 1) / 2;
   if ((long)n_batch * per > 0x7fffffffL) return cudaErrorInvalidValue;
-  sandwich_kernel<C, MODE, U><<<(unsigned)(n_batch * per), 256, 0, s>>>(N, n_w, X, L, O, nt, per);
+  sandwich_kernel<C, MODE, U><<<(unsigned)(n_batch * per), 256, 0, s>>>(N, n_w, X, L, O, nt, per, only);
   return cudaGetLastError();
 }
 
@@ -372,33 +374,33 @@ cudaError_t sandwich_pass_u(int N, int n_batch, int n_w, const double* X, const 
 // largest tile (fewest operand reads) is taken that still gives every SM two
 // CTAs to balance.
 template <bool C, int MODE>
-cudaError_t sandwich_pass(int N, int n_batch, int n_w, const double* X, const double* L, double* O, cudaStream_t s) {
+cudaError_t sandwich_pass(int N, int n_batch, int n_w, const double* X, const double* L, double* O, cudaStream_t s,
+                            const int* only) {
   const long sms = num_sms_fp64();
   auto blocks = [&](int gt) {
     const long nt = (N + gt - 1) / gt;
     return n_batch * (MODE == 0 ? nt * nt : nt * (nt + 1) / 2);
   };
-  if (blocks(64) >= 4 * sms) return sandwich_pass_u<C, MODE, 4>(N, n_batch, n_w, X, L, O, s);
-  if (blocks(32) >= 2 * sms) return sandwich_pass_u<C, MODE, 2>(N, n_batch, n_w, X, L, O, s);
-  return sandwich_pass_u<C, MODE, 1>(N, n_batch, n_w, X, L, O, s);
+  if (blocks(64) >= 4 * sms) return sandwich_pass_u<C, MODE, 4>(N, n_batch, n_w, X, L, O, s, only);
+  if (blocks(32) >= 2 * sms) return sandwich_pass_u<C, MODE, 2>(N, n_batch, n_w, X, L, O, s, only);
+  return sandwich_pass_u<C, MODE, 1>(N, n_batch, n_w, X, L, O, s, only);
 }
 }  // namespace
 
 cudaError_t launch_sandwich(int cplx, int N, int n_batch, int n_w, const double* chi, const double* L, double* T,
-                            double* Y, cudaStream_t s) {
+                            double* Y, cudaStream_t s, const int* only) {
   if (n_batch == 0) return cudaSuccess;
   if (cplx) {
-    if (cudaError_t e = sandwich_pass<true, 0>(N, n_batch, n_w, chi, L, T, s)) return e;
-    return sandwich_pass<true, 1>(N, n_batch, n_w, T, L, Y, s);
+    if (cudaError_t e = sandwich_pass<true, 0>(N, n_batch, n_w, chi, L, T, s, only)) return e;
+    return sandwich_pass<true, 1>(N, n_batch, n_w, T, L, Y, s, only);
   }
-  if (cudaError_t e = sandwich_pass<false, 0>(N, n_batch, n_w, chi, L, T, s)) return e;
-  return sandwich_pass<false, 1>(N, n_batch, n_w, T, L, Y, s);
+  if (cudaError_t e = sandwich_pass<false, 0>(N, n_batch, n_w, chi, L, T, s, only)) return e;
+  return sandwich_pass<false, 1>(N, n_batch, n_w, T, L, Y, s, only);
 }
 
-cudaError_t launch_vinv(int cplx, int N, int n_q, const double* L, double* X, double* Wn, cudaStream_t s) {
-  if (n_q == 0) return cudaSuccess;
-  if (cudaError_t e = launch_trinv(cplx, N, n_q, L, X, s)) return e;
-  return cplx ? sandwich_pass<true, 1>(N, n_q, 1, X, X, Wn, s) : sandwich_pass<false, 1>(N, n_q, 1, X, X, Wn, s);
+cudaError_t launch_gram(int cplx, int N, int n_q, const double* X, double* Wn, cudaStream_t s, const int* only) {
+  return cplx ? sandwich_pass<true, 1>(N, n_q, 1, X, X, Wn, s, only)
+              : sandwich_pass<false, 1>(N, n_q, 1, X, X, Wn, s, only);
 }
 
 cudaError_t launch_energy_reduce(int n_q, int n_w, const double* parts, const double* w_q, const double* zeta_w,

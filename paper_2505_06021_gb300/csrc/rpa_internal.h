@@ -37,7 +37,7 @@ cudaError_t launch_dtab(const BatchGeom& g, const double* eps_occ, const double*
                         const int* kqidx, const double* omega, double zeta_k, double* dtab, cudaStream_t s);
 
 // chi[qb][w] (N x N, full Hermitian) = sum_j sum_t conj(C[qb*n_k+j][P,t]) C[..][Q,t] d[qb][j][w][t].
-// only: null, or device flags per q of the batch; q with a zero flag are left as they are.
+// only: null, or device flags per q of the batch; q without bit 0 are left as they are.
 cudaError_t launch_chi0_fp64(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
                              cudaStream_t s, const int* only = nullptr);
 
@@ -80,16 +80,17 @@ cudaError_t launch_cholesky_ragged(int cplx, const CholTask* tasks, const CholTa
 // launches it takes.
 cudaError_t launch_trinv(int cplx, int N, int n_q, const double* L, double* X, cudaStream_t s);
 int trinv_launches(int N);
-// Wn[q] = -V(q)^-1 (lower triangle) from the Cholesky factors L[q]: X = L^-1
-// into X[q], then -(X^H X).
-cudaError_t launch_vinv(int cplx, int N, int n_q, const double* L, double* X, double* Wn, cudaStream_t s);
+// Wn[q] = -(X[q]^H X[q]), lower triangle: -V(q)^-1 from the inverse Cholesky
+// factors X.  only: null, or a device word per q; those without bit 0 are left.
+cudaError_t launch_gram(int cplx, int N, int n_q, const double* X, double* Wn, cudaStream_t s,
+                        const int* only = nullptr);
 
 // ---- AO -> MO transform (kernels_ao.cu) -----------------------------------
 
 // H[s][n] = sum_nu P[nu][s] c[nu][n0 + n], s < S, n < ncols: the half-
 // transform of one k-point's PADF array P (n_bas x S) with the MO columns
 // [n0, n0 + ncols) of c (n_bas x n_mo).  H is S x ncols.  only: null, or a
-// device word; nothing is done when it is zero.
+// device word; nothing is done unless its bit 0 is set.
 cudaError_t launch_ao_half(int cplx, int n_bas, int S, int n_mo, const double* P, const double* c, int n0, int ncols,
                            double* H, cudaStream_t s, const int* only = nullptr);
 
@@ -152,8 +153,9 @@ cudaError_t launch_proj_finish(int cplx, const ProjPtrs& P, int n_mat, int N, in
 
 // T[b] = chi[b] * L[b / n_w]   (L lower triangular, N x N).
 // Y[b] = -(L[b / n_w]^H T[b]), lower triangle only.
+// only: null, or a device word per matrix; those without bit 0 are left.
 cudaError_t launch_sandwich(int cplx, int N, int n_batch, int n_w, const double* chi, const double* L, double* T,
-                            double* Y, cudaStream_t s);
+                            double* Y, cudaStream_t s, const int* only = nullptr);
 
 // Device-to-device copy by a kernel (a cudaMemcpyAsync when the pointers are
 // not 16-byte aligned or the size is not a multiple of 16): for copies on a

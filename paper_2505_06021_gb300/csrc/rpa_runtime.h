@@ -107,7 +107,7 @@ namespace rpa {
 
 // Workspace of one lane for a job processed in q-batches of qb q-points.
 struct Layout {
-  size_t meta, dtab, chi, T, L, Vc, stageC, stageV, eps, mixed, ao, binmeta, aog, total;
+  size_t meta, dtab, chi, T, L, Vc, stageC, stageV, eps, mixed, ao, binmeta, aog, tail, total;
   size_t slice_cap;  // mixed path: bytes for the weighted operand's digit planes
   int qb;            // q per staging batch (d table, host staging, AO coefficients)
   int qt;            // q per tail batch (chi, L, Vc, T: V factor and log-det)
@@ -141,6 +141,8 @@ struct Bufs {
   char* ao;       // AO-form jobs: fit table, half-transforms, one q's C (ao_internal.h)
   char* binmeta;  // frequency-batched chi0: the job's bin tables, or null
   char* aog;      // AO-form jobs: digit planes of the transforms (AoG64), or null
+  char* tail;     // digit planes of the tail's products (tail_g64_bytes), or null
+  size_t tail_bytes;
 };
 
 void ctx_set_error(rpa_ctx* ctx, const char* fmt, ...);
@@ -165,6 +167,8 @@ void prof_end(rpa_ctx* ctx, Exec* ex, cudaStream_t s, int cls, int n_kernels);
 void prof_collect(rpa_ctx* ctx, Exec* ex);
 // mixed_ws: include the split-precision chi0 workspace (a batch supplies its own).
 // qt: q per tail batch (0: qt = qb).  bj: the job's frequency-batched chi0, if any.
+// Workspace of the tail's products on the tensor cores for nq q at once (0: the FP64 kernels).
+size_t tail_region_bytes(const rpa_job* j, int nq);
 Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt = 0,
                    const BinJob* bj = nullptr, bool g64 = false);
 int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj = nullptr);
