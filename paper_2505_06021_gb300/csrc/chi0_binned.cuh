@@ -279,10 +279,12 @@ __global__ void __launch_bounds__(256) erow_bin_kernel(int cplx, int Npad, int K
 __global__ void __launch_bounds__(256, 2) slice_bin_kernel(SliceBinArgs a) {
   const long total = (long)a.Npad * a.n_kb;
   for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
+    int cv[16];
+    fetch_unit_bin(a, idx, cv);
     if (a.cplx)
-      slice_unit_bin<true>(a, idx);
+      slice_unit_bin<true, false>(a, idx, cv);
     else
-      slice_unit_bin<false>(a, idx);
+      slice_unit_bin<false, false>(a, idx, cv);
   }
 }
 
@@ -306,15 +308,22 @@ struct RedBin {
   int wg;              // frequencies per group (grid y = groups)
 };
 constexpr int RED_WG = 10;
+constexpr int RED_GB = 3;  // skeletons in flight
 
-// (h, l) += a + b (a, b: a float-float product), Knuth TwoSum then renormalise.
+// (h, l) += ph + pl: Knuth's TwoSum on the high parts, the errors gathered in l,
+// renormalised by ff_norm every few terms.
 __device__ __forceinline__ void ff_acc(float& h, float& l, float ph, float pl) {
-  const float s = h + ph;
-  const float bb = s - h;
-  const float e = (h - (s - bb)) + (ph - bb);
-  const float t = e + pl + l;
-  h = s + t;
-  l = t - (h - s);
+  const float s = __fadd_rn(h, ph);
+  const float bb = __fsub_rn(s, h);
+  const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(ph, bb));
+  l = __fadd_rn(l, __fadd_rn(e, pl));
+  h = s;
+}
+
+__device__ __forceinline__ void ff_norm(float& h, float& l) {
+  const float s = __fadd_rn(h, l);
+  l = __fsub_rn(l, __fsub_rn(s, h));
+  h = s;
 }
 
 __global__ void __launch_bounds__(256, 2) reduce_bin_kernel(const __grid_constant__ RedBin rb) {
@@ -341,39 +350,61 @@ __global__ void __launch_bounds__(256, 2) reduce_bin_kernel(const __grid_constan
   for (int w = 0; w < RED_WG; ++w) rh[w] = rl[w] = ih[w] = il[w] = 0.f;
   const int rq = rb.eCraw[Q];
   const int eCQ = rq ? rq - 1022 : -2000;
+  const float* pr = rb.part + (long)r * 128 + c;
   for (int b = 0; b < rb.nb; ++b) {
-    for (int g = 0; g < rb.rank[b]; ++g) {
-      const int ra = rb.eAraw[((long)b * rb.rmax + g) * rb.Npad + P];
-      if (ra <= 0 || rq == 0) continue;  // a zero row or column: no contribution
-      const int g0 = g / rb.G * rb.G, Gs = min(rb.G, rb.rank[b] - g0), gl = g - g0;
-      const long it0 = rb.base[b] + (long)g0 * rb.nks[b] * rb.n_tiles;
-      // x = sum over the split-K partials of (hi + lo), as a float-float pair
-      float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
-      for (int ks = 0; ks < rb.nks[b]; ++ks) {
-        const long item = it0 + ((long)ks * Gs + gl) * rb.n_tiles + tile;
-        const float* pp = rb.part + item * 2 * 128 * 128 + (long)r * 128;
-        ff_acc(xh, xl, pp[c], pp[128 * 128 + c]);
-        if (rb.cplx) ff_acc(yh, yl, pp[64 + c], pp[128 * 128 + 64 + c]);
+    // RED_GB skeletons at a time: their loads are in flight together
+    for (int gb = 0; gb < rb.rank[b]; gb += RED_GB) {
+      float xh[RED_GB], xl[RED_GB], yh[RED_GB], yl[RED_GB];
+      int ra[RED_GB];
+#pragma unroll
+      for (int u = 0; u < RED_GB; ++u) {
+        const int g = gb + u;
+        xh[u] = xl[u] = yh[u] = yl[u] = 0.f;
+        ra[u] = 0;
+        if (g >= rb.rank[b]) continue;
+        ra[u] = rb.eAraw[((long)b * rb.rmax + g) * rb.Npad + P];
+        const int g0 = g / rb.G * rb.G, Gs = min(rb.G, rb.rank[b] - g0);
+        const float* pp = pr + (rb.base[b] + (long)g0 * rb.nks[b] * rb.n_tiles + (long)(g - g0) * rb.n_tiles + tile) *
+                                   (2 * 128 * 128);
+        // x = sum over the split-K partials of (hi + lo), as a float-float pair
+        xh[u] = pp[0];
+        xl[u] = pp[128 * 128];
+        if (rb.cplx) {
+          yh[u] = pp[64];
+          yl[u] = pp[128 * 128 + 64];
+        }
+        for (int ks = 1; ks < rb.nks[b]; ++ks) {
+          pp += (long)Gs * rb.n_tiles * (2 * 128 * 128);
+          ff_acc(xh[u], xl[u], pp[0], pp[128 * 128]);
+          if (rb.cplx) ff_acc(yh[u], yl[u], pp[64], pp[128 * 128 + 64]);
+        }
       }
-      // scale 2^(eA + eC + 1 - 14) with the sign of chi = -sum conj(a) c (exact)
-      const int sh = (ra - 2044 + 1) + eCQ + 1 - 14;
-      xh = -ldexpf(xh, sh);
-      xl = -ldexpf(xl, sh);
-      yh = -ldexpf(yh, sh);
-      yl = -ldexpf(yl, sh);
-      const float2* cf = cs + ((long)b * rb.rmax + g) * rb.n_w + w0;
+#pragma unroll
+      for (int u = 0; u < RED_GB; ++u) {
+        if (ra[u] <= 0 || rq == 0) continue;  // a zero row or column (or no skeleton): no contribution
+        // scale 2^(eA + eC + 1 - 14) with the sign of chi = -sum conj(a) c (exact)
+        const int sh = (ra[u] - 2044 + 1) + eCQ + 1 - 14;
+        const float x0 = -ldexpf(xh[u], sh), x1 = -ldexpf(xl[u], sh);
+        const float y0 = -ldexpf(yh[u], sh), y1 = -ldexpf(yl[u], sh);
+        const float2* cf = cs + ((long)b * rb.rmax + gb + u) * rb.n_w + w0;
+#pragma unroll
+        for (int w = 0; w < RED_WG; ++w) {
+          if (w >= nw) break;
+          const float2 k = cf[w];
+          float ph = __fmul_rn(k.x, x0);
+          float pl = __fadd_rn(fmaf(k.x, x0, -ph), fmaf(k.x, x1, __fmul_rn(k.y, x0)));
+          ff_acc(rh[w], rl[w], ph, pl);
+          if (rb.cplx) {
+            ph = __fmul_rn(k.x, y0);
+            pl = __fadd_rn(fmaf(k.x, y0, -ph), fmaf(k.x, y1, __fmul_rn(k.y, y0)));
+            ff_acc(ih[w], il[w], ph, pl);
+          }
+        }
+      }
 #pragma unroll
       for (int w = 0; w < RED_WG; ++w) {
-        if (w >= nw) break;
-        const float2 k = cf[w];
-        float ph = k.x * xh;
-        float pl = fmaf(k.x, xh, -ph) + fmaf(k.x, xl, k.y * xh);
-        ff_acc(rh[w], rl[w], ph, pl);
-        if (rb.cplx) {
-          ph = k.x * yh;
-          pl = fmaf(k.x, yh, -ph) + fmaf(k.x, yl, k.y * yh);
-          ff_acc(ih[w], il[w], ph, pl);
-        }
+        ff_norm(rh[w], rl[w]);
+        ff_norm(ih[w], il[w]);
       }
     }
   }

@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "slice.cuh"
 #include "tc_ptx.cuh"
 
@@ -390,11 +392,20 @@ __global__ void __launch_bounds__(THREADS, 1) chi0_tc_kernel(const __grid_consta
     const long total = (long)p.sideb.Npad * p.sideb.n_kb;
     const long stride = (long)gridDim.x * NT;
     const long first = (long)blockIdx.x * NT + (threadIdx.x - (THREADS - NT));
-    if (p.sideb.cplx) {
-      for (long idx = first; idx < total; idx += stride) slice_unit_bin<true>(p.sideb, idx);
-    } else {
-      for (long idx = first; idx < total; idx += stride) slice_unit_bin<false>(p.sideb, idx);
-    }
+    auto run = [&](auto cplx) {
+      int cv[16], cn[16] = {};
+      if (first < total) fetch_unit_bin(p.sideb, first, cv);
+      for (long idx = first; idx < total; idx += stride) {
+        if (idx + stride < total) fetch_unit_bin(p.sideb, idx + stride, cn);
+        slice_unit_bin<decltype(cplx)::value, true>(p.sideb, idx, cv);
+#pragma unroll
+        for (int v = 0; v < 16; ++v) cv[v] = cn[v];
+      }
+    };
+    if (p.sideb.cplx)
+      run(std::true_type{});
+    else
+      run(std::false_type{});
   }
   fence_before();
   __syncthreads();

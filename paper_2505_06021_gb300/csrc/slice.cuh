@@ -220,8 +220,25 @@ struct SliceBinArgs {
   long aoff[SB_MAX_BINS];    // bin's plane offset in S (uint16 units)
 };
 
-template <bool CPLX>
-__device__ __forceinline__ void slice_unit_bin(const SliceBinArgs& a, long idx) {
+// The 16 fixed-point values of unit idx (row P = idx mod Npad, K-block idx / Npad).
+__device__ __forceinline__ void fetch_unit_bin(const SliceBinArgs& a, long idx, int (&cv)[16]) {
+  const int P = (int)(idx % a.Npad), kb = (int)(idx / a.Npad);
+  const int4* src = reinterpret_cast<const int4*>(a.cfix + (long)P * a.Kr + (long)kb * 16);
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const int4 x = src[v];
+    cv[4 * v] = x.x;
+    cv[4 * v + 1] = x.y;
+    cv[4 * v + 2] = x.z;
+    cv[4 * v + 3] = x.w;
+  }
+}
+
+// One unit: the planes of its slots.  AHEAD: the next slot's weights and row
+// exponent load during the current one, for the two slicer warps of a
+// tensor-core launch, which have no other warp to hide them behind.
+template <bool CPLX, bool AHEAD>
+__device__ __forceinline__ void slice_unit_bin(const SliceBinArgs& a, long idx, const int (&cv)[16]) {
   constexpr int tpg = CPLX ? 8 : 16;  // positions per K-block
   const int P = (int)(idx % a.Npad);
   const int kb = (int)(idx / a.Npad);
@@ -232,31 +249,32 @@ __device__ __forceinline__ void slice_unit_bin(const SliceBinArgs& a, long idx) 
   const int kbl = kb - a.kb0[b];
   const long nkb = a.kb0[b + 1] - a.kb0[b];
   const long nI = a.Npad / 128;
-  const int4* src = reinterpret_cast<const int4*>(a.cfix + (long)P * a.Kr + (long)kb * 16);
-  int cv[16];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const int4 x = src[v];
-    cv[4 * v] = x.x;
-    cv[4 * v + 1] = x.y;
-    cv[4 * v + 2] = x.z;
-    cv[4 * v + 3] = x.w;
-  }
   const int rc = a.eC[P];
   const int eC = rc ? rc - 1022 : -2000;
-  const long u0 = (long)kb * tpg;
+  const unsigned long long* wr = a.wx + (long)a.g0 * a.Kt + (long)kb * tpg;
+  const int* er = a.eAraw + ((long)b * a.rmax + a.g0) * a.Npad + P;
+  unsigned long long xw[tpg];
+#pragma unroll
+  for (int v = 0; v < tpg; ++v) xw[v] = __ldg(wr + v);
+  int ra = *er;
   for (int gl = 0; gl < G; ++gl) {
-    const int g = a.g0 + gl;
-    const int ra = a.eAraw[((long)b * a.rmax + g) * a.Npad + P];
+    unsigned long long xn[tpg];
+    int rn = 0;
+    if (AHEAD && gl + 1 < G) {
+      wr += a.Kt;
+      er += a.Npad;
+#pragma unroll
+      for (int v = 0; v < tpg; ++v) xn[v] = __ldg(wr + v);
+      rn = *er;
+    }
     const int eA = ra > 0 ? ra - 2044 + 1 : -2000;
     const int shbase = 30 + eA - eC;
-    const unsigned long long* wr = a.wx + (long)g * a.Kt + u0;
     uint32_t px[MAX_S][8];
     long long wm_prev = 0;
     int sh_prev = 0;
 #pragma unroll
     for (int v = 0; v < tpg; ++v) {
-      const unsigned long long x = __ldg(wr + v);
+      const unsigned long long x = xw[v];
       const long long wmv = (long long)(uint32_t)x;
       const int shv = shbase - (int)(uint32_t)(x >> 32);
       if constexpr (CPLX) {
@@ -273,6 +291,17 @@ __device__ __forceinline__ void slice_unit_bin(const SliceBinArgs& a, long idx) 
       if (i >= a.s) break;
       uint16_t* blk = a.S + a.aoff[b] + ((((long)gl * nI + (P >> 7)) * nkb + kbl) * a.s + i) * 2048;
       store_core_rows(blk, P & 127, px[i]);
+    }
+    if constexpr (AHEAD) {
+#pragma unroll
+      for (int v = 0; v < tpg; ++v) xw[v] = xn[v];
+      ra = rn;
+    } else if (gl + 1 < G) {
+      wr += a.Kt;
+      er += a.Npad;
+#pragma unroll
+      for (int v = 0; v < tpg; ++v) xw[v] = __ldg(wr + v);
+      ra = *er;
     }
   }
 }
