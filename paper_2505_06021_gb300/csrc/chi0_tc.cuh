@@ -51,6 +51,31 @@ __device__ __forceinline__ void ff_add4(float& hi, float& lo, float g0, float g1
   lo = f - (hi - t);
 }
 
+// CTAs that share operand rows run the same K range at the same time, but
+// nothing else keeps them together: they drift by more K-blocks than the L2 can
+// bridge (the tiles that run at once advance through 0.5 MB of operands per K-block),
+// and the planes are then read from DRAM several times.  The limits below hold
+// them within about 100 K-blocks.
+constexpr int PACE_KB = 16;
+constexpr unsigned PACE_AHEAD = 4, PACE_RING = 128;
+constexpr int PACE_POLLS = 100;  // at most: the pace is a hint, no condition
+
+__device__ __forceinline__ void pace_add(unsigned* cnt, unsigned n) {
+  asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(cnt), "r"(n) : "memory");
+}
+__device__ __forceinline__ void pace_step(unsigned* cnt, unsigned step, unsigned grid) {
+  if (step >= PACE_AHEAD) {
+    const unsigned m = step - PACE_AHEAD, want = (m / PACE_RING + 1) * grid;
+    for (int i = 0; i < PACE_POLLS; ++i) {
+      unsigned v;
+      asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt + m % PACE_RING) : "memory");
+      if (v >= want) break;
+      __nanosleep(200);
+    }
+  }
+  pace_add(cnt + step % PACE_RING, 1);
+}
+
 // ---------------------------------------------------------- GEMM kernel ----
 // One persistent launch covers several "segments": a segment is one q of one
 // job with G frequencies, its own operand buffers and partial buffer.  The
@@ -74,6 +99,11 @@ struct TcParams {
   int drop_item;  // test hook: the first K-block of this work item is never
                   // loaded (-1: off), so one bounded wait runs out
   int* err;
+  // Pace of the launch (null: none): PACE_RING zeroed counters; step n of a CTA
+  // (PACE_KB K-blocks each) adds one to counter n mod PACE_RING.  A CTA that is
+  // more than PACE_AHEAD steps ahead of the last one waits a little before it
+  // loads on.
+  unsigned* pace;
   int grp_mask;  // accumulator groups that receive MMAs (the host's copy of MmaTable<s>::mask)
   // Side job of the slicer warps: the weighted digit planes of another q
   // (all its frequencies), written while this launch's MMAs run; its inputs
@@ -249,10 +279,12 @@ __global__ void __launch_bounds__(THREADS, 1) chi0_tc_kernel(const __grid_consta
       int armed[STAGES];
       for (int i = 0; i < STAGES; ++i) armed[i] = -1;
       bool ok = true;
+      unsigned step = 0;
       for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
         const ItemPos it = item_pos(p, item);
         const TcSeg& SG = p.seg[it.seg];
         for (int kb = it.kb0; kb < it.kb1 && ok; ++kb) {
+          if (p.pace && (kb - it.kb0) % PACE_KB == 0) pace_step(p.pace, step++, gridDim.x);
           ok = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, p.err, 11, 2000);
           if (!ok) break;
           uint8_t* sa = smem + stage * STAGE_BYTES;
@@ -274,6 +306,9 @@ __global__ void __launch_bounds__(THREADS, 1) chi0_tc_kernel(const __grid_consta
           }
         }
       }
+      // a CTA without more work no longer holds the others' pace
+      if (p.pace)
+        for (unsigned i = 0; i < PACE_RING; ++i) pace_add(p.pace + i, 1u << 24);
       // every armed stage's copy must have landed before the CTA exits
       for (int i = 0; i < STAGES; ++i) {
         if (armed[i] < 0) continue;

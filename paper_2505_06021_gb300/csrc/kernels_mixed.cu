@@ -440,13 +440,21 @@ void launch_slice(int cplx, unsigned grid, cudaStream_t st, const SliceArgs& a) 
 // (slice pairs x padded tiles x padded K of each segment).
 std::atomic<unsigned long long> g_tc_flops{0};
 
-void launch_tc(int s, int grid, size_t smem, cudaStream_t st, const TcParams& tp) {
+void launch_tc(int s, int grid, size_t smem, cudaStream_t st, TcParams& tp) {
   const unsigned long long pairs = (unsigned long long)(s * (s + 1) / 2 + (s == 2 ? 1 : 0));
   unsigned long long f = 0;
   for (int i = 0; i < tp.n_segs; ++i)
     f += (unsigned long long)tp.seg[i].G * tp.seg[i].n_tiles * (unsigned long long)tp.seg[i].n_kb * pairs * 2ull *
          128ull * 128ull * (unsigned long long)KB;
   g_tc_flops += f;
+  // launches whose operands fit the L2 anyway, or that do not fill the GPU, need no pace
+  size_t bytes = 0;
+  for (int i = 0; i < tp.n_segs; ++i)
+    bytes += (size_t)tp.seg[i].n_kb * s * PLANE_BYTES * ((size_t)tp.seg[i].G * tp.seg[i].nI + 1);
+  if (bytes > ((size_t)96 << 20) && grid >= num_sms()) {
+    tp.pace = reinterpret_cast<unsigned*>(tp.err) + 64;  // within the error word's kilobyte
+    cudaMemsetAsync(tp.pace, 0, sizeof(unsigned) * PACE_RING, st);
+  }
   if (s == 2)
     chi0_tc_kernel<2><<<grid, THREADS, smem, st>>>(tp);
   else if (s == 3)
