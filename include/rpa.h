@@ -179,7 +179,9 @@ rpa_status rpa_job_validate(const rpa_job *job, char *msg, size_t msg_len);
  * nodes, residual err[b] <= 1e-10 of the bin's largest |d(., omega_w)| on a
  * dense check grid), so chi0 needs rank[b] contractions over bin b instead of
  * n_w: chi0(w) = sum_b sum_r coef[b][r][w] X_{b,r}, X_{b,r} the contraction of
- * bin b's transitions at omega_{skel[b][r]}.  mode: 0 automatic (n_bins = 0
+ * bin b's transitions at omega_{skel[b][r]}.  (The chi0 of rpa_energy and
+ * rpa_chi0 runs a plan of the same construction and bounds whose number of bins
+ * also weighs the recombination, up to 64.)  mode: 0 automatic (n_bins = 0
  * when the plan saves no work), 2 always.  Outputs (any may be NULL), with
  * B = RPA_FREQ_MAX_BINS: edges [B], rank [B], err [B], skel [B][n_w] (-1 past
  * rank[b]), coef [B][n_w][n_w] (row r of bin b), *work_ratio = modelled

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256) perm_kernel(int n_k, int n_occ, int n_vir
   const long row = (long)blockIdx.x * 8 + warp;
   if (row >= nrow) return;
   const int jj = (int)(row / n_occ), i = (int)(row - (long)jj * n_occ);
-  if (lane < SB_MAX_BINS) run[warp][lane] = 0;
+  for (int b = lane; b < SB_MAX_BINS; b += 32) run[warp][b] = 0;
   __syncwarp();
   const double eo = eps_occ[(long)kidx[jj] * n_occ + i];
   const double* ev = eps_virt + (long)kqidx[jj] * n_virt;

@@ -35,6 +35,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <limits>
 #include <thread>
 #include <vector>
@@ -259,18 +260,19 @@ int count_ge(const double* evs, int n, double e_i, double edge) {
 
 }  // namespace
 
-void freq_parallel_q(int n_q, const std::function<void(int)>& fn) {
+void freq_parallel(int n, const std::function<void(int)>& fn) {
   const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-  const int nt = std::min<int>(n_q, (int)std::min(8u, hw));
-  if (nt <= 1) {
-    for (int q = 0; q < n_q; ++q) fn(q);
-    return;
-  }
+  const int nt = std::min<int>(n, (int)std::min(12u, hw));
+  std::atomic<int> next{0};
+  auto work = [&] {
+    for (int i = next++; i < n; i = next++) fn(i);
+  };
   std::vector<std::thread> th;
-  for (int t = 0; t < nt; ++t)
-    th.emplace_back([&, t] {
-      for (int q = t; q < n_q; q += nt) fn(q);
-    });
+  try {
+    for (int t = 1; t < nt; ++t) th.emplace_back(work);
+  } catch (...) {  // no more threads to be had: this one does the rest
+  }
+  work();
   for (auto& x : th) x.join();
 }
 
@@ -299,7 +301,7 @@ void freq_counts(const rpa_job* j, const FreqPlan& p, int q, const double* eo, c
 }
 
 bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int mode, FreqPlan* out,
-                     std::vector<int>* counts) {
+                     std::vector<int>* counts, int max_bins) {
   FreqPlan& P = *out;
   P = FreqPlan{};
   if (mode == 1 || j->n_w < 2 || j->n_w > 32) return false;
@@ -309,7 +311,7 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
   const std::vector<double> evs = sorted_virt(j, ev);
   const double total = (double)j->n_q * j->n_k * j->n_occ * j->n_virt;
   auto bins_for = [&](double rho) {
-    return std::min(FREQ_MAX_BINS, std::max(1, (int)ceil(log(hi / lo) / log(rho) - 1e-9)));
+    return std::min(max_bins, std::max(1, (int)ceil(log(hi / lo) / log(rho) - 1e-9)));
   };
   auto bin_ends = [&](int nb, int b, double& blo, double& bhi) {
     const double step = pow(hi / lo, 1.0 / nb);
@@ -332,18 +334,20 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
     std::vector<double> kb(nb, 0.0);
     const size_t per_q = (size_t)j->n_k * j->n_occ * nb;
     std::vector<int> cnt(per_q * j->n_q);
-    freq_parallel_q(j->n_q, [&](int q) { freq_counts(j, c, q, eo, evs.data(), cnt.data() + per_q * q); });
+    freq_parallel(j->n_q, [&](int q) { freq_counts(j, c, q, eo, evs.data(), cnt.data() + per_q * q); });
     for (size_t u = 0; u < cnt.size(); ++u) kb[u % nb] += cnt[u];
     if (counts) *counts = std::move(cnt);
     double work = 0.0;
     c.rmax = 0;
     std::vector<BinFit> fits(nb);
-    for (int b = 0; b < nb; ++b) {
+    freq_parallel(nb, [&](int b) {
       double blo, bhi;
       bin_ends(nb, b, blo, bhi);
       if (b > 0) blo = c.edges[b - 1];
       if (b + 1 < nb) bhi = c.edges[b];
       fits[b] = fit_bin(blo, bhi, j->omega, j->n_w, FREQ_TOL, FREQ_AMP);
+    });
+    for (int b = 0; b < nb; ++b) {
       c.rank[b] = fits[b].rank;
       c.err[b] = fits[b].err;
       c.amp[b] = fits[b].amp;
@@ -364,26 +368,43 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
   };
   // Candidate ratios are screened by the mean rank of five sample bins
   // (fitted against a coarse check grid) and the padding of their bin count,
-  // assuming equal populations; only the most promising is planned in full
-  // (the fits and the population counts of every candidate in full took
-  // ~60 ms on the slab job).
-  const double ratios[] = {1.08, 1.1, 1.12, 1.15, 1.2, 1.25, 1.3, 1.5, 1.75, 2.1, 3.0};
+  // assuming equal populations; only the most promising is planned in full.
+  // The plan the chi0 runs also counts the recombination: per element it costs
+  // nb rank n_w float-float multiply-adds against rank K tensor-core terms;
+  // measured, 25 bins of 20 frequencies at K = 114688 take 0.19 of the
+  // contraction's time, i.e. 44 nb n_w / K.  So long contractions take narrow
+  // bins (rank 5 at ratio 1.05 where 1.1 needs 6: slab block chi0 95 -> 79 ms), and
+  // short ones few wide bins.
+  const bool run = max_bins > RPA_FREQ_MAX_BINS;
+  const std::vector<double> ratios = run ? std::vector<double>{1.04, 1.05, 1.065, 1.08, 1.1, 1.12, 1.15, 1.2, 1.25, 1.3, 1.5, 1.75, 2.1, 3.0}
+                                         : std::vector<double>{1.08, 1.1, 1.12, 1.15, 1.2, 1.25, 1.3, 1.5, 1.75, 2.1, 3.0};
+  std::vector<int> rk(ratios.size() * 5);
+  freq_parallel((int)rk.size(), [&](int i) {
+    const int nb = bins_for(ratios[i / 5]);
+    const int at[5] = {0, nb / 4, nb / 2, (3 * nb) / 4, nb - 1};
+    double blo, bhi;
+    bin_ends(nb, at[i % 5], blo, bhi);
+    rk[i] = fit_bin(blo, bhi, j->omega, j->n_w, FREQ_TOL, FREQ_AMP, 101).rank;
+  });
   std::vector<std::pair<double, double>> est;  // (modelled work, rho)
-  for (double rho : ratios) {
-    const int nb = bins_for(rho);
+  for (size_t c = 0; c < ratios.size(); ++c) {
+    const int nb = bins_for(ratios[c]);
     double r = 0.0;
-    int ns = 0;
-    for (int b : {0, nb / 4, nb / 2, (3 * nb) / 4, nb - 1}) {
-      double blo, bhi;
-      bin_ends(nb, b, blo, bhi);
-      r += fit_bin(blo, bhi, j->omega, j->n_w, FREQ_TOL, FREQ_AMP, 101).rank;
-      ++ns;
+    int rm = 0;
+    for (int i = 0; i < 5; ++i) {
+      r += rk[5 * c + i];
+      rm = std::max(rm, rk[5 * c + i]);
     }
-    est.push_back({r / ns * (1.0 + 8.0 * j->n_q * nb / total), rho});
+    // (the recombination keeps the coefficients in 48 KB of shared memory)
+    if (run && nb > RPA_FREQ_MAX_BINS && (size_t)nb * rm * j->n_w * sizeof(double) > 48 * 1024) continue;
+    const double recomb = run ? 44.0 * nb * j->n_w * j->n_q / total : 0.0;
+    est.push_back({r / 5 * (1.0 + 8.0 * j->n_q * nb / total + recomb), ratios[c]});
   }
   std::stable_sort(est.begin(), est.end(),
                    [](const std::pair<double, double>& a, const std::pair<double, double>& b) { return a.first < b.first; });
   P = plan_full(est[0].second);
+  for (size_t c = 1; c < est.size() && (size_t)P.n_bins * P.rmax * j->n_w * sizeof(double) > 48 * 1024; ++c)
+    P = plan_full(est[c].second);
   P.dlo = lo;
   P.dhi = hi;
   if ((size_t)P.n_bins * P.rmax * j->n_w * sizeof(double) > 48 * 1024) {  // coefficients of the reduction
@@ -455,7 +476,7 @@ extern "C" rpa_status rpa_freq_plan(const rpa_job* job, int mode, int* n_bins, d
   if (!job || rpa::validate_job(job, msg, sizeof msg)) return RPA_E_INVAL;
   if (job->mem != RPA_MEM_HOST || mode < 0 || mode > 2) return RPA_E_INVAL;
   rpa::FreqPlan p;
-  rpa::freq_plan_build(job, job->eps_occ, job->eps_virt, mode, &p);
+  rpa::freq_plan_build(job, job->eps_occ, job->eps_virt, mode, &p, nullptr, RPA_FREQ_MAX_BINS);
   if (n_bins) *n_bins = p.n_bins;
   if (work_ratio) *work_ratio = p.n_bins ? p.work_ratio : 1.0;
   for (int b = 0; b < p.n_bins; ++b) {

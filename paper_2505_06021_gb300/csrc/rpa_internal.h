@@ -211,7 +211,7 @@ size_t mixed_seq_workspace_bytes(const BatchGeom& g, int n_slices, size_t slice_
 // bin b the weight of every frequency node is a combination of the weights of
 // rank[b] skeleton nodes, d(D, w) ~= sum_r coef[b][r][w] d(D, w_skel[b][r]),
 // to FREQ_TOL of the bin's largest |d(., w)|.
-constexpr int FREQ_MAX_BINS = 32;
+constexpr int FREQ_MAX_BINS = 64;
 constexpr double FREQ_TOL = 1e-10;
 constexpr double FREQ_AMP = 16.0;
 struct FreqPlan {
@@ -230,11 +230,13 @@ struct FreqPlan {
 // (false when it saves no work), 1 off, 2 always.  Returns whether a plan is
 // to be used.  With counts set it also returns every q's freq_counts for the
 // plan ([q][n_k n_occ][n_bins], the input of freq_bin_q).
+// max_bins: RPA_FREQ_MAX_BINS for the plan rpa_freq_plan reports, FREQ_MAX_BINS
+// for the one the chi0 runs (which also weighs the recombination).
 bool freq_plan_build(const rpa_job* j, const double* eps_occ_h, const double* eps_virt_h, int mode, FreqPlan* out,
-                     std::vector<int>* counts = nullptr);
-// fn(q) for q = 0..n_q-1 on up to 8 host threads (fn must not share state
-// between q).
-void freq_parallel_q(int n_q, const std::function<void(int)>& fn);
+                     std::vector<int>* counts, int max_bins);
+// fn(i) for i = 0..n-1 on up to 12 host threads, handed out one by one (fn must
+// not share state between i).
+void freq_parallel(int n, const std::function<void(int)>& fn);
 // cnt[(jj n_occ + i) n_bins + b]: virtual states of row (k-pair jj, occupied
 // i) of q whose transition falls in bin b.  evs: virtual energies of every
 // k-point sorted ascending.
