@@ -219,48 +219,52 @@ __global__ void __launch_bounds__(256) erow_bin_kernel(int cplx, int Npad, int K
         __ldg(reinterpret_cast<const uint4*>(ewx + (long)g * Kt + u0) + c);
   }
   __syncthreads();
+  const uint32_t* ee2 = reinterpret_cast<const uint32_t*>(ees);  // two positions a word
   for (int rr = 0; rr < EROW_BIN_ROWS / 8; ++rr) {
     const int P = blockIdx.x * EROW_BIN_ROWS + rr * 8 + warp;
     if (P >= Npad) break;
-    int m[MR];
+    // maxima of two positions at a time as 16-bit halves; a zero value counts
+    // as bit length -8000, so that no sum of it passes the test below
+    uint32_t m[MR];
 #pragma unroll
-    for (int g = 0; g < MR; ++g) m[g] = -100000;
-    int* row = cfix + (long)P * Kr;
-    // EROW_ILP positions per lane per step: their loads are issued together
-    for (int ub = 0; ub < len; ub += 32 * EROW_ILP) {
-      int av[EROW_ILP];
+    for (int g = 0; g < MR; ++g) m[g] = 0x8AD08AD0u;  // (-30000, -30000)
+    int* row = cfix + (long)P * Kr + (long)(cplx ? 2 : 1) * u0;
+    // EROW_ILP pairs of positions per lane per step: their loads are issued together
+    for (int ub = 0; ub < len; ub += 64 * EROW_ILP) {
+      int4 av[EROW_ILP];
 #pragma unroll
       for (int k = 0; k < EROW_ILP; ++k) {
-        const int uu = ub + k * 32 + lane;
-        av[k] = 0;
-        if (uu < len && ees[uu] != -2000) {
-          const long u = u0 + uu;
-          if (cplx) {
-            const int2 v = *reinterpret_cast<const int2*>(row + 2 * u);
-            av[k] = max(abs(v.x), abs(v.y));
-          } else {
-            av[k] = abs(row[u]);
-          }
+        const int uu = ub + k * 64 + 2 * lane;
+        av[k] = make_int4(0, 0, 0, 0);
+        if (uu >= len) continue;
+        if (cplx) {
+          av[k] = *reinterpret_cast<const int4*>(row + 2 * uu);
+        } else {
+          const int2 v = *reinterpret_cast<const int2*>(row + uu);
+          av[k] = make_int4(v.x, 0, v.y, 0);
         }
       }
 #pragma unroll
       for (int k = 0; k < EROW_ILP; ++k) {
-        const int uu = ub + k * 32 + lane;
+        const int uu = ub + k * 64 + 2 * lane;
         if (uu >= len) break;
-        if (ees[uu] == -2000) {  // padding position
-          const long u = u0 + uu;
+        const uint32_t e0 = ee2[uu >> 1];
+        const bool pad0 = (int16_t)(e0 & 0xffff) == -2000, pad1 = (int16_t)(e0 >> 16) == -2000;
+        if (pad0 || pad1) {  // padding positions are zeroed
+          if (pad0) av[k].x = av[k].y = 0;
+          if (pad1) av[k].z = av[k].w = 0;
           if (cplx)
-            *reinterpret_cast<int2*>(row + 2 * u) = make_int2(0, 0);
+            *reinterpret_cast<int4*>(row + 2 * uu) = av[k];
           else
-            row[u] = 0;
-          continue;
+            *reinterpret_cast<int2*>(row + uu) = make_int2(av[k].x, av[k].z);
         }
-        if (av[k] == 0) continue;
-        const int bitlen = 32 - __clz(av[k]);
+        const int a0 = max(abs(av[k].x), abs(av[k].y)), a1 = max(abs(av[k].z), abs(av[k].w));
+        const int b0 = a0 ? 32 - __clz(a0) : -8000, b1 = a1 ? 32 - __clz(a1) : -8000;
+        const uint32_t bl = (uint32_t)(b0 & 0xffff) | ((uint32_t)b1 << 16);
 #pragma unroll
         for (int g = 0; g < MR; ++g) {
           if (g >= R) break;
-          m[g] = max(m[g], bitlen + (int)ees[g * len + uu]);
+          m[g] = __viaddmax_s16x2(bl, ee2[(g * len + uu) >> 1], m[g]);
         }
       }
     }
@@ -270,8 +274,8 @@ __global__ void __launch_bounds__(256) erow_bin_kernel(int cplx, int Npad, int K
 #pragma unroll
     for (int g = 0; g < MR; ++g) {
       if (g >= R) break;
-      const int r = __reduce_max_sync(0xffffffffu, m[g]);
-      if (lane == 0 && r > -100000) atomicMax(eAraw + ((long)b * rmax + g) * Npad + P, max(0, r + eC + 2014));
+      const int r = __reduce_max_sync(0xffffffffu, max((int)(int16_t)(m[g] & 0xffff), (int)m[g] >> 16));
+      if (lane == 0 && r > -5000) atomicMax(eAraw + ((long)b * rmax + g) * Npad + P, max(0, r + eC + 2014));
     }
   }
 }
@@ -308,7 +312,7 @@ struct RedBin {
   int wg;              // frequencies per group (grid y = groups)
 };
 constexpr int RED_WG = 10;
-constexpr int RED_GB = 3;  // skeletons in flight
+constexpr int RED_GB = 5;  // skeletons in flight
 
 // (h, l) += ph + pl: Knuth's TwoSum on the high parts, the errors gathered in l,
 // renormalised by ff_norm every few terms.
@@ -326,28 +330,47 @@ __device__ __forceinline__ void ff_norm(float& h, float& l) {
   h = s;
 }
 
-__global__ void __launch_bounds__(256, 2) reduce_bin_kernel(const __grid_constant__ RedBin rb) {
-  extern __shared__ float2 cs[];  // coefficients as (hi, lo) floats
-  const int ncoef = rb.nb * rb.rmax * rb.n_w;
-  for (int i = threadIdx.x; i < ncoef; i += blockDim.x) {
-    const double c = rb.coef[i];
+// (h, l) += (kx + ky)(x0 + x1): the product by Dekker's TwoProd (fmaf) with the
+// cross terms straight into l.
+__device__ __forceinline__ void ff_fma(float& h, float& l, float kx, float ky, float x0, float x1) {
+  const float p = __fmul_rn(kx, x0);
+  const float t = fmaf(kx, x0, -p);
+  l = fmaf(kx, x1, l);
+  l = fmaf(ky, x0, l);
+  const float s = __fadd_rn(h, p);
+  const float bb = __fsub_rn(s, h);
+  const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+  l = __fadd_rn(l, __fadd_rn(e, t));
+  h = s;
+}
+
+// WG: frequencies per group at most.  What bounds it is the FP32 pipe, 12
+// instructions per term, so the frequency loop is branch-free (coefficients past
+// the last frequency are zero) and RED_GB skeletons' loads are in flight.
+template <bool C, int WG>
+__global__ void __launch_bounds__(256, WG > 5 ? 2 : 3) reduce_bin_kernel(const __grid_constant__ RedBin rb) {
+  extern __shared__ float2 cs[];  // this group's coefficients as (hi, lo) floats, [skeleton][WG]
+  const int w0 = blockIdx.y * rb.wg, nw = min(rb.wg, rb.n_w - w0);
+  const int nsk = rb.nb * rb.rmax;
+  for (int i = threadIdx.x; i < nsk * WG; i += blockDim.x) {
+    const int sk = i / WG, w = i - sk * WG;
+    const double c = w < nw ? rb.coef[(long)sk * rb.n_w + w0 + w] : 0.0;
     const float h = (float)c;
     cs[i] = make_float2(h, (float)(c - (double)h));
   }
   __syncthreads();
-  const int ncols = rb.cplx ? 64 : 128;
-  const int per_tile = 128 * ncols / 256;
+  constexpr int ncols = C ? 64 : 128;
+  constexpr int per_tile = 128 * ncols / 256;
   const int tile = blockIdx.x / per_tile;
   const int e = (blockIdx.x - tile * per_tile) * 256 + threadIdx.x;
   const int r = e / ncols, c = e - (e / ncols) * ncols;
   int I, J;
-  tile_ij(rb.cplx, tile, I, J);
+  tile_ij(C, tile, I, J);
   const int P = I * 128 + r, Q = J * ncols + c;
   if (P >= rb.N || Q >= rb.N || Q > P) return;
-  const int w0 = blockIdx.y * rb.wg, nw = min(rb.wg, rb.n_w - w0);
-  float rh[RED_WG], rl[RED_WG], ih[RED_WG], il[RED_WG];
+  float rh[WG], rl[WG], ih[WG], il[WG];
 #pragma unroll
-  for (int w = 0; w < RED_WG; ++w) rh[w] = rl[w] = ih[w] = il[w] = 0.f;
+  for (int w = 0; w < WG; ++w) rh[w] = rl[w] = ih[w] = il[w] = 0.f;
   const int rq = rb.eCraw[Q];
   const int eCQ = rq ? rq - 1022 : -2000;
   const float* pr = rb.part + (long)r * 128 + c;
@@ -369,14 +392,14 @@ __global__ void __launch_bounds__(256, 2) reduce_bin_kernel(const __grid_constan
         // x = sum over the split-K partials of (hi + lo), as a float-float pair
         xh[u] = pp[0];
         xl[u] = pp[128 * 128];
-        if (rb.cplx) {
+        if constexpr (C) {
           yh[u] = pp[64];
           yl[u] = pp[128 * 128 + 64];
         }
         for (int ks = 1; ks < rb.nks[b]; ++ks) {
           pp += (long)Gs * rb.n_tiles * (2 * 128 * 128);
           ff_acc(xh[u], xl[u], pp[0], pp[128 * 128]);
-          if (rb.cplx) ff_acc(yh[u], yl[u], pp[64], pp[128 * 128 + 64]);
+          if constexpr (C) ff_acc(yh[u], yl[u], pp[64], pp[128 * 128 + 64]);
         }
       }
 #pragma unroll
@@ -386,34 +409,27 @@ __global__ void __launch_bounds__(256, 2) reduce_bin_kernel(const __grid_constan
         const int sh = (ra[u] - 2044 + 1) + eCQ + 1 - 14;
         const float x0 = -ldexpf(xh[u], sh), x1 = -ldexpf(xl[u], sh);
         const float y0 = -ldexpf(yh[u], sh), y1 = -ldexpf(yl[u], sh);
-        const float2* cf = cs + ((long)b * rb.rmax + gb + u) * rb.n_w + w0;
+        const float2* cf = cs + (b * rb.rmax + gb + u) * WG;
 #pragma unroll
-        for (int w = 0; w < RED_WG; ++w) {
-          if (w >= nw) break;
+        for (int w = 0; w < WG; ++w) {
           const float2 k = cf[w];
-          float ph = __fmul_rn(k.x, x0);
-          float pl = __fadd_rn(fmaf(k.x, x0, -ph), fmaf(k.x, x1, __fmul_rn(k.y, x0)));
-          ff_acc(rh[w], rl[w], ph, pl);
-          if (rb.cplx) {
-            ph = __fmul_rn(k.x, y0);
-            pl = __fadd_rn(fmaf(k.x, y0, -ph), fmaf(k.x, y1, __fmul_rn(k.y, y0)));
-            ff_acc(ih[w], il[w], ph, pl);
-          }
+          ff_fma(rh[w], rl[w], k.x, k.y, x0, x1);
+          if constexpr (C) ff_fma(ih[w], il[w], k.x, k.y, y0, y1);
         }
       }
 #pragma unroll
-      for (int w = 0; w < RED_WG; ++w) {
+      for (int w = 0; w < WG; ++w) {
         ff_norm(rh[w], rl[w]);
-        ff_norm(ih[w], il[w]);
+        if constexpr (C) ff_norm(ih[w], il[w]);
       }
     }
   }
   const long NN = (long)rb.N * rb.N;
 #pragma unroll
-  for (int w = 0; w < RED_WG; ++w) {
+  for (int w = 0; w < WG; ++w) {
     if (w >= nw) break;
     const double re = (double)rh[w] + (double)rl[w];
-    if (rb.cplx) {
+    if constexpr (C) {
       double2* out = reinterpret_cast<double2*>(rb.chi) + (long)(w0 + w) * NN;
       const double im = P == Q ? 0.0 : (double)ih[w] + (double)il[w];
       out[(long)P * rb.N + Q] = make_double2(re, im);
@@ -423,6 +439,36 @@ __global__ void __launch_bounds__(256, 2) reduce_bin_kernel(const __grid_constan
       out[(long)P * rb.N + Q] = re;
       if (P != Q) out[(long)Q * rb.N + P] = re;
     }
+  }
+}
+
+template <int WG>
+void launch_reduce_wg(const RedBin& rb, dim3 grid, cudaStream_t st) {
+  const size_t smem = sizeof(float2) * (size_t)rb.nb * rb.rmax * WG;
+  if (rb.cplx)
+    reduce_bin_kernel<true, WG><<<grid, 256, smem, st>>>(rb);
+  else
+    reduce_bin_kernel<false, WG><<<grid, 256, smem, st>>>(rb);
+}
+// Groups of at most RED_WG frequencies, as even as they come.
+void launch_reduce_bin(RedBin& rb, cudaStream_t st) {
+  const int per_tile = 128 * (rb.cplx ? 64 : 128) / 256;
+  const int n_groups = (rb.n_w + RED_WG - 1) / RED_WG;
+  rb.wg = (rb.n_w + n_groups - 1) / n_groups;
+  const dim3 grid((unsigned)(rb.n_tiles * per_tile), (unsigned)n_groups);
+  switch (rb.wg) {
+    case 10:
+      return launch_reduce_wg<10>(rb, grid, st);
+    case 9:
+      return launch_reduce_wg<9>(rb, grid, st);
+    case 8:
+      return launch_reduce_wg<8>(rb, grid, st);
+    case 7:
+      return launch_reduce_wg<7>(rb, grid, st);
+    case 6:
+      return launch_reduce_wg<6>(rb, grid, st);
+    default:
+      return launch_reduce_wg<5>(rb, grid, st);
   }
 }
 
@@ -861,12 +907,8 @@ cudaError_t launch_chi0_binned(const MixedBinQ* qs, int n, const FreqPlan& p, in
       rb.eCraw = C.eC;
       rb.coef = C.meta_d + (size_t)p.n_bins * L.rmax;
       rb.chi = q.chi;
-      const int per_tile = 128 * (q.g.cplx ? 64 : 128) / 256;
-      const int n_groups = (q.g.n_w + RED_WG - 1) / RED_WG;
-      rb.wg = (q.g.n_w + n_groups - 1) / n_groups;
       hb();
-      reduce_bin_kernel<<<dim3((unsigned)(L.n_tiles * per_tile), (unsigned)n_groups), 256,
-                          sizeof(float2) * (size_t)p.n_bins * L.rmax * q.g.n_w, st>>>(rb);
+      launch_reduce_bin(rb, st);
       he(RPA_K_CHI0_RED, 1);
       ++nl;
     }
