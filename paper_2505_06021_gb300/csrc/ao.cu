@@ -147,7 +147,8 @@ const double* ao_mo(const rpa_job* j, const AoPlan& p, const char* region, int k
   return (const double*)j->ao->mo[k];
 }
 
-rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p, char* region, cudaStream_t s) {
+rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p, char* region, cudaStream_t s,
+                      char* gws) {
   const rpa_ao* a = j->ao;
   if (!a->overlap) return RPA_OK;
   std::vector<const double*> c(j->n_kpts);
@@ -157,7 +158,7 @@ rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p
     out[k] = (double*)(region + p.off_cproj + p.cproj_bytes * (size_t)k);
   }
   return run_projector(ctx, pex, j->is_complex, j->n_kpts, p.n_bas, a->n_mo, a->overlap, c.data(), out.data(),
-                       a->eps_d, region + p.off_proj, s, nullptr, nullptr);
+                       a->eps_d, region + p.off_proj, s, nullptr, nullptr, gws ? gws + 1024 : nullptr);
 }
 
 // ------------------------------------------------ digit products ----------
@@ -251,6 +252,10 @@ AoG64 ao_g64_plan(const rpa_job* j, const AoPlan& p) {
   const std::vector<AoAtom> at = ao_atoms(j->ao);
   for (const AoAtom& t : at) nb_min = std::min(nb_min, t.nb);
   g.assemble = nb_min * cm >= 32 && f * 2.0 * p.S * j->n_occ * (double)j->n_virt * j->n_k >= 2e8 * at.size();
+  if (j->ao->overlap) {  // the projector's fast start uses the region before the transforms
+    const size_t f = proj_fast_bytes(c, j->n_kpts, p.n_bas);
+    if (f) g.bytes = 1024 + f;
+  }
   if (!g.half && !g.assemble) return g;
   if (g.half) {
     g.rows = p.S;
@@ -275,7 +280,7 @@ AoG64 ao_g64_plan(const rpa_job* j, const AoPlan& p) {
   g.a = (g.a + 1023) & ~(size_t)1023;
   g.b = (g.b + 1023) & ~(size_t)1023;
   g.e = (g.e + 1023) & ~(size_t)1023;
-  g.bytes = 1024 + g.a + g.b + 2 * g.e;
+  g.bytes = std::max(g.bytes, 1024 + g.a + g.b + 2 * g.e);
   return g;
 }
 

@@ -52,7 +52,8 @@ rpa_status ao_enqueue_half(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPl
                            cudaStream_t s, char* gws = nullptr, int* status = nullptr);
 // With overlap matrices: the periodic projector's c~ of every k-point into the
 // region (synchronises s); without: nothing.
-rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p, char* region, cudaStream_t s);
+rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p, char* region, cudaStream_t s,
+                      char* gws = nullptr);
 // The MO coefficients the transform uses for k-point k (c~ or the job's c).
 const double* ao_mo(const rpa_job* j, const AoPlan& p, const char* region, int k);
 // C(q, k_j), j = 0..n_k-1, into out + j * cblk (half-transforms in place).

@@ -823,7 +823,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
     }
   }
   if (job->ao) {
-    if (rpa_status st1 = ao_project(ctx, &ex, job, aop, b.ao, s)) return st1;
+    if (rpa_status st1 = ao_project(ctx, &ex, job, aop, b.ao, s, b.aog)) return st1;
     if (rpa_status st1 = ao_enqueue_half(ctx, &ex, job, aop, b.ao, -1, s, b.aog, b.status)) return st1;
   }
 
@@ -1062,7 +1062,7 @@ rpa_status rpa_chi0(rpa_ctx* ctx, const rpa_job* job, int q, void* chi_out, void
   CK(cudaEventRecord(ex.done, ex.s));
   CK(cudaStreamWaitEvent(s, ex.done, 0));
   if (job->ao) {
-    if (rpa_status st1 = ao_project(ctx, &ex, job, aop, b.ao, s)) return st1;
+    if (rpa_status st1 = ao_project(ctx, &ex, job, aop, b.ao, s, b.aog)) return st1;
     if (rpa_status st1 = ao_enqueue_half(ctx, &ex, job, aop, b.ao, q, s, b.aog, b.status)) return st1;
     if (rpa_status st1 = ao_enqueue_assemble(ctx, &ex, job, aop, b.ao, q, b.ao + aop.off_c, s, b.aog, b.status))
       return st1;
@@ -1106,8 +1106,8 @@ rpa_status rpa_ao2mo(rpa_ctx* ctx, const rpa_job* job, int q, void* C_out, void*
     return RPA_E_NOMEM;
   }
   char* region = (char*)ex.ws;
-  if (rpa_status st = ao_project(ctx, &ex, job, aop, region, s)) return st;
   char* gws = gb ? region + base : nullptr;
+  if (rpa_status st = ao_project(ctx, &ex, job, aop, region, s, gws)) return st;
   int* status = gws ? (int*)(gws + 512) : nullptr;
   ex.status_word() = 0;
   if (status) CK(cudaMemsetAsync(status, 0, sizeof(int), s));

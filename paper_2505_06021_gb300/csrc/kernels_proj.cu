@@ -9,14 +9,23 @@
 // eps/gap even for the tiny eigenvalues the projector removes).  A sweep is
 // Np - 1 rounds of the round-robin (circle) ordering of Np columns (Np = N
 // rounded up to even, a zero padding column); a round rotates Np/2 disjoint
-// column pairs, one CTA per (k-point, pair), so a launch has no inter-CTA
-// dependency and a round is one kernel launch.  Per pair: alpha = |w_p|^2,
-// beta = |w_q|^2, gamma = w_p^H w_q by a block reduction; with
+// column pairs, a CTA or a warp per (k-point, pair), so a launch has no
+// inter-CTA dependency and a round is one kernel launch.  Per pair: alpha =
+// |w_p|^2, beta = |w_q|^2, gamma = w_p^H w_q; with
 // e = conj(gamma)/|gamma|, zeta = (beta - alpha)/(2|gamma|),
 // t = sign(zeta)/(|zeta| + sqrt(1 + zeta^2)), c = 1/sqrt(1 + t^2), s = c t:
 //   w_p <- c w_p - s e w_q,   w_q <- s w_p + c e w_q,
 // which makes the pair orthogonal (the 2 x 2 Hermitian Jacobi rotation).  The
 // largest |gamma|/sqrt(alpha beta) of a sweep decides convergence on the host.
+//
+// Start of the iteration (proj.cu, bases of some size): the sweeps above begin
+// from eigenvectors of nearly full accuracy instead of I.  One-sided Jacobi in FP32
+// (its pipe is 64 times the FP64 one) gives them to about 1e-6; they are
+// refined by matrix products on the tensor cores (g64.cu): Newton-Schulz steps
+// V <- V - V (V^H V - I) / 2 for orthonormality, and first-order corrections
+// V <- V + V E, E_ij = (V^H S V)_ij / (lambda_j - lambda_i) where that is small (the
+// quadratically convergent refinement of Ogita and Aishima, 2018, without its
+// cluster step: what it leaves, the FP64 sweeps finish).
 //
 // Since the eigenvalues are taken in ascending order and R~ is a product over
 // k, R~ removes the m lowest positions at every k-point, m the largest count
@@ -24,6 +33,8 @@
 // eigenvectors of S(k).
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "fp64_elem.cuh"
 #include "rpa_internal.h"
@@ -84,21 +95,25 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// One round r: CTA (pair i, k-point k) rotates columns (p, q) of W[k].
+// The 2 x 2 rotation that makes columns with norms^2 a, b and inner product g
+// orthogonal: c, s, e = conj(g)/|g|.
+__device__ __forceinline__ void pair_rotation(double a, double b, double gr, double gi, double g, double& c, double& s,
+                                              double& er, double& ei) {
+  const double zeta = (b - a) / (2.0 * g);
+  const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+  c = 1.0 / sqrt(1.0 + t * t);
+  s = c * t;
+  er = gr / g;
+  ei = -gi / g;
+}
+
+// |x|^2, |y|^2, conj(x) y over this thread's share of two columns.
 template <bool C>
-__global__ void __launch_bounds__(256) jacobi_round_kernel(int N, int Np, int r, double* __restrict__ W,
-                                                           double* __restrict__ V, double thresh,
-                                                           unsigned long long* __restrict__ off_max) {
-  __shared__ double red[8][4];
-  __shared__ double rot[5];  // c, s, e (re, im), applied flag
-  const int i = blockIdx.x, k = blockIdx.y;
-  int p, q;
-  round_pair(Np, r, i, p, q);
-  double* wp = W + ((size_t)k * Np + p) * N * (C ? 2 : 1);
-  double* wq = W + ((size_t)k * Np + q) * N * (C ? 2 : 1);
-  double a = 0.0, b = 0.0, gr = 0.0, gi = 0.0;
-  for (int mu = threadIdx.x; mu < N; mu += blockDim.x) {
-    const Elem<C> x = ld_elem<C>(wp, mu), y = ld_elem<C>(wq, mu);
+__device__ __forceinline__ void pair_dots(const double* xc, const double* yc, int N, int first, int step, double& a,
+                                          double& b, double& gr, double& gi) {
+  a = b = gr = gi = 0.0;
+  for (int mu = first; mu < N; mu += step) {
+    const Elem<C> x = ld_elem<C>(xc, mu), y = ld_elem<C>(yc, mu);
     if constexpr (C) {
       a = fma(x.re, x.re, fma(x.im, x.im, a));
       b = fma(y.re, y.re, fma(y.im, y.im, b));
@@ -113,8 +128,13 @@ __global__ void __launch_bounds__(256) jacobi_round_kernel(int N, int Np, int r,
   a = warp_sum(a);
   b = warp_sum(b);
   gr = warp_sum(gr);
-  gi = warp_sum(gi);
+  if constexpr (C) gi = warp_sum(gi);
+}
+
+// Sums of the four values over the CTA's warps, valid in every thread.
+__device__ __forceinline__ void cta_join(double (*red)[4], double& a, double& b, double& gr, double& gi) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();  // red is free again
   if (lane == 0) {
     red[wid][0] = a;
     red[wid][1] = b;
@@ -122,39 +142,270 @@ __global__ void __launch_bounds__(256) jacobi_round_kernel(int N, int Np, int r,
     red[wid][3] = gi;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    a = b = gr = gi = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      a += red[w][0];
-      b += red[w][1];
-      gr += red[w][2];
-      gi += red[w][3];
-    }
-    const double g = sqrt(gr * gr + gi * gi);
-    const double off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
-    atomicMax(off_max, (unsigned long long)__double_as_longlong(off));
-    if (off > thresh) {
-      const double zeta = (b - a) / (2.0 * g);
-      const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-      const double c = 1.0 / sqrt(1.0 + t * t);
-      rot[0] = c;
-      rot[1] = c * t;
-      rot[2] = gr / g;  // e = conj(gamma) / |gamma|
-      rot[3] = -gi / g;
-      rot[4] = 1.0;
-    } else {
-      rot[4] = 0.0;
-    }
+  a = b = gr = gi = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    a += red[w][0];
+    b += red[w][1];
+    gr += red[w][2];
+    gi += red[w][3];
   }
-  __syncthreads();
-  if (rot[4] == 0.0) return;
-  const double c = rot[0], s = rot[1], er = rot[2], ei = rot[3];
+}
+
+// One round r: columns (p, q) of pair i of W[k] are rotated, by a CTA each
+// (WARP = false) or, when the pairs of all k-points fill the GPU, by a warp each,
+// four to a CTA: no barriers, and once most pairs are orthogonal a round is
+// the FP64 pipe's time for the inner products.
+template <bool C, bool WARP>
+__global__ void __launch_bounds__(WARP ? 128 : 256) jacobi_round_kernel(int N, int Np, int r, double* __restrict__ W,
+                                                                        double* __restrict__ V, double thresh,
+                                                                        unsigned long long* __restrict__ off_max) {
+  __shared__ double red[8][4];
+  const int lane = threadIdx.x & 31, k = blockIdx.y;
+  const int i = WARP ? blockIdx.x * 4 + (threadIdx.x >> 5) : blockIdx.x;
+  if (i >= Np / 2) return;
+  int p, q;
+  round_pair(Np, r, i, p, q);
+  double* wp = W + ((size_t)k * Np + p) * N * (C ? 2 : 1);
+  double* wq = W + ((size_t)k * Np + q) * N * (C ? 2 : 1);
+  const int first = WARP ? lane : threadIdx.x, step = WARP ? 32 : 256;
+  double a, b, gr, gi;
+  pair_dots<C>(wp, wq, N, first, step, a, b, gr, gi);
+  if constexpr (!WARP) cta_join(red, a, b, gr, gi);
+  const double g = sqrt(gr * gr + gi * gi);
+  const double off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
+  if (first == 0) atomicMax(off_max, (unsigned long long)__double_as_longlong(off));
+  if (!(off > thresh)) return;
+  double c, s, er, ei;
+  pair_rotation(a, b, gr, gi, g, c, s, er, ei);
   double* vp = V + ((size_t)k * Np + p) * N * (C ? 2 : 1);
   double* vq = V + ((size_t)k * Np + q) * N * (C ? 2 : 1);
-  for (int mu = threadIdx.x; mu < N; mu += blockDim.x) {
+  for (int mu = first; mu < N; mu += step) {
     rotate_pair<C>(wp, wq, mu, c, s, er, ei);
     rotate_pair<C>(vp, vq, mu, c, s, er, ei);
   }
+}
+
+// The few columns that the refinement could not tell apart (the eigenvalues
+// far below FP32's resolution, near-degenerate ones): those with a cosine
+// above 1e-3 in G = W^H W, swept among themselves, one CTA per k-point.  More
+// than CLUSTER_MAX are left to the sweeps over all columns.
+constexpr int CLUSTER_MAX = 12;
+template <bool C>
+__global__ void __launch_bounds__(256) proj_cluster_kernel(int N, int Np, const double* __restrict__ G,
+                                                           double* __restrict__ W, double* __restrict__ V,
+                                                           double thresh) {
+  __shared__ double red[8][4];
+  __shared__ int list[CLUSTER_MAX], cnt;
+  extern __shared__ unsigned char mark[];
+  const int k = blockIdx.x, tid = threadIdx.x;
+  const double* g = G + (size_t)k * N * N * (C ? 2 : 1);
+  for (int j = tid; j < N; j += 256) mark[j] = 0;
+  __syncthreads();
+  for (int j = 0; j < N; ++j) {
+    const double gj = ld_elem<C>(g, (long)j * N + j).re;
+    for (int i = tid; i < N; i += 256) {
+      if (i == j) continue;
+      const Elem<C> x = ld_elem<C>(g, (long)j * N + i);
+      double v = x.re * x.re;
+      if constexpr (C) v += x.im * x.im;
+      if (v > 1e-6 * gj * ld_elem<C>(g, (long)i * N + i).re) mark[i] = 1;  // (j is marked as i's partner)
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    int n = 0;
+    for (int j = 0; j < N; ++j)
+      if (mark[j]) {
+        if (n < CLUSTER_MAX) list[n] = j;
+        ++n;
+      }
+    cnt = n;
+  }
+  __syncthreads();
+  if (cnt < 2 || cnt > CLUSTER_MAX) return;
+  double* wk = W + (size_t)k * Np * N * (C ? 2 : 1);
+  double* vk = V + (size_t)k * Np * N * (C ? 2 : 1);
+  for (int sweep = 0; sweep < 12; ++sweep) {
+    double worst = 0.0;
+    for (int u = 0; u < cnt; ++u)
+      for (int v = u + 1; v < cnt; ++v) {
+        const long op = (long)list[u] * N * (C ? 2 : 1), oq = (long)list[v] * N * (C ? 2 : 1);
+        double a, b, gr, gi;
+        pair_dots<C>(wk + op, wk + oq, N, tid, 256, a, b, gr, gi);
+        cta_join(red, a, b, gr, gi);
+        const double h = sqrt(gr * gr + gi * gi);
+        const double off = (a > 0.0 && b > 0.0) ? h / sqrt(a * b) : 0.0;
+        worst = fmax(worst, off);
+        if (!(off > thresh)) continue;
+        double c, s, er, ei;
+        pair_rotation(a, b, gr, gi, h, c, s, er, ei);
+        for (int mu = tid; mu < N; mu += 256) {  // a thread's own elements: no barrier between pairs
+          rotate_pair<C>(wk + op, wk + oq, mu, c, s, er, ei);
+          rotate_pair<C>(vk + op, vk + oq, mu, c, s, er, ei);
+        }
+      }
+    if (worst <= 1e-14) break;
+  }
+}
+
+// ---- FP32 start ----
+
+template <bool C>
+struct Flt;
+template <>
+struct Flt<true> {
+  float re, im;
+};
+template <>
+struct Flt<false> {
+  float re;
+};
+
+// Sum of squares of S(k) (W, N columns of N), one CTA per k-point, fixed order.
+template <bool C>
+__global__ void __launch_bounds__(256) proj_norm_kernel(int N, int Np, const double* __restrict__ W,
+                                                        float* __restrict__ scale) {
+  __shared__ double red[8];
+  const double* w = W + (size_t)blockIdx.x * Np * N * (C ? 2 : 1);
+  const long n = (long)N * N * (C ? 2 : 1);
+  float s = 0.f;
+  for (long i = threadIdx.x; i < n; i += 256) {
+    const float x = (float)w[i];
+    s = fmaf(x, x, s);
+  }
+  const double t = warp_sum((double)s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double u = 0.0;
+    for (int i = 0; i < 8; ++i) u += red[i];
+    scale[blockIdx.x] = (float)(1.0 / sqrt(u / N));  // columns of norm about 1
+  }
+}
+
+// W32 = scale S, V32 = I (Np columns of N each, as in FP64).
+template <bool C>
+__global__ void __launch_bounds__(256) proj_load32_kernel(int N, int Np, const double* __restrict__ W,
+                                                          const float* __restrict__ scale, float* __restrict__ W32,
+                                                          float* __restrict__ V32) {
+  const int k = blockIdx.y, j = blockIdx.x;
+  const size_t c0 = ((size_t)k * Np + j) * N * (C ? 2 : 1);
+  const float sc = scale[k];
+  for (int i = threadIdx.x; i < N * (C ? 2 : 1); i += blockDim.x) {
+    W32[c0 + i] = (float)W[c0 + i] * sc;
+    V32[c0 + i] = i == (C ? 2 : 1) * j ? 1.f : 0.f;
+  }
+}
+
+// One round of the FP32 sweeps: a warp per column pair and k-point.  Columns
+// below 1e-6 of the typical norm (FP32 noise) count as that long.
+template <bool C>
+__global__ void __launch_bounds__(128) jacobi32_round_kernel(int N, int Np, int r, float* __restrict__ W32,
+                                                             float* __restrict__ V32, float thresh,
+                                                             unsigned* __restrict__ off_max) {
+  const int lane = threadIdx.x & 31, i = blockIdx.x * 4 + (threadIdx.x >> 5), k = blockIdx.y;
+  if (i >= Np / 2) return;
+  int p, q;
+  round_pair(Np, r, i, p, q);
+  const size_t m0 = (size_t)k * Np * N * (C ? 2 : 1);
+  Flt<C>* wp = reinterpret_cast<Flt<C>*>(W32 + m0) + (size_t)p * N;
+  Flt<C>* wq = reinterpret_cast<Flt<C>*>(W32 + m0) + (size_t)q * N;
+  float a = 0.f, b = 0.f, gr = 0.f, gi = 0.f;
+  for (int mu = lane; mu < N; mu += 32) {
+    const Flt<C> x = wp[mu], y = wq[mu];
+    a = fmaf(x.re, x.re, a);
+    b = fmaf(y.re, y.re, b);
+    gr = fmaf(x.re, y.re, gr);
+    if constexpr (C) {
+      a = fmaf(x.im, x.im, a);
+      b = fmaf(y.im, y.im, b);
+      gr = fmaf(x.im, y.im, gr);
+      gi = fmaf(x.re, y.im, fmaf(-x.im, y.re, gi));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+    gr += __shfl_xor_sync(0xffffffffu, gr, o);
+    if constexpr (C) gi += __shfl_xor_sync(0xffffffffu, gi, o);
+  }
+  const float g = sqrtf(gr * gr + gi * gi);
+  const float off = g / sqrtf(fmaxf(a, 1e-12f) * fmaxf(b, 1e-12f));
+  if (lane == 0) atomicMax(off_max, __float_as_uint(off));
+  if (!(off > thresh)) return;  // (a NaN ends here too: the start is then rejected)
+  const float zeta = (b - a) / (2.f * g);
+  const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
+  const float c = rsqrtf(1.f + t * t), s = c * t, er = gr / g, ei = -gi / g;
+  auto rot = [&](Flt<C>* xc, Flt<C>* yc) {
+    for (int mu = lane; mu < N; mu += 32) {
+      const Flt<C> x = xc[mu], y = yc[mu];
+      Flt<C> xn, yn;
+      if constexpr (C) {
+        const float eyr = er * y.re - ei * y.im, eyi = er * y.im + ei * y.re;
+        xn.re = c * x.re - s * eyr;
+        xn.im = c * x.im - s * eyi;
+        yn.re = s * x.re + c * eyr;
+        yn.im = s * x.im + c * eyi;
+      } else {
+        xn.re = c * x.re - s * er * y.re;
+        yn.re = s * x.re + c * er * y.re;
+      }
+      xc[mu] = xn;
+      yc[mu] = yn;
+    }
+  };
+  rot(wp, wq);
+  rot(reinterpret_cast<Flt<C>*>(V32 + m0) + (size_t)p * N, reinterpret_cast<Flt<C>*>(V32 + m0) + (size_t)q * N);
+}
+
+__global__ void __launch_bounds__(256) proj_widen_kernel(long n, const float* __restrict__ x, double* __restrict__ y) {
+  for (long i = blockIdx.x * 256L + threadIdx.x; i < n; i += gridDim.x * 256L) y[i] = (double)x[i];
+}
+
+// In place over column j of M(k) (N x N at a stride N^2): ORTHO: -(M - I) / 2,
+// the largest |M - I| into *dev; else the correction
+// E_ij = M_ij / (M_jj - M_ii) where it is below 0.02, zero elsewhere (diag: the
+// M_ii, saved before the launch).
+template <bool C, bool ORTHO>
+__global__ void __launch_bounds__(256) proj_corr_kernel(int N, double* __restrict__ M, const double* __restrict__ diag,
+                                                        unsigned* __restrict__ dev) {
+  const int k = blockIdx.y, j = blockIdx.x;
+  double* col = M + ((size_t)k * N + j) * N * (C ? 2 : 1);
+  const double lj = ORTHO ? 0.0 : diag[(size_t)k * N + j];
+  float dm = 0.f;
+  bool bad = false;
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    Elem<C> e = ld_elem<C>(col, i);
+    double f;
+    if constexpr (ORTHO) {
+      if (i == j) e.re -= 1.0;
+      f = -0.5;
+      float v = fabsf((float)e.re);
+      if constexpr (C) v = fmaxf(v, fabsf((float)e.im));
+      dm = fmaxf(dm, v);
+      bad |= !(v < 1e30f);
+    } else {
+      const double gap = lj - diag[(size_t)k * N + i];
+      float v = fabsf((float)e.re);
+      if constexpr (C) v = fmaxf(v, fabsf((float)e.im));
+      f = i != j && v < 0.02f * fabsf((float)gap) ? 1.0 / gap : 0.0;
+    }
+    e.re *= f;
+    if constexpr (C) e.im *= f;
+    st_elem<C>(col, i, e);
+  }
+  if constexpr (ORTHO) {
+    if (bad) dm = __int_as_float(0x7f800000);
+    dm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dm)));
+    if ((threadIdx.x & 31) == 0) atomicMax(dev, __float_as_uint(dm));
+  }
+}
+
+template <bool C>
+__global__ void __launch_bounds__(256) proj_diag_kernel(int N, const double* __restrict__ M, double* __restrict__ diag) {
+  const int k = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
+  if (i < N) diag[(size_t)k * N + i] = ld_elem<C>(M + (size_t)k * N * N * (C ? 2 : 1), (long)i * N + i).re;
 }
 
 // Per k-point: eigenvalue of column j = |w_j|, ascending rank (ties by index),
@@ -254,13 +505,82 @@ cudaError_t launch_proj_load(int cplx, const ProjPtrs& P, int n_mat, int N, int 
   return cudaGetLastError();
 }
 
+cudaError_t launch_proj_load32(int cplx, int n_mat, int N, int Np, const double* W, float* scale, float* W32, float* V32,
+                               cudaStream_t s) {
+  const dim3 grid(Np, n_mat);
+  if (cplx) {
+    proj_norm_kernel<true><<<n_mat, 256, 0, s>>>(N, Np, W, scale);
+    proj_load32_kernel<true><<<grid, 256, 0, s>>>(N, Np, W, scale, W32, V32);
+  } else {
+    proj_norm_kernel<false><<<n_mat, 256, 0, s>>>(N, Np, W, scale);
+    proj_load32_kernel<false><<<grid, 256, 0, s>>>(N, Np, W, scale, W32, V32);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_jacobi32_round(int cplx, int n_mat, int N, int Np, int r, float* W32, float* V32, float thresh,
+                                  unsigned* off_max, cudaStream_t s) {
+  const dim3 grid((Np / 2 + 3) / 4, n_mat);
+  if (cplx)
+    jacobi32_round_kernel<true><<<grid, 128, 0, s>>>(N, Np, r, W32, V32, thresh, off_max);
+  else
+    jacobi32_round_kernel<false><<<grid, 128, 0, s>>>(N, Np, r, W32, V32, thresh, off_max);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_proj_widen(long n, const float* x, double* y, cudaStream_t s) {
+  proj_widen_kernel<<<(unsigned)std::min<long>((n + 255) / 256, (long)device_sm_count() * 8), 256, 0, s>>>(n, x, y);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_proj_corr(int cplx, int n_mat, int N, bool ortho, double* M, double* diag, unsigned* dev,
+                             cudaStream_t s) {
+  const dim3 grid(N, n_mat), gd((N + 255) / 256, n_mat);
+  if (!ortho) {
+    if (cplx)
+      proj_diag_kernel<true><<<gd, 256, 0, s>>>(N, M, diag);
+    else
+      proj_diag_kernel<false><<<gd, 256, 0, s>>>(N, M, diag);
+  }
+  if (cplx) {
+    if (ortho)
+      proj_corr_kernel<true, true><<<grid, 256, 0, s>>>(N, M, diag, dev);
+    else
+      proj_corr_kernel<true, false><<<grid, 256, 0, s>>>(N, M, diag, dev);
+  } else {
+    if (ortho)
+      proj_corr_kernel<false, true><<<grid, 256, 0, s>>>(N, M, diag, dev);
+    else
+      proj_corr_kernel<false, false><<<grid, 256, 0, s>>>(N, M, diag, dev);
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t launch_jacobi_round(int cplx, int n_mat, int N, int Np, int r, double* W, double* V, double thresh,
                                 unsigned long long* off_max, cudaStream_t s) {
-  const dim3 grid(Np / 2, n_mat);
+  // a warp per pair from eight pairs per SM on
+  if ((long)Np / 2 * n_mat >= 8L * device_sm_count()) {
+    const dim3 grid((Np / 2 + 3) / 4, n_mat);
+    if (cplx)
+      jacobi_round_kernel<true, true><<<grid, 128, 0, s>>>(N, Np, r, W, V, thresh, off_max);
+    else
+      jacobi_round_kernel<false, true><<<grid, 128, 0, s>>>(N, Np, r, W, V, thresh, off_max);
+  } else {
+    const dim3 grid(Np / 2, n_mat);
+    if (cplx)
+      jacobi_round_kernel<true, false><<<grid, 256, 0, s>>>(N, Np, r, W, V, thresh, off_max);
+    else
+      jacobi_round_kernel<false, false><<<grid, 256, 0, s>>>(N, Np, r, W, V, thresh, off_max);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_proj_cluster(int cplx, int n_mat, int N, int Np, const double* G, double* W, double* V, double thresh,
+                                cudaStream_t s) {
   if (cplx)
-    jacobi_round_kernel<true><<<grid, 256, 0, s>>>(N, Np, r, W, V, thresh, off_max);
+    proj_cluster_kernel<true><<<n_mat, 256, N, s>>>(N, Np, G, W, V, thresh);
   else
-    jacobi_round_kernel<false><<<grid, 256, 0, s>>>(N, Np, r, W, V, thresh, off_max);
+    proj_cluster_kernel<false><<<n_mat, 256, N, s>>>(N, Np, G, W, V, thresh);
   return cudaGetLastError();
 }
 

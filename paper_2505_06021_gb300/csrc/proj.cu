@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "g64.h"
 #include "proj_internal.h"
 #include "rpa_internal.h"
 #include "rpa_runtime.h"
@@ -33,9 +34,183 @@ ProjLayout proj_layout(int cplx, int n_mat, int N, int n_mo) {
   return L;
 }
 
+// ------------------------------------------------------- fast start -------
+
+namespace {
+
+// S, one N x N product per k-point, the FP32 columns (W32, V32), diagonals,
+// flags, and the digit planes of a group of k-points.
+struct FastLayout {
+  size_t S, M, f32, diag, flags, ea, eb, pa, pb, bytes;
+  int group;
+};
+FastLayout fast_layout(int cplx, int n_mat, int N) {
+  FastLayout L{};
+  const size_t es = cplx ? 16 : 8, Np = N + (N & 1);
+  L.S = 0;
+  L.M = L.S + al256(es * n_mat * Np * N);
+  L.f32 = L.M + al256(es * n_mat * N * N);
+  L.diag = L.f32 + 2 * al256(es / 2 * n_mat * Np * N);
+  L.flags = L.diag + al256(sizeof(double) * n_mat * N);
+  const size_t a = g64_plane_bytes(cplx, 0, N, N, 1), b = g64_plane_bytes(cplx, 1, N, N, 1);
+  L.group = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_mat, ((size_t)512 << 20) / (a + b)));
+  L.ea = L.flags + 256 + al256(sizeof(float) * n_mat);
+  L.eb = L.ea + al256(sizeof(int) * (size_t)L.group * g64_rpad(cplx, 0, N));
+  L.pa = (L.eb + al256(sizeof(int) * (size_t)L.group * g64_rpad(cplx, 1, N)) + 1023) & ~(size_t)1023;
+  L.pb = L.pa + a * L.group;
+  L.bytes = L.pb + b * L.group;
+  return L;
+}
+
+constexpr int kSweeps32 = 14;
+
+}  // namespace
+
+// Bases below 64 functions need some 60 rounds a sweep: the FP64 sweeps take
+// less than the start's launches.
+size_t proj_fast_bytes(int cplx, int n_mat, int N) {
+  if (N < 64) return 0;
+  const size_t b = fast_layout(cplx, n_mat, N).bytes;
+  return b <= ((size_t)4 << 30) ? b : 0;
+}
+
+// V: eigenvectors of S (= W on entry) to nearly FP64 accuracy, W = S V.  The FP64
+// sweeps from V = I took 13 sweeps of 16 ms on 16 overlaps of 256 functions (208
+// ms); with this start three are left, whose rounds are mostly inner products: 50
+// ms in all.
+// *ok = false (W = S and V = I as before) when the start did not give an
+// orthonormal V: entries out of the FP32 range, no convergence.
+static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, double* W, double* V,
+                             const ProjPtrs& P, char* ws, cudaStream_t s, bool* ok) {
+  const FastLayout L = fast_layout(cplx, n_mat, N);
+  double *S = (double*)(ws + L.S), *M = (double*)(ws + L.M), *diag = (double*)(ws + L.diag);
+  const size_t es = cplx ? 16 : 8, cs = cplx ? 2 : 1;
+  const long cols = (long)Np * N, full = (long)n_mat * cols * (long)cs;
+  float *W32 = (float*)(ws + L.f32), *V32 = (float*)(ws + L.f32 + al256(es / 2 * n_mat * cols));
+  unsigned* off = (unsigned*)(ws + L.flags);       // cosines, then |V^H V - I|
+  int* flag = (int*)(ws + L.flags + 64);           // digit-plane flags (only bit 1 matters here)
+  int* status = (int*)(ws + L.flags + 128);
+  float* scale = (float*)(ws + L.flags + 256);
+  cudaError_t e = cudaSuccess;
+  uint64_t nl = 0;
+  *ok = false;
+  auto fail = [&](const char* what) {
+    ctx_set_error(ctx, "projector: %s failed: %s", what, cudaGetErrorString(e));
+    return RPA_E_CUDA;
+  };
+#define CKP(call)                               \
+  do {                                          \
+    if ((e = (call)) != cudaSuccess) return fail(#call); \
+  } while (0)
+  CKP(cudaMemsetAsync(ws + L.flags, 0, 256, s));
+  CKP(cudaMemcpyAsync(S, W, es * n_mat * cols, cudaMemcpyDeviceToDevice, s));
+  CKP(launch_proj_load32(cplx, n_mat, N, Np, W, scale, W32, V32, s));
+  nl += 2;
+  float off_h = 1.f;
+  for (int sweep = 0; sweep < kSweeps32 && off_h > 3e-6f; ++sweep) {
+    CKP(cudaMemsetAsync(off, 0, sizeof(unsigned), s));
+    for (int r = 0; r < Np - 1; ++r) CKP(launch_jacobi32_round(cplx, n_mat, N, Np, r, W32, V32, 1e-7f, off, s));
+    nl += Np - 1;
+    CKP(cudaMemcpyAsync(&off_h, off, sizeof off_h, cudaMemcpyDeviceToHost, s));
+    CKP(cudaStreamSynchronize(s));
+    if (!(off_h < 1e30f)) {  // W and V are as they were
+      ctx->launches += nl;
+      return RPA_OK;
+    }
+  }
+  CKP(launch_proj_widen(full, V32, V, s));
+  ++nl;
+  // out (columns of N at so per k-point) = or += conj(A) B over rows of A and B
+  auto product = [&](const double* A, long sa, int a_rows, int a_conj, const double* B, long sb, double* out, long so,
+                     int add) -> cudaError_t {
+    for (int k0 = 0; k0 < n_mat; k0 += L.group) {
+      const int nb = std::min(L.group, n_mat - k0);
+      auto src = [&](const double* p, long st, int rows, int cj) {
+        G64Src x{};
+        x.base = p + k0 * st * (long)cs;
+        x.stride = st;
+        x.ld = N;
+        x.by_rows = rows;
+        x.conj = cj;
+        x.nb = nb;
+        x.R = x.K = N;
+        return x;
+      };
+      G64Op a{}, b{};
+      a.planes = (uint16_t*)(ws + L.pa);
+      a.e = (int*)(ws + L.ea);
+      a.stride = (long)(g64_plane_bytes(cplx, 0, N, N, 1) / 2);
+      a.Rpad = g64_rpad(cplx, 0, N);
+      b.planes = (uint16_t*)(ws + L.pb);
+      b.e = (int*)(ws + L.eb);
+      b.stride = (long)(g64_plane_bytes(cplx, 1, N, N, 1) / 2);
+      b.Rpad = g64_rpad(cplx, 1, N);
+      a.n_kb = b.n_kb = g64_nkb(cplx, N);
+      if (cudaError_t x = g64_slice(cplx, 0, src(A, sa, a_rows, a_conj), a, flag, 0, s)) return x;
+      if (cudaError_t x = g64_slice(cplx, 1, src(B, sb, 1, 0), b, flag, 0, s)) return x;
+      G64Out o{};
+      o.base = out + k0 * so * (long)cs;
+      o.stride = so;
+      o.s0 = 1;
+      o.t0 = N;
+      o.rd = o.cd = 1 << 30;
+      o.R = o.C = N;
+      o.add = add;
+      if (cudaError_t x = g64_product(cplx, a, b, G64Index{nullptr, nullptr, 1, 1}, o, nb, 0, nullptr, 0, flag, 0, status,
+                                      &nl, s))
+        return x;
+      nl += 4;
+    }
+    return cudaSuccess;
+  };
+  const long NN = (long)N * N;
+  auto update = [&]() { return product(V, cols, 0, 1, M, NN, V, cols, 1); };  // V += V M
+  auto ortho = [&]() -> cudaError_t {
+    cudaError_t x = cudaMemsetAsync(off, 0, sizeof(unsigned), s);
+    if (x == cudaSuccess) x = product(V, cols, 1, 0, V, cols, M, NN, 0);
+    if (x == cudaSuccess) x = launch_proj_corr(cplx, n_mat, N, true, M, diag, off, s);
+    ++nl;
+    return x == cudaSuccess ? update() : x;
+  };
+  CKP(ortho());
+  CKP(ortho());
+  for (int it = 0; it < 3; ++it) {
+    CKP(product(S, cols, 1, 0, V, cols, W, cols, 0));  // W = S V
+    CKP(product(V, cols, 1, 0, W, cols, M, NN, 0));    // M = V^H S V
+    CKP(launch_proj_corr(cplx, n_mat, N, false, M, diag, off, s));
+    nl += 2;
+    CKP(update());
+    if (it < 2) CKP(ortho());
+  }
+  // orthonormal to rounding: a step squares what it finds
+  float dev = 1.f;
+  for (int it = 0; it < 4 && !(dev < 1e-9f); ++it) {
+    CKP(ortho());
+    CKP(cudaMemcpyAsync(&dev, off, sizeof dev, cudaMemcpyDeviceToHost, s));
+    CKP(cudaStreamSynchronize(s));
+  }
+  CKP(product(S, cols, 1, 0, V, cols, W, cols, 0));
+  CKP(product(W, cols, 1, 0, W, cols, M, NN, 0));
+  CKP(launch_proj_cluster(cplx, n_mat, N, Np, M, W, V, 1e-15, s));
+  ++nl;
+  int st = 0;
+  CKP(cudaMemcpyAsync(&st, status, sizeof st, cudaMemcpyDeviceToHost, s));
+  CKP(cudaStreamSynchronize(s));
+  ctx->launches += nl;
+  if (st) return decode_status(ctx, st, 1);
+  if (dev < 1e-9f) {
+    *ok = true;
+    return RPA_OK;
+  }
+  CKP(launch_proj_load(cplx, P, n_mat, N, Np, W, V, s));
+  ctx->launches += 1;
+  return RPA_OK;
+#undef CKP
+}
+
 rpa_status run_projector(rpa_ctx* ctx, Exec* pex, int cplx, int n_mat, int N, int n_mo, const void* const* S,
                          const double* const* c, double* const* out, double eps_d, char* region, cudaStream_t s,
-                         int* m_out, double* eig_host) {
+                         int* m_out, double* eig_host, char* fast) {
   if (n_mat > ProjPtrs::kMax) {
     ctx_set_error(ctx, "projector: at most %d k-points", ProjPtrs::kMax);
     return RPA_E_INVAL;
@@ -65,6 +240,10 @@ rpa_status run_projector(rpa_ctx* ctx, Exec* pex, int cplx, int n_mat, int N, in
   int sweep = 0;
   double off_h = 1.0;
   prof_begin(ctx, pex, s);
+  if (fast && proj_fast_bytes(cplx, n_mat, N)) {
+    bool ok = false;
+    if (rpa_status st = fast_start(ctx, cplx, n_mat, N, L.Np, W, V, P, fast, s, &ok)) return st;
+  }
   for (; sweep < kMaxSweeps && off_h > conv; ++sweep) {
     if ((e = cudaMemsetAsync(off, 0, sizeof(unsigned long long), s)) != cudaSuccess) return fail(e, "memset");
     for (int r = 0; r < L.Np - 1; ++r)
@@ -132,6 +311,9 @@ extern "C" rpa_status rpa_projector(rpa_ctx* ctx, const rpa_job* job, void* cons
   for (int A = 0; A < a->n_atoms; ++A) n_bas += a->n_bas_atom[A];
   const ProjLayout L = proj_layout(job->is_complex, job->n_kpts, n_bas, a->n_mo);
   Exec& ex = ctx->ex;
+  const size_t base = (L.bytes + 1023) & ~(size_t)1023;
+  size_t fb = proj_fast_bytes(job->is_complex, job->n_kpts, n_bas);
+  if (base + fb > sync_ws_cap(ctx) || (fb && !ex.ensure_ws(base + fb))) fb = 0;
   if (!ex.ensure_ws(L.bytes)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.bytes);
     return RPA_E_NOMEM;
@@ -143,7 +325,8 @@ extern "C" rpa_status rpa_projector(rpa_ctx* ctx, const rpa_job* job, void* cons
     out[k] = (double*)mo_out[k];
   }
   rpa_status st = run_projector(ctx, &ex, job->is_complex, job->n_kpts, n_bas, a->n_mo, a->overlap, c.data(),
-                                out.data(), a->eps_d, (char*)ex.ws, (cudaStream_t)stream, n_removed, eig_out);
+                                out.data(), a->eps_d, (char*)ex.ws, (cudaStream_t)stream, n_removed, eig_out,
+                                fb ? (char*)ex.ws + base : nullptr);
   prof_collect(ctx, &ex);
   return st;
 }

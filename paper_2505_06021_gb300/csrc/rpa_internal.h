@@ -142,6 +142,21 @@ cudaError_t launch_proj_load(int cplx, const ProjPtrs& P, int n_mat, int N, int 
 // double).
 cudaError_t launch_jacobi_round(int cplx, int n_mat, int N, int Np, int r, double* W, double* V, double thresh,
                                 unsigned long long* off_max, cudaStream_t s);
+// FP32 start: W32 = S / (its root mean square column norm), V32 = I from W = S;
+// one round of the FP32 sweeps (largest cosine into *off_max, FP32 bits);
+// y = x in FP64; and, in place over n_mat matrices M (N x N, columns of N):
+// ortho: -(M - I) / 2 with the largest |M - I| in *dev (FP32 bits), else the
+// first-order eigenvector corrections of M = V^H S V (diag: scratch, n_mat N).
+cudaError_t launch_proj_load32(int cplx, int n_mat, int N, int Np, const double* W, float* scale, float* W32, float* V32,
+                               cudaStream_t s);
+cudaError_t launch_jacobi32_round(int cplx, int n_mat, int N, int Np, int r, float* W32, float* V32, float thresh,
+                                  unsigned* off_max, cudaStream_t s);
+cudaError_t launch_proj_widen(long n, const float* x, double* y, cudaStream_t s);
+// Sweeps of W and V over each k-point's few columns with large cosines in G = W^H W.
+cudaError_t launch_proj_cluster(int cplx, int n_mat, int N, int Np, const double* G, double* W, double* V, double thresh,
+                                cudaStream_t s);
+cudaError_t launch_proj_corr(int cplx, int n_mat, int N, bool ortho, double* M, double* diag, unsigned* dev,
+                             cudaStream_t s);
 // Eigenvalues (column norms of W) in ascending order into lam_sorted
 // [n_mat][N], the column of each rank into by_rank, m = the largest count
 // below eps_d over the k-points (into *m, zeroed by the caller), then
