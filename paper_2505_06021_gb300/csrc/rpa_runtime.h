@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <functional>
+
 #include <atomic>
 #include <memory>
 #include <mutex>
@@ -176,7 +178,9 @@ int choose_qt(const rpa_job* j, int qb, int n_slices, size_t cap, const BinJob* 
 // Builds the frequency-batched plan of a split-precision job (band energies
 // read back from the device when they live there) and its per-q tables in
 // ex.hbin; bj.on stays false when the context turns it off or it saves nothing.
-rpa_status bin_job_build(rpa_ctx* ctx, Exec& ex, const rpa_job* j, BinJob& bj);
+// (meanwhile runs between the fetch of the band energies and the host's work on the plan)
+rpa_status bin_job_build(rpa_ctx* ctx, Exec& ex, const rpa_job* j, BinJob& bj,
+                         const std::function<rpa_status()>& meanwhile = nullptr);
 Bufs carve(void* ws, const rpa_job* j, const Layout& L);
 size_t sync_ws_cap(rpa_ctx* ctx);
 size_t tables_bytes(const rpa_job* j);

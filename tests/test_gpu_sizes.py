@@ -1,6 +1,7 @@
 """Sizes at which the launches of the log-det step, the FP64 chi0 and the
 frequency-batched chi0 change shape: panel and tile edges, one matrix and many,
-groups of frequencies, and more energy bins than rpa_freq_plan describes.
+groups of frequencies, more energy bins than rpa_freq_plan describes, and the V
+side that starts before the frequency plan.
 
 Tolerances (from the arithmetic, u = 2^-53):
 * ln det and Tr by Cholesky of a matrix A with 1 <= A <= c: backward error at
@@ -152,3 +153,25 @@ def test_many_bins(rpa):
     """64000 transitions at one q and 10 frequencies: 52 bins of rank 5."""
     _binned(rpa, synth.make_problem("n", is_complex=False, n_aux=40, n_occ=40, n_virt=1600, grid=synth.gamma_grid(),
                                     n_w=10, seed=51), 0)
+
+
+def test_v_side_before_the_plan(rpa):
+    """The first call of a context allocates its workspace after the plan, later
+    calls factor V before it: the same bits, also after a larger job, a smaller
+    one and one of another shape have used the workspace."""
+    def prob(n, n_w, kd, seed):
+        p = synth.make_problem("v", is_complex=True, n_aux=n, n_occ=4, n_virt=30, grid=synth.regular_kq_grid(kd),
+                               n_w=n_w, seed=seed)
+        t = rpa.upload_problem(p)
+        return rpa.job_from_problem(p, t, prec=rpa.PREC_MIXED), t
+
+    specs = [(200, 16, (2, 2, 1), 1), (90, 16, (2, 1, 1), 2), (260, 12, (2, 2, 1), 3), (131, 20, (3, 1, 1), 4)]
+    jobs = [prob(*s) for s in specs]
+    first = []
+    for j, _ in jobs:
+        with rpa.Context(0, chi0_freq=2) as c:
+            first.append(c.energy(j))
+    with rpa.Context(0, chi0_freq=2) as c:
+        for i in (2, 0, 1, 0, 3, 2, 3, 1):
+            r = c.energy(jobs[i][0])
+            assert r["Ec"] == first[i]["Ec"] and np.array_equal(r["lndet"], first[i]["lndet"]), i
