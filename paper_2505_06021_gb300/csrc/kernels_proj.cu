@@ -297,20 +297,14 @@ __global__ void __launch_bounds__(256) proj_load32_kernel(int N, int Np, const d
   }
 }
 
-// One round of the FP32 sweeps: a warp per column pair and k-point.  Columns
-// below 1e-6 of the typical norm (FP32 noise) count as that long.
+// Rotates columns p, q of W and V (N elements each), by one warp, where their
+// cosine is above thresh; returns the cosine.  Columns below 1e-6 of the typical
+// norm (FP32 noise) count as that long.
 template <bool C>
-__global__ void __launch_bounds__(128) jacobi32_round_kernel(int N, int Np, int r, float* __restrict__ W32,
-                                                             float* __restrict__ V32, float thresh,
-                                                             unsigned* __restrict__ off_max) {
-  const int lane = threadIdx.x & 31, i = blockIdx.x * 4 + (threadIdx.x >> 5), k = blockIdx.y;
-  if (i >= Np / 2) return;
-  int p, q;
-  round_pair(Np, r, i, p, q);
-  const size_t m0 = (size_t)k * Np * N * (C ? 2 : 1);
-  Flt<C>* wp = reinterpret_cast<Flt<C>*>(W32 + m0) + (size_t)p * N;
-  Flt<C>* wq = reinterpret_cast<Flt<C>*>(W32 + m0) + (size_t)q * N;
+__device__ __forceinline__ float rotate32(Flt<C>* wp, Flt<C>* wq, Flt<C>* vp, Flt<C>* vq, int N, float thresh) {
+  const int lane = threadIdx.x & 31;
   float a = 0.f, b = 0.f, gr = 0.f, gi = 0.f;
+#pragma unroll 4
   for (int mu = lane; mu < N; mu += 32) {
     const Flt<C> x = wp[mu], y = wq[mu];
     a = fmaf(x.re, x.re, a);
@@ -332,12 +326,12 @@ __global__ void __launch_bounds__(128) jacobi32_round_kernel(int N, int Np, int 
   }
   const float g = sqrtf(gr * gr + gi * gi);
   const float off = g / sqrtf(fmaxf(a, 1e-12f) * fmaxf(b, 1e-12f));
-  if (lane == 0) atomicMax(off_max, __float_as_uint(off));
-  if (!(off > thresh)) return;  // (a NaN ends here too: the start is then rejected)
+  if (!(off > thresh)) return off;  // (a NaN ends here too: the start is then rejected)
   const float zeta = (b - a) / (2.f * g);
   const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
   const float c = rsqrtf(1.f + t * t), s = c * t, er = gr / g, ei = -gi / g;
   auto rot = [&](Flt<C>* xc, Flt<C>* yc) {
+#pragma unroll 4
     for (int mu = lane; mu < N; mu += 32) {
       const Flt<C> x = xc[mu], y = yc[mu];
       Flt<C> xn, yn;
@@ -356,7 +350,82 @@ __global__ void __launch_bounds__(128) jacobi32_round_kernel(int N, int Np, int 
     }
   };
   rot(wp, wq);
-  rot(reinterpret_cast<Flt<C>*>(V32 + m0) + (size_t)p * N, reinterpret_cast<Flt<C>*>(V32 + m0) + (size_t)q * N);
+  rot(vp, vq);
+  return off;
+}
+
+// A block round of the FP32 sweeps: a CTA takes two blocks of B columns of W
+// and V of one k-point into shared memory, rotates every pair across them (B
+// rounds of B disjoint pairs, a warp each) and writes them back; the first block
+// round of a sweep also rotates the pairs within the blocks (2 B - 1 rounds).  A
+// sweep then reads and writes the columns nb - 1 times, not Np - 1, and has as
+// many launches (nb blocks).  What bounds a round inside the CTA is shared
+// memory: 16 warps read W twice, V once and write both.
+template <bool C, int B>
+__global__ void __launch_bounds__(32 * B) jacobi32_block_kernel(int N, int Np, int nb, int br, float* __restrict__ W32,
+                                                                float* __restrict__ V32, float thresh,
+                                                                unsigned* __restrict__ off_max) {
+  extern __shared__ __align__(16) float cols32[];
+  __shared__ unsigned worst;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const size_t m0 = (size_t)blockIdx.y * Np * N;
+  Flt<C>* w = reinterpret_cast<Flt<C>*>(cols32);  // 2 B columns of W, then of V
+  Flt<C>* v = w + (size_t)2 * B * N;
+  Flt<C>* wg = reinterpret_cast<Flt<C>*>(W32) + m0;
+  Flt<C>* vg = reinterpret_cast<Flt<C>*>(V32) + m0;
+  int bp, bq;
+  round_pair(nb, br, blockIdx.x, bp, bq);
+  const Flt<C> zero{};
+  if (threadIdx.x == 0) worst = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {  // (columns past Np count as zero: never rotated)
+    const int col = (h ? bq : bp) * B + wid, lc = h * B + wid;
+#pragma unroll 4
+    for (int mu = lane; mu < N; mu += 32) {
+      w[(size_t)lc * N + mu] = col < Np ? wg[(size_t)col * N + mu] : zero;
+      v[(size_t)lc * N + mu] = col < Np ? vg[(size_t)col * N + mu] : zero;
+    }
+  }
+  __syncthreads();
+  const int rounds = br == 0 ? 2 * B - 1 : B;
+  unsigned mine = 0;
+  for (int r = 0; r < rounds; ++r) {
+    int p = wid, q = B + (wid + r) % B;
+    if (br == 0) round_pair(2 * B, r, wid, p, q);
+    const float off = rotate32<C>(w + (size_t)p * N, w + (size_t)q * N, v + (size_t)p * N, v + (size_t)q * N, N, thresh);
+    mine = max(mine, __float_as_uint(off));
+    __syncthreads();
+  }
+  if (lane == 0) atomicMax(&worst, mine);
+  __syncthreads();
+  if (threadIdx.x == 0) atomicMax(off_max, worst);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int col = (h ? bq : bp) * B + wid, lc = h * B + wid;
+    if (col < Np)
+#pragma unroll 4
+      for (int mu = lane; mu < N; mu += 32) {
+        wg[(size_t)col * N + mu] = w[(size_t)lc * N + mu];
+        vg[(size_t)col * N + mu] = v[(size_t)lc * N + mu];
+      }
+  }
+}
+
+// One round of the FP32 sweeps on columns too long for that: a warp per column
+// pair and k-point, in global memory.
+template <bool C>
+__global__ void __launch_bounds__(128) jacobi32_round_kernel(int N, int Np, int r, float* __restrict__ W32,
+                                                             float* __restrict__ V32, float thresh,
+                                                             unsigned* __restrict__ off_max) {
+  const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (i >= Np / 2) return;
+  int p, q;
+  round_pair(Np, r, i, p, q);
+  const size_t m0 = (size_t)blockIdx.y * Np * N;
+  Flt<C>* w = reinterpret_cast<Flt<C>*>(W32) + m0;
+  Flt<C>* v = reinterpret_cast<Flt<C>*>(V32) + m0;
+  const float off = rotate32<C>(w + (size_t)p * N, w + (size_t)q * N, v + (size_t)p * N, v + (size_t)q * N, N, thresh);
+  if ((threadIdx.x & 31) == 0) atomicMax(off_max, __float_as_uint(off));
 }
 
 __global__ void __launch_bounds__(256) proj_widen_kernel(long n, const float* __restrict__ x, double* __restrict__ y) {
@@ -518,14 +587,38 @@ cudaError_t launch_proj_load32(int cplx, int n_mat, int N, int Np, const double*
   return cudaGetLastError();
 }
 
-cudaError_t launch_jacobi32_round(int cplx, int n_mat, int N, int Np, int r, float* W32, float* V32, float thresh,
-                                  unsigned* off_max, cudaStream_t s) {
-  const dim3 grid((Np / 2 + 3) / 4, n_mat);
-  if (cplx)
-    jacobi32_round_kernel<true><<<grid, 128, 0, s>>>(N, Np, r, W32, V32, thresh, off_max);
-  else
-    jacobi32_round_kernel<false><<<grid, 128, 0, s>>>(N, Np, r, W32, V32, thresh, off_max);
-  return cudaGetLastError();
+// One sweep of the FP32 iteration; returns the launches made, or a negative
+// CUDA error.
+template <bool C, int B>
+static int jacobi32_blocks(int n_mat, int N, int Np, float* W32, float* V32, float thresh, unsigned* off_max,
+                           cudaStream_t s) {
+  const size_t sh = sizeof(Flt<C>) * 4 * B * (size_t)N;
+  cudaError_t e = cudaFuncSetAttribute(jacobi32_block_kernel<C, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  const int nb = 2 * ((Np + 2 * B - 1) / (2 * B));
+  for (int br = 0; br < nb - 1 && e == cudaSuccess; ++br) {
+    jacobi32_block_kernel<C, B><<<dim3(nb / 2, n_mat), 32 * B, sh, s>>>(N, Np, nb, br, W32, V32, thresh, off_max);
+    e = cudaGetLastError();
+  }
+  return e == cudaSuccess ? nb - 1 : -(int)e;
+}
+template <bool C>
+static int jacobi32_sweep(int n_mat, int N, int Np, float* W32, float* V32, float thresh, unsigned* off_max,
+                          cudaStream_t s) {
+  // blocks of 16 columns while 32 columns of W and V fit in shared memory
+  // (complex N <= 450), of 8 up to twice that
+  const size_t col = sizeof(Flt<C>) * 4 * (size_t)N, room = 225 * 1024;
+  if (16 * col <= room) return jacobi32_blocks<C, 16>(n_mat, N, Np, W32, V32, thresh, off_max, s);
+  if (8 * col <= room) return jacobi32_blocks<C, 8>(n_mat, N, Np, W32, V32, thresh, off_max, s);
+  for (int r = 0; r < Np - 1; ++r)
+    jacobi32_round_kernel<C><<<dim3((Np / 2 + 3) / 4, n_mat), 128, 0, s>>>(N, Np, r, W32, V32, thresh, off_max);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? Np - 1 : -(int)e;
+}
+
+int launch_jacobi32_sweep(int cplx, int n_mat, int N, int Np, float* W32, float* V32, float thresh, unsigned* off_max,
+                          cudaStream_t s) {
+  return cplx ? jacobi32_sweep<true>(n_mat, N, Np, W32, V32, thresh, off_max, s)
+              : jacobi32_sweep<false>(n_mat, N, Np, W32, V32, thresh, off_max, s);
 }
 
 cudaError_t launch_proj_widen(long n, const float* x, double* y, cudaStream_t s) {

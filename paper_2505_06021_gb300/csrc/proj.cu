@@ -109,8 +109,9 @@ static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, d
   float off_h = 1.f;
   for (int sweep = 0; sweep < kSweeps32 && off_h > 3e-6f; ++sweep) {
     CKP(cudaMemsetAsync(off, 0, sizeof(unsigned), s));
-    for (int r = 0; r < Np - 1; ++r) CKP(launch_jacobi32_round(cplx, n_mat, N, Np, r, W32, V32, 1e-7f, off, s));
-    nl += Np - 1;
+    const int n = launch_jacobi32_sweep(cplx, n_mat, N, Np, W32, V32, 1e-7f, off, s);
+    if (n < 0) CKP((cudaError_t)-n);
+    nl += n;
     CKP(cudaMemcpyAsync(&off_h, off, sizeof off_h, cudaMemcpyDeviceToHost, s));
     CKP(cudaStreamSynchronize(s));
     if (!(off_h < 1e30f)) {  // W and V are as they were

@@ -143,14 +143,15 @@ cudaError_t launch_proj_load(int cplx, const ProjPtrs& P, int n_mat, int N, int 
 cudaError_t launch_jacobi_round(int cplx, int n_mat, int N, int Np, int r, double* W, double* V, double thresh,
                                 unsigned long long* off_max, cudaStream_t s);
 // FP32 start: W32 = S / (its root mean square column norm), V32 = I from W = S;
-// one round of the FP32 sweeps (largest cosine into *off_max, FP32 bits);
+// one sweep of the FP32 iteration (largest cosine into *off_max, FP32 bits;
+// returns the launches made or a negative CUDA error);
 // y = x in FP64; and, in place over n_mat matrices M (N x N, columns of N):
 // ortho: -(M - I) / 2 with the largest |M - I| in *dev (FP32 bits), else the
 // first-order eigenvector corrections of M = V^H S V (diag: scratch, n_mat N).
 cudaError_t launch_proj_load32(int cplx, int n_mat, int N, int Np, const double* W, float* scale, float* W32, float* V32,
                                cudaStream_t s);
-cudaError_t launch_jacobi32_round(int cplx, int n_mat, int N, int Np, int r, float* W32, float* V32, float thresh,
-                                  unsigned* off_max, cudaStream_t s);
+int launch_jacobi32_sweep(int cplx, int n_mat, int N, int Np, float* W32, float* V32, float thresh, unsigned* off_max,
+                          cudaStream_t s);
 cudaError_t launch_proj_widen(long n, const float* x, double* y, cudaStream_t s);
 // Sweeps of W and V over each k-point's few columns with large cosines in G = W^H W.
 cudaError_t launch_proj_cluster(int cplx, int n_mat, int N, int Np, const double* G, double* W, double* V, double thresh,
