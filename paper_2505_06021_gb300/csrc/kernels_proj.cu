@@ -20,12 +20,20 @@
 //
 // Start of the iteration (proj.cu, bases of some size): the sweeps above begin
 // from eigenvectors of nearly full accuracy instead of I.  One-sided Jacobi in FP32
-// (its pipe is 64 times the FP64 one) gives them to about 1e-6; they are
+// (its pipe is 64 times the FP64 one; in shared memory, 32 columns at a time)
+// gives them to about 1e-6; they are
 // refined by matrix products on the tensor cores (g64.cu): Newton-Schulz steps
 // V <- V - V (V^H V - I) / 2 for orthonormality, and first-order corrections
 // V <- V + V E, E_ij = (V^H S V)_ij / (lambda_j - lambda_i) where that is small (the
 // quadratically convergent refinement of Ogita and Aishima, 2018, without its
-// cluster step: what it leaves, the FP64 sweeps finish).
+// cluster step).  Then the columns of W = S V are made orthogonal to rounding by
+// the same first-order rotations from G = W^H W (whose entries are accurate
+// relative to both columns, so this holds for the tiny eigenvalues too), and the
+// few pairs that need large rotations are rotated one by one; where G still
+// shows a cosine above 1e-14, the FP64 sweeps finish.  Measured, 16 overlaps of 256
+// functions: three FP64 sweeps of 255 rounds (23 us each, 17.8 ms in all) became 0.7
+// ms of products, 29.9 -> 13.1 ms in all; what is left is the FP32 sweeps
+// (7 ms, shared-memory bandwidth) and the refinement's products.
 //
 // Since the eigenvalues are taken in ascending order and R~ is a product over
 // k, R~ removes the m lowest positions at every k-point, m the largest count
@@ -187,9 +195,10 @@ __global__ void __launch_bounds__(WARP ? 128 : 256) jacobi_round_kernel(int N, i
 
 // The few columns that the refinement could not tell apart (the eigenvalues
 // far below FP32's resolution, near-degenerate ones): those with a cosine
-// above 1e-3 in G = W^H W, swept among themselves, one CTA per k-point.  More
-// than CLUSTER_MAX are left to the sweeps over all columns.
-constexpr int CLUSTER_MAX = 12;
+// above 1e-14 in G = W^H W (above 1e-3 where they are too many), swept among
+// themselves, one CTA per k-point.  More than CLUSTER_MAX are left to the sweeps
+// over all columns.
+constexpr int CLUSTER_MAX = 24;
 template <bool C>
 __global__ void __launch_bounds__(256) proj_cluster_kernel(int N, int Np, const double* __restrict__ G,
                                                            double* __restrict__ W, double* __restrict__ V,
@@ -208,17 +217,22 @@ __global__ void __launch_bounds__(256) proj_cluster_kernel(int N, int Np, const 
       const Elem<C> x = ld_elem<C>(g, (long)j * N + i);
       double v = x.re * x.re;
       if constexpr (C) v += x.im * x.im;
-      if (v > 1e-6 * gj * ld_elem<C>(g, (long)i * N + i).re) mark[i] = 1;  // (j is marked as i's partner)
+      const double gg = gj * ld_elem<C>(g, (long)i * N + i).re;
+      if (v > 1e-28 * gg) mark[i] |= v > 1e-6 * gg ? 3 : 1;  // (j is marked as i's partner)
     }
   }
   __syncthreads();
   if (tid == 0) {
     int n = 0;
-    for (int j = 0; j < N; ++j)
-      if (mark[j]) {
-        if (n < CLUSTER_MAX) list[n] = j;
-        ++n;
-      }
+    for (int bits = 1; bits <= 3; bits += 2) {
+      n = 0;
+      for (int j = 0; j < N; ++j)
+        if ((mark[j] & bits) == bits) {
+          if (n < CLUSTER_MAX) list[n] = j;
+          ++n;
+        }
+      if (n <= CLUSTER_MAX) break;
+    }
     cnt = n;
   }
   __syncthreads();
@@ -434,14 +448,15 @@ __global__ void __launch_bounds__(256) proj_widen_kernel(long n, const float* __
 
 // In place over column j of M(k) (N x N at a stride N^2): ORTHO: -(M - I) / 2,
 // the largest |M - I| into *dev; else the correction
-// E_ij = M_ij / (M_jj - M_ii) where it is below 0.02, zero elsewhere (diag: the
-// M_ii, saved before the launch).
+// E_ij = M_ij / (M_jj - M_ii) where it is below lim, zero elsewhere (diag: the
+// M_ii, saved before the launch), and the largest |M_ij| / sqrt(M_ii M_jj)
+// into *dev.
 template <bool C, bool ORTHO>
 __global__ void __launch_bounds__(256) proj_corr_kernel(int N, double* __restrict__ M, const double* __restrict__ diag,
-                                                        unsigned* __restrict__ dev) {
+                                                        float lim, unsigned* __restrict__ dev) {
   const int k = blockIdx.y, j = blockIdx.x;
   double* col = M + ((size_t)k * N + j) * N * (C ? 2 : 1);
-  const double lj = ORTHO ? 0.0 : diag[(size_t)k * N + j];
+  const double lj = ORTHO ? 0.0 : diag[(size_t)k * N + j], inv = ORTHO ? 0.0 : 1.0 / lj;
   float dm = 0.f;
   bool bad = false;
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
@@ -455,20 +470,24 @@ __global__ void __launch_bounds__(256) proj_corr_kernel(int N, double* __restric
       dm = fmaxf(dm, v);
       bad |= !(v < 1e30f);
     } else {
-      const double gap = lj - diag[(size_t)k * N + i];
-      float v = fabsf((float)e.re);
-      if constexpr (C) v = fmaxf(v, fabsf((float)e.im));
-      f = i != j && v < 0.02f * fabsf((float)gap) ? 1.0 / gap : 0.0;
+      // (relative to M_jj, so that the FP32 range holds any scale of M)
+      const double li = diag[(size_t)k * N + i], gap = lj - li;
+      float v = fabsf((float)(e.re * inv));
+      if constexpr (C) v = fmaxf(v, fabsf((float)(e.im * inv)));
+      f = i != j && v < lim * fabsf((float)(gap * inv)) ? 1.0 / gap : 0.0;
+      if (i != j) {
+        const float c = v * rsqrtf((float)(li * inv));
+        dm = fmaxf(dm, c);
+        bad |= !(c < 1e30f);
+      }
     }
     e.re *= f;
     if constexpr (C) e.im *= f;
     st_elem<C>(col, i, e);
   }
-  if constexpr (ORTHO) {
-    if (bad) dm = __int_as_float(0x7f800000);
-    dm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dm)));
-    if ((threadIdx.x & 31) == 0) atomicMax(dev, __float_as_uint(dm));
-  }
+  if (bad) dm = __int_as_float(0x7f800000);
+  dm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dm)));
+  if ((threadIdx.x & 31) == 0) atomicMax(dev, __float_as_uint(dm));
 }
 
 template <bool C>
@@ -626,8 +645,8 @@ cudaError_t launch_proj_widen(long n, const float* x, double* y, cudaStream_t s)
   return cudaGetLastError();
 }
 
-cudaError_t launch_proj_corr(int cplx, int n_mat, int N, bool ortho, double* M, double* diag, unsigned* dev,
-                             cudaStream_t s) {
+cudaError_t launch_proj_corr(int cplx, int n_mat, int N, bool ortho, double* M, double* diag, float lim,
+                             unsigned* dev, cudaStream_t s) {
   const dim3 grid(N, n_mat), gd((N + 255) / 256, n_mat);
   if (!ortho) {
     if (cplx)
@@ -637,14 +656,14 @@ cudaError_t launch_proj_corr(int cplx, int n_mat, int N, bool ortho, double* M, 
   }
   if (cplx) {
     if (ortho)
-      proj_corr_kernel<true, true><<<grid, 256, 0, s>>>(N, M, diag, dev);
+      proj_corr_kernel<true, true><<<grid, 256, 0, s>>>(N, M, diag, lim, dev);
     else
-      proj_corr_kernel<true, false><<<grid, 256, 0, s>>>(N, M, diag, dev);
+      proj_corr_kernel<true, false><<<grid, 256, 0, s>>>(N, M, diag, lim, dev);
   } else {
     if (ortho)
-      proj_corr_kernel<false, true><<<grid, 256, 0, s>>>(N, M, diag, dev);
+      proj_corr_kernel<false, true><<<grid, 256, 0, s>>>(N, M, diag, lim, dev);
     else
-      proj_corr_kernel<false, false><<<grid, 256, 0, s>>>(N, M, diag, dev);
+      proj_corr_kernel<false, false><<<grid, 256, 0, s>>>(N, M, diag, lim, dev);
   }
   return cudaGetLastError();
 }

@@ -63,6 +63,10 @@ FastLayout fast_layout(int cplx, int n_mat, int N) {
 }
 
 constexpr int kSweeps32 = 14;
+constexpr int kPolish = 4;
+// largest cosine at which the columns count as orthogonal without an FP64 sweep
+// that finds them so (the sweeps' own bar is this or wider)
+constexpr float kOrthogonal = 1e-14f;
 
 }  // namespace
 
@@ -74,21 +78,87 @@ size_t proj_fast_bytes(int cplx, int n_mat, int N) {
   return b <= ((size_t)4 << 30) ? b : 0;
 }
 
+// out (columns of N at so per k-point) = or += conj(A) B over rows of A and B,
+// as digit products (A rows or columns of matrices at sa, B columns at sb).
+static cudaError_t fast_product(int cplx, int n_mat, int N, char* ws, const double* A, long sa, int a_rows, int a_conj,
+                                const double* B, long sb, double* out, long so, int add, uint64_t* nl, cudaStream_t s) {
+  const FastLayout L = fast_layout(cplx, n_mat, N);
+  const size_t cs = cplx ? 2 : 1;
+  int* flag = (int*)(ws + L.flags + 64);  // digit-plane flags (only bit 1 matters here)
+  int* status = (int*)(ws + L.flags + 128);
+  for (int k0 = 0; k0 < n_mat; k0 += L.group) {
+    const int nb = std::min(L.group, n_mat - k0);
+    auto src = [&](const double* p, long st, int rows, int cj) {
+      G64Src x{};
+      x.base = p + k0 * st * (long)cs;
+      x.stride = st;
+      x.ld = N;
+      x.by_rows = rows;
+      x.conj = cj;
+      x.nb = nb;
+      x.R = x.K = N;
+      return x;
+    };
+    G64Op a{}, b{};
+    a.planes = (uint16_t*)(ws + L.pa);
+    a.e = (int*)(ws + L.ea);
+    a.stride = (long)(g64_plane_bytes(cplx, 0, N, N, 1) / 2);
+    a.Rpad = g64_rpad(cplx, 0, N);
+    b.planes = (uint16_t*)(ws + L.pb);
+    b.e = (int*)(ws + L.eb);
+    b.stride = (long)(g64_plane_bytes(cplx, 1, N, N, 1) / 2);
+    b.Rpad = g64_rpad(cplx, 1, N);
+    a.n_kb = b.n_kb = g64_nkb(cplx, N);
+    if (cudaError_t x = g64_slice(cplx, 0, src(A, sa, a_rows, a_conj), a, flag, 0, s)) return x;
+    if (cudaError_t x = g64_slice(cplx, 1, src(B, sb, 1, 0), b, flag, 0, s)) return x;
+    G64Out o{};
+    o.base = out + k0 * so * (long)cs;
+    o.stride = so;
+    o.s0 = 1;
+    o.t0 = N;
+    o.rd = o.cd = 1 << 30;
+    o.R = o.C = N;
+    o.add = add;
+    if (cudaError_t x = g64_product(cplx, a, b, G64Index{nullptr, nullptr, 1, 1}, o, nb, 0, nullptr, 0, flag, 0, status,
+                                    nl, s))
+      return x;
+    *nl += 4;
+  }
+  return cudaSuccess;
+}
+
+// The largest cosine between two columns of W (digit planes: rounding at 2^-55
+// of the largest entries), into *cosine; M is left with E for V += V E,
+// W += W E, the first-order rotations of the pairs that take less than 2e-9 (its
+// square, what V then lacks in orthonormality, is below rounding).
+static cudaError_t column_cosine(int cplx, int n_mat, int N, int Np, char* ws, const double* W, float* cosine,
+                                 uint64_t* nl, cudaStream_t s) {
+  const FastLayout L = fast_layout(cplx, n_mat, N);
+  double *M = (double*)(ws + L.M), *diag = (double*)(ws + L.diag);
+  unsigned* off = (unsigned*)(ws + L.flags);
+  const long cols = (long)Np * N;
+  cudaError_t e = cudaMemsetAsync(off, 0, sizeof(unsigned), s);
+  if (e == cudaSuccess) e = fast_product(cplx, n_mat, N, ws, W, cols, 1, 0, W, cols, M, (long)N * N, 0, nl, s);
+  if (e == cudaSuccess) e = launch_proj_corr(cplx, n_mat, N, false, M, diag, 2e-9f, off, s);
+  *nl += 2;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(cosine, off, sizeof *cosine, cudaMemcpyDeviceToHost, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
 // V: eigenvectors of S (= W on entry) to nearly FP64 accuracy, W = S V.  The FP64
 // sweeps from V = I took 13 sweeps of 16 ms on 16 overlaps of 256 functions (208
-// ms); with this start three are left, whose rounds are mostly inner products: 50
-// ms in all.
+// ms); with this start none is left there (or one, where many columns stay close).
 // *ok = false (W = S and V = I as before) when the start did not give an
 // orthonormal V: entries out of the FP32 range, no convergence.
 static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, double* W, double* V,
-                             const ProjPtrs& P, char* ws, cudaStream_t s, bool* ok) {
+                             const ProjPtrs& P, char* ws, cudaStream_t s, bool* ok,
+                             float* cosine) {
   const FastLayout L = fast_layout(cplx, n_mat, N);
   double *S = (double*)(ws + L.S), *M = (double*)(ws + L.M), *diag = (double*)(ws + L.diag);
   const size_t es = cplx ? 16 : 8, cs = cplx ? 2 : 1;
   const long cols = (long)Np * N, full = (long)n_mat * cols * (long)cs;
   float *W32 = (float*)(ws + L.f32), *V32 = (float*)(ws + L.f32 + al256(es / 2 * n_mat * cols));
   unsigned* off = (unsigned*)(ws + L.flags);       // cosines, then |V^H V - I|
-  int* flag = (int*)(ws + L.flags + 64);           // digit-plane flags (only bit 1 matters here)
   int* status = (int*)(ws + L.flags + 128);
   float* scale = (float*)(ws + L.flags + 256);
   cudaError_t e = cudaSuccess;
@@ -121,55 +191,14 @@ static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, d
   }
   CKP(launch_proj_widen(full, V32, V, s));
   ++nl;
-  // out (columns of N at so per k-point) = or += conj(A) B over rows of A and B
   auto product = [&](const double* A, long sa, int a_rows, int a_conj, const double* B, long sb, double* out, long so,
-                     int add) -> cudaError_t {
-    for (int k0 = 0; k0 < n_mat; k0 += L.group) {
-      const int nb = std::min(L.group, n_mat - k0);
-      auto src = [&](const double* p, long st, int rows, int cj) {
-        G64Src x{};
-        x.base = p + k0 * st * (long)cs;
-        x.stride = st;
-        x.ld = N;
-        x.by_rows = rows;
-        x.conj = cj;
-        x.nb = nb;
-        x.R = x.K = N;
-        return x;
-      };
-      G64Op a{}, b{};
-      a.planes = (uint16_t*)(ws + L.pa);
-      a.e = (int*)(ws + L.ea);
-      a.stride = (long)(g64_plane_bytes(cplx, 0, N, N, 1) / 2);
-      a.Rpad = g64_rpad(cplx, 0, N);
-      b.planes = (uint16_t*)(ws + L.pb);
-      b.e = (int*)(ws + L.eb);
-      b.stride = (long)(g64_plane_bytes(cplx, 1, N, N, 1) / 2);
-      b.Rpad = g64_rpad(cplx, 1, N);
-      a.n_kb = b.n_kb = g64_nkb(cplx, N);
-      if (cudaError_t x = g64_slice(cplx, 0, src(A, sa, a_rows, a_conj), a, flag, 0, s)) return x;
-      if (cudaError_t x = g64_slice(cplx, 1, src(B, sb, 1, 0), b, flag, 0, s)) return x;
-      G64Out o{};
-      o.base = out + k0 * so * (long)cs;
-      o.stride = so;
-      o.s0 = 1;
-      o.t0 = N;
-      o.rd = o.cd = 1 << 30;
-      o.R = o.C = N;
-      o.add = add;
-      if (cudaError_t x = g64_product(cplx, a, b, G64Index{nullptr, nullptr, 1, 1}, o, nb, 0, nullptr, 0, flag, 0, status,
-                                      &nl, s))
-        return x;
-      nl += 4;
-    }
-    return cudaSuccess;
-  };
+                     int add) { return fast_product(cplx, n_mat, N, ws, A, sa, a_rows, a_conj, B, sb, out, so, add, &nl, s); };
   const long NN = (long)N * N;
   auto update = [&]() { return product(V, cols, 0, 1, M, NN, V, cols, 1); };  // V += V M
   auto ortho = [&]() -> cudaError_t {
     cudaError_t x = cudaMemsetAsync(off, 0, sizeof(unsigned), s);
     if (x == cudaSuccess) x = product(V, cols, 1, 0, V, cols, M, NN, 0);
-    if (x == cudaSuccess) x = launch_proj_corr(cplx, n_mat, N, true, M, diag, off, s);
+    if (x == cudaSuccess) x = launch_proj_corr(cplx, n_mat, N, true, M, diag, 0.f, off, s);
     ++nl;
     return x == cudaSuccess ? update() : x;
   };
@@ -178,7 +207,7 @@ static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, d
   for (int it = 0; it < 3; ++it) {
     CKP(product(S, cols, 1, 0, V, cols, W, cols, 0));  // W = S V
     CKP(product(V, cols, 1, 0, W, cols, M, NN, 0));    // M = V^H S V
-    CKP(launch_proj_corr(cplx, n_mat, N, false, M, diag, off, s));
+    CKP(launch_proj_corr(cplx, n_mat, N, false, M, diag, 0.02f, off, s));
     nl += 2;
     CKP(update());
     if (it < 2) CKP(ortho());
@@ -191,9 +220,19 @@ static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, d
     CKP(cudaStreamSynchronize(s));
   }
   CKP(product(S, cols, 1, 0, V, cols, W, cols, 0));
-  CKP(product(W, cols, 1, 0, W, cols, M, NN, 0));
-  CKP(launch_proj_cluster(cplx, n_mat, N, Np, M, W, V, 1e-15, s));
-  ++nl;
+  // columns of W orthogonal to FP64 rounding: first-order rotations of all
+  // pairs that take little, full ones among the few columns that remain
+  float last = 2.f;
+  for (int it = 0; dev < 1e-9f; ++it) {
+    CKP(column_cosine(cplx, n_mat, N, Np, ws, W, cosine, &nl, s));
+    if (*cosine <= kOrthogonal || it == kPolish || !(*cosine < 0.5f * last)) break;
+    last = *cosine;
+    CKP(update());
+    CKP(product(W, cols, 0, 1, M, NN, W, cols, 1));
+    CKP(product(W, cols, 1, 0, W, cols, M, NN, 0));
+    CKP(launch_proj_cluster(cplx, n_mat, N, Np, M, W, V, 1e-15, s));
+    ++nl;
+  }
   int st = 0;
   CKP(cudaMemcpyAsync(&st, status, sizeof st, cudaMemcpyDeviceToHost, s));
   CKP(cudaStreamSynchronize(s));
@@ -240,11 +279,14 @@ rpa_status run_projector(rpa_ctx* ctx, Exec* pex, int cplx, int n_mat, int N, in
   const double conv = std::max(1e-14, 4.0 * N * DBL_EPSILON);
   int sweep = 0;
   double off_h = 1.0;
+  bool started = false;
+  float cosine = 1.f;
   prof_begin(ctx, pex, s);
   if (fast && proj_fast_bytes(cplx, n_mat, N)) {
-    bool ok = false;
-    if (rpa_status st = fast_start(ctx, cplx, n_mat, N, L.Np, W, V, P, fast, s, &ok)) return st;
+    if (rpa_status st = fast_start(ctx, cplx, n_mat, N, L.Np, W, V, P, fast, s, &started, &cosine)) return st;
+    if (started && cosine <= kOrthogonal) off_h = cosine;
   }
+
   for (; sweep < kMaxSweeps && off_h > conv; ++sweep) {
     if ((e = cudaMemsetAsync(off, 0, sizeof(unsigned long long), s)) != cudaSuccess) return fail(e, "memset");
     for (int r = 0; r < L.Np - 1; ++r)
@@ -256,6 +298,14 @@ rpa_status run_projector(rpa_ctx* ctx, Exec* pex, int cplx, int n_mat, int N, in
       return fail(e, "copy");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e, "sync");
     memcpy(&off_h, &bits, sizeof off_h);
+    // the sweep that would only find the columns orthogonal is a Gram product
+    if (started && off_h > conv) {
+      uint64_t nl = 0;
+      if ((e = column_cosine(cplx, n_mat, N, L.Np, fast, W, &cosine, &nl, s)) != cudaSuccess)
+        return fail(e, "Gram product");
+      ctx->launches += nl;
+      if (cosine <= kOrthogonal) off_h = cosine;
+    }
   }
   prof_end(ctx, pex, s, RPA_K_PROJ, sweep * (L.Np - 1));
   if (off_h > conv) {

@@ -147,7 +147,8 @@ cudaError_t launch_jacobi_round(int cplx, int n_mat, int N, int Np, int r, doubl
 // returns the launches made or a negative CUDA error);
 // y = x in FP64; and, in place over n_mat matrices M (N x N, columns of N):
 // ortho: -(M - I) / 2 with the largest |M - I| in *dev (FP32 bits), else the
-// first-order eigenvector corrections of M = V^H S V (diag: scratch, n_mat N).
+// first-order corrections below lim of M = V^H S V or W^H W (diag: scratch,
+// n_mat N) with the largest |M_ij| / sqrt(M_ii M_jj) in *dev.
 cudaError_t launch_proj_load32(int cplx, int n_mat, int N, int Np, const double* W, float* scale, float* W32, float* V32,
                                cudaStream_t s);
 int launch_jacobi32_sweep(int cplx, int n_mat, int N, int Np, float* W32, float* V32, float thresh, unsigned* off_max,
@@ -156,8 +157,8 @@ cudaError_t launch_proj_widen(long n, const float* x, double* y, cudaStream_t s)
 // Sweeps of W and V over each k-point's few columns with large cosines in G = W^H W.
 cudaError_t launch_proj_cluster(int cplx, int n_mat, int N, int Np, const double* G, double* W, double* V, double thresh,
                                 cudaStream_t s);
-cudaError_t launch_proj_corr(int cplx, int n_mat, int N, bool ortho, double* M, double* diag, unsigned* dev,
-                             cudaStream_t s);
+cudaError_t launch_proj_corr(int cplx, int n_mat, int N, bool ortho, double* M, double* diag, float lim,
+                             unsigned* dev, cudaStream_t s);
 // Eigenvalues (column norms of W) in ascending order into lam_sorted
 // [n_mat][N], the column of each rank into by_rank, m = the largest count
 // below eps_d over the k-points (into *m, zeroed by the caller), then

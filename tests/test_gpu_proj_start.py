@@ -80,3 +80,11 @@ def test_projector_start_matches_plain_sweeps(rpa, cplx, nb, ovl, scale):
         assert np.array_equal(ea, eb)
     for k in range(p.n_kpts):
         assert float((a[k] - b[k]).abs().max()) <= 20 * tol
+
+
+@pytest.mark.parametrize("cplx,nb", [(True, (32, 32)), (False, (33, 32)), (True, (225, 225)), (True, (226, 227)),
+                                     (True, (451, 454))])
+def test_projector_start_column_blocks(rpa, cplx, nb):
+    """The smallest basis of the start, the edge between blocks of 16 and 8
+    columns, and columns too long for either."""
+    test_projector_start_matches_plain_sweeps(rpa, cplx, nb, None, 1.0)
