@@ -63,7 +63,7 @@ typedef int rpa_status;
 
 /* Arithmetic of the chi0 contraction.  The sandwich, the factorisation and
  * all sums are FP64 in every mode. */
-#define RPA_PREC_FP64 0  /* chi0 in FP64 (DFMA) */
+#define RPA_PREC_FP64 0  /* chi0 to FP64 rounding (exact digit products, DFMA) */
 #define RPA_PREC_MIXED 1 /* chi0 on tcgen05 tensor cores from BF16 slices of
                             the FP64 operands, FP32 accumulation in exact
                             chunks, FP64 result (split-precision, Ozaki-style) */

@@ -20,7 +20,7 @@
 //      reads B at its own K offset);
 //   8. reduce_bin_kernel: per element the split-K partials of every (b, r),
 //      scaled by their exponents and combined with coef into all n_w
-//      frequencies in FP64, Hermitian store.
+//      frequencies in float-float arithmetic, Hermitian store.
 // With all skeletons in one round and two workspace regions, q+1's weighted
 // planes are written by the slicer warps of q's tensor-core launch (its
 // steps 1-6 run before that launch).  Included by kernels_mixed.cu.

@@ -2,13 +2,15 @@
 //
 // GB300 executes FP64 at about 1/58 of its FP32 rate (1.2 TFLOP/s measured
 // for DFMA and DGEMM), so every kernel here is bound by the FP64 pipe and is
-// organised to issue as few FP64 instructions per useful result as possible:
+// organised to issue as few FP64 instructions per useful result as possible.
+// Larger chi0 and sandwich calls run as digit products on the tensor cores
+// (g64.cu) and come here only for matrices those cannot hold (`only` flags).
 //   * chi0: the product conj(C_P,t) C_Q,t is formed once per t and reused for
 //     a group of G frequencies (2 DFMA per frequency instead of 4), and only
 //     the lower triangle of tiles is computed (chi0 is Hermitian);
 //   * the sandwich uses the Cholesky factor L of V (triangular operands, lower
 //     output only) instead of the dense V^(1/2);
-//   * the factorisation of 1 - Pi keeps the diagonal in "pivot minus one"
+//   * the factorisation of 1 - Pi (cholesky.cu) keeps the diagonal in "pivot minus one"
 //     form so that ln det = sum log1p(u) keeps its digits as Pi -> 0;
 //   * the inverse form used with the split-precision chi0 needs no sandwich at
 //     all: det(1 - V^(1/2) chi V^(1/2)) = det(V^-1 - chi) det V and
