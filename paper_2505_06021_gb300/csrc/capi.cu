@@ -594,10 +594,13 @@ static rpa_status stage_logdet(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
   if (b.Vc) {
     // inverse form: one Cholesky of V^-1 - chi per (q, w); no sandwich
     prof_begin(ctx, pex, s);
+    int nc = 0;
+    const CholOuter co{b.tail, b.tail_bytes};
     CK(launch_cholesky(j->is_complex, j->n_aux, nq * j->n_w, b.chi, mstride, 2, b.parts + (size_t)2 * q0 * j->n_w,
-                       b.status, q0 * j->n_w, s, b.L, b.Vc, b.ldV + q0, j->n_w));
-    prof_end(ctx, pex, s, RPA_K_LOGDET, cholesky_launches(j->n_aux, nq * j->n_w, 2));
-    ctx->launches += cholesky_launches(j->n_aux, nq * j->n_w, 2);
+                       b.status, q0 * j->n_w, s, b.L, b.Vc, b.ldV + q0, j->n_w,
+                       b.tail && chol_g64_use(j->is_complex, j->n_aux, nq * j->n_w, 2) ? &co : nullptr, &nc));
+    prof_end(ctx, pex, s, RPA_K_LOGDET, nc);
+    ctx->launches += nc;
     return RPA_OK;
   }
   // Y = -(L^H chi L) (lower triangle), overwriting chi's storage
@@ -608,10 +611,13 @@ static rpa_status stage_logdet(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const 
   ctx->launches += nl;
   // 1 - Pi' = 1 + Y: Cholesky, ln det, Tr
   prof_begin(ctx, pex, s);
+  int nc = 0;
+  const CholOuter co{b.tail, b.tail_bytes};
   CK(launch_cholesky(j->is_complex, j->n_aux, nq * j->n_w, b.chi, mstride, 0, b.parts + (size_t)2 * q0 * j->n_w,
-                     b.status, q0 * j->n_w, s));
-  prof_end(ctx, pex, s, RPA_K_LOGDET, cholesky_launches(j->n_aux, nq * j->n_w, 0));
-  ctx->launches += cholesky_launches(j->n_aux, nq * j->n_w, 0);
+                     b.status, q0 * j->n_w, s, nullptr, nullptr, nullptr, j->n_w,
+                     b.tail && chol_g64_use(j->is_complex, j->n_aux, j->n_w, 0) ? &co : nullptr, &nc));
+  prof_end(ctx, pex, s, RPA_K_LOGDET, nc);
+  ctx->launches += nc;
   return RPA_OK;
 }
 
@@ -1190,15 +1196,18 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   prof_begin(ctx, &ex, s);
   CK(launch_cholesky(job->is_complex, job->n_aux, 1, b.L, (long)(NN * (es / 8)), 1, nullptr, b.status,
                      (1 << 29) + q, s));
-  const int nv = cholesky_launches(job->n_aux, 1, 1), nd = cholesky_launches(job->n_aux, job->n_w, 0);
+  const int nv = cholesky_launches(job->n_aux, 1, 1);
+  int nd = 0;
+  const CholOuter co{b.tail, b.tail_bytes};
   prof_end(ctx, &ex, s, RPA_K_VFACTOR, nv);
   prof_begin(ctx, &ex, s);
   uint64_t nsw = 0;
   CK(sandwich(job->is_complex, job->n_aux, job->n_w, job->n_w, b, (const double*)chi, b.chi, &nsw, s));
   prof_end(ctx, &ex, s, RPA_K_SANDWICH, (int)nsw);
   prof_begin(ctx, &ex, s);
-  CK(launch_cholesky(job->is_complex, job->n_aux, job->n_w, b.chi, (long)(NN * (es / 8)), 0, b.parts, b.status, 0,
-                     s));
+  CK(launch_cholesky(job->is_complex, job->n_aux, job->n_w, b.chi, (long)(NN * (es / 8)), 0, b.parts, b.status, 0, s,
+                     nullptr, nullptr, nullptr, job->n_w,
+                     b.tail && chol_g64_use(job->is_complex, job->n_aux, job->n_w, 0) ? &co : nullptr, &nd));
   prof_end(ctx, &ex, s, RPA_K_LOGDET, nd);
   ctx->launches += nv + nsw + nd;
   if (!ex.hres.reserve(64 + sizeof(double) * 2 * job->n_w)) return RPA_E_NOMEM;

@@ -29,9 +29,12 @@
 // launches now: one complex N = 768 factor of V 19.9 -> 2.4 ms; 16 matrices of
 // N = 768 in FP64 30.1 -> 9.7 ms; 32 in the inverse form 17.6 -> 8.8 ms; 320 of
 // N = 512 in the inverse form 34.7 -> 19.4 ms; 64 of N = 300 18.6 -> 1.6 ms; 16
-// real ones of N = 64 0.285 -> 0.065 ms.  What is left is the FP64 pipe (the 16
-// FP64 matrices need 7.6 ms of it) and, for few matrices, two launches of some
-// 20 us each per panel.
+// real ones of N = 64 0.285 -> 0.065 ms.  There the 16 FP64 matrices need 7.6 ms of
+// the FP64 pipe and take 9.7, so larger batches (chol_g64_use) leave all but 1/(N /
+// 128) of the trailing updates to the tensor cores, one block column of 128
+// columns at a time: 16 of N = 768 9.9 -> 4.4 ms, 320 of N = 512 in the inverse form
+// 19.3 -> 14.4 ms.  What is left is the FP64 work inside the block columns and, for few
+// matrices, two launches of some 20 us each per panel.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -42,6 +45,7 @@
 #include <vector>
 
 #include "fp64_elem.cuh"
+#include "g64.h"
 #include "rpa_internal.h"
 
 namespace rpa {
@@ -306,16 +310,16 @@ __global__ void __launch_bounds__(256) chol_init_kernel(const __grid_constant__ 
   }
 }
 
-// The first diagonal block of every matrix, and the traces (mode 0: Tr Pi =
-// -sum Y_jj; mode 2: the partial sums of chol_init_kernel).
+// The diagonal block at kb of every matrix, and with the first (kb = 0) the
+// traces (mode 0: Tr Pi = -sum Y_jj; mode 2: the partial sums of chol_init_kernel).
 template <bool C, int NB>
-__global__ void __launch_bounds__(256) chol_first_kernel(const __grid_constant__ CholBatch B, int nblk) {
+__global__ void __launch_bounds__(256) chol_first_kernel(const __grid_constant__ CholBatch B, int nblk, int kb) {
   __shared__ Elem<C> D[NB][CB + 1];
   __shared__ DiagShared<C, NB> S;
   __shared__ double red[8];
   const CholTask t = task_of<C>(B, blockIdx.x);
-  const int N = t.N, tid = threadIdx.x, nb = min(NB, N);
-  if (t.mode != 1) {
+  const int N = t.N, tid = threadIdx.x, nb = min(NB, N - kb);
+  if (t.mode != 1 && kb == 0) {
     double s = 0.0;
     if (t.mode == 0) {
       for (int j = tid; j < N; j += 256) s -= ld_elem<C>(t.A, (long)j * N + j).re;
@@ -327,11 +331,57 @@ __global__ void __launch_bounds__(256) chol_first_kernel(const __grid_constant__
   }
   for (int i = tid; i < NB * NB; i += 256) {
     const int r = i / NB, c = i % NB;
-    if (r < nb && c <= r) D[r][c] = ld_elem<C>(t.A, (long)r * N + c);
+    if (r < nb && c <= r) D[r][c] = ld_elem<C>(t.A, (long)(kb + r) * N + kb + c);
   }
   __syncthreads();
-  const double lg = diag_factor<C, NB>(D, S, nb, t.mode, t.A, N);
-  if (tid == 0) diag_report(t, lg, S.bad, true, N <= NB);
+  const double lg = diag_factor<C, NB>(D, S, nb, t.mode, t.A + ((long)kb * N + kb) * (C ? 2 : 1), N);
+  if (tid == 0) diag_report(t, lg, S.bad, kb == 0, N - kb <= NB);
+}
+
+// Block columns (chol_outer below) of matrices out of the digit split's range:
+// A[r][c] -= sum_{k < J0} L[r][k] conj(L[c][k]), J0 <= c < cend, in FP64.
+template <bool C>
+__global__ void __launch_bounds__(256) chol_outer_kernel(int N, double* __restrict__ mats, long bstride, int J0,
+                                                         int cend, int per, const int* __restrict__ only) {
+  constexpr int T = 32, KS = 16;
+  __shared__ Elem<C> S1[T][KS + 1], S2[T][KS + 1];
+  const int b = blockIdx.x / per, tile = blockIdx.x % per;
+  if (!(only[b] & 1)) return;
+  const int nc = (cend - J0 + T - 1) / T, TI = tile / nc, TJ = tile % nc;
+  if (TI < TJ) return;
+  double* A = mats + (long)b * bstride;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  Elem<C> o[2][2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const int r = J0 + TI * T + ty + 16 * u, c = J0 + TJ * T + tx + 16 * v;
+      o[u][v] = r < N && c < N ? ld_elem<C>(A, (long)r * N + c) : zero_elem<C>();
+    }
+  for (int k0 = 0; k0 < J0; k0 += KS) {
+    for (int i = tid; i < T * KS; i += 256) {
+      const int r = i / KS, k = k0 + i % KS;
+      const int ri = J0 + TI * T + r, rj = J0 + TJ * T + r;
+      S1[r][i % KS] = ri < N && k < J0 ? ld_elem<C>(A, (long)ri * N + k) : zero_elem<C>();
+      S2[r][i % KS] = rj < N && k < J0 ? ld_elem<C>(A, (long)rj * N + k) : zero_elem<C>();
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < KS; ++k)
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) msub_conj<C>(o[u][v], S1[ty + 16 * u][k], S2[tx + 16 * v][k]);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const int r = J0 + TI * T + ty + 16 * u, c = J0 + TJ * T + tx + 16 * v;
+      if (r < N && c < cend && c <= r) st_elem<C>(A, (long)r * N + c, o[u][v]);
+    }
 }
 
 // Panel rows below the diagonal block at kb (full panels only: kb + NB < N).
@@ -371,10 +421,11 @@ __global__ void __launch_bounds__(32 * WARPS) chol_panel_kernel(const __grid_con
 // triangle beyond it, U x U outputs per thread; FP64 (FF = false) or, on the
 // split-precision path, float-float on the FP32 pipe (about 2^-45 of the
 // update, five times the FP64 pipe's rate).  Tile (0, 0) goes on to factor
-// the next diagonal block.
+// the next diagonal block.  Only columns below cend (a multiple of the panel
+// width, or at least N).
 template <bool C, bool FF, int NB, int U>
 __global__ void __launch_bounds__(256, FF ? 3 : 2)
-    chol_update_kernel(const __grid_constant__ CholBatch B, int kb, int per) {
+    chol_update_kernel(const __grid_constant__ CholBatch B, int kb, int per, int cend) {
   static_assert(NB <= 16 * U, "the first tile holds the next diagonal block");
   constexpr int T = 16 * U, SR = NB > T ? NB : T;
   __shared__ Elem<C> S1[SR][CB + 1];
@@ -385,9 +436,16 @@ __global__ void __launch_bounds__(256, FF ? 3 : 2)
   const int N = t.N, m0 = kb + NB, m = N - m0;
   if (m <= 0) return;
   const int nt = (m + T - 1) / T;
-  if (tile >= nt * (nt + 1) / 2) return;
   int TI, TJ;
-  tri_ij(tile, TI, TJ);
+  if (cend < N) {
+    const int nc = (cend - m0 + T - 1) / T;
+    TI = tile / nc;
+    TJ = tile % nc;
+    if (TI >= nt || TI < TJ) return;
+  } else {
+    if (tile >= nt * (nt + 1) / 2) return;
+    tri_ij(tile, TI, TJ);
+  }
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   double* A = t.A;
   Elem<C> o[U][U];  // the tile's own values, in flight during the product
@@ -462,7 +520,7 @@ __global__ void __launch_bounds__(256, FF ? 3 : 2)
       const int r = m0 + TI * T + lr, c = m0 + TJ * T + lc;
       if (diag && lr < NB && lc < NB)
         S1[lr][lc] = o[u][v];
-      else if (r < N && c <= r)
+      else if (r < N && c <= r && c < cend)
         st_elem<C>(A, (long)r * N + c, o[u][v]);
     }
   if (!diag) return;
@@ -707,11 +765,100 @@ bool panel32(int N, long n_mat) {
   return n_mat * h * (h + 1) / 2 >= 8L * device_sm_count();
 }
 
+// Block columns of OUTER columns (modes 0 and 2 with planes): the panels update
+// only inside their block column, and each block column takes everything to its
+// left at once as a digit product on the tensor cores (g64.cu),
+// A[J0.., J] -= L[J0.., < J0] L[J, < J0]^H, whose planes are made of the finished columns.
+constexpr int OUTER = 128;
+
+struct OuterBytes {
+  size_t a, b, ea, eb, one;  // planes and exponents of one matrix, the largest block column
+};
+OuterBytes outer_bytes(int cplx, int N) {
+  OuterBytes o{};
+  for (int J0 = OUTER; J0 < N; J0 += OUTER) {
+    o.a = std::max(o.a, g64_plane_bytes(cplx, 0, N - J0, J0, 1));
+    o.b = std::max(o.b, g64_plane_bytes(cplx, 1, std::min(OUTER, N - J0), J0, 1));
+  }
+  o.ea = sizeof(int) * (size_t)g64_rpad(cplx, 0, N);
+  o.eb = sizeof(int) * (size_t)g64_rpad(cplx, 1, OUTER);
+  o.one = o.a + o.b + o.ea + o.eb;
+  return o;
+}
+
+cudaError_t chol_outer(int cplx, int N, int n_mat, double* mats, long bstride, int J0, const CholOuter& x, int* status,
+                       cudaStream_t s) {
+  const OuterBytes t = outer_bytes(cplx, N);
+  const long cs = cplx ? 2 : 1;
+  const int C = std::min(OUTER, N - J0), R = N - J0;
+  const size_t fb = ((sizeof(int) * (size_t)n_mat + 1023) / 1024) * 1024;
+  int* flag = (int*)x.work;
+  if (x.bytes < fb + t.one) return cudaErrorInvalidValue;
+  const int room = (int)std::min<size_t>((size_t)n_mat, (x.bytes - fb) / t.one);
+  if (cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int) * (size_t)n_mat, s)) return e;
+  for (int b0 = 0; b0 < n_mat; b0 += room) {
+    const int nb = std::min(room, n_mat - b0);
+    char* p = (char*)x.work + fb;
+    double* Ab = mats + b0 * bstride;
+    // conj(L) by rows, its rows J0.. and J0 .. J0 + C - 1
+    auto src = [&](int rows) {
+      G64Src g{};
+      g.base = Ab + (long)J0 * N * cs;
+      g.stride = bstride / cs;
+      g.ld = N;
+      g.by_rows = 1;
+      g.conj = 1;
+      g.nb = nb;
+      g.R = rows;
+      g.K = J0;
+      return g;
+    };
+    G64Op oa{}, ob{};
+    oa.planes = (uint16_t*)p;
+    ob.planes = (uint16_t*)(p + t.a * (size_t)nb);
+    oa.e = (int*)(p + (t.a + t.b) * (size_t)nb);
+    ob.e = (int*)(p + (t.a + t.b + t.ea) * (size_t)nb);
+    oa.stride = (long)(g64_plane_bytes(cplx, 0, R, J0, 1) / 2);
+    ob.stride = (long)(g64_plane_bytes(cplx, 1, C, J0, 1) / 2);
+    oa.Rpad = g64_rpad(cplx, 0, R);
+    ob.Rpad = g64_rpad(cplx, 1, C);
+    oa.n_kb = ob.n_kb = g64_nkb(cplx, J0);
+    if (cudaError_t e = g64_slice(cplx, 0, src(R), oa, flag + b0, 1, s)) return e;
+    if (cudaError_t e = g64_slice(cplx, 1, src(C), ob, flag + b0, 1, s)) return e;
+    G64Out o{};
+    o.base = Ab + ((long)J0 * N + J0) * cs;
+    o.stride = bstride / cs;
+    o.s0 = N;
+    o.t0 = 1;
+    o.rd = o.cd = 1 << 30;
+    o.R = R;
+    o.C = C;
+    o.add = o.neg = 1;
+    o.tri = 2;
+    if (cudaError_t e = g64_product(cplx, oa, ob, G64Index{nullptr, nullptr, 1, 1}, o, nb, 0, nullptr, 0, flag + b0, 1,
+                                    status, nullptr, s))
+      return e;
+    const int per = ((R + 31) / 32) * ((C + 31) / 32);
+    if (cplx)
+      chol_outer_kernel<true><<<(unsigned)(nb * per), 256, 0, s>>>(N, Ab, bstride, J0, J0 + C, per, flag + b0);
+    else
+      chol_outer_kernel<false><<<(unsigned)(nb * per), 256, 0, s>>>(N, Ab, bstride, J0, J0 + C, per, flag + b0);
+  }
+  return cudaGetLastError();
+}
+int outer_launches(int cplx, int N, int n_mat, size_t bytes) {
+  const OuterBytes t = outer_bytes(cplx, N);
+  const size_t fb = ((sizeof(int) * (size_t)n_mat + 1023) / 1024) * 1024;
+  const int room = (int)std::min<size_t>((size_t)n_mat, (bytes - fb) / t.one);
+  return (n_mat + room - 1) / room * 6;
+}
+
 // Launches of one batch whose largest matrix is N (tasks sorted by size,
 // largest first, when ragged: Ns[b] is task b's size, so that each panel
 // covers only the prefix that still has one).
 template <bool C>
-cudaError_t chol_run(const CholBatch& B, int N, int n_mat, const int* Ns, int mode, cudaStream_t s, int* n_launch) {
+cudaError_t chol_run(const CholBatch& B, int N, int n_mat, const int* Ns, int mode, cudaStream_t s, int* n_launch,
+                     const CholOuter* outer) {
   int nl = 0;
   if (N <= SMALL_N) {
     if (cudaError_t e = small_attr<C>()) return e;
@@ -725,9 +872,9 @@ cudaError_t chol_run(const CholBatch& B, int N, int n_mat, const int* Ns, int mo
   }
   const bool wide = mode == 2 && panel32(N, n_mat);
   if (wide)
-    chol_first_kernel<C, 32><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS);
+    chol_first_kernel<C, 32><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS, 0);
   else
-    chol_first_kernel<C, 16><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS);
+    chol_first_kernel<C, 16><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS, 0);
   ++nl;
   const long sms = device_sm_count();
   const int NB = wide ? 32 : 16;
@@ -750,23 +897,41 @@ cudaError_t chol_run(const CholBatch& B, int N, int n_mat, const int* Ns, int mo
       else
         chol_panel_kernel<C, 16, 4, 8><<<(unsigned)(live * per64), 256, 0, s>>>(B, kb, per64);
     }
+    ++nl;
     const long n32 = (m + 31) / 32, n16 = (m + 15) / 16;
-    const int per32 = (int)(n32 * (n32 + 1) / 2), per16 = (int)(n16 * (n16 + 1) / 2);
+    int per32 = (int)(n32 * (n32 + 1) / 2), per16 = (int)(n16 * (n16 + 1) / 2), cend = N;
+    if (outer) {
+      cend = std::min(N, (kb / OUTER + 1) * OUTER);
+      if (kb + NB == cend) {  // the next block column
+        if (cudaError_t e = chol_outer(C ? 1 : 0, N, n_mat, B.mats, B.bstride, cend, *outer, B.status, s)) return e;
+        if (wide)
+          chol_first_kernel<C, 32><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS, cend);
+        else
+          chol_first_kernel<C, 16><<<n_mat, 256, 0, s>>>(B, INIT_BLOCKS, cend);
+        nl += 1 + outer_launches(C ? 1 : 0, N, n_mat, outer->bytes);
+        continue;
+      }
+      if (cend < N) {
+        const int w = cend - kb - NB;
+        per32 = (int)(n32 * ((w + 31) / 32));
+        per16 = (int)(n16 * ((w + 15) / 16));
+      }
+    }
     // 16 x 16 tiles until 32 x 32 ones give every SM two (they read less)
     const bool t32 = live * (long)per32 >= 2 * sms;
     if (mode == 2) {
       if (wide)
-        chol_update_kernel<C, true, 32, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32);
+        chol_update_kernel<C, true, 32, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32, cend);
       else if (t32)
-        chol_update_kernel<C, true, 16, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32);
+        chol_update_kernel<C, true, 16, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32, cend);
       else
-        chol_update_kernel<C, true, 16, 1><<<(unsigned)(live * per16), 256, 0, s>>>(B, kb, per16);
+        chol_update_kernel<C, true, 16, 1><<<(unsigned)(live * per16), 256, 0, s>>>(B, kb, per16, cend);
     } else if (t32) {
-      chol_update_kernel<C, false, 16, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32);
+      chol_update_kernel<C, false, 16, 2><<<(unsigned)(live * per32), 256, 0, s>>>(B, kb, per32, cend);
     } else {
-      chol_update_kernel<C, false, 16, 1><<<(unsigned)(live * per16), 256, 0, s>>>(B, kb, per16);
+      chol_update_kernel<C, false, 16, 1><<<(unsigned)(live * per16), 256, 0, s>>>(B, kb, per16, cend);
     }
-    nl += 2;
+    ++nl;
   }
   if (n_launch) *n_launch = nl;
   return cudaGetLastError();
@@ -776,15 +941,27 @@ cudaError_t chol_run(const CholBatch& B, int N, int n_mat, const int* Ns, int mo
 
 cudaError_t launch_cholesky(int cplx, int N, int n_mat, double* mats, long bstride, int mode, double* out,
                             int* status, int status_base, cudaStream_t s, const double* Wn, const double* Vc,
-                            const double* ldV, int n_w) {
+                            const double* ldV, int n_w, const CholOuter* outer, int* n_launch) {
   if (n_mat == 0) return cudaSuccess;
   if (mode == 2 && (!Wn || !Vc || !ldV || n_w <= 0)) return cudaErrorInvalidValue;
   if (mode != 1 && !out) return cudaErrorInvalidValue;
   const long nt = (N + 15) / 16;
   if ((long)n_mat * std::max<long>(nt * (nt + 1) / 2, INIT_BLOCKS) > 0x7fffffffL) return cudaErrorInvalidValue;
   const CholBatch B{nullptr, mats, bstride, out, status, Wn, Vc, ldV, N, mode, status_base, std::max(n_w, 1)};
-  return cplx ? chol_run<true>(B, N, n_mat, nullptr, mode, s, nullptr)
-              : chol_run<false>(B, N, n_mat, nullptr, mode, s, nullptr);
+  if (outer && (N <= OUTER || mode == 1 || !outer->work)) outer = nullptr;
+  return cplx ? chol_run<true>(B, N, n_mat, nullptr, mode, s, n_launch, outer)
+              : chol_run<false>(B, N, n_mat, nullptr, mode, s, n_launch, outer);
+}
+
+// The digit products save FP64 work (mode 0) or a fifth of it on the FP32 pipe (mode
+// 2) and add some 60 us of launches per block column.  Measured, log-det step of
+// one q with and without: complex N = 384, 8 frequencies 2.07 and 2.25 ms, N = 512,
+// 16 4.07 and 5.39, N = 768, 8 5.71 and 8.29; real N = 384, 16 equal, N = 512, 16
+// 2.36 and 2.54, N = 768, 16 4.15 and 5.15.  Inverse form: 16 real of N = 733 2.12 and
+// 1.65 (not taken), 32 complex of N = 768 7.4 and 9.2, 320 of N = 512 14.4 and 19.3.
+bool chol_g64_use(int cplx, int N, int n, int mode) {
+  const double macs = (cplx ? 4.0 : 1.0) * N * (double)N * N * n;
+  return N >= 384 && n >= 8 && macs >= (mode == 2 ? 2.5e10 : 1.5e9);
 }
 
 int cholesky_launches(int N, int n_mat, int mode) {
@@ -812,8 +989,8 @@ cudaError_t launch_cholesky_ragged(int cplx, const CholTask* tasks, const CholTa
     CholBatch B{};
     B.tasks = tasks + lo;
     int nl = 0;
-    const cudaError_t e = cplx ? chol_run<true>(B, Ns[lo], n, Ns.data() + lo, mode, s, &nl)
-                               : chol_run<false>(B, Ns[lo], n, Ns.data() + lo, mode, s, &nl);
+    const cudaError_t e = cplx ? chol_run<true>(B, Ns[lo], n, Ns.data() + lo, mode, s, &nl, nullptr)
+                               : chol_run<false>(B, Ns[lo], n, Ns.data() + lo, mode, s, &nl, nullptr);
     if (e != cudaSuccess) return e;
     total += nl;
   }

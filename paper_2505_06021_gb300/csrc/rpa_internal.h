@@ -55,9 +55,20 @@ cudaError_t launch_chi0_fp64(const BatchGeom& g, const double* const* Cptrs, con
 // the matrix is abandoned.
 cudaError_t launch_cholesky(int cplx, int N, int n_mat, double* mats, long bstride, int mode, double* out,
                             int* status, int status_base, cudaStream_t s, const double* Wn = nullptr,
-                            const double* Vc = nullptr, const double* ldV = nullptr, int n_w = 0);
+                            const double* Vc = nullptr, const double* ldV = nullptr, int n_w = 0,
+                            const struct CholOuter* outer = nullptr, int* n_launch = nullptr);
+// Workspace for the trailing updates of modes 0 and 2 as digit products on the
+// tensor cores (tail_g64_bytes of any number of matrices is enough), and whether n
+// matrices of size N take them (mode 0: n per q, since its answer decides the bits
+// of an FP64 job; mode 2: all of the launch).
+struct CholOuter {
+  void* work;
+  size_t bytes;
+};
+bool chol_g64_use(int cplx, int N, int n, int mode);
 
-// Kernel launches launch_cholesky makes for n_mat matrices of size N.
+// Kernel launches launch_cholesky makes for n_mat matrices of size N without `outer`
+// (with it: *n_launch).
 int cholesky_launches(int N, int n_mat, int mode);
 
 // One matrix of a ragged Cholesky launch (matrices of different sizes).

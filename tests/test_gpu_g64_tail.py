@@ -102,3 +102,41 @@ def test_inverse_form_energy_matches(rpa, n):
             r.append(c.energy(job))
     assert np.max(np.abs(r[0]["lndet"] - r[1]["lndet"])) <= 1e-11
     assert abs(r[0]["Ec"] - r[1]["Ec"]) <= 1e-11 * abs(r[1]["Ec"])
+
+
+@pytest.mark.parametrize("cplx,n,n_w", [(True, 384, 8), (True, 385, 9), (True, 513, 8), (False, 400, 20), (False, 640, 8)])
+def test_block_columns_match_fp64_kernels(rpa, cplx, n, n_w):
+    """Sizes whose Cholesky factors take their block columns as digit products
+    (twice the tolerance: N to 640)."""
+    V, chi = _inputs(cplx, n, n_w, 94)
+    a, b = _both(rpa, cplx, n, n_w, V, chi)
+    assert np.all(np.abs(a - b) <= 2 * TOL * np.abs(b)), np.max(np.abs(a - b) / np.abs(b))
+
+
+@pytest.mark.parametrize("far", [2.0 ** 12, 2.0 ** 80])
+def test_block_columns_spread_row(rpa, far):
+    """V = 1 and a pair of rows whose factor holds one entry far above the others."""
+    _, chi = _inputs(True, 400, 8, 95)
+    V = torch.eye(400, dtype=torch.complex128, device="cuda")
+    chi[2, 5, 300] = chi[2, 300, 5] = -far
+    chi[2, 5, 5] -= 2.0 * far
+    chi[2, 300, 300] -= 2.0 * far
+    a, b = _both(rpa, True, 400, 8, V, chi)
+    assert np.all(np.abs(a - b) <= 2 * TOL * np.abs(b)), np.max(np.abs(a - b) / np.abs(b))
+
+
+@pytest.mark.parametrize("n,n_w", [(400, 25), (512, 16)])
+def test_inverse_form_block_columns(rpa, n, n_w):
+    """Split-precision job with digit-product block columns against the FP64
+    kernels' tail on the same chi0 plan; the float-float updates of the latter keep
+    about 2^-45 of each update: 400 pivots of 2^-45 at most, 1e-11 of ln det."""
+    from paper_2505_06021_gb300 import synth
+
+    p = synth.make_problem("tailb", is_complex=True, n_aux=n, n_occ=3, n_virt=12, grid=synth.regular_kq_grid((2, 2, 1)),
+                           n_w=n_w, seed=96)
+    job = rpa.job_from_problem(p, rpa.upload_problem(p), prec=rpa.PREC_MIXED)
+    r = []
+    for cap in (0, 1 << 20):
+        with rpa.Context(0, hbm_cap_bytes=cap, chi0_freq=1) as c:
+            r.append(c.energy(job))
+    assert np.max(np.abs(r[0]["lndet"] - r[1]["lndet"])) <= 2e-11 * max(1.0, np.max(np.abs(r[1]["lndet"])))
