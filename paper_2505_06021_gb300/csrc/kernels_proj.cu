@@ -33,7 +33,7 @@
 // shows a cosine above 1e-14, the FP64 sweeps finish.  Measured, 16 overlaps of 256
 // functions: three FP64 sweeps of 255 rounds (23 us each, 17.8 ms in all) became 0.7
 // ms of products, 29.9 -> 13.1 ms in all; what is left is the FP32 sweeps
-// (7 ms, shared-memory bandwidth) and the refinement's products.
+// (7 ms) and the refinement's products.
 //
 // Since the eigenvalues are taken in ascending order and R~ is a product over
 // k, R~ removes the m lowest positions at every k-point, m the largest count
@@ -373,8 +373,10 @@ __device__ __forceinline__ float rotate32(Flt<C>* wp, Flt<C>* wq, Flt<C>* vp, Fl
 // rounds of B disjoint pairs, a warp each) and writes them back; the first block
 // round of a sweep also rotates the pairs within the blocks (2 B - 1 rounds).  A
 // sweep then reads and writes the columns nb - 1 times, not Np - 1, and has as
-// many launches (nb blocks).  What bounds a round inside the CTA is shared
-// memory: 16 warps read W twice, V once and write both.
+// many launches (nb blocks).  What bounds a round inside the CTA is each warp's
+// chain of loads, sums and rotation (2.8 us; shared memory 44 % and issue 47 %
+// busy).  16 overlaps of 256 functions: 50.8 -> 29.9 ms in all against a
+// launch per round in global memory.
 template <bool C, int B>
 __global__ void __launch_bounds__(32 * B) jacobi32_block_kernel(int N, int Np, int nb, int br, float* __restrict__ W32,
                                                                 float* __restrict__ V32, float thresh,
