@@ -139,10 +139,15 @@ __device__ __forceinline__ void pair_dots(const double* xc, const double* yc, in
   if constexpr (C) gi = warp_sum(gi);
 }
 
-// Sums of the four values over the CTA's warps, valid in every thread.
-__device__ __forceinline__ void cta_join(double (*red)[4], double& a, double& b, double& gr, double& gi) {
+// The rotation of a CTA's column pair from its warps' sums, by thread 0 alone: its
+// roots, divisions and sums are FP64 instructions of one warp (64 clocks of a
+// sub-partition each, however few lanes take part), and seven more warps that
+// repeat them would share the same four pipes.  rot: c, s, e (re, im), 1 if the
+// cosine is above thresh; returns the cosine (thread 0), 0 elsewhere.
+__device__ __forceinline__ double cta_rotation(double (*red)[4], double* rot, double a, double b, double gr, double gi,
+                                               double thresh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();  // red is free again
+  double off = 0.0;
   if (lane == 0) {
     red[wid][0] = a;
     red[wid][1] = b;
@@ -150,24 +155,37 @@ __device__ __forceinline__ void cta_join(double (*red)[4], double& a, double& b,
     red[wid][3] = gi;
   }
   __syncthreads();
-  a = b = gr = gi = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-    a += red[w][0];
-    b += red[w][1];
-    gr += red[w][2];
-    gi += red[w][3];
+  if (threadIdx.x == 0) {
+    a = b = gr = gi = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      a += red[w][0];
+      b += red[w][1];
+      gr += red[w][2];
+      gi += red[w][3];
+    }
+    const double g = sqrt(gr * gr + gi * gi);
+    off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
+    rot[4] = 0.0;
+    if (off > thresh) {
+      pair_rotation(a, b, gr, gi, g, rot[0], rot[1], rot[2], rot[3]);
+      rot[4] = 1.0;
+    }
   }
+  __syncthreads();
+  return off;
 }
 
 // One round r: columns (p, q) of pair i of W[k] are rotated, by a CTA each
 // (WARP = false) or, when the pairs of all k-points fill the GPU, by a warp each,
 // four to a CTA: no barriers, and once most pairs are orthogonal a round is
-// the FP64 pipe's time for the inner products.
+// the FP64 pipe's time for the inner products.  Calls on 63 functions and 1, 9 and
+// 16 k-points: 7.1, 8.6 and 12 ms (9.7, 17.2 and 29.8 with the rotation in all eight
+// warps of the CTA).
 template <bool C, bool WARP>
 __global__ void __launch_bounds__(WARP ? 128 : 256) jacobi_round_kernel(int N, int Np, int r, double* __restrict__ W,
                                                                         double* __restrict__ V, double thresh,
                                                                         unsigned long long* __restrict__ off_max) {
-  __shared__ double red[8][4];
+  __shared__ double red[8][4], rot[5];
   const int lane = threadIdx.x & 31, k = blockIdx.y;
   const int i = WARP ? blockIdx.x * 4 + (threadIdx.x >> 5) : blockIdx.x;
   if (i >= Np / 2) return;
@@ -176,15 +194,25 @@ __global__ void __launch_bounds__(WARP ? 128 : 256) jacobi_round_kernel(int N, i
   double* wp = W + ((size_t)k * Np + p) * N * (C ? 2 : 1);
   double* wq = W + ((size_t)k * Np + q) * N * (C ? 2 : 1);
   const int first = WARP ? lane : threadIdx.x, step = WARP ? 32 : 256;
-  double a, b, gr, gi;
+  double a, b, gr, gi, off, c, s, er, ei;
   pair_dots<C>(wp, wq, N, first, step, a, b, gr, gi);
-  if constexpr (!WARP) cta_join(red, a, b, gr, gi);
-  const double g = sqrt(gr * gr + gi * gi);
-  const double off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
+  if constexpr (WARP) {
+    const double g = sqrt(gr * gr + gi * gi);
+    off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
+    if (off > thresh) pair_rotation(a, b, gr, gi, g, c, s, er, ei);
+  } else {
+    off = cta_rotation(red, rot, a, b, gr, gi, thresh);
+  }
   if (first == 0) atomicMax(off_max, (unsigned long long)__double_as_longlong(off));
-  if (!(off > thresh)) return;
-  double c, s, er, ei;
-  pair_rotation(a, b, gr, gi, g, c, s, er, ei);
+  if constexpr (WARP) {
+    if (!(off > thresh)) return;
+  } else {
+    if (rot[4] == 0.0) return;
+    c = rot[0];
+    s = rot[1];
+    er = rot[2];
+    ei = rot[3];
+  }
   double* vp = V + ((size_t)k * Np + p) * N * (C ? 2 : 1);
   double* vq = V + ((size_t)k * Np + q) * N * (C ? 2 : 1);
   for (int mu = first; mu < N; mu += step) {
@@ -203,7 +231,7 @@ template <bool C>
 __global__ void __launch_bounds__(256) proj_cluster_kernel(int N, int Np, const double* __restrict__ G,
                                                            double* __restrict__ W, double* __restrict__ V,
                                                            double thresh) {
-  __shared__ double red[8][4];
+  __shared__ double red[8][4], rot[5], offs;
   __shared__ int list[CLUSTER_MAX], cnt;
   extern __shared__ unsigned char mark[];
   const int k = blockIdx.x, tid = threadIdx.x;
@@ -246,19 +274,19 @@ __global__ void __launch_bounds__(256) proj_cluster_kernel(int N, int Np, const 
         const long op = (long)list[u] * N * (C ? 2 : 1), oq = (long)list[v] * N * (C ? 2 : 1);
         double a, b, gr, gi;
         pair_dots<C>(wk + op, wk + oq, N, tid, 256, a, b, gr, gi);
-        cta_join(red, a, b, gr, gi);
-        const double h = sqrt(gr * gr + gi * gi);
-        const double off = (a > 0.0 && b > 0.0) ? h / sqrt(a * b) : 0.0;
-        worst = fmax(worst, off);
-        if (!(off > thresh)) continue;
-        double c, s, er, ei;
-        pair_rotation(a, b, gr, gi, h, c, s, er, ei);
+        worst = fmax(worst, cta_rotation(red, rot, a, b, gr, gi, thresh));
+        const double c = rot[0], s = rot[1], er = rot[2], ei = rot[3];
+        const bool turn = rot[4] != 0.0;
+        __syncthreads();  // rot and red are free again
+        if (!turn) continue;
         for (int mu = tid; mu < N; mu += 256) {  // a thread's own elements: no barrier between pairs
           rotate_pair<C>(wk + op, wk + oq, mu, c, s, er, ei);
           rotate_pair<C>(vk + op, vk + oq, mu, c, s, er, ei);
         }
       }
-    if (worst <= 1e-14) break;
+    if (tid == 0) offs = worst;
+    __syncthreads();
+    if (offs <= 1e-14) break;
   }
 }
 
