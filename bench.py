@@ -838,7 +838,7 @@ _V_CACHE = {}  # V(q) depends only on the shape here: shared by jobs of one shap
 
 
 def plan_of(rpa, p, mode):
-    """The frequency-batched chi0 plan of a problem (rpa_freq_plan on a host
+    """The frequency-batched chi0 plan of a problem (rpa_chi0_plan on a host
     descriptor with placeholder C/V pointers: the plan reads only the shapes,
     pairs, frequencies and band energies)."""
     import numpy as np
@@ -848,7 +848,7 @@ def plan_of(rpa, p, mode):
     t = {"C": [ph] * (p.n_q * p.n_k), "V": [ph] * p.n_q,
          "eps_occ": torch.from_numpy(np.ascontiguousarray(p.eps_occ, np.float64)),
          "eps_virt": torch.from_numpy(np.ascontiguousarray(p.eps_virt, np.float64))}
-    pl = rpa.job_from_problem(p, t, prec=rpa.PREC_MIXED, mem=rpa.MEM_HOST).freq_plan(2 if mode == 2 else 0)
+    pl = rpa.job_from_problem(p, t, prec=rpa.PREC_MIXED, mem=rpa.MEM_HOST).chi0_plan(2 if mode == 2 else 0)
     if mode == 1 or pl["n_bins"] == 0:
         return {"used": False}
     return {"used": True, "n_bins": pl["n_bins"], "rank": [int(x) for x in pl["rank"]],

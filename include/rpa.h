@@ -179,9 +179,9 @@ rpa_status rpa_job_validate(const rpa_job *job, char *msg, size_t msg_len);
  * nodes, residual err[b] <= 1e-10 of the bin's largest |d(., omega_w)| on a
  * dense check grid), so chi0 needs rank[b] contractions over bin b instead of
  * n_w: chi0(w) = sum_b sum_r coef[b][r][w] X_{b,r}, X_{b,r} the contraction of
- * bin b's transitions at omega_{skel[b][r]}.  (The chi0 of rpa_energy and
- * rpa_chi0 runs a plan of the same construction and bounds whose number of bins
- * also weighs the recombination, up to 64.)  mode: 0 automatic (n_bins = 0
+ * bin b's transitions at omega_{skel[b][r]}.  (rpa_chi0_plan reports the plan
+ * that rpa_energy and rpa_chi0 run: the same construction and bounds, its number
+ * of bins also weighed by the recombination.)  mode: 0 automatic (n_bins = 0
  * when the plan saves no work), 2 always.  Outputs (any may be NULL), with
  * B = RPA_FREQ_MAX_BINS: edges [B], rank [B], err [B], skel [B][n_w] (-1 past
  * rank[b]), coef [B][n_w][n_w] (row r of bin b), *work_ratio = modelled
@@ -189,6 +189,13 @@ rpa_status rpa_job_validate(const rpa_job *job, char *msg, size_t msg_len);
  * mem != RPA_MEM_HOST. */
 #define RPA_FREQ_MAX_BINS 32
 rpa_status rpa_freq_plan(const rpa_job *job, int mode, int *n_bins, double *edges, int *rank, int *skel,
+                         double *coef, double *err, double *work_ratio);
+
+/* As rpa_freq_plan, for the plan that the chi0 of rpa_energy and rpa_chi0 runs on
+ * this job (mode as the context's chi0_freq: 0 or 2; n_bins = 0: every frequency
+ * is contracted), with B = RPA_CHI0_MAX_BINS. */
+#define RPA_CHI0_MAX_BINS 64
+rpa_status rpa_chi0_plan(const rpa_job *job, int mode, int *n_bins, double *edges, int *rank, int *skel,
                          double *coef, double *err, double *work_ratio);
 
 /* Host-only: device bytes the job occupies while it runs (its inputs when

@@ -20,13 +20,14 @@ LIB_PATH = os.path.join(HERE, "lib", "librpa.so")
 RPA_OK, RPA_E_INVAL, RPA_E_NOMEM, RPA_E_CUDA, RPA_E_NOTPD, RPA_E_TIMEOUT, RPA_E_BUSY, RPA_E_NOTREADY = range(8)
 PREC_FP64, PREC_MIXED = 0, 1
 MEM_DEVICE, MEM_HOST = 0, 1
-FREQ_MAX_BINS = 32  # RPA_FREQ_MAX_BINS: energy bins of the frequency-batched chi0 at most
+FREQ_MAX_BINS = 32  # RPA_FREQ_MAX_BINS: energy bins of rpa_freq_plan at most
+CHI0_MAX_BINS = 64  # RPA_CHI0_MAX_BINS: of the plan that the frequency-batched chi0 runs
 
 STATUS_NAMES = {0: "OK", 1: "INVAL", 2: "NOMEM", 3: "CUDA", 4: "NOTPD", 5: "TIMEOUT", 6: "BUSY", 7: "NOTREADY"}
 
 # Entry points declared in include/rpa.h
 EXPORTS = ("rpa_create", "rpa_destroy", "rpa_last_error", "rpa_job_validate", "rpa_job_footprint", "rpa_freq_plan",
-           "rpa_chi0",
+           "rpa_chi0_plan", "rpa_chi0",
            "rpa_ao2mo", "rpa_projector", "rpa_logdet", "rpa_energy", "rpa_energy_batch", "rpa_submit", "rpa_poll",
            "rpa_wait",
            "rpa_serving_stats", "rpa_serving_peak", "rpa_test_drop_copy", "rpa_kernel_launches", "rpa_stream",
@@ -91,6 +92,8 @@ def load_library(path: str = LIB_PATH):
         "rpa_job_validate": (I, [J, ctypes.c_char_p, S]),
         "rpa_job_footprint": (I, [J, ctypes.POINTER(S)]),
         "rpa_freq_plan": (I, [J, I, ctypes.POINTER(I), ctypes.POINTER(D), ctypes.POINTER(I), ctypes.POINTER(I),
+                              ctypes.POINTER(D), ctypes.POINTER(D), ctypes.POINTER(D)]),
+        "rpa_chi0_plan": (I, [J, I, ctypes.POINTER(I), ctypes.POINTER(D), ctypes.POINTER(I), ctypes.POINTER(I),
                               ctypes.POINTER(D), ctypes.POINTER(D), ctypes.POINTER(D)]),
         "rpa_chi0": (I, [P, J, I, P, P]),
         "rpa_ao2mo": (I, [P, J, I, P, P]),
@@ -219,23 +222,31 @@ class Job:
     def freq_plan(self, mode: int = 0) -> Dict[str, object]:
         """rpa_freq_plan (host-only; needs a MEM_HOST job): the frequency
         factorisation of the split-precision chi0."""
+        return self._plan("rpa_freq_plan", FREQ_MAX_BINS, mode)
+
+    def chi0_plan(self, mode: int = 0) -> Dict[str, object]:
+        """rpa_chi0_plan (host-only; needs a MEM_HOST job): the factorisation
+        that rpa_energy and rpa_chi0 run."""
+        return self._plan("rpa_chi0_plan", CHI0_MAX_BINS, mode)
+
+    def _plan(self, entry: str, n_max: int, mode: int) -> Dict[str, object]:
         nb = ctypes.c_int()
         nw = self.s.n_w
-        edges = np.zeros(FREQ_MAX_BINS)
-        rank = np.zeros(FREQ_MAX_BINS, np.int32)
-        skel = np.zeros(FREQ_MAX_BINS * nw, np.int32)
-        coef = np.zeros(FREQ_MAX_BINS * nw * nw)
-        err = np.zeros(FREQ_MAX_BINS)
+        edges = np.zeros(n_max)
+        rank = np.zeros(n_max, np.int32)
+        skel = np.zeros(n_max * nw, np.int32)
+        coef = np.zeros(n_max * nw * nw)
+        err = np.zeros(n_max)
         wr = ctypes.c_double()
         ip = ctypes.POINTER(ctypes.c_int)
-        st = load_library().rpa_freq_plan(ctypes.byref(self.s), int(mode), ctypes.byref(nb), _dptr(edges),
-                                          rank.ctypes.data_as(ip), skel.ctypes.data_as(ip), _dptr(coef), _dptr(err),
-                                          ctypes.byref(wr))
+        st = getattr(load_library(), entry)(ctypes.byref(self.s), int(mode), ctypes.byref(nb), _dptr(edges),
+                                            rank.ctypes.data_as(ip), skel.ctypes.data_as(ip), _dptr(coef), _dptr(err),
+                                            ctypes.byref(wr))
         if st:
-            raise RpaError(st, "rpa_freq_plan failed")
+            raise RpaError(st, entry + " failed")
         n = int(nb.value)
         return {"n_bins": n, "edges": edges[:max(0, n - 1)].copy(), "rank": rank[:n].copy(),
-                "skel": skel.reshape(FREQ_MAX_BINS, nw)[:n].copy(), "coef": coef.reshape(FREQ_MAX_BINS, nw, nw)[:n].copy(),
+                "skel": skel.reshape(n_max, nw)[:n].copy(), "coef": coef.reshape(n_max, nw, nw)[:n].copy(),
                 "err": err[:n].copy(), "work_ratio": float(wr.value)}
 
     def footprint(self) -> int:

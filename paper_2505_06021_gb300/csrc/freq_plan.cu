@@ -470,13 +470,15 @@ void freq_meta_d(const rpa_job* j, const FreqPlan& p, std::vector<double>& img) 
 
 // ============================================================== C ABI =====
 
-extern "C" rpa_status rpa_freq_plan(const rpa_job* job, int mode, int* n_bins, double* edges, int* rank,
-                                    int* skel, double* coef, double* err, double* work_ratio) {
+static_assert(RPA_CHI0_MAX_BINS == rpa::FREQ_MAX_BINS, "rpa_chi0_plan reports every bin");
+
+static rpa_status report_plan(const rpa_job* job, int mode, int max_bins, int* n_bins, double* edges, int* rank,
+                              int* skel, double* coef, double* err, double* work_ratio) {
   char msg[256];
   if (!job || rpa::validate_job(job, msg, sizeof msg)) return RPA_E_INVAL;
   if (job->mem != RPA_MEM_HOST || mode < 0 || mode > 2) return RPA_E_INVAL;
   rpa::FreqPlan p;
-  rpa::freq_plan_build(job, job->eps_occ, job->eps_virt, mode, &p, nullptr, RPA_FREQ_MAX_BINS);
+  rpa::freq_plan_build(job, job->eps_occ, job->eps_virt, mode, &p, nullptr, max_bins);
   if (n_bins) *n_bins = p.n_bins;
   if (work_ratio) *work_ratio = p.n_bins ? p.work_ratio : 1.0;
   for (int b = 0; b < p.n_bins; ++b) {
@@ -491,4 +493,14 @@ extern "C" rpa_status rpa_freq_plan(const rpa_job* job, int mode, int* n_bins, d
     }
   }
   return RPA_OK;
+}
+
+extern "C" rpa_status rpa_freq_plan(const rpa_job* job, int mode, int* n_bins, double* edges, int* rank,
+                                    int* skel, double* coef, double* err, double* work_ratio) {
+  return report_plan(job, mode, RPA_FREQ_MAX_BINS, n_bins, edges, rank, skel, coef, err, work_ratio);
+}
+
+extern "C" rpa_status rpa_chi0_plan(const rpa_job* job, int mode, int* n_bins, double* edges, int* rank,
+                                    int* skel, double* coef, double* err, double* work_ratio) {
+  return report_plan(job, mode, RPA_CHI0_MAX_BINS, n_bins, edges, rank, skel, coef, err, work_ratio);
 }
