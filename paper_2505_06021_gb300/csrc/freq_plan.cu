@@ -400,6 +400,7 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
     const double recomb = run ? 44.0 * nb * j->n_w * j->n_q / total : 0.0;
     est.push_back({r / 5 * (1.0 + 8.0 * j->n_q * nb / total + recomb), ratios[c]});
   }
+  if (est.empty()) return false;  // no ratio's coefficients fit (an energy range of many decades)
   std::stable_sort(est.begin(), est.end(),
                    [](const std::pair<double, double>& a, const std::pair<double, double>& b) { return a.first < b.first; });
   P = plan_full(est[0].second);

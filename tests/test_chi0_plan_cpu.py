@@ -55,3 +55,19 @@ def test_long_contractions_take_more_bins(rpa):
     long_, base = _host_job(rpa, p).chi0_plan(), _host_job(rpa, p).freq_plan()
     assert 0 < short["n_bins"] < long_["n_bins"] and long_["n_bins"] > 32
     assert long_["work_ratio"] < base["work_ratio"]
+
+
+@pytest.mark.parametrize("n_w", [24, 32])
+@pytest.mark.parametrize("mode", [0, 2])
+def test_gap_so_small_that_no_plan_fits(rpa, n_w, mode):
+    """A gap of 1e-16 puts 17 decades of transition energies into the bins: even at
+    the widest ratio their coefficients exceed the recombination's shared memory,
+    and every frequency is contracted on its own."""
+    p = synth.make_problem("gap", is_complex=False, n_aux=12, n_occ=4, n_virt=28, grid=synth.gamma_grid(), n_w=n_w, seed=5)
+    t = rpa.upload_problem(p, device="cpu")
+    t["eps_occ"] -= t["eps_occ"].max()
+    t["eps_virt"] += 1e-16 - t["eps_virt"].min()
+    t["eps_virt"][0, int(t["eps_virt"][0].argmin())] = 1e-16
+    job = rpa.job_from_problem(p, t, prec=rpa.PREC_MIXED, mem=rpa.MEM_HOST)
+    assert job.chi0_plan(mode)["n_bins"] == 0
+    assert job.freq_plan(mode)["n_bins"] == 0
