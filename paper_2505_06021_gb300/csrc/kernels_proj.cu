@@ -43,6 +43,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "fp64_elem.cuh"
 #include "rpa_internal.h"
@@ -636,13 +637,33 @@ cudaError_t launch_proj_load32(int cplx, int n_mat, int N, int Np, const double*
   return cudaGetLastError();
 }
 
+// Shared memory of a block round at most (2 B columns of W and V).
+constexpr size_t J32_SMEM = 225 * 1024;
+
+// The launch limit of a block kernel, per device and set once to the most any
+// basis takes: it belongs to the function, which the contexts of all threads share.
+template <bool C, int B>
+static cudaError_t jacobi32_attr() {
+  static std::mutex mu;
+  static bool done[MAX_DEVICES] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= MAX_DEVICES) dev = 0;
+  std::lock_guard<std::mutex> lk(mu);
+  if (done[dev]) return cudaSuccess;
+  const cudaError_t e =
+      cudaFuncSetAttribute(jacobi32_block_kernel<C, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)J32_SMEM);
+  done[dev] = e == cudaSuccess;
+  return e;
+}
+
 // One sweep of the FP32 iteration; returns the launches made, or a negative
 // CUDA error.
 template <bool C, int B>
 static int jacobi32_blocks(int n_mat, int N, int Np, float* W32, float* V32, float thresh, unsigned* off_max,
                            cudaStream_t s) {
   const size_t sh = sizeof(Flt<C>) * 4 * B * (size_t)N;
-  cudaError_t e = cudaFuncSetAttribute(jacobi32_block_kernel<C, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  cudaError_t e = jacobi32_attr<C, B>();
   const int nb = 2 * ((Np + 2 * B - 1) / (2 * B));
   for (int br = 0; br < nb - 1 && e == cudaSuccess; ++br) {
     jacobi32_block_kernel<C, B><<<dim3(nb / 2, n_mat), 32 * B, sh, s>>>(N, Np, nb, br, W32, V32, thresh, off_max);
@@ -655,7 +676,7 @@ static int jacobi32_sweep(int n_mat, int N, int Np, float* W32, float* V32, floa
                           cudaStream_t s) {
   // blocks of 16 columns while 32 columns of W and V fit in shared memory
   // (complex N <= 450), of 8 up to twice that
-  const size_t col = sizeof(Flt<C>) * 4 * (size_t)N, room = 225 * 1024;
+  const size_t col = sizeof(Flt<C>) * 4 * (size_t)N, room = J32_SMEM;
   if (16 * col <= room) return jacobi32_blocks<C, 16>(n_mat, N, Np, W32, V32, thresh, off_max, s);
   if (8 * col <= room) return jacobi32_blocks<C, 8>(n_mat, N, Np, W32, V32, thresh, off_max, s);
   for (int r = 0; r < Np - 1; ++r)

@@ -1,5 +1,6 @@
 """The projector's sweeps as launches: what a column pair costs its SM, and
 contexts that share the device."""
+import threading
 import time
 
 import pytest
@@ -47,3 +48,33 @@ def test_small_basis_pairs_share_an_sm(rpa):
                 best = min(best, (time.perf_counter() - t0) / (c.launches - n0))
             per_launch.append(best)
     assert per_launch[1] <= 2.3 * per_launch[0], per_launch
+
+
+def test_two_contexts_with_different_bases(rpa):
+    """Two contexts in two threads on one device, a block kernel launch of 16
+    columns each with other shared memory: every call succeeds and gives what it
+    gives alone."""
+    jobs = [_job(rpa, n, (2, 1, 1)) for n in (256, 64)]
+    alone, errors, results = [], [], [[], []]
+    for job in jobs:
+        with rpa.Context(0) as c:
+            alone.append(c.projector(job)[2].tobytes())
+    torch.cuda.synchronize()
+    gate = threading.Barrier(2)
+
+    def work(i):
+        try:
+            with rpa.Context(0) as c, torch.cuda.stream(torch.cuda.Stream()):
+                gate.wait(60)
+                for _ in range(60):
+                    results[i].append(c.projector(jobs[i])[2].tobytes())
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    assert all(r == a for a, rs in zip(alone, results) for r in rs)
