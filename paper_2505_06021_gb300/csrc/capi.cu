@@ -254,7 +254,7 @@ size_t tail_region_bytes(const rpa_job* j, int nq) {
 }
 
 Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt, const BinJob* bj,
-                   bool g64) {
+                   int g64) {
   Layout L{};
   if (qt < qb) qt = qb;
   const size_t es = j->is_complex ? 16 : 8;
@@ -289,21 +289,21 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
   if (binned) L.binmeta = al(bj->meta_bytes);
   L.total = L.meta + L.dtab + L.chi + L.T + L.L + L.Vc + 2 * (L.stageC + L.stageV) + L.eps + L.mixed + L.ao +
             L.binmeta;
-  if (g64 && j->ao) {
+  if ((g64 & G64_AO) && j->ao) {
     const size_t m = al(ao_g64_plan(j, ao_plan(j, qb)).bytes);
     if (L.total + m <= ws_cap) {
       L.aog = m;
       L.total += m;
     }
   }
-  if (g64) {
+  if (g64 & G64_TAIL) {
     const size_t m = tail_region_bytes(j, qt);
     if (L.total + m <= ws_cap) {
       L.tail = m;
       L.total += m;
     }
   }
-  if (g64 && j->prec == RPA_PREC_FP64) {
+  if ((g64 & G64_CHI) && j->prec == RPA_PREC_FP64) {
     // the FP64 chi0 on the tensor cores, where its planes fit under the cap
     BatchGeom g{j->is_complex, j->n_aux, j->n_occ, j->n_virt, (int)nov, j->n_k, j->n_w, qb};
     if (chi0_g64_use(g)) {
@@ -802,7 +802,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
   const void* v_ws = nullptr;
   size_t v_bytes = 0;
   auto v_side = [&]() -> rpa_status {
-    Lv = plan_layout(job, job->n_q, ctx->n_slices, ws_cap, false, job->n_q, nullptr, true);
+    Lv = plan_layout(job, job->n_q, ctx->n_slices, ws_cap, false, job->n_q, nullptr, G64_ALL);
     const size_t need = Lv.meta + Lv.chi + Lv.T + Lv.L + Lv.Vc + Lv.tail;
     if (!ex.ws || ex.ws_bytes < need) return RPA_OK;
     const Bufs bv = carve(ex.ws, job, Lv);
@@ -820,7 +820,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
       return stb;
   const int qb = choose_qb(job, ctx->n_slices, ws_cap, &bj);
   const int qt = choose_qt(job, qb, ctx->n_slices, ws_cap, &bj);
-  Layout L = plan_layout(job, qb, ctx->n_slices, ws_cap, true, qt, &bj, allow_bin);
+  Layout L = plan_layout(job, qb, ctx->n_slices, ws_cap, true, qt, &bj, allow_bin ? G64_ALL : 0);
   if (!ex.ensure_ws(L.total)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
     return RPA_E_NOMEM;
@@ -1087,7 +1087,7 @@ rpa_status rpa_chi0(rpa_ctx* ctx, const rpa_job* job, int q, void* chi_out, void
   cudaStream_t s = (cudaStream_t)stream;
   BinJob bj;
   if (rpa_status stb = bin_job_build(ctx, ex, job, bj)) return stb;
-  Layout L = plan_layout(job, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, &bj, true);
+  Layout L = plan_layout(job, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, &bj, G64_AO | G64_CHI);
   if (!ex.ensure_ws(L.total)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
     return RPA_E_NOMEM;
@@ -1183,7 +1183,7 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   rpa_job j1 = *job;
   j1.prec = RPA_PREC_FP64;
   j1.ao = nullptr;  // only the tail's buffers are used
-  Layout L = plan_layout(&j1, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, nullptr, true);
+  Layout L = plan_layout(&j1, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, nullptr, G64_TAIL);
   if (!ex.ensure_ws(L.total)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
     return RPA_E_NOMEM;

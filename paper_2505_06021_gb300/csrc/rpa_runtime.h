@@ -167,12 +167,14 @@ rpa_status wait_event(rpa_ctx* ctx, cudaEvent_t ev, double timeout_s);
 void prof_begin(rpa_ctx* ctx, Exec* ex, cudaStream_t s);
 void prof_end(rpa_ctx* ctx, Exec* ex, cudaStream_t s, int cls, int n_kernels);
 void prof_collect(rpa_ctx* ctx, Exec* ex);
-// mixed_ws: include the split-precision chi0 workspace (a batch supplies its own).
-// qt: q per tail batch (0: qt = qb).  bj: the job's frequency-batched chi0, if any.
 // Workspace of the tail's products on the tensor cores for nq q at once (0: the FP64 kernels).
 size_t tail_region_bytes(const rpa_job* j, int nq);
+// Parts whose digit planes a call uses (plan_layout's g64).
+enum { G64_AO = 1, G64_TAIL = 2, G64_CHI = 4, G64_ALL = 7 };
+// mixed_ws: include the split-precision chi0 workspace (a batch supplies its own).
+// qt: q per tail batch (0: qt = qb).  bj: the job's frequency-batched chi0, if any.
 Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt = 0,
-                   const BinJob* bj = nullptr, bool g64 = false);
+                   const BinJob* bj = nullptr, int g64 = 0);
 int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj = nullptr);
 int choose_qt(const rpa_job* j, int qb, int n_slices, size_t cap, const BinJob* bj = nullptr);
 // Builds the frequency-batched plan of a split-precision job (band energies

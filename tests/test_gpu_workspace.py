@@ -1,0 +1,53 @@
+"""Device memory of the calls: what a call reserves, and calls on a device whose
+memory is nearly used up."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rpa():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2505_06021_gb300 as m
+    from paper_2505_06021_gb300 import build as b
+
+    b.build()
+    return m
+
+
+def _free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _big_job(rpa, n_q=1):
+    """Jobs whose chi0 planes are about 3 GB: N_aux 768, 9 k-points, 1536 band pairs."""
+    n_aux, n_occ, n_virt, n_k, n_w = 768, 16, 96, 9, 16
+    g = torch.Generator(device="cuda").manual_seed(3)
+    nov = n_occ * n_virt
+    C = [torch.view_as_complex(torch.randn((n_aux, nov, 2), generator=g, device="cuda", dtype=torch.float64) /
+                               (2.0 * nov) ** 0.5) for _ in range(n_k)] * n_q
+    eo = torch.rand((n_k, n_occ), generator=g, device="cuda", dtype=torch.float64) - 1.3
+    ev = torch.rand((n_k, n_virt), generator=g, device="cuda", dtype=torch.float64) + 0.1
+    pair = np.tile(np.arange(n_k, dtype=np.int32), (n_q, 1))
+    om = np.linspace(0.1, 4.0, n_w)
+    return rpa.Job(is_complex=True, n_aux=n_aux, n_occ=n_occ, n_virt=n_virt, pair_k=pair, pair_kq=pair,
+                   w_q=np.ones(n_q) / n_q, zeta_k=1.0 / n_k, omega=om, zeta_w=np.full(n_w, 0.25), eps_occ=eo,
+                   eps_virt=ev, C=C, V=[torch.eye(n_aux, dtype=torch.complex128, device="cuda")] * n_q)
+
+
+def test_calls_reserve_only_the_planes_they_use(rpa):
+    """The log-det step holds no chi0 planes (16 frequencies' chi0, chi0 L and factors
+    are 0.3 GB, its own planes 1 GB at most), the chi0 step no tail planes."""
+    job = _big_job(rpa)
+    with rpa.Context(0) as c:
+        chi = c.chi0(job, 0)
+        torch.cuda.empty_cache()
+    with rpa.Context(0) as c:
+        f0 = _free()
+        c.logdet(job, 0, chi)
+        used = f0 - _free()
+    assert used < 1.6 * 2 ** 30, used
