@@ -381,6 +381,11 @@ extern "C" rpa_status rpa_energy_batch(rpa_ctx* ctx, const rpa_job* jobs, int n_
     bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap, true);
     bc.plan->sig = sig;
   }
+  if (!bc.mem.ensure_ws(bc.plan->ws_bytes) && !known) {
+    // no room on the device for the digit planes: without them
+    bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap);
+    bc.plan->sig = sig;
+  }
   Plan& p = *bc.plan;
   if (!bc.mem.ensure_ws(p.ws_bytes)) {
     ctx_set_error(ctx, "cannot allocate %zu bytes of batch workspace", p.ws_bytes);

@@ -495,6 +495,18 @@ rpa_status enqueue_table_copies(rpa_ctx* ctx, const rpa_job* j, const Bufs& b, c
   return RPA_OK;
 }
 
+// Workspace for a layout with the parts g64 as digit products; where the device has no room
+// for their planes (memory held outside the cap), without them.
+static rpa_status layout_ws(rpa_ctx* ctx, Exec& ex, int g64, const std::function<Layout(int)>& plan, Layout* out) {
+  for (int g : {g64, 0}) {
+    *out = plan(g);
+    if (ex.ensure_ws(out->total)) return RPA_OK;
+    if (!g) break;
+  }
+  ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", out->total);
+  return RPA_E_NOMEM;
+}
+
 static rpa_status upload_tables(rpa_ctx* ctx, Exec& ex, const rpa_job* j, const Bufs& b, const void* const* Cdev) {
   if (!ex.hstage.reserve(tables_bytes(j) + 64)) {
     ctx_set_error(ctx, "cannot allocate pinned host staging");
@@ -820,11 +832,11 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
       return stb;
   const int qb = choose_qb(job, ctx->n_slices, ws_cap, &bj);
   const int qt = choose_qt(job, qb, ctx->n_slices, ws_cap, &bj);
-  Layout L = plan_layout(job, qb, ctx->n_slices, ws_cap, true, qt, &bj, allow_bin ? G64_ALL : 0);
-  if (!ex.ensure_ws(L.total)) {
-    ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
-    return RPA_E_NOMEM;
-  }
+  Layout L;
+  if (rpa_status st = layout_ws(ctx, ex, allow_bin ? G64_ALL : 0, [&](int g) {
+        return plan_layout(job, qb, ctx->n_slices, ws_cap, true, qt, &bj, g);
+      }, &L))
+    return st;
   Bufs b = carve(ex.ws, job, L);
   // the early V side holds if this layout has its buffers in the same place
   const bool v_done = v_ws && v_ws == ex.ws && v_bytes == ex.ws_bytes && qb == job->n_q && qt == job->n_q &&
@@ -1087,11 +1099,11 @@ rpa_status rpa_chi0(rpa_ctx* ctx, const rpa_job* job, int q, void* chi_out, void
   cudaStream_t s = (cudaStream_t)stream;
   BinJob bj;
   if (rpa_status stb = bin_job_build(ctx, ex, job, bj)) return stb;
-  Layout L = plan_layout(job, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, &bj, G64_AO | G64_CHI);
-  if (!ex.ensure_ws(L.total)) {
-    ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
-    return RPA_E_NOMEM;
-  }
+  Layout L;
+  if (rpa_status st = layout_ws(ctx, ex, G64_AO | G64_CHI, [&](int g) {
+        return plan_layout(job, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, &bj, g);
+      }, &L))
+    return st;
   Bufs b = carve(ex.ws, job, L);
   std::vector<const void*> cp;
   AoPlan aop;
@@ -1183,11 +1195,11 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   rpa_job j1 = *job;
   j1.prec = RPA_PREC_FP64;
   j1.ao = nullptr;  // only the tail's buffers are used
-  Layout L = plan_layout(&j1, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, nullptr, G64_TAIL);
-  if (!ex.ensure_ws(L.total)) {
-    ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", L.total);
-    return RPA_E_NOMEM;
-  }
+  Layout L;
+  if (rpa_status st = layout_ws(ctx, ex, G64_TAIL, [&](int g) {
+        return plan_layout(&j1, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, nullptr, g);
+      }, &L))
+    return st;
   Bufs b = carve(ex.ws, &j1, L);
   const size_t es = job->is_complex ? 16 : 8;
   const size_t NN = (size_t)job->n_aux * job->n_aux;

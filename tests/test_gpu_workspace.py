@@ -51,3 +51,40 @@ def test_calls_reserve_only_the_planes_they_use(rpa):
         c.logdet(job, 0, chi)
         used = f0 - _free()
     assert used < 1.6 * 2 ** 30, used
+
+
+def _leave(n):
+    """Holds the device's memory but for n bytes."""
+    torch.cuda.empty_cache()
+    return torch.empty(_free() - n, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("left", [0.75, 0.95])
+def test_calls_fit_beside_what_the_caller_holds(rpa, left):
+    """With less memory left than the digit planes need (3 GB for chi0, 1 GB for the
+    log-det, which itself needs 0.35), the calls run without them; the results
+    agree to rounding (1e-13 of sums over 13824 transitions and 768 pivots)."""
+    job = _big_job(rpa)
+
+    def calls(hold):
+        out = []
+        for what in (lambda c: c.chi0(job, 0, out=chi).clone().cpu(), lambda c: torch.from_numpy(c.logdet(job, 0, chi0)),
+                     lambda c: torch.from_numpy(c.energy(job)["eps"]), lambda c: torch.from_numpy(c.energy_batch([job]))):
+            with rpa.Context(0) as c:
+                c.logdet(small, 0, torch.zeros((1, 8, 8), dtype=torch.complex128, device="cuda"))  # kernels loaded
+                h = _leave(int(left * 2 ** 30)) if hold else None
+                out.append(what(c))
+                del h
+        return out
+
+    one = torch.ones((1, 1), dtype=torch.float64, device="cuda")
+    z = np.zeros((1, 1), np.int32)
+    small = rpa.Job(is_complex=True, n_aux=8, n_occ=1, n_virt=1, pair_k=z, pair_kq=z, w_q=np.ones(1), zeta_k=1.0,
+                    omega=np.ones(1), zeta_w=np.ones(1), eps_occ=-one, eps_virt=one,
+                    C=[torch.ones((8, 1), dtype=torch.complex128, device="cuda")],
+                    V=[torch.eye(8, dtype=torch.complex128, device="cuda")])
+    chi = torch.empty((16, 768, 768), dtype=torch.complex128, device="cuda")
+    with rpa.Context(0) as c:
+        chi0 = c.chi0(job, 0)
+    for a, b in zip(calls(False), calls(True)):
+        assert float((a - b).abs().max()) <= 1e-13 * float(a.abs().max())
