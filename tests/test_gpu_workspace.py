@@ -18,6 +18,12 @@ def rpa():
     return m
 
 
+@pytest.fixture(autouse=True)
+def give_back():
+    yield
+    torch.cuda.empty_cache()  # what _leave held
+
+
 def _free():
     torch.cuda.synchronize()
     return torch.cuda.mem_get_info()[0]
