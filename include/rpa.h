@@ -37,7 +37,10 @@
  * - Streams: a `void *stream` argument is a cudaStream_t (0 = legacy default
  *   stream), e.g. torch.cuda.current_stream().cuda_stream.
  * - Determinism: in RPA_FP64 mode the same job gives bit-identical results
- *   whatever else runs on the device; all reductions have a fixed order.
+ *   through rpa_energy, rpa_energy_batch and rpa_submit, whatever else runs on
+ *   the device; all reductions have a fixed order.  (Where the context's cap, or
+ *   the device's memory, has no room for the digit planes of a job's products,
+ *   the job runs on the FP64 kernels instead: the same to rounding.)
  */
 #ifndef RPA_H
 #define RPA_H

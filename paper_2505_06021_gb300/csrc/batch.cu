@@ -73,7 +73,8 @@ std::vector<uint64_t> signature(const rpa_job* jobs, int n, int n_slices) {
 
 }  // namespace
 
-std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget, bool g64) {
+std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget, const int* g64,
+                                 size_t tail_most) {
   std::unique_ptr<Plan> p(new Plan);
   p->jobs.resize(n);
   size_t pin = 0;
@@ -83,15 +84,20 @@ std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_
     jp.mixed = 0;
     jp.g64 = 0;
     jp.tail = 0;
-    if (g64) {
-      // the tails run side by side, each with planes of its own
-      const size_t m = a1k(tail_region_bytes(&jobs[i], jobs[i].n_q));
-      if (m && a1k(jp.L.total) + m + 2048 <= budget / 2) jp.tail = m;
+    // (an FP64 job's planes do not depend on the room, only their size does)
+    const int gi = g64 ? g64[i] : 0, nqi = jobs[i].n_q;
+    const bool f64 = jobs[i].prec == RPA_PREC_FP64, least = gi & G64_LEAST;
+    if (gi & G64_TAIL) {
+      const size_t m = a1k(tail_region_bytes(&jobs[i], nqi, least && f64 ? 0 : tail_most));
+      if (a1k(jp.L.total) + m + 2048 <= budget / 2)
+        jp.tail = m;
+      else if (f64)
+        jp.tail = a1k(tail_region_bytes(&jobs[i], nqi, 0));
     }
-    if (g64 && jobs[i].prec == RPA_PREC_FP64) {
-      BatchGeom ga = geom_q(jobs[i]);
-      ga.n_qb = jobs[i].n_q;
-      if (chi0_g64_use(ga) && a1k(jp.L.total) + jp.tail + chi0_g64_bytes(ga) + 2048 <= budget) jp.g64 = a1k(chi0_g64_bytes(ga));
+    if ((gi & G64_CHI) && f64) {
+      int f = least || chi_region_bytes(&jobs[i], nqi, 1) == 0 ? 1 : chi0_g64_freqs(geom_q(jobs[i]));
+      while (f > 1 && a1k(jp.L.total) + jp.tail + chi_region_bytes(&jobs[i], nqi, f) + 2048 > budget) --f;
+      jp.g64 = a1k(chi_region_bytes(&jobs[i], nqi, f));
     }
     if (jobs[i].prec == RPA_PREC_MIXED) {
       const size_t per_q = a1k(mixed_workspace_bytes(geom_q(jobs[i]), n_slices, kBatchSliceCap));
@@ -378,12 +384,16 @@ extern "C" rpa_status rpa_energy_batch(rpa_ctx* ctx, const rpa_job* jobs, int n_
   const bool known = bc.plan && bc.plan->exec && bc.plan->sig == sig;
   const bool replay = known && !ctx->prof;
   if (!known) {
-    bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap, true);
-    bc.plan->sig = sig;
-  }
-  if (!bc.mem.ensure_ws(bc.plan->ws_bytes) && !known) {
-    // no room on the device for the digit planes: without them
-    bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap);
+    std::vector<int> g64(n_jobs);
+    for (int i = 0; i < n_jobs; ++i) g64[i] = job_g64(&jobs[i], ctx->n_slices, sync_ws_cap(ctx));
+    bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap, g64.data(), G64_TAIL_MOST);
+    // no room on the device for the planes: the smallest, then none
+    if (!bc.mem.ensure_ws(bc.plan->ws_bytes)) {
+      for (int& g : g64) g |= G64_LEAST;
+      bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap, g64.data(), G64_TAIL_MOST);
+      if (!bc.mem.ensure_ws(bc.plan->ws_bytes))
+        bc.plan = batch_plan(jobs, n_jobs, ctx->n_slices, ctx->cap, nullptr, 0);
+    }
     bc.plan->sig = sig;
   }
   Plan& p = *bc.plan;

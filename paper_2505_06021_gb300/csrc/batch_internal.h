@@ -57,11 +57,12 @@ struct SideStreams {
   void release();
 };
 
-// Plan for n jobs; groups of jobs whose workspace fits `budget`.  g64: FP64
-// jobs may take chi0 to the tensor cores (their planes share the mixed region;
-// not set by the serving lanes, whose admission counts the FP64 kernel's
-// workspace).
-std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget, bool g64 = false);
+// Plan for n jobs; groups of jobs whose workspace fits `budget`.  g64[i]: the
+// parts of job i that run as digit products (job_g64; null: none).  The chi0 planes of
+// FP64 jobs share the mixed region; the tails run side by side, each with planes of
+// its own (tail_most bytes at most).
+std::unique_ptr<Plan> batch_plan(const rpa_job* jobs, int n, int n_slices, size_t budget, const int* g64,
+                                 size_t tail_most);
 // Writes every job's small tables into the pinned buffer (tables_bytes each).
 void batch_fill_tables(const Plan& p, const rpa_job* jobs, int n, char* pin);
 // Issues the batch on `s` (tables already filled); results land in `pin` at

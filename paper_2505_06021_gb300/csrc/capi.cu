@@ -245,12 +245,21 @@ static size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 // Workspace cap of the synchronous calls (the serving lanes use a smaller one).
 size_t sync_ws_cap(rpa_ctx* ctx) { return std::min<size_t>(ctx->cap, (size_t)192 << 30); }
 
-size_t tail_region_bytes(const rpa_job* j, int nq) {
+size_t tail_region_bytes(const rpa_job* j, int nq, size_t most) {
   // the sandwich of an FP64 job (per q and frequency), the Gram product of the
   // inverse form otherwise (per q)
   const bool f64 = j->prec == RPA_PREC_FP64;
   if (!tail_g64_use(j->is_complex, j->n_aux, f64 ? j->n_w : nq)) return 0;
-  return al(tail_g64_bytes(j->is_complex, j->n_aux, f64 ? nq * j->n_w : nq));
+  return al(tail_g64_bytes(j->is_complex, j->n_aux, f64 ? nq * j->n_w : nq, most));
+}
+
+static BatchGeom geom_of(const rpa_job* j, int qb) {
+  return BatchGeom{j->is_complex, j->n_aux, j->n_occ, j->n_virt, j->n_occ * j->n_virt, j->n_k, j->n_w, qb};
+}
+
+size_t chi_region_bytes(const rpa_job* j, int qb, int n_freq) {
+  const BatchGeom g = geom_of(j, qb);
+  return j->prec == RPA_PREC_FP64 && chi0_g64_use(g) ? al(chi0_g64_bytes(g, n_freq)) : 0;
 }
 
 Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt, const BinJob* bj,
@@ -289,30 +298,29 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
   if (binned) L.binmeta = al(bj->meta_bytes);
   L.total = L.meta + L.dtab + L.chi + L.T + L.L + L.Vc + 2 * (L.stageC + L.stageV) + L.eps + L.mixed + L.ao +
             L.binmeta;
-  if ((g64 & G64_AO) && j->ao) {
-    const size_t m = al(ao_g64_plan(j, ao_plan(j, qb)).bytes);
-    if (L.total + m <= ws_cap) {
-      L.aog = m;
-      L.total += m;
+  // Digit planes.  Split-precision jobs take what fits under the cap; FP64 jobs
+  // (job_g64) always, the smallest first and then what the cap has room for.
+  const bool f64 = j->prec == RPA_PREC_FP64;
+  auto take = [&](size_t& part, size_t m) {
+    if (!f64 && L.total + m > ws_cap) return;
+    part = m;
+    L.total += m;
+  };
+  if ((g64 & G64_AO) && j->ao) take(L.aog, al(ao_g64_plan(j, ao_plan(j, qb)).bytes));
+  if (g64 & G64_TAIL) take(L.tail, tail_region_bytes(j, qt, f64 ? 0 : G64_TAIL_MOST));
+  if ((g64 & G64_CHI) && f64) take(L.mixed, chi_region_bytes(j, qb, 1));
+  if (f64 && !(g64 & G64_LEAST)) {
+    auto grow = [&](size_t& part, size_t m) {
+      if (!part || m <= part || L.total + (m - part) > ws_cap) return false;
+      L.total += m - part;
+      part = m;
+      return true;
+    };
+    for (size_t most = G64_TAIL_MOST; most >= ((size_t)1 << 24) && !grow(L.tail, tail_region_bytes(j, qt, most)); most /= 2) {
     }
-  }
-  if (g64 & G64_TAIL) {
-    const size_t m = tail_region_bytes(j, qt);
-    if (L.total + m <= ws_cap) {
-      L.tail = m;
-      L.total += m;
-    }
-  }
-  if ((g64 & G64_CHI) && j->prec == RPA_PREC_FP64) {
-    // the FP64 chi0 on the tensor cores, where its planes fit under the cap
-    BatchGeom g{j->is_complex, j->n_aux, j->n_occ, j->n_virt, (int)nov, j->n_k, j->n_w, qb};
-    if (chi0_g64_use(g)) {
-      const size_t m = al(chi0_g64_bytes(g));
-      if (L.total + m <= ws_cap) {
-        L.mixed = m;
-        L.total += m;
+    if (L.mixed)
+      for (int f = chi0_g64_freqs(geom_of(j, qb)); f > 1 && !grow(L.mixed, chi_region_bytes(j, qb, f)); --f) {
       }
-    }
   }
   if (mixed_ws && binned) {
     // the frequency-batched chi0 takes what the cap leaves (pipelined when that suffices)
@@ -333,13 +341,23 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
   return L;
 }
 
-int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj) {
+int job_g64(const rpa_job* j, int n_slices, size_t cap) {
+  if (j->prec != RPA_PREC_FP64) return G64_ALL;
+  int m = 0;
+  for (int part : {G64_AO, G64_TAIL, G64_CHI})
+    if (plan_layout(j, 1, n_slices, cap, true, 0, nullptr, m | part | G64_LEAST).total <= cap) m |= part;
+  return m;
+}
+
+int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj, int g64) {
   int qb = j->n_q;
   if (j->ao) {  // AO form: the MO-basis coefficients of a few q at a time (<= 4 GB)
     const size_t per_q = (j->is_complex ? 16 : 8) * (size_t)j->n_aux * j->n_occ * j->n_virt * j->n_k;
     qb = (int)std::max<size_t>(1, std::min<size_t>((size_t)j->n_q, ((size_t)4 << 30) / std::max<size_t>(per_q, 1)));
   }
-  while (qb > 1 && plan_layout(j, qb, n_slices, cap, true, 0, bj).total > cap) qb = (qb + 1) / 2;
+  // (a split-precision job's planes are taken from what is left)
+  g64 = j->prec == RPA_PREC_FP64 ? g64 | G64_LEAST : 0;
+  while (qb > 1 && plan_layout(j, qb, n_slices, cap, true, 0, bj, g64).total > cap) qb = (qb + 1) / 2;
   // host-resident inputs: at least four q-batches, so that the copies of one
   // batch overlap the compute of the previous one.  With the frequency-batched
   // chi0, fewer q per batch while that keeps all skeletons in one round (the
@@ -367,32 +385,31 @@ int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj) {
   return qb;
 }
 
-int choose_qt(const rpa_job* j, int qb, int n_slices, size_t cap, const BinJob* bj) {
+int choose_qt(const rpa_job* j, int qb, int n_slices, size_t cap, const BinJob* bj, int g64) {
   // host-staged and AO-form jobs compute chi0 per staging batch; their tail
   // (V factor, log-det) runs over as many q as fit, so that its Cholesky
   // launches fill the GPU
   if (j->mem != RPA_MEM_HOST && !j->ao) return qb;
   int m = (j->n_q + qb - 1) / qb;
-  while (m > 1 && plan_layout(j, qb, n_slices, cap, true, std::min(j->n_q, m * qb), bj).total > cap)
+  g64 = j->prec == RPA_PREC_FP64 ? g64 | G64_LEAST : 0;
+  while (m > 1 && plan_layout(j, qb, n_slices, cap, true, std::min(j->n_q, m * qb), bj, g64).total > cap)
     m = (m + 1) / 2;
   return std::min(j->n_q, m * qb);
 }
 
-size_t job_workspace(const rpa_job* j, int n_slices, size_t ws_cap) {
-  const int qb = choose_qb(j, n_slices, ws_cap);
-  return plan_layout(j, qb, n_slices, ws_cap, true, choose_qt(j, qb, n_slices, ws_cap)).total;
+size_t job_workspace(const rpa_job* j, int n_slices, size_t ws_cap, int g64) {
+  const int qb = choose_qb(j, n_slices, ws_cap, nullptr, g64);
+  return plan_layout(j, qb, n_slices, ws_cap, true, choose_qt(j, qb, n_slices, ws_cap, nullptr, g64), nullptr, g64).total;
 }
 
-size_t job_footprint(const rpa_job* j, int n_slices, size_t ws_cap) {
-  const int qb = choose_qb(j, n_slices, ws_cap);
-  Layout L = plan_layout(j, qb, n_slices, ws_cap, true, choose_qt(j, qb, n_slices, ws_cap));
+size_t job_footprint(const rpa_job* j, int n_slices, size_t ws_cap, int g64) {
   size_t in = 0;
   if (j->mem == RPA_MEM_DEVICE) {
     const size_t es = j->is_complex ? 16 : 8;
     in = j->ao ? ao_input_bytes(j) : es * (size_t)j->n_aux * j->n_occ * j->n_virt * j->n_q * j->n_k;
     in += es * (size_t)j->n_aux * j->n_aux * j->n_q;
   }
-  return in + L.total;
+  return in + job_workspace(j, n_slices, ws_cap, g64);
 }
 
 Bufs carve(void* ws, const rpa_job* j, const Layout& L) {
@@ -496,12 +513,11 @@ rpa_status enqueue_table_copies(rpa_ctx* ctx, const rpa_job* j, const Bufs& b, c
 }
 
 // Workspace for a layout with the parts g64 as digit products; where the device has no room
-// for their planes (memory held outside the cap), without them.
+// for their planes (memory held outside the cap), with the smallest ones or without them.
 static rpa_status layout_ws(rpa_ctx* ctx, Exec& ex, int g64, const std::function<Layout(int)>& plan, Layout* out) {
-  for (int g : {g64, 0}) {
+  for (int g : {g64, g64 | G64_LEAST, 0}) {
     *out = plan(g);
     if (ex.ensure_ws(out->total)) return RPA_OK;
-    if (!g) break;
   }
   ctx_set_error(ctx, "cannot allocate %zu bytes of workspace", out->total);
   return RPA_E_NOMEM;
@@ -790,7 +806,7 @@ rpa_status bin_job_build(rpa_ctx* ctx, Exec& ex, const rpa_job* j, BinJob& bj,
   return RPA_OK;
 }
 
-rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_cap, bool allow_bin) {
+rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_cap, bool allow_bin, int g64) {
   char msg[512];
   if (validate_job(job, msg, sizeof msg)) {
     ctx_set_error(ctx, "%s", msg);
@@ -801,6 +817,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
     return RPA_E_INVAL;
   }
   CK(cudaSetDevice(ctx->device));
+  if (g64 < 0) g64 = job_g64(job, ctx->n_slices, sync_ws_cap(ctx));
   cudaStream_t s = ex.s;
   BinJob bj;
   // Device-resident split-precision jobs: the V side of all q (V = L L^H, V^-1)
@@ -814,7 +831,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
   const void* v_ws = nullptr;
   size_t v_bytes = 0;
   auto v_side = [&]() -> rpa_status {
-    Lv = plan_layout(job, job->n_q, ctx->n_slices, ws_cap, false, job->n_q, nullptr, G64_ALL);
+    Lv = plan_layout(job, job->n_q, ctx->n_slices, ws_cap, false, job->n_q, nullptr, g64);
     const size_t need = Lv.meta + Lv.chi + Lv.T + Lv.L + Lv.Vc + Lv.tail;
     if (!ex.ws || ex.ws_bytes < need) return RPA_OK;
     const Bufs bv = carve(ex.ws, job, Lv);
@@ -826,14 +843,14 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
     return RPA_OK;
   };
   const bool v_early = allow_bin && job->prec == RPA_PREC_MIXED && job->mem == RPA_MEM_DEVICE && !job->ao &&
-                       choose_qb(job, ctx->n_slices, ws_cap) == job->n_q;
+                       choose_qb(job, ctx->n_slices, ws_cap, nullptr, g64) == job->n_q;
   if (allow_bin)
     if (rpa_status stb = bin_job_build(ctx, ex, job, bj, v_early ? std::function<rpa_status()>(v_side) : nullptr))
       return stb;
-  const int qb = choose_qb(job, ctx->n_slices, ws_cap, &bj);
-  const int qt = choose_qt(job, qb, ctx->n_slices, ws_cap, &bj);
+  const int qb = choose_qb(job, ctx->n_slices, ws_cap, &bj, g64);
+  const int qt = choose_qt(job, qb, ctx->n_slices, ws_cap, &bj, g64);
   Layout L;
-  if (rpa_status st = layout_ws(ctx, ex, allow_bin ? G64_ALL : 0, [&](int g) {
+  if (rpa_status st = layout_ws(ctx, ex, g64, [&](int g) {
         return plan_layout(job, qb, ctx->n_slices, ws_cap, true, qt, &bj, g);
       }, &L))
     return st;
@@ -1033,7 +1050,7 @@ rpa_status rpa_job_validate(const rpa_job* job, char* msg, size_t msg_len) {
 rpa_status rpa_job_footprint(const rpa_job* job, size_t* bytes) {
   if (!bytes) return RPA_E_INVAL;
   if (rpa_status st = validate_job(job, nullptr, 0)) return st;
-  *bytes = job_footprint(job, 4, (size_t)24 << 30);
+  *bytes = job_footprint(job, 4, (size_t)24 << 30, job->prec == RPA_PREC_FP64 && !job->ao ? job_g64(job, 4, (size_t)120 << 30) : 0);
   return RPA_OK;
 }
 
@@ -1100,7 +1117,7 @@ rpa_status rpa_chi0(rpa_ctx* ctx, const rpa_job* job, int q, void* chi_out, void
   BinJob bj;
   if (rpa_status stb = bin_job_build(ctx, ex, job, bj)) return stb;
   Layout L;
-  if (rpa_status st = layout_ws(ctx, ex, G64_AO | G64_CHI, [&](int g) {
+  if (rpa_status st = layout_ws(ctx, ex, job_g64(job, ctx->n_slices, sync_ws_cap(ctx)) & ~G64_TAIL, [&](int g) {
         return plan_layout(job, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, &bj, g);
       }, &L))
     return st;
@@ -1196,7 +1213,7 @@ rpa_status rpa_logdet(rpa_ctx* ctx, const rpa_job* job, int q, const void* chi, 
   j1.prec = RPA_PREC_FP64;
   j1.ao = nullptr;  // only the tail's buffers are used
   Layout L;
-  if (rpa_status st = layout_ws(ctx, ex, G64_TAIL, [&](int g) {
+  if (rpa_status st = layout_ws(ctx, ex, job_g64(&j1, ctx->n_slices, sync_ws_cap(ctx)) & G64_TAIL, [&](int g) {
         return plan_layout(&j1, 1, ctx->n_slices, sync_ws_cap(ctx), true, 0, nullptr, g);
       }, &L))
     return st;
@@ -1251,7 +1268,7 @@ rpa_status rpa_test_drop_copy(rpa_ctx* ctx, int item) {
 rpa_status rpa_energy(rpa_ctx* ctx, const rpa_job* job, double* Ec, double* eps_qw, double* parts) {
   if (!ctx || !Ec) return RPA_E_INVAL;
   std::lock_guard<std::mutex> lk(ctx->mu);
-  if (rpa_status st = rpa::energy_enqueue(ctx, ctx->ex, job, rpa::sync_ws_cap(ctx), true)) return st;
+  if (rpa_status st = rpa::energy_enqueue(ctx, ctx->ex, job, rpa::sync_ws_cap(ctx), true, -1)) return st;
   // bounded wait: scaled with the job's chi0 work at a conservative 0.2 TFLOP/s
   const double work = 8.0 * job->n_aux * (double)job->n_aux * job->n_occ * job->n_virt * job->n_q * job->n_k *
                       job->n_w / (job->is_complex ? 1.0 : 4.0);

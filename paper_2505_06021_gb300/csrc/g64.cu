@@ -819,9 +819,9 @@ bool tail_g64_use(int cplx, int N, int n) {
   return N >= 128 && (cplx ? 1.0 : 0.25) * N * (double)N * N * n >= 2.5e7;
 }
 
-size_t tail_g64_bytes(int cplx, int N, int n_mat) {
+size_t tail_g64_bytes(int cplx, int N, int n_mat, size_t most) {
   const size_t one = tail_bytes(cplx, N).one;
-  return al1k(sizeof(int) * (size_t)n_mat) + std::max(2 * one, std::min<size_t>((size_t)1 << 30, one * (size_t)n_mat));
+  return al1k(sizeof(int) * (size_t)n_mat) + std::max(2 * one, std::min(most, one * (size_t)n_mat));
 }
 
 cudaError_t launch_sandwich_g64(int cplx, int N, int n_batch, int n_w, const double* chi, const double* L, double* T,
@@ -1083,9 +1083,10 @@ struct ChiPanel {
   long T;        // transitions per panel
   size_t a, b, ea, eb, ep, part, flag, total;
 };
-// The panel depends on the geometry of one q alone, so the result does not
-// depend on what shares the workspace.
-ChiPanel chi0_panel(const BatchGeom& g) {
+// The panel (T) depends on the geometry of one q alone, so the result does not
+// depend on what shares the workspace; G frequencies per pass (0: as many as
+// CHI_PLANES holds) change only its size.
+ChiPanel chi0_panel(const BatchGeom& g, int G = 0) {
   ChiPanel L{};
   const long Kt = (long)g.n_k * g.n_ov;
   const long unit = g.cplx ? KBC * 8 : KBC * 16;  // transitions of one exact accumulation
@@ -1099,11 +1100,12 @@ ChiPanel chi0_panel(const BatchGeom& g) {
   const long panels = (all + units - 1) / units;
   units = (all + panels - 1) / panels;
   L.T = units * unit;
+  if (G > 0) L.G = std::min(L.G, G);
   const int K = (int)std::min(L.T, Kt);
   L.KP = (int)std::max<long>(1, std::min<long>(64, K / 512));
   L.a = al1k(g64_plane_bytes(g.cplx, 0, g.n_aux, K, L.G));
   L.b = al1k(g64_plane_bytes(g.cplx, 1, g.n_aux, K, 1));
-  L.ea = al1k(sizeof(int) * (size_t)RA * L.G);
+  L.ea = al1k(sizeof(int) * (size_t)RA * g.n_w);
   L.eb = al1k(sizeof(int) * (size_t)RB);
   L.ep = al1k(sizeof(RowStat) * (size_t)(L.G + 1) * L.KP * std::max(RA, RB));
   L.flag = al1k(sizeof(int) * (size_t)std::max(1, g.n_qb));
@@ -1117,8 +1119,10 @@ ChiPanel chi0_panel(const BatchGeom& g) {
 
 template <bool C>
 cudaError_t chi0_g64_run(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi, void* work,
-                         int* status, uint64_t* n_launch, cudaStream_t s) {
-  const ChiPanel L = chi0_panel(g);
+                         size_t work_bytes, int* status, uint64_t* n_launch, cudaStream_t s) {
+  ChiPanel L = chi0_panel(g);
+  while (L.G > 1 && L.total > work_bytes) L = chi0_panel(g, L.G - 1);
+  if (L.total > work_bytes) return cudaErrorInvalidValue;
   char* p = (char*)work;
   int* flag = (int*)p;
   p += L.flag;
@@ -1127,7 +1131,7 @@ cudaError_t chi0_g64_run(const BatchGeom& g, const double* const* Cptrs, const d
   p += L.a;
   B.planes = (uint16_t*)p;
   p += L.b;
-  A.e = (int*)p;
+  int* eA = (int*)p;
   p += L.ea;
   B.e = (int*)p;
   p += L.eb;
@@ -1148,17 +1152,24 @@ cudaError_t chi0_g64_run(const BatchGeom& g, const double* const* Cptrs, const d
       A.n_kb = B.n_kb = g64_nkb(C, K);
       A.stride = (long)(A.Rpad / 128) * A.n_kb * (A_BLOCK / 2);
       B.stride = 0;
+      // every frequency's exponents before the first product: the flags that the
+      // products read are then those of the whole panel, however many passes it takes
       for (int w0 = 0; w0 < g.n_w; w0 += L.G) {
         const int G = std::min(L.G, g.n_w - w0);
         chi_exp_kernel<C><<<dim3((unsigned)((Npad + 7) / 8), (unsigned)L.KP, (unsigned)(1 + (G + CHI_W - 1) / CHI_W)), 256, 0,
                          s>>>(g.n_aux, Npad, g.n_ov, g.n_w, w0, G, t0, t1, Cq, dq, ep, flag + q);
-        chi_exp_final_kernel<<<((G + 1) * Npad + 255) / 256, 256, 0, s>>>(g.n_aux, A.Rpad, B.Rpad, Npad, G, L.KP, ep, A.e,
-                                                                         B.e, flag + q);
+        chi_exp_final_kernel<<<((G + 1) * Npad + 255) / 256, 256, 0, s>>>(g.n_aux, A.Rpad, B.Rpad, Npad, G, L.KP, ep,
+                                                                         eA + (size_t)w0 * A.Rpad, B.e, flag + q);
+        nl += 2;
+      }
+      for (int w0 = 0; w0 < g.n_w; w0 += L.G) {
+        const int G = std::min(L.G, g.n_w - w0);
+        A.e = eA + (size_t)w0 * A.Rpad;
         if (w0 == 0)
           chi_slice_b_kernel<C><<<grid_for((long)B.Rpad * B.n_kb, 16), 256, 0, s>>>(g.n_aux, g.n_ov, t0, t1, Cq, B);
         chi_slice_a_kernel<C><<<grid_for((long)A.Rpad * A.n_kb, 16), 256, 0, s>>>(g.n_aux, g.n_ov, g.n_w, w0, G, t0, t1, Cq,
                                                                                 dq, A);
-        nl += w0 == 0 ? 4 : 3;
+        nl += w0 == 0 ? 2 : 1;
         G64Out o{};
         o.base = chi + ((long)q * g.n_w + w0) * NN * (C ? 2 : 1);
         o.stride = NN;
@@ -1192,13 +1203,13 @@ bool chi0_g64_use(const BatchGeom& g) {
   return (g.cplx ? 4.0 : 1.0) * g.n_aux * (g.n_aux + 1.0) * K * g.n_w >= 5e8 && K * (g.cplx ? 2 : 1) >= 128;
 }
 
-size_t chi0_g64_bytes(const BatchGeom& g) { return chi0_panel(g).total; }
+int chi0_g64_freqs(const BatchGeom& g) { return chi0_panel(g).G; }
+size_t chi0_g64_bytes(const BatchGeom& g, int n_freq) { return chi0_panel(g, n_freq).total; }
 
 cudaError_t launch_chi0_g64(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
                             void* work, size_t work_bytes, int* status, uint64_t* n_launch, cudaStream_t s) {
-  if (work_bytes < chi0_g64_bytes(g)) return cudaErrorInvalidValue;
-  return g.cplx ? chi0_g64_run<true>(g, Cptrs, dtab, chi, work, status, n_launch, s)
-                : chi0_g64_run<false>(g, Cptrs, dtab, chi, work, status, n_launch, s);
+  return g.cplx ? chi0_g64_run<true>(g, Cptrs, dtab, chi, work, work_bytes, status, n_launch, s)
+                : chi0_g64_run<false>(g, Cptrs, dtab, chi, work, work_bytes, status, n_launch, s);
 }
 
 }  // namespace rpa

@@ -89,7 +89,7 @@ cudaError_t g64_product(int cplx, const G64Op& A, const G64Op& B, const G64Index
 // kernels.  n in tail_g64_use: matrices per q (its answer decides the bits of
 // an FP64 job, so it may not depend on how many q share the call).
 bool tail_g64_use(int cplx, int N, int n);
-size_t tail_g64_bytes(int cplx, int N, int n_mat);
+size_t tail_g64_bytes(int cplx, int N, int n_mat, size_t most = (size_t)1 << 30);
 cudaError_t launch_sandwich_g64(int cplx, int N, int n_batch, int n_w, const double* chi, const double* L, double* T,
                                 double* Y, void* work, size_t work_bytes, int* status, uint64_t* n_launch,
                                 cudaStream_t s);
@@ -98,8 +98,11 @@ cudaError_t launch_gram_g64(int cplx, int N, int n_q, const double* X, double* W
 
 // FP64 chi0 on this product: whether the size takes it, its workspace, and
 // the launch for all q of g (q out of the split's range are redone by the FP64 kernel).
+// The workspace holds the planes of some frequencies at a time (chi0_g64_freqs at
+// most, one at least); the result does not depend on how many.
 bool chi0_g64_use(const BatchGeom& g);
-size_t chi0_g64_bytes(const BatchGeom& g);
+int chi0_g64_freqs(const BatchGeom& g);
+size_t chi0_g64_bytes(const BatchGeom& g, int n_freq);
 cudaError_t launch_chi0_g64(const BatchGeom& g, const double* const* Cptrs, const double* dtab, double* chi,
                             void* work, size_t work_bytes, int* status, uint64_t* n_launch, cudaStream_t s);
 

@@ -149,14 +149,15 @@ struct Bufs {
 
 void ctx_set_error(rpa_ctx* ctx, const char* fmt, ...);
 rpa_status validate_job(const rpa_job* j, char* msg, size_t len);
-size_t job_footprint(const rpa_job* j, int n_slices, size_t ws_cap);
+size_t job_footprint(const rpa_job* j, int n_slices, size_t ws_cap, int g64);
 // Device workspace a lane needs for the job (part of job_footprint).
-size_t job_workspace(const rpa_job* j, int n_slices, size_t ws_cap);
+size_t job_workspace(const rpa_job* j, int n_slices, size_t ws_cap, int g64);
 // Enqueues the whole hot path of `job` on lane `ex` (no host wait) and records
 // ex.done after the results were copied into ex.hres.
 // allow_bin: use the frequency-batched chi0 when the context's setting and
 // the job's plan allow it (the synchronous entry point; serving lanes do not).
-rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_cap, bool allow_bin = false);
+// (g64 < 0: job_g64)
+rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_cap, bool allow_bin, int g64);
 // After ex.done has completed: decodes the device status and copies results.
 rpa_status energy_finish(rpa_ctx* ctx, Exec& ex, const rpa_job* job, double* Ec, double* eps_qw, double* parts);
 // Bounded wait for an event (RPA_E_TIMEOUT after timeout_s).
@@ -168,15 +169,24 @@ void prof_begin(rpa_ctx* ctx, Exec* ex, cudaStream_t s);
 void prof_end(rpa_ctx* ctx, Exec* ex, cudaStream_t s, int cls, int n_kernels);
 void prof_collect(rpa_ctx* ctx, Exec* ex);
 // Workspace of the tail's products on the tensor cores for nq q at once (0: the FP64 kernels).
-size_t tail_region_bytes(const rpa_job* j, int nq);
-// Parts whose digit planes a call uses (plan_layout's g64).
-enum { G64_AO = 1, G64_TAIL = 2, G64_CHI = 4, G64_ALL = 7 };
+// (at most `most` bytes of planes, but two matrices' at least)
+size_t tail_region_bytes(const rpa_job* j, int nq, size_t most);
+// Workspace of the chi0 on the tensor cores for qb q with n_freq frequencies per pass (0: all that
+// CHI_PLANES holds); 0 where the FP64 kernel is taken.
+size_t chi_region_bytes(const rpa_job* j, int qb, int n_freq);
+// Parts that run as digit products (plan_layout's g64); LEAST: with the smallest planes.
+enum { G64_AO = 1, G64_TAIL = 2, G64_CHI = 4, G64_ALL = 7, G64_LEAST = 8 };
+constexpr size_t G64_TAIL_MOST = (size_t)1 << 30;
+// The parts that job j runs as digit products under a workspace cap (the synchronous calls', for
+// every entry point).  It decides the bits of an FP64 job: there it depends on the job's shape and the
+// cap alone, and every layout of the job holds those parts' planes, if need be the smallest.
+int job_g64(const rpa_job* j, int n_slices, size_t cap);
 // mixed_ws: include the split-precision chi0 workspace (a batch supplies its own).
 // qt: q per tail batch (0: qt = qb).  bj: the job's frequency-batched chi0, if any.
 Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool mixed_ws, int qt = 0,
                    const BinJob* bj = nullptr, int g64 = 0);
-int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj = nullptr);
-int choose_qt(const rpa_job* j, int qb, int n_slices, size_t cap, const BinJob* bj = nullptr);
+int choose_qb(const rpa_job* j, int n_slices, size_t cap, const BinJob* bj, int g64);
+int choose_qt(const rpa_job* j, int qb, int n_slices, size_t cap, const BinJob* bj, int g64);
 // Builds the frequency-batched plan of a split-precision job (band energies
 // read back from the device when they live there) and its per-q tables in
 // ex.hbin; bj.on stays false when the context turns it off or it saves nothing.

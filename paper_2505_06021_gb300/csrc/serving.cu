@@ -48,6 +48,7 @@ struct ServeJob {
   std::vector<const void*> C, V;
   size_t footprint = 0;  // inputs + workspace
   size_t ws_need = 0;    // workspace part
+  int g64 = 0;           // parts that run as digit products (FP64 jobs)
   bool batchable = false;  // device-resident and small enough to share a micro-batch
   double t_submit = 0, t_admit = 0, t_done = 0;
   int state = 0;  // 0 pending, 1 running, 2 done
@@ -68,6 +69,7 @@ struct ServeLane {
 struct ServeBatch {
   std::vector<std::shared_ptr<ServeJob>> jobs;
   std::vector<rpa_job> desc;    // their descriptors, in batch order
+  std::vector<int> g64;         // and the parts of each that run as digit products
   std::unique_ptr<Plan> plan;   // null: a single host-memory job (energy_enqueue)
   ServeLane* lane = nullptr;
   size_t inputs = 0;
@@ -165,6 +167,10 @@ static size_t release_idle(ServeState* S, ServeLane* keep, size_t want) {
 
 static size_t lane_ws_cap(rpa_ctx* ctx) { return std::min<size_t>(ctx->cap / 4, (size_t)24 << 30); }
 
+// (many jobs' tails run side by side in a micro-batch: a few matrices' planes each)
+static std::unique_ptr<Plan> lane_plan(rpa_ctx* ctx, const rpa_job* jobs, int n, const int* g64) {
+  return batch_plan(jobs, n, ctx->n_slices, lane_ws_cap(ctx), g64, (size_t)256 << 20);
+}
 
 static void scheduler(rpa_ctx* ctx) {
   ServeState* S = ctx->serve;
@@ -197,8 +203,11 @@ static void scheduler(rpa_ctx* ctx) {
           est += add;
           B->inputs += j->footprint - j->ws_need;
         }
-        for (const auto& j : B->jobs) B->desc.push_back(j->job);
-        B->plan = batch_plan(B->desc.data(), (int)B->desc.size(), ctx->n_slices, lane_ws_cap(ctx));
+        for (const auto& j : B->jobs) {
+          B->desc.push_back(j->job);
+          B->g64.push_back(j->g64);
+        }
+        B->plan = lane_plan(ctx, B->desc.data(), (int)B->desc.size(), B->g64.data());
         ws_need = B->plan->ws_bytes;
       }
       size_t extra = 0;
@@ -212,7 +221,8 @@ static void scheduler(rpa_ctx* ctx) {
           B->inputs -= B->jobs.back()->footprint - B->jobs.back()->ws_need;
           B->jobs.pop_back();
           B->desc.pop_back();
-          B->plan = batch_plan(B->desc.data(), (int)B->desc.size(), ctx->n_slices, lane_ws_cap(ctx));
+          B->g64.pop_back();
+          B->plan = lane_plan(ctx, B->desc.data(), (int)B->desc.size(), B->g64.data());
           ws_need = B->plan->ws_bytes;
           lane = pick_lane(S, ws_need, &extra);
           if (!lane) break;  // the lane was free a moment ago: cannot happen, but stay safe
@@ -257,10 +267,25 @@ static void scheduler(rpa_ctx* ctx) {
       S->running.push_back(std::move(B));
       lk.unlock();
       rpa_status st = RPA_OK;
-      bool no_memory = false;
+      bool no_memory = false, replanned = false;
+      auto fits = [&]() {
+        return lane->ex.ensure_ws(Bp->plan->ws_bytes) && lane->ex.hstage.reserve(Bp->plan->pin_bytes + 64);
+      };
+      bool ready = Bp->plan && fits();
+      if (Bp->plan && !ready && S->running.size() == 1) {
+        // nothing else will free memory: smaller digit planes, then none
+        replanned = true;
+        for (int& g : Bp->g64) g |= G64_LEAST;
+        Bp->plan = lane_plan(ctx, Bp->desc.data(), (int)Bp->desc.size(), Bp->g64.data());
+        ready = fits();
+        if (!ready) {
+          Bp->plan = lane_plan(ctx, Bp->desc.data(), (int)Bp->desc.size(), nullptr);
+          ready = fits();
+        }
+      }
       if (!Bp->plan) {
-        st = energy_enqueue(ctx, lane->ex, &Bp->jobs[0]->job, lane_ws_cap(ctx));
-      } else if (!lane->ex.ensure_ws(Bp->plan->ws_bytes) || !lane->ex.hstage.reserve(Bp->plan->pin_bytes + 64)) {
+        st = energy_enqueue(ctx, lane->ex, &Bp->jobs[0]->job, lane_ws_cap(ctx), false, Bp->jobs[0]->g64);
+      } else if (!ready) {
         ctx_set_error(ctx, "cannot allocate the serving batch's workspace");
         st = RPA_E_NOMEM;
         no_memory = true;
@@ -273,7 +298,7 @@ static void scheduler(rpa_ctx* ctx) {
         if (st == RPA_OK && cudaEventRecord(lane->ex.done, lane->ex.s) != cudaSuccess) st = RPA_E_CUDA;
       }
       lk.lock();
-      if (no_memory) S->ws_total = lanes_ws(S);  // the lane may have given up its old workspace
+      if (no_memory || replanned) S->ws_total = lanes_ws(S);  // the lane may have given up its old workspace
       if (no_memory && S->running.size() > 1) {
         // the device is short (memory held outside the cap): put the jobs back
         // at the head of the queue and admit again when a running batch ends
@@ -421,15 +446,23 @@ rpa_status rpa_submit(rpa_ctx* ctx, const rpa_job* job, uint64_t* ticket) {
   j->job.zeta_w = j->zeta_w.data();
   j->job.C = j->C.data();
   j->job.V = j->V.data();
-  j->footprint = job_footprint(job, ctx->n_slices, lane_ws_cap(ctx));
-  j->ws_need = job_workspace(job, ctx->n_slices, lane_ws_cap(ctx));
+  // An FP64 job takes the digit products that rpa_energy takes, so that both give the
+  // same bits, in smaller planes or without them only where the cap has no room for
+  // them beside the job's inputs.
+  const int g64 = job->prec == RPA_PREC_FP64 ? job_g64(job, ctx->n_slices, sync_ws_cap(ctx)) : 0;
+  for (int g : {g64, g64 | G64_LEAST, 0}) {
+    j->g64 = g;
+    j->footprint = job_footprint(job, ctx->n_slices, lane_ws_cap(ctx), g);
+    j->ws_need = job_workspace(job, ctx->n_slices, lane_ws_cap(ctx), g);
+    if (j->footprint <= ctx->cap) break;
+  }
   if (job->mem == RPA_MEM_DEVICE) {
     // the batch engine holds every q's split-precision workspace at once:
     // jobs whose batch workspace stays within a lane's cap share micro-batches,
     // larger ones run alone q-batch by q-batch
     const size_t inputs = j->footprint - j->ws_need;
-    const size_t ws_b = batch_plan(&j->job, 1, ctx->n_slices, lane_ws_cap(ctx))->ws_bytes;
-    if (ws_b <= lane_ws_cap(ctx)) {
+    const size_t ws_b = lane_plan(ctx, &j->job, 1, &j->g64)->ws_bytes;
+    if (ws_b <= lane_ws_cap(ctx) && (!j->g64 || inputs + ws_b <= ctx->cap)) {
       j->batchable = true;
       j->ws_need = ws_b;
       j->footprint = inputs + ws_b;
