@@ -127,12 +127,14 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;
 }
 
-// 1 / x for a normal positive x: the hardware approximation and two
-// Newton-Raphson steps r += r (1 - x r), four FP64 instructions on the serial
-// chain of a panel; other values go through the division.
+// 1 / x, correctly rounded: for a normal positive x the hardware approximation and
+// two Newton-Raphson steps r += r (1 - x r), four FP64 instructions on the serial
+// chain of a panel.  The last step rounds r (1 + e) with e exact up to its own rounding, which is
+// the nearest value but for the significand 2 - 2^-52, whose reciprocal lies next to a
+// midpoint (Markstein, 1990); it and the values outside the range go through the division.
 __device__ __forceinline__ double fast_rcp(double x) {
   const int hi = __double2hiint(x);
-  if (hi < (2 << 20) || hi >= (2044 << 20)) return 1.0 / x;
+  if (hi < (2 << 20) || hi >= (2044 << 20) || ((hi | 0xFFF00000) & __double2loint(x)) == -1) return 1.0 / x;
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   r = fma(r, fma(-x, r, 1.0), r);
