@@ -297,8 +297,9 @@ __global__ void __launch_bounds__(256, 2) slice_bin_kernel(SliceBinArgs a) {
 // (n_w x sum_b rank_b multiply-adds per element) runs in float-float
 // arithmetic on the FP32 pipe (GB300's FP64 pipe is 1/58 of it): coef is held
 // as an unevaluated sum of two floats, each product is formed exactly by
-// Dekker's TwoProd (fmaf), and sums use Knuth's TwoSum; about 2^-44 relative,
-// far below the split-precision error of the partials.  Frequencies are
+// Dekker's TwoProd (fmaf), and sums use Knuth's TwoSum, skeletons in pairs, with a
+// renormalisation per pair (ff.h); about 2^-49 of the sum of the terms' magnitudes, far
+// below the split-precision error of the partials.  Frequencies are
 // taken in groups of at most RED_WG along grid y (registers).
 struct RedBin {
   int cplx, N, Npad, n_tiles, nb, rmax, n_w, G;  // G: skeleton slots per round
@@ -314,37 +315,7 @@ struct RedBin {
 constexpr int RED_WG = 10;
 constexpr int RED_GB = 5;  // skeletons in flight
 
-// (h, l) += ph + pl: Knuth's TwoSum on the high parts, the errors gathered in l,
-// renormalised by ff_norm every few terms.
-__device__ __forceinline__ void ff_acc(float& h, float& l, float ph, float pl) {
-  const float s = __fadd_rn(h, ph);
-  const float bb = __fsub_rn(s, h);
-  const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(ph, bb));
-  l = __fadd_rn(l, __fadd_rn(e, pl));
-  h = s;
-}
-
-__device__ __forceinline__ void ff_norm(float& h, float& l) {
-  const float s = __fadd_rn(h, l);
-  l = __fsub_rn(l, __fsub_rn(s, h));
-  h = s;
-}
-
-// (h, l) += (kx + ky)(x0 + x1): the product by Dekker's TwoProd (fmaf) with the
-// cross terms straight into l.
-__device__ __forceinline__ void ff_fma(float& h, float& l, float kx, float ky, float x0, float x1) {
-  const float p = __fmul_rn(kx, x0);
-  const float t = fmaf(kx, x0, -p);
-  l = fmaf(kx, x1, l);
-  l = fmaf(ky, x0, l);
-  const float s = __fadd_rn(h, p);
-  const float bb = __fsub_rn(s, h);
-  const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  l = __fadd_rn(l, __fadd_rn(e, t));
-  h = s;
-}
-
-// WG: frequencies per group at most.  What bounds it is the FP32 pipe, 12
+// WG: frequencies per group at most.  What bounds it is the FP32 pipe, 13.5
 // instructions per term, so the frequency loop is branch-free (coefficients past
 // the last frequency are zero) and RED_GB skeletons' loads are in flight.
 template <bool C, int WG>
@@ -392,9 +363,11 @@ __global__ void __launch_bounds__(256, WG > 5 ? 2 : 3) reduce_bin_kernel(const _
         // x = sum over the split-K partials of (hi + lo), as a float-float pair
         xh[u] = pp[0];
         xl[u] = pp[128 * 128];
+        ff_norm(xh[u], xl[u]);
         if constexpr (C) {
           yh[u] = pp[64];
           yl[u] = pp[128 * 128 + 64];
+          ff_norm(yh[u], yl[u]);
         }
         for (int ks = 1; ks < rb.nks[b]; ++ks) {
           pp += (long)Gs * rb.n_tiles * (2 * 128 * 128);
@@ -403,24 +376,34 @@ __global__ void __launch_bounds__(256, WG > 5 ? 2 : 3) reduce_bin_kernel(const _
         }
       }
 #pragma unroll
-      for (int u = 0; u < RED_GB; ++u) {
-        if (ra[u] <= 0 || rq == 0) continue;  // a zero row or column (or no skeleton): no contribution
+      for (int u = 0; u < RED_GB; u += 2) {
+        // (a zero row or column, or no skeleton: no contribution)
+        const int v = u + 1 < RED_GB ? u + 1 : u;
+        const bool one = ra[u] > 0 && rq != 0, two = v > u && ra[v] > 0 && rq != 0;
+        if (!one && !two) continue;
         // scale 2^(eA + eC + 1 - 14) with the sign of chi = -sum conj(a) c (exact)
-        const int sh = (ra[u] - 2044 + 1) + eCQ + 1 - 14;
-        const float x0 = -ldexpf(xh[u], sh), x1 = -ldexpf(xl[u], sh);
-        const float y0 = -ldexpf(yh[u], sh), y1 = -ldexpf(yl[u], sh);
-        const float2* cf = cs + (b * rb.rmax + gb + u) * WG;
+        const int su = (ra[u] - 2044 + 1) + eCQ + 1 - 14, sv = (ra[v] - 2044 + 1) + eCQ + 1 - 14;
+        float x[4] = {-ldexpf(xh[u], su), -ldexpf(xl[u], su), -ldexpf(yh[u], su), -ldexpf(yl[u], su)};
+        const float y[4] = {-ldexpf(xh[v], sv), -ldexpf(xl[v], sv), -ldexpf(yh[v], sv), -ldexpf(yl[v], sv)};
+        if (!one)
 #pragma unroll
-        for (int w = 0; w < WG; ++w) {
-          const float2 k = cf[w];
-          ff_fma(rh[w], rl[w], k.x, k.y, x0, x1);
-          if constexpr (C) ff_fma(ih[w], il[w], k.x, k.y, y0, y1);
+          for (int i = 0; i < 4; ++i) x[i] = y[i];
+        const float2* cf = cs + (b * rb.rmax + gb + (one ? u : v)) * WG;
+        if (one && two) {
+#pragma unroll
+          for (int w = 0; w < WG; ++w) {
+            const float2 k = cf[w], m = cf[w + WG];
+            ff_fma2(rh[w], rl[w], k.x, k.y, x[0], x[1], m.x, m.y, y[0], y[1]);
+            if constexpr (C) ff_fma2(ih[w], il[w], k.x, k.y, x[2], x[3], m.x, m.y, y[2], y[3]);
+          }
+        } else {
+#pragma unroll
+          for (int w = 0; w < WG; ++w) {
+            const float2 k = cf[w];
+            ff_fma(rh[w], rl[w], k.x, k.y, x[0], x[1]);
+            if constexpr (C) ff_fma(ih[w], il[w], k.x, k.y, x[2], x[3]);
+          }
         }
-      }
-#pragma unroll
-      for (int w = 0; w < WG; ++w) {
-        ff_norm(rh[w], rl[w]);
-        if constexpr (C) ff_norm(ih[w], il[w]);
       }
     }
   }

@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "chi0_tc.cuh"
+#include "ff.h"
 #include "rpa_internal.h"
 
 namespace rpa {
