@@ -129,11 +129,12 @@ static cudaError_t fast_product(int cplx, int n_mat, int N, char* ws, const doub
 }
 
 // The largest cosine between two columns of W (digit planes: rounding at 2^-55
-// of the largest entries), into *cosine; M is left with E for V += V E,
+// of the largest entries), into *cosine, and the products' status word (a wait that
+// ran out: the cosine means nothing) into *status_h; M is left with E for V += V E,
 // W += W E, the first-order rotations of the pairs that take less than 2e-9 (its
 // square, what V then lacks in orthonormality, is below rounding).
 static cudaError_t column_cosine(int cplx, int n_mat, int N, int Np, char* ws, const double* W, float* cosine,
-                                 uint64_t* nl, cudaStream_t s) {
+                                 int* status_h, uint64_t* nl, cudaStream_t s) {
   const FastLayout L = fast_layout(cplx, n_mat, N);
   double *M = (double*)(ws + L.M), *diag = (double*)(ws + L.diag);
   unsigned* off = (unsigned*)(ws + L.flags);
@@ -143,6 +144,8 @@ static cudaError_t column_cosine(int cplx, int n_mat, int N, int Np, char* ws, c
   if (e == cudaSuccess) e = launch_proj_corr(cplx, n_mat, N, false, M, diag, 2e-9f, off, s);
   *nl += 2;
   if (e == cudaSuccess) e = cudaMemcpyAsync(cosine, off, sizeof *cosine, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(status_h, ws + L.flags + 128, sizeof *status_h, cudaMemcpyDeviceToHost, s);
   return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
@@ -224,9 +227,10 @@ static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, d
   // columns of W orthogonal to FP64 rounding: first-order rotations of all
   // pairs that take little, full ones among the few columns that remain
   float last = 2.f;
+  int st = 0;
   for (int it = 0; dev < 1e-9f; ++it) {
-    CKP(column_cosine(cplx, n_mat, N, Np, ws, W, cosine, &nl, s));
-    if (*cosine <= kOrthogonal || it == kPolish || !(*cosine < 0.5f * last)) break;
+    CKP(column_cosine(cplx, n_mat, N, Np, ws, W, cosine, &st, &nl, s));
+    if (st || *cosine <= kOrthogonal || it == kPolish || !(*cosine < 0.5f * last)) break;
     last = *cosine;
     CKP(update());
     CKP(product(W, cols, 0, 1, M, NN, W, cols, 1));
@@ -234,7 +238,6 @@ static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, d
     CKP(launch_proj_cluster(cplx, n_mat, N, Np, M, W, V, 1e-15, s));
     ++nl;
   }
-  int st = 0;
   CKP(cudaMemcpyAsync(&st, status, sizeof st, cudaMemcpyDeviceToHost, s));
   CKP(cudaStreamSynchronize(s));
   ctx->launches += nl;
@@ -302,9 +305,11 @@ rpa_status run_projector(rpa_ctx* ctx, Exec* pex, int cplx, int n_mat, int N, in
     // the sweep that would only find the columns orthogonal is a Gram product
     if (started && off_h > conv) {
       uint64_t nl = 0;
-      if ((e = column_cosine(cplx, n_mat, N, L.Np, fast, W, &cosine, &nl, s)) != cudaSuccess)
+      int st = 0;
+      if ((e = column_cosine(cplx, n_mat, N, L.Np, fast, W, &cosine, &st, &nl, s)) != cudaSuccess)
         return fail(e, "Gram product");
       ctx->launches += nl;
+      if (st) return decode_status(ctx, st, 1);
       if (cosine <= kOrthogonal) off_h = cosine;
     }
   }
