@@ -304,7 +304,10 @@ struct Flt<false> {
   float re;
 };
 
-// Sum of squares of S(k) (W, N columns of N), one CTA per k-point, fixed order.
+// Sum of squares of S(k) (W, N columns of N), one CTA per k-point, fixed order, and
+// from it the scale of the FP32 start.  Columns of a root mean square norm outside
+// [2^-50, 2^60] get a NaN, which rejects the start: beyond it the FP32 sum or the digit
+// products' range may not hold S.
 template <bool C>
 __global__ void __launch_bounds__(256) proj_norm_kernel(int N, int Np, const double* __restrict__ W,
                                                         float* __restrict__ scale) {
@@ -322,7 +325,8 @@ __global__ void __launch_bounds__(256) proj_norm_kernel(int N, int Np, const dou
   if (threadIdx.x == 0) {
     double u = 0.0;
     for (int i = 0; i < 8; ++i) u += red[i];
-    scale[blockIdx.x] = (float)(1.0 / sqrt(u / N));  // columns of norm about 1
+    const double norm = sqrt(u / N);
+    scale[blockIdx.x] = norm >= 0x1p-50 && norm <= 0x1p60 ? (float)(1.0 / norm) : __int_as_float(0x7fffffff);
   }
 }
 

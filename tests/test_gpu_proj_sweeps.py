@@ -6,6 +6,7 @@ import time
 import pytest
 
 from paper_2505_06021_gb300 import synth
+from test_gpu_proj_start import test_projector_start_matches_plain_sweeps as start_matches_plain_sweeps
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -78,3 +79,10 @@ def test_two_contexts_with_different_bases(rpa):
         t.join()
     assert not errors, errors
     assert all(r == a for a, rs in zip(alone, results) for r in rs)
+
+
+@pytest.mark.parametrize("scale", [1e21, 1e30, 1e-22])
+def test_overlaps_beyond_the_start(rpa, scale):
+    """Overlaps whose squares leave the FP32 range while their entries do not (and
+    such as leave the digit products' range) take the plain sweeps, bit for bit."""
+    start_matches_plain_sweeps(rpa, True, (40, 45), None, scale)
