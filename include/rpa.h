@@ -65,7 +65,14 @@ typedef int rpa_status;
 #define RPA_E_NOTREADY 7 /* submitted job not finished yet */
 
 /* Arithmetic of the chi0 contraction.  The sandwich, the factorisation and
- * all sums are FP64 in every mode. */
+ * all sums are to FP64 rounding in every mode.  FP64 products of some size run
+ * as digit products on the tensor cores: exact integer sums of the operands' rows
+ * in 55-bit fixed point, so the error of an element is about 2^-55 sqrt(K) of the two
+ * rows' largest entries, by norm less than a chain of FP64 multiply-adds makes.
+ * Elements much smaller than their rows keep an error of at most some 3 2^-53 of
+ * the sum of their terms' magnitudes in chi0 and in the AO -> MO transform: rows
+ * whose entries spread further go through the FP64 kernels, as do values outside
+ * 2^+-60, infinities and NaN. */
 #define RPA_PREC_FP64 0  /* chi0 to FP64 rounding (exact digit products, DFMA) */
 #define RPA_PREC_MIXED 1 /* chi0 on tcgen05 tensor cores from BF16 slices of
                             the FP64 operands, FP32 accumulation in exact

@@ -228,6 +228,7 @@ G64Op op_of(int cplx, int role, int R, int K, char* planes, char* e) {
 G64Src src_of(int by_rows, int conj, int R, int K, long ld, int nb) {
   G64Src s{};
   s.use_tab = 1;
+  s.by_element = 1;
   s.by_rows = by_rows;
   s.conj = conj;
   s.R = R;

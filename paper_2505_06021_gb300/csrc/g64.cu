@@ -167,24 +167,42 @@ struct RowStat {
 // Bit 0 (FP64 kernels): an infinity, a NaN, values outside 2^+-60, or a mean
 // binary exponent more than 1.5 + log2(K) / 2 below the largest entry's: then
 // 2^-56 max|a| |b| can exceed the DFMA chain's error, about 2^-53 sqrt(K) / 5
-// of |a| |b| for typical entries.  (Gaussian rows: 3 at K = 128, 3.2 at 34560.
+// of |a| |b| for typical entries.  (Gaussian rows: 2.4 at K = 128, 2.8 at 8192.
 // Sums of less than 64 terms, the short ends of triangular operands: 8, as
 // their few exponents scatter.)
 // Bit 1 (level 8 too): (max / rms)^2 above `spread` sqrt(K / 128), where the
 // dropped levels could exceed it.
+//
+// These bounds are for the norm of an output row.  A single element sum_k a_k b_k can
+// be far smaller than |a| |b| where the large entries of one row meet the small ones
+// of the other (halves scaled by 2^-g in turn: mean gap 2.5 + g / 2), and the split's
+// error is not.  Operands whose products are results of their own (`by_element`: the
+// unweighted rows of chi0, AO -> MO) are held to the gap up to which the error per element,
+// over sum_k |a_k b_k|, stays within about twice a DFMA chain's.  Emulated, split over
+// chain at g = 0, 2, 4, 6, 8, levels to 7: K = 128 0.57, 1.9, 7, 31, 130, K = 2048 0.19, 0.6, 2.6,
+// 9, 39; with level 8 0.09, 0.34, 1.4, 5.5, 23 and 0.03, 0.1, 0.3, 1.6, 5.3.  So level 8
+// from a gap of 4.25 (one Gaussian row in 10^6 has one), the FP64 kernels
+// from 4.6 at K = 128, a quarter more per factor of two.
 constexpr float SPREAD = 40.f;            // as given: Gaussian rows reach 20
 constexpr float SPREAD_WEIGHTED = 100.f;  // times the smooth frequency weights (a factor 2 of spread of their own)
 constexpr float TINY = 8.7e-19f;          // 2^-60
-__device__ __forceinline__ int row_flags(const RowStat& r, float spread) {
+__device__ __forceinline__ int row_flags(const RowStat& r, float spread, bool by_element) {
   const float m = __uint_as_float(r.m), n = (float)max(r.nz, 1);
   if (r.m >= 0x7f800000u || !(m < 1.1e18f) || !(m > TINY)) return 1;
-  if ((float)(r.m >> 23) - (float)r.es / n > (n < 64.f ? 8.f : 1.5f + 0.5f * log2f(n))) return 1;
+  const float gap = (float)(r.m >> 23) - (float)r.es / n, lg = log2f(n);
+  if (by_element) {
+    if (gap > (n < 16.f ? 8.f : n < 64.f ? 5.2f : 4.6f + 0.25f * fmaxf(lg - 7.f, 0.f))) return 1;
+    if (gap > 4.25f) return 2;
+  } else if (gap > (n < 64.f ? 8.f : 1.5f + 0.5f * lg)) {
+    return 1;
+  }
   return m * m <= spread * sqrtf(n * (1.0f / 128.0f)) * r.ss / n ? 0 : 2;
 }
 // The row's exponent; raises its flags.
-__device__ __forceinline__ int row_exponent(const RowStat& r, float spread, int* flag, int nflag = 1) {
+__device__ __forceinline__ int row_exponent(const RowStat& r, float spread, bool by_element, int* flag,
+                                            int nflag = 1) {
   if (r.m == 0) return E_ZERO;
-  if (const int bits = row_flags(r, spread))
+  if (const int bits = row_flags(r, spread, by_element))
     for (int i = 0; i < nflag; ++i) atomicOr(flag + i, bits);
   if (r.m >= 0x7f800000u) return 1100;
   return (int)(__float_as_uint(__uint_as_float(r.m) * 1.000001f) >> 23) - 126;
@@ -221,7 +239,8 @@ __global__ void __launch_bounds__(256) g64_exp_kernel(const __grid_constant__ G6
     for (int w = 1; w < 8; ++w) st.join(sr[w][lane]);
   }
   if (r < Rpad)
-    e[(long)b * Rpad + r] = r < src.R ? row_exponent(st, SPREAD, flag + (long)b * frep, max(frep, 1)) : E_ZERO;
+    e[(long)b * Rpad + r] = r < src.R ? row_exponent(st, SPREAD, src.by_element, flag + (long)b * frep, max(frep, 1))
+                                         : E_ZERO;
 }
 
 // One thread per (matrix, row, K-block); consecutive threads take consecutive
@@ -979,7 +998,7 @@ __global__ void __launch_bounds__(256) chi_exp_final_kernel(int N, int NpadA, in
   RowStat st;
   if (P < N)
     for (int kp = 0; kp < KP; ++kp) st.join(part[((long)slot * KP + kp) * Npad + P]);
-  const int e = row_exponent(st, slot ? SPREAD_WEIGHTED : SPREAD, flag);
+  const int e = row_exponent(st, slot ? SPREAD_WEIGHTED : SPREAD, slot == 0, flag);
   if (slot == 0) {
     if (P < NpadB) eB[P] = e;
   } else if (P < NpadA) {

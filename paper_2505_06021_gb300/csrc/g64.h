@@ -20,6 +20,7 @@ struct G64Src {
   long stride, ld;
   int use_tab, by_rows, conj, nb, R, K;
   int no_diag;  // element (r, r) counts as zero (g64_product adds its terms, see G64Diag)
+  int by_element;  // the rows' spread is bounded so that single elements keep their accuracy (g64.cu)
 };
 
 // A sliced operand in device memory: planes, one exponent per row (|x| < 2^e).
