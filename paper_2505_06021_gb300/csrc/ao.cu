@@ -164,8 +164,8 @@ rpa_status ao_project(rpa_ctx* ctx, Exec* pex, const rpa_job* j, const AoPlan& p
 // ------------------------------------------------ digit products ----------
 // Both transforms are contractions of FP64 arrays whose FP64 form is bound by
 // the FP64 pipe (0.98 of it).  One q of 2 x (96 basis, 192 fit), 16 k-points,
-// 192 orbitals: 180 ms in FP64, 10.7 ms here (slicing and stores about half of
-// it); error against 113-bit sums 9.9e-16 and 4.0e-16.  As digit products
+// 192 orbitals: 180 ms in FP64, 11.7 ms here (slicing and stores about half of
+// it); error against 113-bit sums 9.9e-16 in FP64, 4.0e-16 here.  As digit products
 // (g64.cu):
 //   half:  H[s][n] = sum_nu P[nu][s] c[nu][n]; left rows s, right rows n; the PADF
 //          planes serve the occupied and the virtual columns.

@@ -823,8 +823,8 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
   // Device-resident split-precision jobs: the V side of all q (V = L L^H, V^-1)
   // runs on the GPU while the host makes the frequency plan, where the workspace
   // is there already and all q fit in one batch.  Gamma-point job (real, N = 733,
-  // plan 1.2 ms, V side 1.4): 5.59 -> 4.32 ms; 2-D periodic job (16 q, N = 512,
-  // plan 4.6 ms, V side 8): 134.2 -> 132.0 ms.  Buffers that the V side uses
+  // plan 1.2 ms, V side 1.4): 4.32 ms, 5.59 with the V side after it; 2-D periodic job
+  // (16 q, N = 512, plan 4.6 ms, V side 8): 2 ms of 132.  Buffers that the V side uses
   // stand at the head of the workspace, so that the plan, made later, cannot
   // move them; where the final layout differs all the same, it runs again.
   Layout Lv{};

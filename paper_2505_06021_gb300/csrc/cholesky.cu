@@ -25,15 +25,15 @@
 // trailing tiles fill the GPU, since each panel converts and adds the whole
 // trailing matrix in FP64.
 //
-// Measured on GB300, one CTA or an 8-CTA cluster per matrix before, panel
-// launches now: one complex N = 768 factor of V 19.9 -> 2.4 ms; 16 matrices of
-// N = 768 in FP64 30.1 -> 9.7 ms; 32 in the inverse form 17.6 -> 8.8 ms; 320 of
-// N = 512 in the inverse form 34.7 -> 19.4 ms; 64 of N = 300 18.6 -> 1.6 ms; 16
-// real ones of N = 64 0.285 -> 0.065 ms.  There the 16 FP64 matrices need 7.6 ms of
-// the FP64 pipe and take 9.7, so larger batches (chol_g64_use) leave all but 1/(N /
+// Measured on GB300, panel launches (and one CTA or an 8-CTA cluster per matrix
+// instead): one complex N = 768 factor of V 1.5 ms (19.9); 16 matrices of
+// N = 768 in FP64 9.7 ms (30.1); 32 in the inverse form 8.8 ms (17.6); 320 of
+// N = 512 in the inverse form 19.4 ms (34.7); 64 of N = 300 1.6 ms (18.6); 16
+// real ones of N = 64 0.065 ms (0.285).  The 16 FP64 matrices need 7.6 ms of
+// the FP64 pipe, so larger batches (chol_g64_use) leave all but 1/(N /
 // 128) of the trailing updates to the tensor cores, one block column of 128
-// columns at a time: 16 of N = 768 9.9 -> 4.4 ms, 320 of N = 512 in the inverse form
-// 19.3 -> 14.4 ms.  What is left is the FP64 work inside the block columns and, for few
+// columns at a time: 16 of N = 768 4.4 ms (9.9 without), 320 of N = 512 in the inverse
+// form 14.4 (19.3).  What is left is the FP64 work inside the block columns and, for few
 // matrices, two launches of some 20 us each per panel.
 #include <cuda_runtime.h>
 #include <math.h>

@@ -373,7 +373,7 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
   // nb rank n_w float-float multiply-adds against rank K tensor-core terms;
   // measured, 25 bins of 20 frequencies at K = 114688 take 0.19 of the
   // contraction's time, i.e. 44 nb n_w / K.  So long contractions take narrow
-  // bins (rank 5 at ratio 1.05 where 1.1 needs 6: slab block chi0 95 -> 79 ms), and
+  // bins (rank 5 at ratio 1.05 where 1.1 needs 6: slab block chi0 79 ms, 95 at 1.1), and
   // short ones few wide bins.
   const bool run = max_bins > RPA_FREQ_MAX_BINS;
   const std::vector<double> ratios = run ? std::vector<double>{1.04, 1.05, 1.065, 1.08, 1.1, 1.12, 1.15, 1.2, 1.25, 1.3, 1.5, 1.75, 2.1, 3.0}

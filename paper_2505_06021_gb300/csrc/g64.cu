@@ -830,8 +830,8 @@ G64Out square_out(double* base, int N, int neg, int tri) {
 }  // namespace
 
 // Measured: the sandwich of 16 matrices of N = 768 40.6 ms in FP64 (its pipe
-// needs 33), 1.9 ms here; 48 of N = 150 1.69 -> 0.40 ms; V^-1 = X^H X of 16 of N =
-// 512 3.5 -> 0.45 ms.  Small matrices leave the tiles (128 rows) mostly padding; below 2.5e7 complex
+// needs 33), 1.9 ms here; 48 of N = 150 1.69 and 0.40 ms; V^-1 = X^H X of 16 of N =
+// 512 3.5 and 0.45 ms.  Small matrices leave the tiles (128 rows) mostly padding; below 2.5e7 complex
 // multiply-adds per q (N = 150, 12 frequencies: 0.42 ms in FP64) the FP64 kernels
 // take little more than the launches.
 bool tail_g64_use(int cplx, int N, int n) {
@@ -1213,8 +1213,8 @@ cudaError_t chi0_g64_run(const BatchGeom& g, const double* const* Cptrs, const d
 
 // The split needs some six launches per panel and K long enough for its error
 // bound.  Measured: one q of N_aux 320, 9 k, N_ov 1920, 16 frequencies (113
-// GFLOP) 66.2 -> 4.65 ms; N_aux 150, 4 k, N_ov 252, 12 frequencies (1.1 GFLOP
-// per q) 0.98 -> 0.21 ms per q.  At 5e8 flops the FP64 kernel takes about 0.3
+// GFLOP) 5.0 ms, 66.2 on the FP64 kernel; N_aux 150, 4 k, N_ov 252, 12 frequencies (1.1
+// GFLOP per q) 0.21 ms per q and 0.98.  At 5e8 flops the FP64 kernel takes about 0.3
 // ms, little more than the launches here.  Error against 64-bit sums at the
 // first size: 2.5e-16, the FP64 kernel's 3.7e-15.
 bool chi0_g64_use(const BatchGeom& g) {

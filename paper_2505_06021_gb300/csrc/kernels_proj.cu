@@ -31,8 +31,8 @@
 // relative to both columns, so this holds for the tiny eigenvalues too), and the
 // few pairs that need large rotations are rotated one by one; where G still
 // shows a cosine above 1e-14, the FP64 sweeps finish.  Measured, 16 overlaps of 256
-// functions: three FP64 sweeps of 255 rounds (23 us each, 17.8 ms in all) became 0.7
-// ms of products, 29.9 -> 13.1 ms in all; what is left is the FP32 sweeps
+// functions: 0.7 ms of products stand for three FP64 sweeps of 255 rounds (23 us each,
+// 17.8 ms), 13.1 ms in all instead of 29.9; the most of it is the FP32 sweeps
 // (7 ms) and the refinement's products.
 //
 // Since the eigenvalues are taken in ascending order and R~ is a product over
@@ -408,8 +408,8 @@ __device__ __forceinline__ float rotate32(Flt<C>* wp, Flt<C>* wq, Flt<C>* vp, Fl
 // sweep then reads and writes the columns nb - 1 times, not Np - 1, and has as
 // many launches (nb blocks).  What bounds a round inside the CTA is each warp's
 // chain of loads, sums and rotation (2.8 us; shared memory 44 % and issue 47 %
-// busy).  16 overlaps of 256 functions: 50.8 -> 29.9 ms in all against a
-// launch per round in global memory.
+// busy).  Sweeps of 16 overlaps of 256 functions: 21 ms less than with a launch per
+// round in global memory.
 template <bool C, int B>
 __global__ void __launch_bounds__(32 * B) jacobi32_block_kernel(int N, int Np, int nb, int br, float* __restrict__ W32,
                                                                 float* __restrict__ V32, float thresh,

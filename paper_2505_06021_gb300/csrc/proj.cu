@@ -152,8 +152,8 @@ static cudaError_t column_cosine(int cplx, int n_mat, int N, int Np, char* ws, c
 // V: eigenvectors of S (= W on entry) to nearly FP64 accuracy, W = S V.  The FP64
 // sweeps from V = I took 13 sweeps of 16 ms on 16 overlaps of 256 functions (208
 // ms); with this start none is left there (or one, where many columns stay close).
-// *ok = false (W = S and V = I as before) when the start did not give an
-// orthonormal V: entries out of the FP32 range, no convergence.
+// *ok = false (W = S and V = I again) when the start did not give an
+// orthonormal V: columns outside its range (proj_norm_kernel), no convergence.
 static rpa_status fast_start(rpa_ctx* ctx, int cplx, int n_mat, int N, int Np, double* W, double* V,
                              const ProjPtrs& P, char* ws, cudaStream_t s, bool* ok,
                              float* cosine) {
