@@ -363,11 +363,9 @@ __global__ void __launch_bounds__(256, WG > 5 ? 2 : 3) reduce_bin_kernel(const _
         // x = sum over the split-K partials of (hi + lo), as a float-float pair
         xh[u] = pp[0];
         xl[u] = pp[128 * 128];
-        ff_norm(xh[u], xl[u]);
         if constexpr (C) {
           yh[u] = pp[64];
           yl[u] = pp[128 * 128 + 64];
-          ff_norm(yh[u], yl[u]);
         }
         for (int ks = 1; ks < rb.nks[b]; ++ks) {
           pp += (long)Gs * rb.n_tiles * (2 * 128 * 128);
@@ -381,6 +379,13 @@ __global__ void __launch_bounds__(256, WG > 5 ? 2 : 3) reduce_bin_kernel(const _
         const int v = u + 1 < RED_GB ? u + 1 : u;
         const bool one = ra[u] > 0 && rq != 0, two = v > u && ra[v] > 0 && rq != 0;
         if (!one && !two) continue;
+        // (renormalised here, not above: the loads of all RED_GB skeletons stay in flight)
+        ff_norm(xh[u], xl[u]);
+        if (v > u) ff_norm(xh[v], xl[v]);
+        if constexpr (C) {
+          ff_norm(yh[u], yl[u]);
+          if (v > u) ff_norm(yh[v], yl[v]);
+        }
         // scale 2^(eA + eC + 1 - 14) with the sign of chi = -sum conj(a) c (exact)
         const int su = (ra[u] - 2044 + 1) + eCQ + 1 - 14, sv = (ra[v] - 2044 + 1) + eCQ + 1 - 14;
         float x[4] = {-ldexpf(xh[u], su), -ldexpf(xl[u], su), -ldexpf(yh[u], su), -ldexpf(yl[u], su)};
