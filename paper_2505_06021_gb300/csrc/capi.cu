@@ -316,7 +316,7 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
       part = m;
       return true;
     };
-    for (size_t most = G64_TAIL_MOST; most >= ((size_t)1 << 24) && !grow(L.tail, tail_region_bytes(j, qt, most)); most /= 2) {
+    for (size_t most = G64_TAIL_MOST; L.tail && most >= ((size_t)1 << 24) && !grow(L.tail, tail_region_bytes(j, qt, most)); most /= 2) {
     }
     if (L.mixed)
       for (int f = chi0_g64_freqs(geom_of(j, qb)); f > 1 && !grow(L.mixed, chi_region_bytes(j, qb, f)); --f) {
@@ -343,9 +343,16 @@ Layout plan_layout(const rpa_job* j, int qb, int n_slices, size_t ws_cap, bool m
 
 int job_g64(const rpa_job* j, int n_slices, size_t cap) {
   if (j->prec != RPA_PREC_FP64) return G64_ALL;
+  const size_t least[3] = {j->ao ? al(ao_g64_plan(j, ao_plan(j, 1)).bytes) : 0, tail_region_bytes(j, 1, 0),
+                           chi_region_bytes(j, 1, 1)};
+  if (!least[0] && !least[1] && !least[2]) return 0;
+  size_t total = plan_layout(j, 1, n_slices, cap, true).total;
   int m = 0;
-  for (int part : {G64_AO, G64_TAIL, G64_CHI})
-    if (plan_layout(j, 1, n_slices, cap, true, 0, nullptr, m | part | G64_LEAST).total <= cap) m |= part;
+  for (int i = 0; i < 3; ++i)
+    if (least[i] && total + least[i] <= cap) {
+      total += least[i];
+      m |= 1 << i;  // G64_AO, G64_TAIL, G64_CHI
+    }
   return m;
 }
 
