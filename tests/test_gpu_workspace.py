@@ -94,3 +94,22 @@ def test_calls_fit_beside_what_the_caller_holds(rpa, left):
         chi0 = c.chi0(job, 0)
     for a, b in zip(calls(False), calls(True)):
         assert float((a - b).abs().max()) <= 1e-13 * float(a.abs().max())
+
+
+@pytest.mark.parametrize("left,same", [(0.75, False), (1.9, True)])
+def test_served_job_fits_beside_what_the_caller_holds(rpa, left, same):
+    """A lane that cannot hold a job's planes runs it with the smallest ones (the same
+    bits: 1.1 GB here) or without them."""
+    job = _big_job(rpa)
+    with rpa.Context(0) as c:
+        ref = c.energy(job)
+    with rpa.Context(0) as c:
+        h = _leave(int(left * 2 ** 30))
+        Ec, eps = c.wait(c.submit(job), 300.0, job)
+        del h
+    eps = eps.reshape(ref["eps"].shape)
+    if same:
+        assert Ec == ref["Ec"] and np.array_equal(eps, ref["eps"])
+    else:
+        assert not np.array_equal(eps, ref["eps"])
+        assert np.abs(eps - ref["eps"]).max() <= 1e-13 * np.abs(ref["eps"]).max()
