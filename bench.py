@@ -413,6 +413,23 @@ def served_latency(args, local, n_jobs):
                       "rpa_submit/rpa_poll, mixed chi0" % n_jobs}
 
 
+def fp64_roofline(achieved, dfma_kernel, **more):
+    """Roofline record of an FP64 product step: the digit products on the tensor
+    cores issue 36 BF16 flops per FP64 flop; their peak is the measured BF16 rate
+    over that.  A rate above the FP64 pipe's can only be theirs."""
+    if achieved <= FP64_PEAK_TFLOPS:
+        return dict({"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                     "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None, "kernel": dfma_kernel,
+                     "peak_source": "derived FP64 DFMA peak: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz "
+                                    "(microbenchmark measured 1.205 TFLOP/s)"}, **more)
+    path = os.path.join(ROOT, "MEASURED_PEAKS.json")
+    bf16 = json.load(open(path)).get("bf16_tflops_sustained", 1700.0) if os.path.exists(path) else 1700.0
+    return dict({"bound": "tensor", "achieved": achieved, "peak": bf16 / 36, "unit": "TFLOP/s",
+                 "frac": 36 * achieved / bf16, "traffic": None,
+                 "kernel": "g64_kernel (tcgen05, eight 7-bit digit planes, 36 digit pairs per product) with its slicing",
+                 "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained / 36 (of measured)"}, **more)
+
+
 def chi0_roofline(prec, prof, cnt, chi0_flops, steps, name, slices):
     """Roofline record of the dominant kernel (the chi0 contraction) from the
     library's CUDA-event profile: `chi0_flops` algorithmic FP64-equivalent
@@ -425,13 +442,7 @@ def chi0_roofline(prec, prof, cnt, chi0_flops, steps, name, slices):
                 "4N(N+1)N_ov per (q, k, omega), complex; all n_w frequencies) per launch / the launch's mean "
                 "CUDA-event time")
     if prec == "fp64":
-        return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_PEAK_TFLOPS,
-                "traffic": traffic_for("chi0_fp64") if name == "periodic2d" else None,
-                "kernel": "chi0_fp64_kernel", "peak_source": "derived FP64 DFMA peak: 152 SMs x 2 DFMA/clk x "
-                "2 flop x 2.07 GHz (microbenchmark measured 1.205 TFLOP/s)", "counting": counting,
-                "note": "the kernel forms conj(C_P)C_Q once per t and reuses it over a group of frequencies, so "
-                        "it executes fewer FP64 instructions than the algorithmic count"}, achieved
+        return fp64_roofline(achieved, "chi0_fp64_kernel", counting=counting), achieved
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
     peak = peaks.get("bf16_tflops_sustained", 1700.0)
@@ -776,8 +787,7 @@ def run_batch(args):
                 "timing": "one profiled eager batch step: CUDA events around every tensor-core launch"}
     else:
         ach = alg / (chi_ms / 1e3) / 1e12
-        roof = {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": ach / FP64_PEAK_TFLOPS, "traffic": None, "kernel": "chi0_fp64_kernel"}
+        roof = fp64_roofline(ach, "chi0_fp64_kernel")
     line = {"metric": METRIC, "value": val, "unit": "jobs/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64" if prec == "fp64" else "bf16-slices->f64",
@@ -1129,11 +1139,8 @@ def run_ao(args):
     half, asm = ao_flops(p)
     ao_ms, ao_n = prof["ao2mo"]
     ach = (half + asm) * args.steps / (ao_ms / 1e3) / 1e12
-    roof = {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": ach / FP64_PEAK_TFLOPS, "traffic": None,
-            "kernel": "ao_half_kernel + ao_assemble_kernel (AO -> MO transform, FP64)",
-            "peak_source": "derived FP64 DFMA peak: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz",
-            "algorithmic_tflop_per_job": (half + asm) / 1e12, "launches_per_job": ao_n // max(args.steps, 1)}
+    roof = fp64_roofline(ach, "ao_half_kernel + ao_assemble_kernel (AO -> MO transform, FP64)",
+                         algorithmic_tflop_per_job=(half + asm) / 1e12, launches_per_job=ao_n // max(args.steps, 1))
     kernel_ms = {k: {"ms": v[0] / args.steps, "launches": v[1] // max(args.steps, 1)} for k, v in prof.items()
                  if v[1]}
     line = {"metric": METRIC, "value": jobs_per_s, "unit": "jobs/s", "n_gpus": world, "steps": args.steps,
