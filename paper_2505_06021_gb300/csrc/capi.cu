@@ -100,6 +100,7 @@ bool Exec::ensure_ws(size_t bytes) {
     return false;
   }
   ws_bytes = want;
+  ++ws_gen;
   return true;
 }
 
@@ -835,8 +836,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
   // stand at the head of the workspace, so that the plan, made later, cannot
   // move them; where the final layout differs all the same, it runs again.
   Layout Lv{};
-  const void* v_ws = nullptr;
-  size_t v_bytes = 0;
+  unsigned v_gen = 0;  // the workspace that holds it (0: not run)
   auto v_side = [&]() -> rpa_status {
     Lv = plan_layout(job, job->n_q, ctx->n_slices, ws_cap, false, job->n_q, nullptr, g64);
     const size_t need = Lv.meta + Lv.chi + Lv.T + Lv.L + Lv.Vc + Lv.tail;
@@ -845,8 +845,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
     if (rpa_status st = upload_tables(ctx, ex, job, bv, job->C)) return st;
     if (rpa_status st = vside_copy(ctx, job, bv, 0, job->n_q, job->V, s)) return st;
     if (rpa_status st = vside_factor(ctx, &ex, job, bv, 0, job->n_q, s)) return st;
-    v_ws = ex.ws;
-    v_bytes = ex.ws_bytes;
+    v_gen = ex.ws_gen;
     return RPA_OK;
   };
   const bool v_early = allow_bin && job->prec == RPA_PREC_MIXED && job->mem == RPA_MEM_DEVICE && !job->ao &&
@@ -863,7 +862,7 @@ rpa_status energy_enqueue(rpa_ctx* ctx, Exec& ex, const rpa_job* job, size_t ws_
     return st;
   Bufs b = carve(ex.ws, job, L);
   // the early V side holds if this layout has its buffers in the same place
-  const bool v_done = v_ws && v_ws == ex.ws && v_bytes == ex.ws_bytes && qb == job->n_q && qt == job->n_q &&
+  const bool v_done = v_gen && v_gen == ex.ws_gen && qb == job->n_q && qt == job->n_q &&
                       L.meta == Lv.meta && L.chi == Lv.chi && L.T == Lv.T && L.L == Lv.L && L.Vc == Lv.Vc &&
                       L.tail == Lv.tail;
   const size_t es = job->is_complex ? 16 : 8;

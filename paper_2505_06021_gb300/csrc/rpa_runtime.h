@@ -51,6 +51,7 @@ struct Exec {
   cudaEvent_t done = nullptr;
   void* ws = nullptr;
   size_t ws_bytes = 0;
+  unsigned ws_gen = 0;  // allocations made: what an earlier one held is gone, whatever its address
   // per-kernel timing: (class, start, end) recorded on the launching stream
   struct Mark {
     int cls, n;
