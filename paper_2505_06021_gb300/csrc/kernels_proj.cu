@@ -144,9 +144,10 @@ __device__ __forceinline__ void pair_dots(const double* xc, const double* yc, in
 // roots, divisions and sums are FP64 instructions of one warp (64 clocks of a
 // sub-partition each, however few lanes take part), and seven more warps that
 // repeat them would share the same four pipes.  rot: c, s, e (re, im), 1 if the
-// cosine is above thresh; returns the cosine (thread 0), 0 elsewhere.
+// cosine is above thresh; returns the cosine (thread 0), 0 elsewhere.  off_max (or null)
+// takes the cosine before the rotation is computed.
 __device__ __forceinline__ double cta_rotation(double (*red)[4], double* rot, double a, double b, double gr, double gi,
-                                               double thresh) {
+                                               double thresh, unsigned long long* off_max) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double off = 0.0;
   if (lane == 0) {
@@ -166,10 +167,17 @@ __device__ __forceinline__ double cta_rotation(double (*red)[4], double* rot, do
     }
     const double g = sqrt(gr * gr + gi * gi);
     off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
-    rot[4] = 0.0;
+    if (off_max) atomicMax(off_max, (unsigned long long)__double_as_longlong(off));
     if (off > thresh) {
-      pair_rotation(a, b, gr, gi, g, rot[0], rot[1], rot[2], rot[3]);
+      double c, s, er, ei;
+      pair_rotation(a, b, gr, gi, g, c, s, er, ei);
+      rot[0] = c;
+      rot[1] = s;
+      rot[2] = er;
+      rot[3] = ei;
       rot[4] = 1.0;
+    } else {
+      rot[4] = 0.0;
     }
   }
   __syncthreads();
@@ -195,19 +203,16 @@ __global__ void __launch_bounds__(WARP ? 128 : 256) jacobi_round_kernel(int N, i
   double* wp = W + ((size_t)k * Np + p) * N * (C ? 2 : 1);
   double* wq = W + ((size_t)k * Np + q) * N * (C ? 2 : 1);
   const int first = WARP ? lane : threadIdx.x, step = WARP ? 32 : 256;
-  double a, b, gr, gi, off, c, s, er, ei;
+  double a, b, gr, gi, c, s, er, ei;
   pair_dots<C>(wp, wq, N, first, step, a, b, gr, gi);
   if constexpr (WARP) {
     const double g = sqrt(gr * gr + gi * gi);
-    off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
-    if (off > thresh) pair_rotation(a, b, gr, gi, g, c, s, er, ei);
-  } else {
-    off = cta_rotation(red, rot, a, b, gr, gi, thresh);
-  }
-  if (first == 0) atomicMax(off_max, (unsigned long long)__double_as_longlong(off));
-  if constexpr (WARP) {
+    const double off = (a > 0.0 && b > 0.0) ? g / sqrt(a * b) : 0.0;
+    if (first == 0) atomicMax(off_max, (unsigned long long)__double_as_longlong(off));
     if (!(off > thresh)) return;
+    pair_rotation(a, b, gr, gi, g, c, s, er, ei);
   } else {
+    cta_rotation(red, rot, a, b, gr, gi, thresh, off_max);
     if (rot[4] == 0.0) return;
     c = rot[0];
     s = rot[1];
@@ -275,7 +280,7 @@ __global__ void __launch_bounds__(256) proj_cluster_kernel(int N, int Np, const 
         const long op = (long)list[u] * N * (C ? 2 : 1), oq = (long)list[v] * N * (C ? 2 : 1);
         double a, b, gr, gi;
         pair_dots<C>(wk + op, wk + oq, N, tid, 256, a, b, gr, gi);
-        worst = fmax(worst, cta_rotation(red, rot, a, b, gr, gi, thresh));
+        worst = fmax(worst, cta_rotation(red, rot, a, b, gr, gi, thresh, nullptr));
         const double c = rot[0], s = rot[1], er = rot[2], ei = rot[3];
         const bool turn = rot[4] != 0.0;
         __syncthreads();  // rot and red are free again
