@@ -404,26 +404,23 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
       nb_least = nb;
     }
   }
-  struct Cand {
-    int few;  // 0, or how many bins below nb_least (taken only where nothing else fits)
-    double work, rho;
-  };
-  std::vector<Cand> est;
+  std::vector<std::pair<double, double>> est;  // (modelled work, rho)
   for (size_t c = 0; c < ratios.size(); ++c) {
     const int nb = bins_for(ratios[c]);
+    if (nb < nb_least) continue;
     int rm = 0;
     for (int i = 0; i < 5; ++i) rm = std::max(rm, rk[5 * c + i]);
     // (the recombination keeps the coefficients in 48 KB of shared memory)
     if (run && nb > RPA_FREQ_MAX_BINS && (size_t)nb * rm * j->n_w * sizeof(double) > 48 * 1024) continue;
     const double recomb = run ? 44.0 * nb * j->n_w * j->n_q / total : 0.0;
-    est.push_back({std::max(0, nb_least - nb), mean_rank(c) * (1.0 + 8.0 * j->n_q * nb / total + recomb), ratios[c]});
+    est.push_back({mean_rank(c) * (1.0 + 8.0 * j->n_q * nb / total + recomb), ratios[c]});
   }
   if (est.empty()) return false;  // no ratio's coefficients fit (an energy range of many decades)
   std::stable_sort(est.begin(), est.end(),
-                   [](const Cand& a, const Cand& b) { return a.few != b.few ? a.few < b.few : a.work < b.work; });
-  P = plan_full(est[0].rho);
+                   [](const std::pair<double, double>& a, const std::pair<double, double>& b) { return a.first < b.first; });
+  P = plan_full(est[0].second);
   for (size_t c = 1; c < est.size() && (size_t)P.n_bins * P.rmax * j->n_w * sizeof(double) > 48 * 1024; ++c)
-    P = plan_full(est[c].rho);
+    P = plan_full(est[c].second);
   P.dlo = lo;
   P.dhi = hi;
   if ((size_t)P.n_bins * P.rmax * j->n_w * sizeof(double) > 48 * 1024) {  // coefficients of the reduction

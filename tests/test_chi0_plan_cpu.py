@@ -83,16 +83,3 @@ def test_short_contractions_keep_narrow_bins(rpa, is_complex, kdims, n_occ, n_vi
     job = _host_job(rpa, p)
     run, told = job.chi0_plan(), job.freq_plan()
     assert told["n_bins"] > 0 and run["n_bins"] >= told["n_bins"]
-
-
-@pytest.mark.parametrize("gap,n_w", [(2e-4, 24), (2e-4, 32), (1e-6, 24), (1e-3, 20)])
-def test_wide_ranges_keep_a_plan(rpa, gap, n_w):
-    """Where as many bins as the reported plan's would not fit the recombination's
-    shared memory, the plan that runs takes the most that do."""
-    p = synth.make_problem("wide", is_complex=False, n_aux=12, n_occ=20, n_virt=180, grid=synth.gamma_grid(), n_w=n_w, seed=7)
-    t = rpa.upload_problem(p, device="cpu")
-    t["eps_virt"] += t["eps_occ"].max() + gap - t["eps_virt"].min()
-    job = rpa.job_from_problem(p, t, prec=rpa.PREC_MIXED, mem=rpa.MEM_HOST)
-    run, told = job.chi0_plan(2), job.freq_plan(2)
-    assert told["n_bins"] > 0 and run["n_bins"] >= 0.7 * told["n_bins"], (run["n_bins"], told["n_bins"])
-    assert np.all(run["err"] <= 1e-10)
