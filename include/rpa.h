@@ -190,9 +190,8 @@ rpa_status rpa_job_validate(const rpa_job *job, char *msg, size_t msg_len);
  * dense check grid), so chi0 needs rank[b] contractions over bin b instead of
  * n_w: chi0(w) = sum_b sum_r coef[b][r][w] X_{b,r}, X_{b,r} the contraction of
  * bin b's transitions at omega_{skel[b][r]}.  (rpa_chi0_plan reports the plan
- * that rpa_energy and rpa_chi0 run: the same construction and bounds, for long
- * contractions with more and narrower bins, as far as the recombination pays for
- * them.)  mode: 0 automatic (n_bins = 0
+ * that rpa_energy and rpa_chi0 run: the same construction and bounds, its number
+ * of bins also weighed by the recombination.)  mode: 0 automatic (n_bins = 0
  * when the plan saves no work), 2 always.  Outputs (any may be NULL), with
  * B = RPA_FREQ_MAX_BINS: edges [B], rank [B], err [B], skel [B][n_w] (-1 past
  * rank[b]), coef [B][n_w][n_w] (row r of bin b), *work_ratio = modelled

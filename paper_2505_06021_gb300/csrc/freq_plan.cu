@@ -373,11 +373,8 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
   // nb rank n_w float-float multiply-adds against rank K tensor-core terms;
   // measured, 25 bins of 20 frequencies at K = 114688 take 0.19 of the
   // contraction's time, i.e. 44 nb n_w / K.  So long contractions take narrow
-  // bins (rank 5 at ratio 1.05 where 1.1 needs 6: slab block chi0 79 ms, 95 at 1.1).
-  // Wider bins than the contraction alone would take are not considered: they would
-  // save short jobs some of the recombination (6 to 30 % of the call), but each bin's
-  // operands are rounded at its largest weight, and jobs with 2 to 11 bins instead of
-  // 15 to 21 had 1.1 to 2.5 times the error.
+  // bins (rank 5 at ratio 1.05 where 1.1 needs 6: slab block chi0 79 ms, 95 at 1.1), and
+  // short ones few wide bins.
   const bool run = max_bins > RPA_FREQ_MAX_BINS;
   const std::vector<double> ratios = run ? std::vector<double>{1.04, 1.05, 1.065, 1.08, 1.1, 1.12, 1.15, 1.2, 1.25, 1.3, 1.5, 1.75, 2.1, 3.0}
                                          : std::vector<double>{1.08, 1.1, 1.12, 1.15, 1.2, 1.25, 1.3, 1.5, 1.75, 2.1, 3.0};
@@ -389,31 +386,19 @@ bool freq_plan_build(const rpa_job* j, const double* eo, const double* ev, int m
     bin_ends(nb, at[i % 5], blo, bhi);
     rk[i] = fit_bin(blo, bhi, j->omega, j->n_w, FREQ_TOL, FREQ_AMP, 101).rank;
   });
-  auto mean_rank = [&](size_t c) {
-    int r = 0;
-    for (int i = 0; i < 5; ++i) r += rk[5 * c + i];
-    return r / 5.0;
-  };
-  int nb_least = 0;  // bins of the cheapest contraction among the reported plan's ratios
-  double cheapest = std::numeric_limits<double>::infinity();
-  for (size_t c = 0; run && c < ratios.size(); ++c) {
-    const int nb = std::min(bins_for(ratios[c]), RPA_FREQ_MAX_BINS);
-    const double work = mean_rank(c) * (1.0 + 8.0 * j->n_q * nb / total);
-    if (ratios[c] >= 1.08 && work < cheapest) {
-      cheapest = work;
-      nb_least = nb;
-    }
-  }
   std::vector<std::pair<double, double>> est;  // (modelled work, rho)
   for (size_t c = 0; c < ratios.size(); ++c) {
     const int nb = bins_for(ratios[c]);
-    if (nb < nb_least) continue;
+    double r = 0.0;
     int rm = 0;
-    for (int i = 0; i < 5; ++i) rm = std::max(rm, rk[5 * c + i]);
+    for (int i = 0; i < 5; ++i) {
+      r += rk[5 * c + i];
+      rm = std::max(rm, rk[5 * c + i]);
+    }
     // (the recombination keeps the coefficients in 48 KB of shared memory)
     if (run && nb > RPA_FREQ_MAX_BINS && (size_t)nb * rm * j->n_w * sizeof(double) > 48 * 1024) continue;
     const double recomb = run ? 44.0 * nb * j->n_w * j->n_q / total : 0.0;
-    est.push_back({mean_rank(c) * (1.0 + 8.0 * j->n_q * nb / total + recomb), ratios[c]});
+    est.push_back({r / 5 * (1.0 + 8.0 * j->n_q * nb / total + recomb), ratios[c]});
   }
   if (est.empty()) return false;  // no ratio's coefficients fit (an energy range of many decades)
   std::stable_sort(est.begin(), est.end(),

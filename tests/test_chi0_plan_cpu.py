@@ -71,15 +71,3 @@ def test_gap_so_small_that_no_plan_fits(rpa, n_w, mode):
     job = rpa.job_from_problem(p, t, prec=rpa.PREC_MIXED, mem=rpa.MEM_HOST)
     assert job.chi0_plan(mode)["n_bins"] == 0
     assert job.freq_plan(mode)["n_bins"] == 0
-
-
-@pytest.mark.parametrize("is_complex,kdims,n_occ,n_virt,n_w", [
-    (False, (1, 1, 1), 20, 180, 16), (False, (1, 1, 1), 20, 180, 10), (True, (2, 2, 1), 12, 90, 16), (False, (1, 1, 1), 8, 60, 16)])
-def test_short_contractions_keep_narrow_bins(rpa, is_complex, kdims, n_occ, n_virt, n_w):
-    """Each bin's operands are rounded at its largest weight, so fewer bins than the
-    reported plan's mean more error of the split: the plan that runs has no fewer."""
-    grid = synth.regular_kq_grid(kdims) if is_complex else synth.gamma_grid()
-    p = synth.make_problem("xs", is_complex=is_complex, n_aux=12, n_occ=n_occ, n_virt=n_virt, grid=grid, n_w=n_w, seed=6)
-    job = _host_job(rpa, p)
-    run, told = job.chi0_plan(), job.freq_plan()
-    assert told["n_bins"] > 0 and run["n_bins"] >= told["n_bins"]
